@@ -438,7 +438,7 @@ int run_plan(msa_plan *plan, const char *d_residues, const int32_t *d_subst, int
     L.spin_ns = spin_ms * 1000000LL;
     L.withhold = withhold;
     L.nprob = 1;
-    L.tab_ints = plan->hp.A * (plan->hp.A + 1) * 32;  // table plus the sentinel column
+    L.tab_ints = plan->hp.A * (plan->hp.A + 1);  // table plus the sentinel column
     L.corner = plan->hp.check_corner;
     if (tagged_faces(plan->hp.kernel)) {
         if (plan->epoch >= 32767) {  // column kernel tags (epoch << 16) + T would wrap: start over from cleared faces
@@ -535,7 +535,9 @@ int msa_plan_read_tb(msa_plan *plan, void *host_dst, int64_t bytes) {
                 const int64_t dst = base + x2;
                 if (dst >= bytes) continue;
                 const int T = x2 + l + rho;  // CTA time of the cell
-                out[dst] = col[((int64_t)((T + c3::U) * c3::W + w) * 32 + l) * c3::R + r];
+                // the stored tag's mask; a byte that is no tag is passed on (a cell the fill left out)
+                const int tag = col[((int64_t)((T + c3::U) * c3::W + w) * 32 + l) * c3::R + r];
+                out[dst] = (uint8_t)(tag > 7 ? tag : (x0 | x1 | x2) == 0 ? 0 : c3::mask_of_tag(tag));
             }
         }
     }

@@ -11,21 +11,40 @@
 //   e01, e12            are lane l-1 at time T-1      (shuffled at time T)
 //   e02                 is row rho-1 at time T-1
 //   e012                is lane l-1, row rho-1 at time T-2 (shuffled at time T-1)
-// so each step first finishes its own cells -- the max of a pre-reduced candidate
-// P and the freshly shuffled e1 candidate, then the tie-bit strip -- and then
-// prepares P for time T+1 and the e02/e012 pair D for time T+2 from values it
-// already holds. Only the shuffle, one max and the strip sit on the step-to-step
-// dependency chain.
+// so each step first finishes its own cells -- one fused add-max of a pre-reduced
+// candidate P and the freshly shuffled e1 candidate, then the tag is cut off --
+// and then prepares P for time T+1 and the e02/e012 pair D for time T+2 from
+// values it already holds. Only the shuffle, that add-max and the cut sit on the
+// step-to-step dependency chain.
+//
+// Keys. The kernel carries V = 8 H'(x) (the packed key of internal.h without its
+// W part: the low three bits are zero) and adds to the candidate of move m a tag
+// t(m), falling in m, so that one max finds the best value and, in its low three
+// bits, the lowest mask among equals:
+//     m    1 2 3 4 5 6 7
+//     t(m) 7 5 4 3 2 1 0
+// t(1) = 7 instead of 6 (no two moves share a tag, the order is the masks') makes
+// t(1) - t(5) = t(3) + t(6) - t(7): with 7 on row -1's value, 4 on p01, 1 on p12
+// and -5 on p02 every candidate gets its tag from a sum that is formed anyway,
+// and e0 and e02 share vm + 7. Traceback bytes hold the tags; readers decode
+// them (c3::mask_of_tag). Against keys with W in them (three instructions to
+// recover the mask and rebuild the key) the cut is one, on the chain and off it.
+//
+// Pair scores never need an address in the step. p12 (row-independent, by lane
+// and position) is looked up once per CTA by a staging warp, which fills a ring
+// indexed by CTA time and lane; p02 (by row and position) by each warp for its own
+// R rows, one block of steps ahead, into a ring indexed by tau = x2 + r, so that a
+// lane reads its R rows of a step with R / 4 16-byte loads.
 //
 // Communication, all indexed by CTA time T (so every index inside an unrolled
 // block of U steps is a compile-time offset):
 //   ring[w][T]  row -1 of warp w at time T: (value, tag T) written by warp w-1
-//               (its last row), or by the staging warp for w = 0 (the column
-//               above, face F0 at its time T + WR). A reader accepts an entry
-//               when its tag is T, so warps never wait on a barrier.
+//               (its last row), or by the row staging warp for w = 0 (the
+//               column above, face F0 at its time T + WR). A reader accepts an
+//               entry when its tag is T, so warps never wait on a barrier.
 //   f1r[T]      lane 0's inputs from the column to the left (its lane 31 at
 //               time T + 31) and the corner from the column above-left, copied
-//               by the staging warp, which publishes how far it got.
+//               by the column staging warp, which publishes how far it got.
 //   F0, F1      global faces of this column, (value, tag) 8-byte entries whose
 //               tag carries the launch epoch: no flags and no fences.
 // A column runs CTA times -U .. nsteps - 1; the first block computes cells at
@@ -39,18 +58,38 @@
 // check keeps that margin); the origin's pre-reduced candidate is set to
 // H(0) = 0 when time 0 begins.
 //
-// Cell update with pair scores scaled by 2^3 (packed keys, see internal.h): the
-// max over the seven moves gives the key, then m* = (W(x) - max) mod 8 and
-// Q(x) = max + m*; m* is the traceback byte. Each lane stores its R bytes of a
-// step as one word, 32 * R contiguous bytes per warp step.
+// Each lane stores its R traceback bytes of a step as one word, 32 * R contiguous
+// bytes per warp step.
+//
+// What bounds it: the chain of columns. A step takes about 295 cycles (one warp per
+// scheduler, 156 instructions, 80 of them on the half-rate integer pipe, 54 % of
+// its cycles), a column starts about 56 steps after each of its producers (32 of
+// them the skew, the rest the L2 round trip, the staging batch and the lag of the
+// warps), and 528 columns of 152 at a time are 4,000 steps even at a lag of 32.
+// Measured (ms, 700 x 760 x 800 / 128^3): 0.642 / 0.099, against 0.792 / 0.120 for
+// the kernel with W in its keys, 8 warps of 4 rows, table addresses in the step and
+// one staging warp. On the way: 4 rows x 8 warps 0.654 / 0.107; lane 31 storing
+// face F1 itself, one entry pair at a time, 0.94 / 0.15; the shuffles of a step at
+// its start instead of the step before, row -1 read when needed 0.96 / 0.145; two
+// CTAs per SM 0.734 / 0.099 (each column's steps get slower, and the chain with
+// them); staging batches of 8 / 4 rows on both axes 0.671 / 0.69; a 16-step block
+// 1.06 (instruction fetch), 4-step groups 0.80; two steps per ring vote 0.70.
 #include "api_internal.h"
 #include "device_common.cuh"
+
+#include <utility>
 
 namespace msadp {
 
 struct C3Smem {
     unsigned long long ring[c3::W][c3::SI][32];  // row -1 of warp w by CTA time: (value, tag)
-    int32_t f1r[c3::SF][c3::F1S];                // lane-0 inputs by CTA time: [3 + rho'], rho' = -1 .. WR-1
+    int32_t f1r[c3::SF + 1][c3::F1S];            // lane-0 inputs by CTA time: [3 + rho'], rho' = -1 .. WR-1
+    int32_t p12r[c3::SP + c3::U][32];            // pair score (x1 of lane, x2) + 1 by x2 + lane, the first
+                                                 // U rows again after the last
+    int32_t p02r[c3::W][c3::R / 4][c3::SQ + c3::U][4];  // per warp: pair score (x0 of row r, x2) - 5 by r / 4,
+                                                        // x2 + r and r mod 4, the first U slots again after the
+                                                        // last (16-byte reads of consecutive slots: no conflict)
+    int32_t f1b[c3::W][2][32];                   // per warp: lane 31's values of HF steps, twice
     int32_t prog[c3::W];                         // compute warp w has finished the steps < prog[w]
     int32_t staged;                              // f1r rows < staged hold this column's values
     int32_t failed;                              // a wait ran out: every warp leaves the column
@@ -59,7 +98,7 @@ struct C3Smem {
     int32_t pad[3];
 };
 
-int col3_warps_per_cta() { return c3::W + 1; }
+int col3_warps_per_cta() { return c3::W + 2; }
 
 namespace {
 
@@ -86,9 +125,6 @@ __device__ __forceinline__ void vstore(int32_t *p, int v) { *reinterpret_cast<vo
 __device__ __forceinline__ void st_entry(unsigned long long *p, unsigned long long v) {
     asm volatile("st.relaxed.gpu.u64 [%0], %1;" ::"l"(p), "l"(v));
 }
-__device__ __forceinline__ void st_global_v2(unsigned long long *p, unsigned long long a, unsigned long long b) {
-    asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(p), "l"(a), "l"(b));
-}
 __device__ __forceinline__ unsigned long long ld_global_relaxed(const unsigned long long *p) {
     unsigned long long v;
     asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p));
@@ -99,9 +135,6 @@ __device__ __forceinline__ ulonglong2 ld_global_relaxed_v2(const unsigned long l
     asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "l"(p));
     return v;
 }
-__device__ __forceinline__ int ldtab(const char *tab, int byte_off) {
-    return *reinterpret_cast<const int *>(tab + byte_off);
-}
 
 // Mark the column failed (first failure wins the launch status).
 __device__ void c3_fail(C3Smem &sm, const LaunchDesc &L) {
@@ -109,20 +142,42 @@ __device__ void c3_fail(C3Smem &sm, const LaunchDesc &L) {
     atomicCAS(L.err, 0, MSA_ETIMEOUT);
 }
 
-// Slow path of a ring read: wait (bounded) until every lane's entry carries tag T.
-__device__ __noinline__ unsigned long long c3_ring_wait(const unsigned long long *p, int T, C3Smem &sm,
-                                                       const LaunchDesc &L) {
-    const uint64_t t0 = global_ns();
-    unsigned long long e = lds_u64_volatile(p);
-    while (__any_sync(kFull, (int)(e >> 32) != T)) {
-        if (vload(&sm.failed) || (int64_t)(global_ns() - t0) > L.spin_ns) {
-            if ((threadIdx.x & 31) == 0) c3_fail(sm, L);
-            return pack_entry(kNeg, T);
+// The ring entries of a chunk of CH consecutive CTA times.
+constexpr int CH = c3::CH;
+struct C3Chunk {
+    unsigned long long e[CH];
+};
+__device__ __forceinline__ C3Chunk c3_ring_load(const unsigned long long *p) {
+    C3Chunk k;
+#pragma unroll
+    for (int j = 0; j < CH; ++j) k.e[j] = lds_u64_volatile(p + j * 32);
+    return k;
+}
+__device__ __forceinline__ bool c3_ring_ready(const C3Chunk &k, int T) {  // this lane's entries carry T, T + 1, ..
+    bool ok = true;
+#pragma unroll
+    for (int j = 0; j < CH; ++j) ok = ok && (int)(k.e[j] >> 32) == T + j;
+    return ok;
+}
+
+// Slow path of a ring read: wait (bounded) until every lane's entries of the chunk carry their tags.
+__device__ __noinline__ C3Chunk c3_ring_wait(const unsigned long long *p, int T, C3Smem &sm, const LaunchDesc &L) {
+    C3Chunk k = c3_ring_load(p);
+    uint64_t t0 = 0;
+    for (int polls = 0; !__all_sync(kFull, c3_ring_ready(k, T)); ++polls) {
+        if (polls >= 8) {
+            if (t0 == 0) t0 = global_ns();
+            if (vload(&sm.failed) || (int64_t)(global_ns() - t0) > L.spin_ns) {
+                if ((threadIdx.x & 31) == 0) c3_fail(sm, L);
+#pragma unroll
+                for (int j = 0; j < CH; ++j) k.e[j] = pack_entry(kNeg, T + j);
+                return k;
+            }
+            __nanosleep(20);
         }
-        __nanosleep(20);
-        e = lds_u64_volatile(p);
+        k = c3_ring_load(p);
     }
-    return e;
+    return k;
 }
 
 // Registers of one compute lane that change from step to step.
@@ -130,119 +185,185 @@ struct C3St {
     int V[c3::R];       // V(T-1, r) on entry to step T, V(T, r) after it
     int P[c3::R];       // max over every candidate of cell (T, r) but e1
     int D[c3::R];       // max of the e02 and e012 candidates of cell (T+1, r)
-    int cc[2 * c3::R];  // byte offsets of axis-2 codes: shift register by position
-    int pp[2 * c3::R];  // pair scores (x1, x2) of those positions
-    int VM;             // V(T-1, -1): the ring entry of the previous step
+    int pp[c3::R];      // p12 + 1 of the last R positions: shift register by position
+    int S[c3::R];       // lane l-1's V(T-1, r), shuffled as soon as step T-1 had it
+    int SM;             // lane l-1's V(T-1, -1)
+    int f[c3::R];       // lane 0's inputs of step T (the staged face), loaded a step ahead
+    int fm;
+    C3Chunk cur, nxt;   // row -1 of this chunk's times and of the next chunk's
+    int st_seen, dn_seen, fail_seen;  // the staged times, the warp below's progress and the column's failure,
+                                      // read a step before their use
+    int q;              // p02 entry of the next block on its way into the ring
 };
 
 // Constants of one compute lane for a column.
 struct C3Ln {
-    int p01[c3::R];     // pair score (x0, x1) per row
-    int rowb[c3::R];    // byte offset of row r's table row (code of x0) plus 4 * lane
-    int laneb;          // byte offset of this lane's table row (code of x1) plus 4 * lane
-    int Wl;             // W(x) = Wl + 4T - 3r
+    int p01[c3::R];     // pair score (x0, x1) + 4 per row
     int wR;             // first CTA row of the warp
     int tagout;         // tag base of ring-out entries (0: shared ring, epoch << 16: global face)
     int tagf1;          // tag base of this column's F1 entries
-    bool last;          // lane 31 writes the F1 face
+    bool last;          // lane 31's values are the F1 face
+    int *f1b;           // f1b[w]
+    int f1t;            // the step (of HF) of the F1 entry this lane writes
     int ctime;          // CTA time at which this lane computes the far corner (else never)
     int crow;           // the corner's row among this lane's R rows
+    int N;              // CTA times of the column
+    const int32_t *prog_dn;  // progress of the warp below (the last warp: its own)
+    int wcorner;        // W of the far corner: the recorded key is V + W
     int32_t *qcorner;   // where the corner's key goes (for the traceback's cross-check)
 };
 
-// Per-block addresses (block = U steps starting at CTA time T0).
+// Addresses of the block of U steps starting at CTA time T0.
 struct C3Blk {
     const unsigned long long *rin;  // ring[w][T0 mod SI][lane]
+    const unsigned long long *rin2; // ring[w][(T0 + U) mod SI][lane]
     unsigned long long *rout;       // ring[w+1][T0 mod SI][lane] or F0[T0][lane] (generic)
     const int *f1row;               // f1r[T0 mod SF]
     unsigned char *tbp;             // traceback bytes of (T0, w, lane): R bytes
-    unsigned long long *f1o;        // F1[T0][wR]
-    const uint16_t *c2p;            // code offset of x2 = T0 + 2 - lane - wR
+    unsigned long long *f1o;        // this lane's entry of F1[T0 ..][wR ..]
+    const int *p02;                 // p02r[w][0][(T0 + 2 - wR - lane) mod SQ]
+    const int *p12;                 // p12r[(T0 + 2 - wR) mod SP][lane]
 };
 
-template <int s>
-__device__ __forceinline__ void c3_step(C3St &g, const C3Ln &c, const char *tab, const C3Blk &b, int T0, int lane,
-                                        C3Smem &sm, const LaunchDesc &L) {
-    constexpr int M = 2 * c3::R - 1;
-    constexpr int R = c3::R;
-    static_assert(R == 2 || R == 4, "rows per warp: 2 or 4");
-    const int T = T0 + s;
-    // U(T, r) from lane l-1 (lane 0: the staged face)
-    const int *fr = b.f1row + s * c3::F1S;
-    int fv[R];
-    if constexpr (R == 4) {
-        const int4 f = *reinterpret_cast<const int4 *>(fr + 4 + c.wR);
-        fv[0] = f.x, fv[1] = f.y, fv[2] = f.z, fv[3] = f.w;
-    } else {
-        const int2 f = *reinterpret_cast<const int2 *>(fr + 4 + c.wR);
-        fv[0] = f.x, fv[1] = f.y;
+// Every HF steps a warp handles HF x R = 32 entries, one a lane: of face F1, and of
+// its p02 ring, which is filled a block ahead: for the HF steps starting at CTA time
+// T0 this lane's entry is row lane mod R at tau = T0 + 2 - wR + lane / R.
+constexpr int HF = 32 / c3::R;
+struct C3Fill {
+    const uint16_t *c2;   // c2off entry of this lane's tau at T0 = 0
+    const int *row;       // table row of the code of this lane's row
+    int tau;              // this lane's tau at T0 = 0
+    int *ring;            // p02r[w] of this lane's row
+};
+__device__ __forceinline__ void c3_fill_store(const C3Fill &f, int T0, int v) {
+    const int slot = (f.tau + T0) & (c3::SQ - 1);
+    f.ring[slot * 4] = v;
+    f.ring[(slot < c3::U ? slot + c3::SQ : slot) * 4] = v;  // no branch: the step stays one basic block
+}
+__device__ __forceinline__ int c3_fill_load(const C3Fill &f, int T0) { return f.row[f.c2[T0]] - 5; }
+
+// Lane 0's inputs of the step with staged-face row fr.
+__device__ __forceinline__ void c3_load_face(C3St &g, const int *fr, int wR) {
+#pragma unroll
+    for (int r = 0; r < c3::R; r += 4) {
+        const int4 v = *reinterpret_cast<const int4 *>(fr + 4 + wR + r);
+        g.f[r] = v.x, g.f[r + 1] = v.y, g.f[r + 2] = v.z, g.f[r + 3] = v.w;
     }
-    const int fm = fr[3 + c.wR];
+    g.fm = fr[3 + wR];
+}
+
+// One step. Everything with a latency is started a step or more before its use:
+// the shuffles of this step's values (for the next step) as soon as they exist,
+// the staged face a step ahead, row -1 a chunk ahead with one vote per chunk.
+template <int s>
+__device__ __forceinline__ void c3_step(C3St &g, const C3Ln &c, const C3Fill &f, const C3Blk &b, int T0, int lane,
+                                        C3Smem &sm, const LaunchDesc &L) {
+    constexpr int R = c3::R, H = c3::U, M = R - 1;
+    static_assert(R == 4 || R == 8, "rows per warp: 4 or 8");
+    static_assert(H % CH == 0 && H % R == 0 && H % HF == 0, "a block is a whole number of pair-score shifts");
+    const int T = T0 + s;
+    // p12 of the position x2 = T + 2 - lane - wR (row 0 of time T + 2), p02 of every row of time T + 2
+    const int ppR = g.pp[s & M];  // position s - R, the last row's e12 pair
+    g.pp[s & M] = b.p12[s * 32];
+    int p02[R];
+#pragma unroll
+    for (int r = 0; r < R; r += 4) {
+        const int4 v = *reinterpret_cast<const int4 *>(b.p02 + r * (c3::SQ + c3::U) + s * 4);
+        p02[r] = v.x, p02[r + 1] = v.y, p02[r + 2] = v.z, p02[r + 3] = v.w;
+    }
+    // row -1 of the next chunk
+    if constexpr (s % CH == 0)
+        g.nxt = c3_ring_load(s + CH < H ? b.rin + (s + CH) * 32 : b.rin2 + (s + CH - H) * 32);
+    // U(T, r) from lane l-1 (lane 0: the staged face)
     int Un[R];
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-        const int v = __shfl_up_sync(kFull, g.V[r], 1);
-        Un[r] = lane == 0 ? fv[r] : v;
-    }
-    int UMn = __shfl_up_sync(kFull, g.VM, 1);
-    if (lane == 0) UMn = fm;
-    // the cells of time T
-    const int WT = c.Wl + 4 * T;
-    unsigned pk = 0;
+    for (int r = 0; r < R; ++r) Un[r] = lane == 0 ? g.f[r] : g.S[r];
+    const int UMn = lane == 0 ? g.fm : g.SM;
+    const int VMn = (int)(unsigned)g.cur.e[s % CH];
+    // the cells of time T: best candidate and its tag; the tags are the traceback bytes
+    int acc[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-        const int acc = max(g.P[r], Un[r]);
-        const int m = (WT - 3 * r - acc) & 7;
-        g.V[r] = acc + m;
-        pk |= (unsigned)m << (8 * r);
+        acc[r] = __viaddmax_s32(Un[r], 5, g.P[r]);
+        g.V[r] = acc[r] & ~7;
+        g.S[r] = __shfl_up_sync(kFull, g.V[r], 1);
     }
+    g.SM = __shfl_up_sync(kFull, VMn, 1);
     // outputs: last row to the warp below (or face F0), traceback bytes, lane 31 to face F1
     st_entry(b.rout + s * 32, pack_entry(g.V[R - 1], c.tagout + T));
-    if constexpr (R == 4)
-        *reinterpret_cast<uint32_t *>(b.tbp + s * (c3::W * 32 * R)) = pk;
-    else
-        *reinterpret_cast<uint16_t *>(b.tbp + s * (c3::W * 32 * R)) = (uint16_t)pk;
-    if (c.last) {
-        const int tg = c.tagf1 + T;
+    c3_load_face(g, b.f1row + (s + 1) * c3::F1S, c.wR);
+    unsigned pk[R / 4];
 #pragma unroll
-        for (int r = 0; r < R; r += 2)
-            st_global_v2(b.f1o + s * c3::WR + r, pack_entry(g.V[r], tg), pack_entry(g.V[r + 1], tg));
+    for (int r = 0; r < R; r += 4)
+        pk[r / 4] = __byte_perm(__byte_perm((unsigned)acc[r], (unsigned)acc[r + 1], 0x0040),
+                                __byte_perm((unsigned)acc[r + 2], (unsigned)acc[r + 3], 0x0040), 0x5410) &
+                    0x07070707u;
+    if constexpr (R == 4)
+        *reinterpret_cast<uint32_t *>(b.tbp + s * (c3::W * 32 * R)) = pk[0];
+    else
+        *reinterpret_cast<uint2 *>(b.tbp + s * (c3::W * 32 * R)) = make_uint2(pk[0], pk[R / 4 - 1]);
+    // a p02 entry of the next block: looked up in the first of HF steps, stored in the last
+    if constexpr (s % HF == 0) g.q = c3_fill_load(f, T + H);
+    if constexpr (s % HF == HF - 1) c3_fill_store(f, T - HF + 1 + H, g.q);
+    // lane 31's values are the warp's part of face F1: laid out in shared memory and,
+    // every HF steps, written by the whole warp, an entry per lane
+    if (c.last) {
+#pragma unroll
+        for (int r = 0; r < R; r += 4)
+            *reinterpret_cast<int4 *>(c.f1b + s % (2 * HF) * R + r) = make_int4(g.V[r], g.V[r + 1], g.V[r + 2], g.V[r + 3]);
     }
-    // code of the position x2 = T + 2 - lane - wR (row 0 of time T + 2)
-    const int cn = b.c2p[s];
-    g.cc[s & M] = cn;
-    g.pp[s & M] = ldtab(tab, c.laneb + cn);
-    // row -1: V(T, -1) from the ring (written by the warp above at its time T)
-    unsigned long long e = lds_u64_volatile(b.rin + s * 32);
-    if (__any_sync(kFull, (int)(e >> 32) != T)) e = c3_ring_wait(b.rin + s * 32, T, sm, L);
-    const int VMn = (int)(unsigned)e;
+    int fo = 0;
+    if constexpr (s % HF == HF - 1) {
+        __syncwarp();
+        fo = c.f1b[s / HF % 2 * 32 + lane];
+    }
+    if constexpr (s == H - 1) {
+        g.st_seen = ld_acquire_shared(&sm.staged);
+        g.dn_seen = ld_acquire_shared(c.prog_dn);
+        g.fail_seen = vload(&sm.failed);
+    }
     // P of time T + 1 and D of time T + 2
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-        const int vm = r ? g.V[r - 1] : VMn;
-        const int um = r ? Un[r - 1] : UMn;
-        const int y = um + c.p01[r];
-        int pn = max(max(g.D[r], vm), max(g.V[r], y));
-        pn = max(pn, Un[r] + g.pp[(s - r - 1) & M]);
-        const int p02 = ldtab(tab, c.rowb[r] + g.cc[(s - r) & M]);
-        const int p12 = g.pp[(s - r) & M];
-        g.D[r] = max(vm + p02, y + p02 + p12);
-        g.P[r] = pn;
+        const int vm = (r ? g.V[r - 1] : VMn) + 7;
+        const int y = (r ? Un[r - 1] : UMn) + c.p01[r];
+        int pn = __viaddmax_s32(g.V[r], 3, y);
+        pn = __viaddmax_s32(Un[r], r + 1 < R ? g.pp[(s - r - 1) & M] : ppR, pn);
+        g.P[r] = __vimax3_s32(pn, g.D[r], vm);
+        g.D[r] = __viaddmax_s32(y, g.pp[(s - r) & M], vm) + p02[r];
     }
-    g.VM = VMn;
+    if constexpr (s % HF == HF - 1) st_entry(b.f1o + (s - HF + 1) * c3::WR, pack_entry(fo, c.tagf1 + T - HF + 1 + c.f1t));
+    if constexpr (s % CH == CH - 1) {
+        if (s + 1 < H || T + 1 < c.N) {  // no entry follows the column's last time
+            if (__any_sync(kFull, !c3_ring_ready(g.nxt, T + 1)))
+                g.nxt = c3_ring_wait(s + 1 < H ? b.rin + (s + 1) * 32 : b.rin2, T + 1, sm, L);
+        }
+        g.cur = g.nxt;
+    }
 }
 
 // A step of the block that holds the far corner's CTA time (kernels that record
 // the corner): the plain step, then the corner's lane stores its row's key.
 template <int s>
-__device__ __forceinline__ void c3_capture_step(C3St &g, const C3Ln &c, const char *tab, const C3Blk &b, int T0,
+__device__ __forceinline__ void c3_capture_step(C3St &g, const C3Ln &c, const C3Fill &f, const C3Blk &b, int T0,
                                                 int lane, C3Smem &sm, const LaunchDesc &L) {
-    c3_step<s>(g, c, tab, b, T0, lane, sm, L);
+    c3_step<s>(g, c, f, b, T0, lane, sm, L);
     if (T0 + s == c.ctime) {
-        // a select chain (R is 2 or 4): a loop over r would index the registers dynamically
-        const int v = c.crow == 0 ? g.V[0] : c.crow == 1 ? g.V[1] : c.crow == 2 ? g.V[2 % c3::R] : g.V[c3::R - 1];
-        __stcg(c.qcorner, v);
+        int v = g.V[0];  // a select chain: a loop with a dynamic index would put the registers in memory
+#pragma unroll
+        for (int r = 1; r < c3::R; ++r) v = c.crow == r ? g.V[r] : v;
+        __stcg(c.qcorner, v + c.wcorner);
     }
+}
+
+// The unrolled steps of a block.
+template <bool CAP, int... S>
+__device__ __forceinline__ void c3_steps(C3St &g, const C3Ln &c, const C3Fill &f, const C3Blk &b, int T0, int lane,
+                                         C3Smem &sm, const LaunchDesc &L, std::integer_sequence<int, S...>) {
+    if constexpr (CAP)
+        (c3_capture_step<S>(g, c, f, b, T0, lane, sm, L), ...);
+    else
+        (c3_step<S>(g, c, f, b, T0, lane, sm, L), ...);
 }
 
 struct C3Col {
@@ -250,160 +371,155 @@ struct C3Col {
     const unsigned long long *f0up, *f1left, *f1diag;  // producer faces (nullptr: none)
     unsigned long long *f0dst, *f1dst;                  // this column's faces
     int tagbase;                                        // (epoch << 16) of this launch
+    const int *row1;                                    // table row of the code of x1 = 32B + lane
+    const uint16_t *c2;                                 // c2off entry of x2 = -lane
 };
 
-// Staging warp: copy the column's inputs from the producer columns' faces into
-// ring[0] and f1r, as soon as their tags show this launch's values, and publish
-// the number of CTA-time rows staged. Positions a producer never computes (past
-// its last step, or no producer at all) are staged as kNeg. A batch covers SB
-// rows: every load of the batch is issued before any tag is checked (one L2 round
-// trip per batch). Loads are 16-byte pairs of entries: an F0 row (32 entries) is
-// read by half a warp, an F1 row (WR entries) by WR / 2 lanes.
-__device__ void c3_stager(C3Smem &sm, const C3Col &cc, int lane, const LaunchDesc &L) {
-    constexpr int SB = 8;                        // rows per batch (one block: measured best)
-    constexpr int NL0 = SB / 2;                  // F0 loads per lane and batch (2 rows per load)
-    constexpr int LPR1 = c3::WR / 2;             // lanes per F1 row
-    constexpr int RPI1 = 32 / LPR1;              // F1 rows per load
-    constexpr int NL1 = SB / RPI1;               // F1 loads per lane and batch
-    static_assert(SB <= c3::SI - c3::U && SB <= c3::SF - c3::U, "staging batch exceeds the rings");
-    static_assert(SB % RPI1 == 0 && 32 % LPR1 == 0, "F1 rows per load");
-    const int half = lane >> 4, pair0 = 2 * (lane & 15);            // F0: row parity, first entry
-    const int sub1 = lane / LPR1, pair1 = 2 * (lane % LPR1);        // F1: row in the load, first entry
-    const unsigned rowmask1 = LPR1 == 32 ? 0xffffffffu : ((1u << LPR1) - 1);
-    int Ts = -c3::U;
-    uint64_t t_progress = global_ns();
-    while (Ts < cc.N) {
-        // the slots to fill must have been read by the compute warps
-        {
-            const int need0 = Ts + SB - c3::SI, needall = Ts + SB - c3::SF;
-            int ok;
-            while (true) {
-                const int pw = lane < c3::W ? ld_acquire_shared(&sm.prog[lane]) : (1 << 30);
-                const int pmin = __reduce_min_sync(kFull, pw);
-                const int p0 = __shfl_sync(kFull, pw, 0);
-                ok = p0 >= need0 && pmin >= needall;
-                if (ok) break;
-                if (vload(&sm.failed) || (int64_t)(global_ns() - t_progress) > L.spin_ns) break;
-                __nanosleep(64);
-            }
-            if (!ok) {
-                if (lane == 0 && !vload(&sm.failed)) c3_fail(sm, L);
-                return;
-            }
-        }
-        // issue every load of the batch
-        ulonglong2 a[NL0], b[NL1];
-        unsigned long long d = pack_entry(kNeg, 0);
-        const ulonglong2 none = make_ulonglong2(pack_entry(kNeg, 0), pack_entry(kNeg, 0));
+// Staging warps: they copy the column's inputs from the producer columns' faces as
+// soon as the entries' tags show this launch's values. Positions a producer never
+// computes (past its last step, or no producer at all) are staged as kNeg.
+//
+// Waits of the staging warps, every sixteenth poll: true when the column failed or the limit ran out.
+__device__ __forceinline__ bool c3_stage_expired(C3Smem &sm, uint64_t &t0, int lane, const LaunchDesc &L) {
+    if (t0 == 0) t0 = global_ns();
+    const bool end = vload(&sm.failed) || ld_volatile(L.err) != 0 || (int64_t)(global_ns() - t0) > L.spin_ns;
+    if (!__any_sync(kFull, end)) return false;
+    if (lane == 0 && !vload(&sm.failed)) c3_fail(sm, L);
+    return true;
+}
+// Bounded wait until the first n of prog have reached need.
+__device__ __forceinline__ bool c3_wait_room(C3Smem &sm, const int32_t *prog, int n, int need, int lane,
+                                             const LaunchDesc &L) {
+    uint64_t t0 = 0;
+    for (int polls = 0; !__all_sync(kFull, lane >= n || ld_acquire_shared(prog + lane) >= need); ++polls) {
+        if ((polls & 15) == 15 && c3_stage_expired(sm, t0, lane, L)) return false;
+        __nanosleep(100);
+    }
+    return true;
+}
+
+// Row warp: face F0 of the column above into ring[0], SB CTA times a batch. The
+// ring's entries carry their own tags, so a lane stores what it has.
+__device__ void c3_stage_rows(C3Smem &sm, const C3Col &cc, int lane, const LaunchDesc &L) {
+    constexpr int SB = c3::SB, NL = SB / 2;                // loads per lane and batch (2 rows per load)
+    const int half = lane >> 4, pair = 2 * (lane & 15);    // row parity, first entry
+    const ulonglong2 none = make_ulonglong2(pack_entry(kNeg, 0), pack_entry(kNeg, 0));
+    ulonglong2 e[NL];
+    int room = -c3::U + c3::SI;  // ring slots of the CTA times below are free
+    for (int Ts = -c3::U; Ts < cc.N; Ts += SB) {
+        // the slots to fill must have been read by warp 0
+        if (room < Ts + SB && !c3_wait_room(sm, &sm.prog[0], 1, Ts + SB - c3::SI, lane, L)) return;
+        room = ld_acquire_shared(&sm.prog[0]) + c3::SI;
+        uint64_t t0 = 0;
+        for (int polls = 0;; ++polls) {
+            bool ok = true;
 #pragma unroll
-        for (int i = 0; i < NL0; ++i) {
+            for (int i = 0; i < NL; ++i) {
+                const int T = Ts + 2 * i + half;
+                e[i] = none;
+                if (cc.f0up && T + c3::WR < cc.N)
+                    e[i] = ld_global_relaxed_v2(cc.f0up + (int64_t)(T + c3::WR + c3::U) * 32 + pair);
+            }
+#pragma unroll
+            for (int i = 0; i < NL; ++i) {
+                const int T = Ts + 2 * i + half, want = cc.tagbase + T + c3::WR;
+                if (cc.f0up && T + c3::WR < cc.N)
+                    ok = ok && (int)(e[i].x >> 32) == want && (int)(e[i].y >> 32) == want;
+            }
+            if (__all_sync(kFull, ok)) break;
+            if ((polls & 15) == 15 && c3_stage_expired(sm, t0, lane, L)) return;
+        }
+#pragma unroll
+        for (int i = 0; i < NL; ++i) {
             const int T = Ts + 2 * i + half;
-            a[i] = none;
-            if (cc.f0up && T + c3::WR < cc.N)
-                a[i] = ld_global_relaxed_v2(cc.f0up + (int64_t)(T + c3::WR + c3::U) * 32 + pair0);
+            *reinterpret_cast<ulonglong2 *>(&sm.ring[0][T & (c3::SI - 1)][pair]) =
+                make_ulonglong2(pack_entry((int)(unsigned)e[i].x, T), pack_entry((int)(unsigned)e[i].y, T));
         }
+    }
+}
+
+// Column warp: face F1 of the column to the left and the corner of the column
+// above-left into f1r, and the (axis 1, axis 2) pair scores into p12r; it
+// publishes how many CTA times are staged.
+__device__ void c3_stage_cols(C3Smem &sm, const C3Col &cc, int lane, const LaunchDesc &L) {
+    constexpr int SB = c3::SBC;
+    constexpr int LPR = c3::WR / 2, RPL = 32 / LPR, NL = SB / RPL;  // lanes per row, rows per load, loads
+    static_assert(SB % RPL == 0 && 32 % LPR == 0, "F1 rows per load");
+    const int sub = lane / LPR, pair = 2 * (lane % LPR);
+    const ulonglong2 none = make_ulonglong2(pack_entry(kNeg, 0), pack_entry(kNeg, 0));
+    for (int Ts = -c3::U; Ts < cc.N; Ts += SB) {
+        // the slots to fill must have been read by every compute warp
+        if (!c3_wait_room(sm, sm.prog, c3::W, Ts + SB - c3::SF, lane, L)) return;
+        ulonglong2 e[NL];
+        unsigned long long d;  // lane i: the corner of the batch's row i
+        uint64_t t0 = 0;
+        for (int polls = 0;; ++polls) {
 #pragma unroll
-        for (int i = 0; i < NL1; ++i) {
-            const int T = Ts + RPI1 * i + sub1;
-            b[i] = none;
-            if (cc.f1left && T + 31 < cc.N)
-                b[i] = ld_global_relaxed_v2(cc.f1left + (int64_t)(T + 31 + c3::U) * c3::WR + pair1);
-        }
-        {
-            const int T = Ts + lane;  // lane i fetches the corner of row Ts + i
-            if (lane < SB && cc.f1diag && T + 31 + c3::WR < cc.N)
-                d = ld_global_relaxed(cc.f1diag + (int64_t)(T + 31 + c3::WR + c3::U) * c3::WR + c3::WR - 1);
-        }
-        // rows whose entries all carry this launch's tag
-        unsigned rows_ok = 0;
-#pragma unroll
-        for (int i = 0; i < NL0; ++i) {
-            const int T = Ts + 2 * i + half;
-            bool v = true;
-            if (cc.f0up && T + c3::WR < cc.N) {
-                const int want = cc.tagbase + T + c3::WR;
-                v = (int)(a[i].x >> 32) == want && (int)(a[i].y >> 32) == want;
+            for (int i = 0; i < NL; ++i) {
+                const int T = Ts + RPL * i + sub;
+                e[i] = none;
+                if (cc.f1left && T + 31 < cc.N)
+                    e[i] = ld_global_relaxed_v2(cc.f1left + (int64_t)(T + 31 + c3::U) * c3::WR + pair);
             }
-            const unsigned bal = __ballot_sync(kFull, v);
-            rows_ok |= ((bal & 0xffffu) == 0xffffu ? 1u : 0u) << (2 * i);
-            rows_ok |= ((bal >> 16) == 0xffffu ? 1u : 0u) << (2 * i + 1);
-        }
-        unsigned rows_ok1 = 0;
+            const int Td = Ts + lane;
+            d = pack_entry(kNeg, 0);
+            const bool corner = lane < SB && cc.f1diag && Td + 31 + c3::WR < cc.N;
+            if (corner) d = ld_global_relaxed(cc.f1diag + (int64_t)(Td + 31 + c3::WR + c3::U) * c3::WR + c3::WR - 1);
+            if (polls == 0) {
+                // p12 of the batch's rows (warp 0 reads row T + 2 at time T), while the loads fly
 #pragma unroll
-        for (int i = 0; i < NL1; ++i) {
-            const int T = Ts + RPI1 * i + sub1;
-            bool v = true;
-            if (cc.f1left && T + 31 < cc.N) {
-                const int want = cc.tagbase + T + 31;
-                v = (int)(b[i].x >> 32) == want && (int)(b[i].y >> 32) == want;
+                for (int i = 0; i < SB; ++i) {
+                    const int t = Ts + i + 2;
+                    const int slot = t & (c3::SP - 1), v = cc.row1[cc.c2[t]] + 1;
+                    sm.p12r[slot][lane] = v;
+                    if (slot < c3::U) sm.p12r[slot + c3::SP][lane] = v;
+                }
             }
-            const unsigned bal = __ballot_sync(kFull, v);
+            bool ok = !corner || (int)(d >> 32) == cc.tagbase + Td + 31 + c3::WR;
 #pragma unroll
-            for (int q = 0; q < RPI1; ++q)
-                rows_ok1 |= (((bal >> (q * LPR1)) & rowmask1) == rowmask1 ? 1u : 0u) << (RPI1 * i + q);
-        }
-        rows_ok &= rows_ok1;
-        {
-            const int T = Ts + lane;
-            const bool v = lane >= SB || !cc.f1diag || T + 31 + c3::WR >= cc.N ||
-                           (int)(d >> 32) == cc.tagbase + T + 31 + c3::WR;
-            rows_ok &= __ballot_sync(kFull, v) & ((1u << SB) - 1);
-        }
-        const int n = rows_ok == (1u << SB) - 1 ? SB : __ffs(~rows_ok) - 1;  // rows ready, in order
-#pragma unroll
-        for (int i = 0; i < NL0; ++i) {
-            const int r = 2 * i + half;
-            if (r < n) {
-                const int T = Ts + r;
-                *reinterpret_cast<ulonglong2 *>(&sm.ring[0][T & (c3::SI - 1)][pair0]) =
-                    make_ulonglong2(pack_entry((int)(unsigned)a[i].x, T), pack_entry((int)(unsigned)a[i].y, T));
+            for (int i = 0; i < NL; ++i) {
+                const int T = Ts + RPL * i + sub, want = cc.tagbase + T + 31;
+                if (cc.f1left && T + 31 < cc.N)
+                    ok = ok && (int)(e[i].x >> 32) == want && (int)(e[i].y >> 32) == want;
             }
+            if (__all_sync(kFull, ok)) break;
+            if ((polls & 15) == 15 && c3_stage_expired(sm, t0, lane, L)) return;
         }
 #pragma unroll
-        for (int i = 0; i < NL1; ++i) {
-            const int r = RPI1 * i + sub1;
-            if (r < n) {
-                const int T = Ts + r;
-                *reinterpret_cast<int2 *>(&sm.f1r[T & (c3::SF - 1)][4 + pair1]) =
-                    make_int2((int)(unsigned)b[i].x, (int)(unsigned)b[i].y);
-            }
+        for (int i = 0; i < NL; ++i) {
+            const int T = Ts + RPL * i + sub;
+            *reinterpret_cast<int2 *>(&sm.f1r[T & (c3::SF - 1)][4 + pair]) =
+                make_int2((int)(unsigned)e[i].x, (int)(unsigned)e[i].y);
         }
-        if (lane < n) sm.f1r[(Ts + lane) & (c3::SF - 1)][3] = (int)(unsigned)d;
-        if (n > 0) {
-            Ts += n;
-            __syncwarp();
-            if (lane == 0) st_release_shared(&sm.staged, Ts);
-            t_progress = global_ns();
-        } else {
-            if (vload(&sm.failed) || ld_volatile(L.err) != 0 || (int64_t)(global_ns() - t_progress) > L.spin_ns) {
-                if (lane == 0 && !vload(&sm.failed)) c3_fail(sm, L);
-                return;
-            }
-            __nanosleep(64);
-        }
+        if (lane < SB) sm.f1r[(Ts + lane) & (c3::SF - 1)][3] = (int)(unsigned)d;
+        __syncwarp();
+        if (lane == 0) st_release_shared(&sm.staged, Ts + SB);
     }
 }
 
 // Block prologue of a compute warp: publish progress, then wait (bounded) until
 // the staged face covers the block and the warp below has freed the ring slots.
-__device__ __forceinline__ bool c3_block_wait(C3Smem &sm, int w, int T0, const LaunchDesc &L) {
+// The values seen are loads of the previous block's end.
+__device__ __forceinline__ bool c3_block_wait(C3Smem &sm, const C3Ln &c, int w, int T0, const C3St &g,
+                                              const LaunchDesc &L) {
     __syncwarp();
     if ((threadIdx.x & 31) == 0) st_release_shared(&sm.prog[w], T0);
     const int need_st = T0 + c3::U;
-    const int need_dn = T0 + c3::U - c3::SI;
-    const bool lastw = w == c3::W - 1;
-    if (ld_acquire_shared(&sm.staged) >= need_st && (lastw || ld_acquire_shared(&sm.prog[w + 1]) >= need_dn))
-        return true;
-    const uint64_t t0 = global_ns();
-    while (true) {
-        __nanosleep(32);
-        if (ld_acquire_shared(&sm.staged) >= need_st && (lastw || ld_acquire_shared(&sm.prog[w + 1]) >= need_dn))
+    const int need_dn = w == c3::W - 1 ? -(1 << 30) : T0 + c3::U - c3::SI;
+    if (__all_sync(kFull, g.st_seen >= need_st && g.dn_seen >= need_dn && !g.fail_seen)) return true;
+    uint64_t t0 = 0;
+    for (int polls = 0;; ++polls) {
+        if (!__any_sync(kFull, vload(&sm.failed) != 0) &&
+            __all_sync(kFull, ld_acquire_shared(&sm.staged) >= need_st && ld_acquire_shared(c.prog_dn) >= need_dn))
             return true;
-        if (vload(&sm.failed)) return false;
-        if ((int64_t)(global_ns() - t0) > L.spin_ns) {
+        if (__any_sync(kFull, vload(&sm.failed) != 0)) return false;
+        if (polls < 4) continue;
+        if (t0 == 0) t0 = global_ns();
+        if (__any_sync(kFull, (int64_t)(global_ns() - t0) > L.spin_ns)) {
             if ((threadIdx.x & 31) == 0) c3_fail(sm, L);
             return false;
         }
+        __nanosleep(32);
     }
 }
 
@@ -413,14 +529,13 @@ __device__ __forceinline__ bool c3_block_wait(C3Smem &sm, int w, int T0, const L
 // cross-check; the block holding it runs a capturing copy of the steps (which
 // costs registers, so plain launches use the kernel without it).
 template <bool CAP>
-__global__ void __launch_bounds__(c3::THREADS, 1) fill_col3_kernel(const LaunchDesc L) {
+__global__ void __launch_bounds__(c3::THREADS, c3::CTAS) fill_col3_kernel(const LaunchDesc L) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C3Smem &sm = *reinterpret_cast<C3Smem *>(smem_raw);
     int *tabr = reinterpret_cast<int *>(smem_raw + sizeof(C3Smem));
-    uint16_t *c2off = reinterpret_cast<uint16_t *>(tabr + L.tab_ints);  // axis-2 code offsets by x2 + CODEPAD
+    uint16_t *c2off = reinterpret_cast<uint16_t *>(tabr + L.tab_ints);  // axis-2 codes by x2 + CODEPAD
 
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-    const bool stager = w == c3::W;
     if (tid == 0) sm.cur_prob = -1;
     __syncthreads();
 
@@ -458,13 +573,12 @@ __global__ void __launch_bounds__(c3::THREADS, 1) fill_col3_kernel(const LaunchD
         const int tag_faces = (int64_t)ticket == L.withhold ? 0 : cc.tagbase;
 
         const int A = P.A;
-        // replicated pair table (entry-major, one copy per lane) with a sentinel
-        // code A for positions x2 <= 0, and the axis-2 code offsets
+        // pair table with a sentinel code A for positions x2 <= 0, and the axis-2 codes
         const int have = sm.cur_prob;
         __syncthreads();
         if (have != pidx)
-            for (int i = tid; i < A * (A + 1) * 32; i += c3::THREADS) {
-                const int c0 = i / ((A + 1) * 32), c2 = (i >> 5) % (A + 1);
+            for (int i = tid; i < A * (A + 1); i += c3::THREADS) {
+                const int c0 = i / (A + 1), c2 = i % (A + 1);
                 tabr[i] = c2 == A ? c3::kSentinelPair : P.tab[c0 * A + c2];
             }
         if (tid == 0) {
@@ -476,44 +590,58 @@ __global__ void __launch_bounds__(c3::THREADS, 1) fill_col3_kernel(const LaunchD
         const int len2 = P.len[2];
         for (int i = tid; i < P.rho[2] + 2 * c3::CODEPAD + 16; i += c3::THREADS) {
             const int x2 = i - c3::CODEPAD;  // position x2 consumes residue x2 - 1
-            const int code = x2 <= 0 ? A : x2 <= len2 ? P.codes[P.cofs[2] + x2 - 1] : 0;
-            c2off[i] = (uint16_t)(code * 128);
+            c2off[i] = (uint16_t)(x2 <= 0 ? A : x2 <= len2 ? P.codes[P.cofs[2] + x2 - 1] : 0);
         }
+        // pair scores before the first block belong to positions x2 < 0
+        for (int i = tid; i < (c3::SP + c3::U) * 32; i += c3::THREADS) (&sm.p12r[0][0])[i] = c3::kSentinelPair;
+        for (int i = tid; i < c3::W * (c3::SQ + c3::U) * c3::R; i += c3::THREADS)
+            (&sm.p02r[0][0][0][0])[i] = c3::kSentinelPair;
         // ring entries start with a tag no step uses
         for (int i = tid; i < c3::W * c3::SI * 32; i += c3::THREADS)
             (&sm.ring[0][0][0])[i] = pack_entry(kNeg, 0x7fffffff);
         __syncthreads();
 
-        if (stager) {
-            c3_stager(sm, cc, lane, L);
+        const int x1 = cc.B * 32 + lane;
+        const int code1 = (x1 >= 1 && x1 <= P.len[1]) ? P.codes[P.cofs[1] + x1 - 1] : 0;
+        if (w == c3::W) {
+            c3_stage_rows(sm, cc, lane, L);
+        } else if (w > c3::W) {
+            cc.row1 = tabr + code1 * (A + 1);
+            cc.c2 = c2off + c3::CODEPAD - lane;
+            c3_stage_cols(sm, cc, lane, L);
         } else {
             const bool lastw = w == c3::W - 1;
             C3Ln c;
             c.wR = w * c3::R;
             c.last = lane == 31;
+            c.f1b = &sm.f1b[w][0][0];
+            c.f1t = lane / c3::R;
             c.tagout = lastw ? tag_faces : 0;
             c.tagf1 = tag_faces;
-            const int x1 = cc.B * 32 + lane;
-            const int code1 = (x1 >= 1 && x1 <= P.len[1]) ? P.codes[P.cofs[1] + x1 - 1] : 0;
+            c.N = cc.N;
+            c.prog_dn = &sm.prog[lastw ? w : w + 1];
             const int x0b = cc.A * c3::WR + c.wR;
-#pragma unroll
-            for (int r = 0; r < c3::R; ++r) {
+            auto code0 = [&](int r) {
                 const int x0 = x0b + r;
-                const int code0 = (x0 >= 1 && x0 <= P.len[0]) ? P.codes[P.cofs[0] + x0 - 1] : 0;
-                c.rowb[r] = (code0 * (A + 1) * 32 + lane) * 4;
-                c.p01[r] = P.tab[code0 * A + code1];
-            }
-            c.laneb = (code1 * (A + 1) * 32 + lane) * 4;
-            c.Wl = cc.A * c3::WR + 64 * cc.B - 2 * lane - 3 * c.wR;
+                return (x0 >= 1 && x0 <= P.len[0]) ? (int)P.codes[P.cofs[0] + x0 - 1] : 0;
+            };
+#pragma unroll
+            for (int r = 0; r < c3::R; ++r) c.p01[r] = P.tab[code0(r) * A + code1] + 4;
+            C3Fill f;
+            f.row = tabr + code0(lane % c3::R) * (A + 1);
+            f.tau = 2 - c.wR + lane / c3::R;
+            f.c2 = c2off + c3::CODEPAD + f.tau - lane % c3::R;
+            f.ring = &sm.p02r[w][lane % c3::R / 4][0][lane % 4];
+#pragma unroll
+            for (int n = -c3::U; n < 0; n += HF) c3_fill_store(f, n, c3_fill_load(f, n));
             {  // the far corner (len0, len1, len2): row rho of lane l at CTA time len2 + l + rho
                 const int rhoc = P.len[0] - cc.A * c3::WR, lc = P.len[1] - 32 * cc.B;
                 const bool mine = rhoc >= c.wR && rhoc < c.wR + c3::R && lc == lane;
                 c.ctime = mine ? P.len[2] + lc + rhoc : (int)0x80000000;
                 c.crow = rhoc - c.wR;
+                c.wcorner = P.w_corner;
                 c.qcorner = P.qcorner;
             }
-            const char *tab = reinterpret_cast<const char *>(tabr);
-            const uint16_t *c2lane = c2off + c3::CODEPAD + 2 - lane - c.wR;  // x2 = T + 2 - lane - wR at T
 
             C3St g;
 #pragma unroll
@@ -521,17 +649,16 @@ __global__ void __launch_bounds__(c3::THREADS, 1) fill_col3_kernel(const LaunchD
                 g.V[r] = kNeg;
                 g.P[r] = kNeg;
                 g.D[r] = kNeg;
+                g.S[r] = kNeg;
             }
             const bool origin = cc.A == 0 && cc.B == 0 && w == 0 && lane == 0;
-            g.VM = kNeg;
-            // shift registers before time -U: positions x2 = 2 - U - lane - wR - j, j = 1 .. 2R-1
+            g.SM = kNeg;
+            g.st_seen = g.dn_seen = -(1 << 30);
+            g.fail_seen = 0;
+            g.cur = c3_ring_wait(&sm.ring[w][-c3::U & (c3::SI - 1)][lane], -c3::U, sm, L);
+            // p12 of the positions before time -U, all below 0
 #pragma unroll
-            for (int j = 1; j < 2 * c3::R; ++j) {
-                const int cj = c2lane[-c3::U - j];
-                g.cc[(-j) & (2 * c3::R - 1)] = cj;
-                g.pp[(-j) & (2 * c3::R - 1)] = ldtab(tab, c.laneb + cj);
-            }
-            g.cc[0] = g.pp[0] = 0;
+            for (int j = 0; j < c3::R; ++j) g.pp[j] = c3::kSentinelPair;
 
             unsigned long long *ringout = lastw ? cc.f0dst + lane : &sm.ring[w + 1][0][lane];
             unsigned char *tbw = P.tb + (int64_t)lin * c3::tb_col_bytes(P.rho[2]) + (w * 32 + lane) * c3::R;
@@ -541,35 +668,35 @@ __global__ void __launch_bounds__(c3::THREADS, 1) fill_col3_kernel(const LaunchD
                 const int ct = __shfl_sync(kFull, c.ctime, (P.len[1] - 32 * cc.B) & 31);
                 if (ct != (int)0x80000000) T0c = ct / c3::U * c3::U;
             }
+            C3Blk b;
+            b.rin2 = &sm.ring[w][-c3::U & (c3::SI - 1)][lane];
+            b.rout = ringout + (lastw ? 0 : (-c3::U & (c3::SI - 1)) * 32);
+            b.f1row = &sm.f1r[-c3::U & (c3::SF - 1)][0];
+            b.tbp = tbw;
+            b.f1o = cc.f1dst + (int64_t)c.f1t * c3::WR + c.wR + lane % c3::R;
+            b.p02 = &sm.p02r[w][0][(-c3::U + 2 - c.wR - lane) & (c3::SQ - 1)][0];
+            b.p12 = &sm.p12r[(-c3::U + 2 - c.wR) & (c3::SP - 1)][lane];
             for (int T0 = -c3::U; T0 < cc.N; T0 += c3::U) {
-                if (!c3_block_wait(sm, w, T0, L)) break;
+                if (!c3_block_wait(sm, c, w, T0, g, L)) break;
                 if (T0 == 0 && origin) g.P[0] = 0;  // H(0) = 0, no move
-                C3Blk b;
-                b.rin = &sm.ring[w][T0 & (c3::SI - 1)][lane];
-                b.rout = lastw ? ringout + (int64_t)(T0 + c3::U) * 32 : ringout + (T0 & (c3::SI - 1)) * 32;
-                b.f1row = &sm.f1r[T0 & (c3::SF - 1)][0];
-                b.tbp = tbw + (int64_t)(T0 + c3::U) * (c3::W * 32 * c3::R);
-                b.f1o = cc.f1dst + (int64_t)(T0 + c3::U) * c3::WR + c.wR;
-                b.c2p = c2lane + T0;
-                if (!CAP || T0 != T0c) {
-                    c3_step<0>(g, c, tab, b, T0, lane, sm, L);
-                    c3_step<1>(g, c, tab, b, T0, lane, sm, L);
-                    c3_step<2>(g, c, tab, b, T0, lane, sm, L);
-                    c3_step<3>(g, c, tab, b, T0, lane, sm, L);
-                    c3_step<4>(g, c, tab, b, T0, lane, sm, L);
-                    c3_step<5>(g, c, tab, b, T0, lane, sm, L);
-                    c3_step<6>(g, c, tab, b, T0, lane, sm, L);
-                    c3_step<7>(g, c, tab, b, T0, lane, sm, L);
-                } else {
-                    c3_capture_step<0>(g, c, tab, b, T0, lane, sm, L);
-                    c3_capture_step<1>(g, c, tab, b, T0, lane, sm, L);
-                    c3_capture_step<2>(g, c, tab, b, T0, lane, sm, L);
-                    c3_capture_step<3>(g, c, tab, b, T0, lane, sm, L);
-                    c3_capture_step<4>(g, c, tab, b, T0, lane, sm, L);
-                    c3_capture_step<5>(g, c, tab, b, T0, lane, sm, L);
-                    c3_capture_step<6>(g, c, tab, b, T0, lane, sm, L);
-                    c3_capture_step<7>(g, c, tab, b, T0, lane, sm, L);
-                }
+                c3_load_face(g, b.f1row, c.wR);
+                b.rin = b.rin2;
+                b.rin2 = &sm.ring[w][(T0 + c3::U) & (c3::SI - 1)][lane];
+                // the next block's addresses, formed while this one runs
+                C3Blk n;
+                const int Tn = T0 + c3::U;
+                n.rin2 = b.rin2;
+                n.rout = lastw ? b.rout + c3::U * 32 : ringout + (Tn & (c3::SI - 1)) * 32;
+                n.f1row = &sm.f1r[Tn & (c3::SF - 1)][0];
+                n.tbp = b.tbp + c3::U * (c3::W * 32 * c3::R);
+                n.f1o = b.f1o + c3::U * c3::WR;
+                n.p02 = &sm.p02r[w][0][(Tn + 2 - c.wR - lane) & (c3::SQ - 1)][0];
+                n.p12 = &sm.p12r[(Tn + 2 - c.wR) & (c3::SP - 1)][lane];
+                if (!CAP || T0 != T0c)
+                    c3_steps<false>(g, c, f, b, T0, lane, sm, L, std::make_integer_sequence<int, c3::U>{});
+                else
+                    c3_steps<true>(g, c, f, b, T0, lane, sm, L, std::make_integer_sequence<int, c3::U>{});
+                b = n;
             }
             __syncwarp();
             if (lane == 0) st_release_shared(&sm.prog[w], 1 << 30);
@@ -579,10 +706,10 @@ __global__ void __launch_bounds__(c3::THREADS, 1) fill_col3_kernel(const LaunchD
     }
 }
 
-// Dynamic shared memory: rings and staged faces, the replicated pair table with
-// its sentinel column (A*(A+1) entries x 32 lanes) and the axis-2 code offsets.
+// Dynamic shared memory: rings and staged faces, the pair table with its sentinel
+// column (A*(A+1) entries) and the axis-2 codes.
 int col3_smem_bytes(int alphabet_size) {
-    return (int)sizeof(C3Smem) + alphabet_size * (alphabet_size + 1) * 32 * 4 +
+    return (int)sizeof(C3Smem) + alphabet_size * (alphabet_size + 1) * 4 +
            (c3::MAXRHO2 + 2 * c3::CODEPAD + 16) * 2 + 16;
 }
 

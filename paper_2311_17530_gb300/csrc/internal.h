@@ -208,19 +208,25 @@ constexpr int kBand2RowsPerLane = 4;
 // or T-2 (same lane, lane l-1, or row rho-1), so rings indexed by T connect the
 // warps of a CTA and faces indexed by T connect neighbouring columns.
 namespace c3 {
-constexpr int R = 4;          // rows per warp (registers)
-constexpr int W = 8;          // compute warps per CTA
+constexpr int R = 8;          // rows per warp (registers)
+constexpr int W = 4;          // compute warps per CTA
+constexpr int CTAS = 1;       // resident CTAs per SM the registers are sized for
 constexpr int WR = R * W;     // rows per CTA
-constexpr int U = 8;          // steps per block (the unrolled loop body), a multiple of 2R
+constexpr int U = 8;          // steps per block (the unrolled loop body), a multiple of R
+constexpr int CH = 1;         // steps per ring read (one tag vote each), divides U
+constexpr int SB = 4;         // CTA times per staging batch of axis-0 faces, divides U
+constexpr int SBC = 8;        // CTA times per staging batch of axis-1 faces, divides U
 constexpr int SI = 32;        // depth of the rings into each warp (CTA-time entries), multiple of U
 constexpr int SF = 64;        // depth of the staged axis-1 face ring, multiple of U
+constexpr int SP = 128;       // depth of the ring of (axis 1, axis 2) pair scores, by x2 + lane
+constexpr int SQ = 64;        // depth of each warp's ring of (axis 0, axis 2) pair scores, by x2 + row
 constexpr int F1S = WR + 4;   // ints per staged axis-1 face row: [3] row -1, [4 + rho] row rho
-constexpr int THREADS = 32 * (W + 1);  // compute warps + one staging warp
-constexpr int MAXA = 24;      // largest alphabet (replicated pair table)
+constexpr int THREADS = 32 * (W + 2);  // compute warps + two staging warps
+constexpr int MAXA = 24;      // largest alphabet
 constexpr int MAXRHO2 = 4096; // largest axis-2 extent (staged codes)
 constexpr int CODEPAD = 96;   // axis-2 code staging pad on both sides
 constexpr int kSentinelPair = -(1 << 27);  // pair score of a move into x2 <= 0 (no residue)
-static_assert(U % (2 * R) == 0 && SI % U == 0 && SF % U == 0 && (WR == 16 || WR == 32), "column geometry");
+static_assert(U >= R && U % CH == 0 && SP >= SF + WR + 16 && SQ >= 31 + 2 * U + 1 && SI % U == 0 && SF % U == 0 && (WR == 16 || WR == 32), "column geometry");
 // CTA-time steps of one column: the last cell x2 = rho2 - 1 of lane 31, row
 // WR - 1 is computed at T = rho2 + WR + 29; rounded up to whole blocks. A column
 // runs T = -U .. nsteps - 1: the first block only fills the pipeline (its cells
@@ -239,7 +245,9 @@ __host__ __device__ constexpr int face1_rows(int rho2) { return nsteps(rho2) + U
 // (nsteps(rho2) + U) * W * 32 * R bytes, and the move of cell (x0 = A*WR + w*R + r,
 // x1 = 32B + l, x2) sits at (((T + U)*W + w)*32 + l)*R + r with
 // T = x2 + l + w*R + r, so each warp step stores one contiguous run of 32 lanes x
-// R bytes.
+// R bytes. A byte is the tag of the winning move (fill_col3.cu): tags 7 5 4 3 2 1 0
+// are the masks 1 .. 7, tag 6 is no move; the origin's byte is not read.
+__host__ __device__ constexpr int mask_of_tag(int t) { return t == 7 ? 1 : t == 6 ? 0 : 7 - t; }
 __host__ __device__ constexpr int64_t tb_col_bytes(int rho2) { return (int64_t)(nsteps(rho2) + U) * W * 32 * R; }
 }  // namespace c3
 

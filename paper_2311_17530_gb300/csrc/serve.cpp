@@ -571,7 +571,7 @@ int Server::launch(Slot &sl, std::vector<ServeReq *> &batch, const Settings &cfg
         L.spin_ns = cfg.spin_ms * 1000000LL;
         L.withhold = -1;
         L.nprob = g.count;
-        L.tab_ints = g.maxA * (g.maxA + 1) * 32;
+        L.tab_ints = g.maxA * (g.maxA + 1);
         L.epoch = epoch_;
         for (int j = 0; j < g.count; ++j) L.corner |= batch[g.first + j]->hp.check_corner;
         e = g.kernel == kKernelCol3    ? launch_fill_col3(L, g.grid, col3_smem_bytes(g.maxA), s)

@@ -125,7 +125,7 @@ struct ColWindow {
 };
 
 __device__ void walk_col3(const ProblemDesc &P, const IODesc &io, unsigned char *win, WalkState &ws) {
-    static_assert(c3::WR == 32 && c3::R == 4, "index arithmetic below assumes WR = 32, R = 4");
+    static_assert(c3::WR == 32 && (c3::R == 4 || c3::R == 8), "index arithmetic below assumes WR = 32, R = 4 or 8");
     constexpr int kRowB = c3::W * 32 * c3::R;         // bytes of one CTA time of a column
     static_assert(kRowB == 1024, "the walk steps T by shifting the move count by 10");
     constexpr int kBuf = kTracebackSmem / 2;          // one window buffer
@@ -220,20 +220,26 @@ __device__ void walk_col3(const ProblemDesc &P, const IODesc &io, unsigned char 
         // The next cell's byte is loaded before this move's checks branch, so the
         // branches resolve under the load's latency; an address below the window
         // is clamped to its first byte (in bounds, unused: the walk leaves).
-        unsigned a = wbase + (unsigned)(T * kRowB + (rho >> 2) * (32 * c3::R) + l * c3::R + (rho & 3));
-        int m = lds_u8(a);
+        unsigned a = wbase + (unsigned)(T * kRowB + rho / c3::R * (32 * c3::R) + l * c3::R + rho % c3::R);
+        int mt = lds_u8(a);
         while (true) {
-            // next address: every moved axis lowers T (kRowB bytes); axis 0 also
-            // lowers the row (1 byte, or 125 when it crosses a warp block of R
-            // rows), axis 1 the lane (R bytes). The part below kRowB is a byte
-            // table indexed by the mask (selected by the row's position in its block).
-            const int mm = m & 7;
-            const unsigned small = __byte_perm((x0 & 3) ? 0x05040100u : 0x81047d00u,
-                                               (x0 & 3) ? 0x05040100u : 0x81047d00u, (unsigned)mm);
-            const unsigned an = (unsigned)max((int)a - (__popc(mm) << 10) - (int)small, (int)wlo);
+            // next address: every moved axis lowers T (kRowB = 4 x 256 bytes); axis 0
+            // also lowers the row (1 byte, or 249 when it crosses a warp block of R
+            // rows), axis 1 the lane (R bytes; 249 + 8 carries 1 into the 256s). The
+            // stored byte is the move's tag (c3::mask_of_tag); the mask, the 256s and
+            // the rest of the step are byte tables indexed by it, byte 6 (no move)
+            // being 0.
+            const unsigned sel = ((unsigned)mt & 7u) | 0x6660u;
+            const bool cross = x0 % c3::R == 0;
+            const unsigned lo = c3::R == 8 ? __byte_perm(cross ? 0x00f90801u : 0x00010809u, cross ? 0xf9000801u : 0x01000809u, sel)
+                                           : __byte_perm(cross ? 0x007d0481u : 0x00010405u, cross ? 0x7d000481u : 0x01000405u, sel);
+            const unsigned hi = __byte_perm(cross && c3::R == 8 ? 0x0408080du : 0x0408080cu,
+                                            cross && c3::R == 8 ? 0x04000409u : 0x04000408u, sel);
+            const unsigned an = (unsigned)max((int)a - (int)(hi << 8) - (int)lo, (int)wlo);
             const int mn = lds_u8(an);
+            const int m = (int)__byte_perm(0x04050607u, 0x01000203u, sel);
             const int zero = (x0 == 0) | ((x1 == 0) << 1) | ((x2 == 0) << 2);
-            const bool bad = ((unsigned)(m - 1) > 6u) | ((m & zero) != 0) | (ncols >= len_sum);
+            const bool bad = ((unsigned)mt > 7u) | (m == 0) | ((m & zero) != 0) | (ncols >= len_sum);
             const int y0 = x0 - (m & 1), y1 = x1 - ((m >> 1) & 1), y2 = x2 - (m >> 2);
             const bool in = ((y0 >> 5) == A) & ((y1 >> 5) == B) & (y2 + (y1 & 31) + (y0 & 31) >= t_lo) &
                             ((y0 | y1 | y2) != 0);
@@ -247,7 +253,7 @@ __device__ void walk_col3(const ProblemDesc &P, const IODesc &io, unsigned char 
             x1 = y1;
             x2 = y2;
             if (!in) break;
-            m = mn;
+            mt = mn;
             a = an;
         }
         if (ncols == before) fail = true;  // a window must advance the walk
