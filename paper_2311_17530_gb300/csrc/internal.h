@@ -215,7 +215,6 @@ constexpr int WR = R * W;     // rows per CTA
 constexpr int U = 8;          // steps per block (the unrolled loop body), a multiple of R
 constexpr int CH = 1;         // steps per ring read (one tag vote each), divides U
 constexpr int SB = 4;         // CTA times per staging batch of axis-0 faces, divides U
-constexpr int SBC = 8;        // CTA times per staging batch of axis-1 faces, divides U
 constexpr int SI = 32;        // depth of the rings into each warp (CTA-time entries), multiple of U
 constexpr int SF = 64;        // depth of the staged axis-1 face ring, multiple of U
 constexpr int SP = 128;       // depth of the ring of (axis 1, axis 2) pair scores, by x2 + lane
