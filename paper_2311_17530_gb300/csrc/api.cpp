@@ -695,7 +695,7 @@ int msa_near_optimal(int k, const char *const *seqs, const int32_t *lens, const 
     const size_t o_res = take(total + 16), o_sub = take((size_t)A * A * 4), o_out = take(sizeof(msa_device_result)),
                  o_mask1 = take(total + 16), o_masks = take((size_t)max_count * total + 16),
                  o_ncols = take((size_t)max_count * 4), o_scores = take((size_t)max_count * 8), o_cm = take(8),
-                 o_path = take(total + 16), o_acc = take((total + 1) * 8), o_next = take((total + 1) * 4);
+                 o_work = take(near_optimal_work_bytes(k, (int64_t)total));
     char *d = nullptr;
     cudaError_t e = cudaMalloc(&d, off);
     if (e != cudaSuccess) {
@@ -724,9 +724,8 @@ int msa_near_optimal(int k, const char *const *seqs, const int32_t *lens, const 
                   reinterpret_cast<msa_device_result *>(d + o_out), reinterpret_cast<uint8_t *>(d + o_mask1), gap, 0};
         NearOut no{reinterpret_cast<uint8_t *>(d + o_masks), reinterpret_cast<int32_t *>(d + o_ncols),
                    reinterpret_cast<int64_t *>(d + o_scores), reinterpret_cast<int32_t *>(d + o_cm),
-                   reinterpret_cast<uint8_t *>(d + o_path), reinterpret_cast<int64_t *>(d + o_acc),
-                   reinterpret_cast<int32_t *>(d + o_next)};
-        e = launch_near_optimal(plan->pp.prob, io, delta, max_count, no, s);
+                   reinterpret_cast<unsigned char *>(d + o_work)};
+        e = launch_near_optimal(k, (int64_t)total, plan->pp.prob, io, delta, max_count, no, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) rc = cuda_error(e, "near-optimal enumeration");
     }

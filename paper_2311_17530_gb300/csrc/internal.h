@@ -305,21 +305,20 @@ int fill_stream_ctas_per_sm(int k);
 int fill_band2_ctas_per_sm();
 int fill_band2_warps_per_cta();
 int col3_smem_bytes(int alphabet_size);
-// Outputs and stack of the near-optimal enumeration (near_optimal.cu), device memory:
+// Outputs of the near-optimal enumeration (near_optimal.cu), device memory:
 // masks max_count x len_sum (first column first), ncols and scores per alignment,
-// count_more[2] = {alignments stored, 1 when more were left (2: walk inconsistent)},
-// and per depth (len_sum + 1 entries) the move taken, the score so far and the next mask.
+// count_more[2] = {alignments stored, 1 when more were left (2: walk inconsistent)};
+// work holds near_optimal_work_bytes of tables and stack (0: they fit in shared memory).
 struct NearOut {
     uint8_t *masks;
     int32_t *ncols;
     int64_t *scores;
     int32_t *count_more;
-    uint8_t *path;
-    int64_t *acc;
-    int32_t *next;
+    unsigned char *work;
 };
-cudaError_t launch_near_optimal(const ProblemDesc *d_prob, IODesc io, int64_t delta, int32_t max_count, NearOut o,
-                                cudaStream_t s);
+size_t near_optimal_work_bytes(int k, int64_t len_sum);
+cudaError_t launch_near_optimal(int k, int64_t len_sum, const ProblemDesc *d_prob, IODesc io, int64_t delta,
+                                int32_t max_count, NearOut o, cudaStream_t s);
 
 // Exact pruning (prune.cu): the pairwise tables of every pair i < j, the largest
 // fwd + bwd of every tile rectangle, the tiles' bounds and, against a lower

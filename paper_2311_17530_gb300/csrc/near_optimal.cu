@@ -14,140 +14,230 @@
 // The fill is the generic tile kernel, which keeps the packed key of every cell:
 // Q(x) = H'(x) 2^k + W(x) with H'(x) = H(x) - gap (k - 1) |x|_1 and
 // W(x) = sum_i 2^i x_i, so H(x) = (Q(x) - W(x)) / 2^k + gap (k - 1) |x|_1
-// exactly. One warp walks: at each depth its 32 lanes judge 32 consecutive
-// masks at once and a ballot picks the lowest one that qualifies.
+// exactly (and in 32 bits: every sum compared below is the score of an alignment,
+// which the encode step's range check keeps in range).
+//
+// One warp walks, and what bounds it is the chain of one node: residue codes and
+// offsets from shared memory, one score per lane, a ballot. At a node every mask is
+// judged at once, a lane per mask (and 32 masks per round), and the set that
+// qualifies goes on the stack, so going back costs no judging: the lanes look 32
+// depths at a time for the deepest one with a mask left and count the moves to undo
+// with one ballot per axis. The offset of a cell is a sum of one term per axis in
+// every layout of the scores, so the terms are tabulated per coordinate once.
+// 256 alignments of 120 x 110 x 130 (9,100 moves followed): 24.6 ms when the walk
+// went back one column at a time, judging again, with positions in local memory.
 #include "device_common.cuh"
 
 namespace msadp {
 
-// Element offset of cell x in the tile kernel's score tensor: row-major
+namespace {
+
+constexpr int kNearThreads = 256;
+constexpr int kNearSmem = 160 * 1024;  // tables and stack beyond this stay in global memory
+
+// Term of coordinate v of axis i in the element offset of a cell's score: row-major
 // (qstride) for k <= 3, tile-major (the traceback's layout 2) for k >= 4.
-__device__ __forceinline__ int64_t score_cell(const ProblemDesc &P, const int *x) {
-    int64_t g = 0;
-    if (P.tb_layout == 2) {
-        int64_t t = 0, loc = 0;
-        for (int i = 0; i < P.k; ++i) {
-            const int e = P.E[i], q = x[i] / e;
-            t += (int64_t)q * P.gstride[i];
-            loc += (int64_t)(x[i] - q * e) * P.lst[i];
-        }
-        g = t * P.tb_block + loc;
-    } else {
-        for (int i = 0; i < P.k; ++i) g += (int64_t)x[i] * P.qstride[i];
-    }
-    return g;
+__device__ __forceinline__ int64_t axis_offset(const ProblemDesc &P, int i, int v) {
+    if (P.tb_layout != 2) return (int64_t)v * P.qstride[i];
+    const int q = v / P.E[i];
+    return (int64_t)q * P.gstride[i] * P.tb_block + (int64_t)(v - q * P.E[i]) * P.lst[i];
 }
 
-__device__ __forceinline__ int64_t forward_score(const ProblemDesc &P, const int *x, int64_t u) {
-    int64_t w = 0, s = 0;
-    for (int i = 0; i < P.k; ++i) {
-        w += (int64_t)x[i] << i;
-        s += x[i];
-    }
-    return (((int64_t)P.Q[score_cell(P, x)] - w) >> P.k) + u * s;
+__host__ __device__ constexpr int near_words(int K) { return K <= 5 ? 1 : 1 << (K - 5); }  // 32-mask rounds: lane l judges mask 32 w + l
+
+// Bytes of the walk's tables and stack (8-byte terms, hit sets, scores, codes, moves).
+size_t near_bytes(int k, int64_t len_sum) {
+    const size_t depth = (size_t)len_sum + 1;
+    return ((size_t)len_sum + k) * 8 + depth * 4 * near_words(k) + depth * 4 + (size_t)len_sum + 16 + depth + 64;
 }
 
-__global__ void __launch_bounds__(32) near_optimal_kernel(const ProblemDesc *probs, IODesc io, int64_t delta,
-                                                          int32_t max_count, NearOut o) {
+template <int K>
+__global__ void __launch_bounds__(kNearThreads) near_optimal_kernel(const ProblemDesc *probs, IODesc io, int64_t delta,
+                                                                    int32_t max_count, NearOut o, int in_smem) {
+    constexpr int NW = near_words(K), NM = 1 << K, NP = K * (K - 1) / 2;
+    extern __shared__ __align__(16) unsigned char near_smem[];
+    __shared__ int sub[MSA_MAX_ALPHABET * MSA_MAX_ALPHABET];
     const ProblemDesc &P = probs[0];
-    const int lane = threadIdx.x;
-    const int k = P.k, A = P.A, total = P.len_sum, nm = (1 << k) - 1;
+    const int lane = threadIdx.x & 31;
+    const int A = P.A, total = P.len_sum, depths = total + 1;
     if (ld_volatile(&P.istat->status) != 0) {  // the fill did not complete: nothing to enumerate
-        if (lane == 0) {
+        if (threadIdx.x == 0) {
             o.count_more[0] = 0;
             o.count_more[1] = 0;
         }
         return;
     }
-    const int64_t u = (int64_t)io.gap * (k - 1);
-    int x[MSA_MAX_K];
-    for (int i = 0; i < k; ++i) x[i] = P.len[i];
-    const int64_t thr = forward_score(P, x, u) - delta;  // OPT - delta
+    // tables: per axis the offset term of every coordinate; the residue codes; the pair scores
+    unsigned char *base = in_smem ? near_smem : o.work;
+    int64_t *off = reinterpret_cast<int64_t *>(base);
+    unsigned *hits = reinterpret_cast<unsigned *>(off + total + K);
+    int *accs = reinterpret_cast<int *>(hits + (size_t)depths * NW);
+    uint8_t *codes = reinterpret_cast<uint8_t *>(accs + depths);
+    uint8_t *path = codes + ((total + 15) & ~15);
+    int cofs[K], at[K];  // first code of sequence i, first entry of axis i in off
+#pragma unroll
+    for (int i = 0; i < K; ++i) {
+        cofs[i] = P.cofs[i];
+        at[i] = cofs[i] + i;
+    }
+#pragma unroll
+    for (int i = 0; i < K; ++i)
+        for (int v = threadIdx.x; v < P.rho[i]; v += kNearThreads) off[at[i] + v] = axis_offset(P, i, v);
+    for (int c = threadIdx.x; c < total; c += kNearThreads) codes[c] = P.codes[c];
+    for (int c = threadIdx.x; c < A * A; c += kNearThreads) sub[c] = io.subst[c];
+    __syncthreads();
+    if (threadIdx.x >= 32) return;
+
+    const int gap = io.gap, u = gap * (K - 1);
+    int x[K], S = 0, W = 0;
+    int64_t corner = 0;
+#pragma unroll
+    for (int i = 0; i < K; ++i) {
+        x[i] = P.len[i];
+        S += x[i];
+        W += x[i] << i;
+        corner += off[at[i] + x[i]];
+    }
+    const int32_t *Q = P.Q;
+    const int opt = ((Q[corner] - W) >> K) + u * S;
+    // OPT - delta (no alignment scores below the 32-bit range)
+    const int thr = delta > (int64_t)opt - INT32_MIN ? INT32_MIN : (int)(opt - delta);
     int d = 0, count = 0, more = 0;
-    int64_t acc = 0;  // score of the columns fixed so far (depth d)
-    int nxt = 1;      // next mask to try at depth d
+    int acc = 0;  // score of the columns fixed so far (depth d)
     // Every move followed leads to at least one qualifying alignment (H(p) is
-    // reached by some path), so the walk takes at most 2 (total + 1) steps per
-    // alignment it stores, plus one; the bound below only guards that argument.
-    const int64_t limit = 2 * ((int64_t)total + 1) * ((int64_t)max_count + 1) + 2;
-    for (int64_t it = 0; d >= 0; ++it) {
+    // reached by some path), so at most total + 1 nodes are judged per alignment
+    // stored, plus one walk; the bound below only guards that argument.
+    const int64_t limit = ((int64_t)total + 1) * ((int64_t)max_count + 1) + 2;
+    for (int64_t it = 0;; ++it) {
         if (it > limit) {
             more = 2;  // reported as an inconsistent tensor
             break;
         }
-        bool origin = true;
-        for (int i = 0; i < k; ++i) origin = origin && x[i] == 0;
-        int mstar = 0;
-        int64_t spstar = 0;
-        if (origin) {
-            if (count == max_count) {
-                more = 1;
-                break;
-            }
+        if (S == 0) {
+            __syncwarp();  // lane 0's moves
             uint8_t *dst = o.masks + (int64_t)count * total;
-            for (int c = lane; c < d; c += 32) dst[c] = o.path[d - 1 - c];
+            for (int c = lane; c < d; c += 32) dst[c] = path[d - 1 - c];
             if (lane == 0) {
                 o.ncols[count] = d;
                 o.scores[count] = acc;
             }
             ++count;
         } else {
-            // residues at x (the column a move consumes)
-            int code[MSA_MAX_K];
-            for (int i = 0; i < k; ++i) code[i] = x[i] >= 1 ? P.codes[P.cofs[i] + x[i] - 1] : 0;
-            for (int base = nxt; base <= nm && !mstar; base += 32) {
-                const int m = base + lane;
-                bool ok = m <= nm;
-                int64_t sp = 0;
+            // the pair scores of the residues at x and the axes that can still move
+            int open = 0, code[K];
+#pragma unroll
+            for (int i = 0; i < K; ++i) {
+                open |= (x[i] > 0) << i;
+                code[i] = codes[min(cofs[i] + max(x[i] - 1, 0), total - 1)];  // at x_i = 0 unused, but a code
+            }
+            int pair[NP];
+            {
+                int p = 0;
+#pragma unroll
+                for (int i = 0; i < K; ++i)
+#pragma unroll
+                    for (int j = i + 1; j < K; ++j) pair[p++] = sub[code[i] * A + code[j]] - 2 * gap;
+            }
+            int first = 0, spfirst = 0;
+            unsigned mine[NW];
+#pragma unroll
+            for (int w = 0; w < NW; ++w) {
+                const int m = 32 * w + lane;
+                const bool ok = m > 0 && m < NM && (m & ~open) == 0;
+                int sp = u * __popc(m);  // gap terms: u per residue, less 2 gap per pair of residues
+                int p = 0;
+                int64_t g = 0;
+#pragma unroll
+                for (int i = 0; i < K; ++i) {
+                    const int bi = (m >> i) & 1;
+                    g += off[at[i] + x[i] - (ok ? bi : 0)];
+#pragma unroll
+                    for (int j = i + 1; j < K; ++j, ++p)
+                        if (bi & (m >> j)) sp += pair[p];
+                }
+                bool hit = false;
                 if (ok) {
-                    int y[MSA_MAX_K];
-                    for (int i = 0; i < k; ++i) {
-                        const int b = (m >> i) & 1;
-                        ok = ok && (!b || x[i] >= 1);
-                        y[i] = x[i] - b;
-                    }
-                    if (ok) {
-                        for (int i = 0; i < k; ++i)
-                            for (int j = i + 1; j < k; ++j) {
-                                const int bi = (m >> i) & 1, bj = (m >> j) & 1;
-                                if (bi && bj)
-                                    sp += io.subst[code[i] * A + code[j]];
-                                else if (bi || bj)
-                                    sp += io.gap;
-                            }
-                        ok = forward_score(P, y, u) + sp + acc >= thr;
-                    }
+                    const int h = ((Q[g] - (W - m)) >> K) + u * (S - __popc(m));
+                    hit = h + sp + acc >= thr;
                 }
-                const unsigned hit = __ballot_sync(kFull, ok);
-                if (hit) {
-                    const int src = __ffs(hit) - 1;
-                    mstar = base + src;
-                    spstar = __shfl_sync(kFull, sp, src);
+                mine[w] = __ballot_sync(kFull, hit);
+                if (!first && mine[w]) {  // uniform
+                    const int l = __ffs(mine[w]) - 1;
+                    first = 32 * w + l;
+                    spfirst = __shfl_sync(kFull, sp, l);
+                    mine[w] &= mine[w] - 1;
                 }
+            }
+            if (first) {  // follow the lowest mask, the others stay on the stack
+                if (lane == 0) {
+#pragma unroll
+                    for (int w = 0; w < NW; ++w) hits[(size_t)d * NW + w] = mine[w];
+                    accs[d] = acc;
+                    path[d] = (uint8_t)first;
+                }
+#pragma unroll
+                for (int i = 0; i < K; ++i) x[i] -= (first >> i) & 1;
+                S -= __popc(first);
+                W -= first;
+                acc += spfirst;
+                ++d;
+                continue;
             }
         }
+        // back to the deepest depth with a mask left, 32 depths at a time
         __syncwarp();
-        if (mstar) {  // descend
-            if (lane == 0) {
-                o.path[d] = (uint8_t)mstar;
-                o.next[d] = mstar + 1;
-                o.acc[d] = acc;
+        int found = -1;
+        while (d > 0 && found < 0) {
+            const int j = d - 1 - lane;
+            unsigned any = 0;
+            int pm = 0;
+            if (j >= 0) {
+#pragma unroll
+                for (int w = 0; w < NW; ++w) any |= hits[(size_t)j * NW + w];
+                pm = path[j];
             }
-            for (int i = 0; i < k; ++i) x[i] -= (mstar >> i) & 1;
-            acc += spstar;
-            nxt = 1;
-            ++d;
-        } else {  // back to the previous depth (its move undone, its next mask resumed)
-            --d;
-            if (d >= 0) {
+            const unsigned has = __ballot_sync(kFull, any != 0);
+            const int n = has ? __ffs(has) : min(d, 32);  // depths to undo
+#pragma unroll
+            for (int i = 0; i < K; ++i) {
+                const unsigned moved = __ballot_sync(kFull, (pm >> i) & 1) & (n == 32 ? kFull : (1u << n) - 1);
+                x[i] += __popc(moved);
+                S += __popc(moved);
+                W += __popc(moved) << i;
+            }
+            d -= n;
+            if (has) found = d;
+        }
+        if (found < 0) break;  // nothing left
+        if (count == max_count) {
+            more = 1;
+            break;
+        }
+        // its lowest mask left: the column's score from its residues
+        int m = 0;
+#pragma unroll
+        for (int w = 0; w < NW; ++w) {
+            const unsigned h = hits[(size_t)d * NW + w];
+            if (!m && h) {
+                m = 32 * w + __ffs(h) - 1;
                 __syncwarp();
-                const int m = o.path[d];
-                for (int i = 0; i < k; ++i) x[i] += (m >> i) & 1;
-                acc = o.acc[d];
-                nxt = o.next[d];
+                if (lane == 0) hits[(size_t)d * NW + w] = h & (h - 1);
             }
         }
+        acc = accs[d] + u * __popc(m);
+#pragma unroll
+        for (int i = 0; i < K; ++i)
+#pragma unroll
+            for (int j = i + 1; j < K; ++j)
+                if ((m >> i) & (m >> j) & 1)
+                    acc += sub[codes[cofs[i] + x[i] - 1] * A + codes[cofs[j] + x[j] - 1]] - 2 * gap;
         __syncwarp();
+        if (lane == 0) path[d] = (uint8_t)m;
+#pragma unroll
+        for (int i = 0; i < K; ++i) x[i] -= (m >> i) & 1;
+        S -= __popc(m);
+        W -= m;
+        ++d;
     }
     if (lane == 0) {
         o.count_more[0] = count;
@@ -155,10 +245,36 @@ __global__ void __launch_bounds__(32) near_optimal_kernel(const ProblemDesc *pro
     }
 }
 
-cudaError_t launch_near_optimal(const ProblemDesc *d_prob, IODesc io, int64_t delta, int32_t max_count, NearOut o,
-                                cudaStream_t s) {
-    near_optimal_kernel<<<1, 32, 0, s>>>(d_prob, io, delta, max_count, o);
+template <int K>
+cudaError_t launch_near(const ProblemDesc *d_prob, IODesc io, int64_t delta, int32_t max_count, NearOut o, size_t bytes,
+                        cudaStream_t s) {
+    const int in_smem = bytes <= (size_t)kNearSmem;
+    cudaError_t e = cudaFuncSetAttribute(near_optimal_kernel<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, kNearSmem);
+    if (e != cudaSuccess) return e;
+    near_optimal_kernel<K><<<1, kNearThreads, in_smem ? bytes : 0, s>>>(d_prob, io, delta, max_count, o, in_smem);
     return cudaGetLastError();
+}
+
+}  // namespace
+
+size_t near_optimal_work_bytes(int k, int64_t len_sum) {
+    const size_t b = near_bytes(k, len_sum);
+    return b <= (size_t)kNearSmem ? 0 : b;
+}
+
+cudaError_t launch_near_optimal(int k, int64_t len_sum, const ProblemDesc *d_prob, IODesc io, int64_t delta,
+                                int32_t max_count, NearOut o, cudaStream_t s) {
+    const size_t bytes = near_bytes(k, len_sum);
+    switch (k) {
+        case 2: return launch_near<2>(d_prob, io, delta, max_count, o, bytes, s);
+        case 3: return launch_near<3>(d_prob, io, delta, max_count, o, bytes, s);
+        case 4: return launch_near<4>(d_prob, io, delta, max_count, o, bytes, s);
+        case 5: return launch_near<5>(d_prob, io, delta, max_count, o, bytes, s);
+        case 6: return launch_near<6>(d_prob, io, delta, max_count, o, bytes, s);
+        case 7: return launch_near<7>(d_prob, io, delta, max_count, o, bytes, s);
+        case 8: return launch_near<8>(d_prob, io, delta, max_count, o, bytes, s);
+        default: return cudaErrorInvalidValue;
+    }
 }
 
 }  // namespace msadp

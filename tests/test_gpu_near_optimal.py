@@ -70,3 +70,15 @@ def test_bad_arguments():
     with pytest.raises(msa.MsaError) as ei:
         msadp.msa_near_optimal(p.seqs, p.alphabet, p.subst, p.gap, 0, 0)
     assert ei.value.code == msa.MSA_EINVAL
+
+
+@pytest.mark.parametrize("lens", [(3, 2, 2, 3, 2, 3), (2, 2, 1, 2, 2, 1, 2), (1, 2, 1, 1, 2, 1, 1, 2)])
+def test_more_masks_than_lanes(lens):
+    """k = 6 .. 8: a node's masks take two, four and eight rounds of 32."""
+    for seed, delta, count in [(8500, 0, 60), (8501, 3, 200)]:
+        check(inputs.random_problem(seed + len(lens), len(lens), list(lens), table=PAPER_TABLE, gap=-1), delta, count)
+
+
+def test_stack_beyond_shared_memory():
+    """Sequences whose tables and stack do not fit in shared memory (kept in global memory)."""
+    check(inputs.random_problem(8600, 2, [4700, 4650], alphabet=inputs.PROTEIN, related=True), 2, 40)
