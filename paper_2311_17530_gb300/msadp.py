@@ -143,8 +143,9 @@ def _i32(values) -> ctypes.Array:
 
 
 def _table(subst) -> ctypes.Array:
-    t = np.ascontiguousarray(np.asarray(subst, dtype=np.int64).reshape(-1))
-    return _i32(t.tolist())
+    # one array conversion: element by element it was two thirds of a submit's 50 us (20 letters)
+    t = np.asarray(subst, dtype=np.int64).reshape(-1).astype(np.int32)
+    return (ctypes.c_int32 * t.size).from_buffer(t) if t.size else _i32([])
 
 
 def _rows(buf: bytes, k: int, stride: int) -> List[str]:
@@ -186,18 +187,19 @@ def msa_near_optimal(seqs: Sequence[str], alphabet: str, subst, gap: int, delta:
     _check(L.msa_near_optimal(k, arr, lens, alphabet.encode(), _table(subst), int(gap), int(delta), int(max_count),
                               masks.ctypes.data, ncols.ctypes.data, scores.ctypes.data, ctypes.byref(count),
                               ctypes.byref(more)))
+    # all rows at once: a consumed residue is the sequence's next one, so column c of row i takes
+    # residue (number of moves of i up to c) - 1 (column by column this was 14 ms for 256 alignments)
+    n = count.value
+    used = np.arange(masks.shape[1]) < ncols[:n, None]
+    rows = []
+    for i, s in enumerate(enc):
+        moved = ((masks[:n] >> i) & 1 != 0) & used
+        text = np.frombuffer(s + b"-", dtype=np.uint8)[np.cumsum(moved, axis=1) - 1]
+        rows.append(np.where(moved, text, np.uint8(ord("-"))))
     out = []
-    for a in range(count.value):
-        ms = [int(m) for m in masks[a, : ncols[a]]]
-        rows, pos = [[] for _ in range(k)], [0] * k
-        for m in ms:
-            for i in range(k):
-                if (m >> i) & 1:
-                    rows[i].append(seqs[i][pos[i]])
-                    pos[i] += 1
-                else:
-                    rows[i].append("-")
-        out.append((int(scores[a]), ms, ["".join(r) for r in rows]))
+    for a in range(n):
+        c = int(ncols[a])
+        out.append((int(scores[a]), masks[a, :c].tolist(), [r[a, :c].tobytes().decode() for r in rows]))
     return out, bool(more.value)
 
 
