@@ -111,18 +111,19 @@ int msa_near_optimal(int k, const char *const *seqs, const int32_t *lens, const 
  * where an optimal alignment can lie). Any alignment through cell x scores at
  * most U(x) = sum over pairs i < j of fwd_ij(x_i, x_j) + bwd_ij(x_i, x_j), the
  * optimal pairwise scores of the prefixes and suffixes (Eq. 1 on each pair; gap
- * against gap scores 0, section 5.2). The fill is the generic tile kernel; a
- * tile whose bound -- the sum over pairs of the largest fwd + bwd over the tile's
- * rectangle -- is below a lower bound L on the optimum holds no cell of an
- * optimal alignment and is left out. The score and alignment equal msa_align's
- * (the same tie rule) whenever L does not exceed the optimum.
+ * against gap scores 0, section 5.2). A tile of the generic tile kernel whose
+ * bound -- the sum over pairs of the largest fwd + bwd over the tile's rectangle
+ * -- is below a lower bound L on the optimum holds no cell of an optimal
+ * alignment: the fill may leave it out, and does (with that kernel) where this is
+ * faster than a kernel that fills every cell. The score and alignment equal
+ * msa_align's (the same tie rule) whenever L does not exceed the optimum.
  *
  *   have_lower_bound  0: L is the score of a feasible alignment the device builds
  *                     from the origin, taking at each cell the move to the
  *                     neighbour with the largest U (ties: lowest mask);
  *                     1: L = lower_bound (e.g. the score of a heuristic alignment)
  *   out_score, out_alignment  as for msa_align
- *   out_stats         (may be NULL) the bound used and what was left out
+ *   out_stats         (may be NULL) the bound used and what it leaves out
  *
  * Sequences of at most 16383 residues. Host buffers; allocates device memory for
  * the call; synchronous. MSA_EINVAL also when a given lower bound exceeds the
@@ -130,8 +131,8 @@ int msa_near_optimal(int k, const char *const *seqs, const int32_t *lens, const 
  */
 typedef struct msa_prune_stats {
     int64_t lower_bound;   /* L */
-    int64_t tiles;         /* tiles of the fill */
-    int64_t tiles_skipped; /* tiles left out */
+    int64_t tiles;         /* tiles of the generic tile kernel */
+    int64_t tiles_skipped; /* tiles the bound leaves out */
     int64_t cells_skipped; /* cells of the tensor in them */
     int64_t cells;         /* cells of the tensor */
 } msa_prune_stats;

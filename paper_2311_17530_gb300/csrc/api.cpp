@@ -384,17 +384,6 @@ extern "C" {
 
 int msa_plan_execute(msa_plan *plan, const char *d_residues, const int32_t *d_subst, int32_t gap,
                      msa_device_result *d_result, uint8_t *d_masks, void *stream) {
-    return msadp::run_plan(plan, d_residues, d_subst, gap, d_result, d_masks, stream, nullptr);
-}
-
-}  // extern "C"
-
-namespace msadp {
-
-// msa_plan_execute's steps; with `prune`, its kernels run between the encode
-// step and the fill (the plan's problem descriptor then points at prune->skip).
-int run_plan(msa_plan *plan, const char *d_residues, const int32_t *d_subst, int32_t gap, msa_device_result *d_result,
-             uint8_t *d_masks, void *stream, const PruneDesc *prune) {
     if (!plan || !d_subst || !d_result || (plan->hp.len_sum > 0 && (!d_residues || !d_masks)))
         return set_error(MSA_EINVAL, "NULL plan or device pointer");
     cudaStream_t s = (cudaStream_t)stream;
@@ -423,10 +412,6 @@ int run_plan(msa_plan *plan, const char *d_residues, const int32_t *d_subst, int
     IODesc io{d_residues, d_subst, d_result, d_masks, gap, 0};
     e = launch_encode(plan->pp.prob, 1, plan->hp.len_sum, nullptr, io, s);
     if (e != cudaSuccess) return cuda_error(e, "encode launch");
-    if (prune) {
-        e = launch_prune(*prune, prune->greedy != 0, s);
-        if (e != cudaSuccess) return cuda_error(e, "pruning kernels");
-    }
     LaunchDesc L;
     memset(&L, 0, sizeof L);
     L.probs = plan->pp.prob;
@@ -460,10 +445,6 @@ int run_plan(msa_plan *plan, const char *d_residues, const int32_t *d_subst, int
     }
     return MSA_OK;
 }
-
-}  // namespace msadp
-
-extern "C" {
 
 int msa_plan_timings(msa_plan *plan, float out_ms[3]) {
     if (!plan || !out_ms) return set_error(MSA_EINVAL, "NULL plan or output");
@@ -808,13 +789,18 @@ size_t prune_layout(const HostPlan &hp, const int32_t *E, char *base, PruneDesc 
     return o;
 }
 
-// Shared set-up: request checks, a generic-tile-kernel plan, the pruning
-// descriptor, one device buffer holding inputs, outputs and the pruning arrays.
+// Shared set-up: request checks, the generic tile kernel's tile grid, the pruning
+// descriptor, one device buffer holding inputs, outputs, the pruning arrays and what
+// the encode step needs (a problem descriptor without tensors).
 struct PruneRun {
     msa_plan *plan = nullptr;
+    HostPlan hp;      // shape and tile grid of the generic tile kernel
+    PlanPointers pp;  // of the descriptor
+    size_t reset_bytes = 0;
+    char *ws = nullptr;
     char *d = nullptr;
     PruneDesc D;
-    size_t o_res = 0, o_sub = 0, o_out = 0, o_masks = 0, o_prune = 0;
+    size_t o_res = 0, o_sub = 0, o_out = 0, o_masks = 0, o_prune = 0, o_ws = 0;
     ~PruneRun() {
         if (d) cudaFree(d);
         if (plan) msa_plan_destroy(plan);
@@ -828,12 +814,16 @@ int prune_setup(int k, const char *const *seqs, const int32_t *lens, const char 
     if (rc) return rc;
     for (int i = 0; i < k; ++i)
         if (lens[i] > 16383) return set_error(MSA_ETOOBIG, "pruning takes sequences of at most 16383 residues");
-    rc = plan_create(k, lens, alphabet, kKernelTiles, -1, &R.plan);
-    if (rc) return rc;
-    const HostPlan &hp = R.plan->hp;
+    std::string err;
+    rc = plan_shape(k, lens, (int)strlen(alphabet), kKernelTiles, R.hp, err);
+    if (rc) return set_error(rc, "%s", err.c_str());
+    const HostPlan &hp = R.hp;
     if (E)
         for (int i = 0; i < k; ++i)
             if (E[i] < 1) return set_error(MSA_EINVAL, "tile extent %d of axis %d is below 1", E[i], i);
+    HostPlan bare = hp;  // no tickets, no tensors
+    bare.ntiles = bare.tb_dev_bytes = bare.qelems = bare.aux_elems = 0;
+    const size_t wbytes = plan_layout(bare, nullptr, nullptr, &R.reset_bytes);
     const size_t pbytes = prune_layout(hp, E ? E : hp.E, nullptr, R.D);
     const size_t total = (size_t)hp.len_sum, A = (size_t)hp.A;
     size_t off = 0;
@@ -846,6 +836,7 @@ int prune_setup(int k, const char *const *seqs, const int32_t *lens, const char 
     R.o_sub = take(A * A * 4);
     R.o_out = take(sizeof(msa_device_result));
     R.o_masks = take(total + 16);
+    R.o_ws = take(wbytes);
     R.o_prune = take(pbytes);
     cudaError_t e = cudaMalloc(&R.d, off);
     if (e != cudaSuccess) {
@@ -853,8 +844,11 @@ int prune_setup(int k, const char *const *seqs, const int32_t *lens, const char 
         R.d = nullptr;
         return set_error(MSA_ENOMEM, "pruning buffers: %s", cudaGetErrorString(e));
     }
+    R.ws = R.d + R.o_ws;
+    size_t rb = 0;
+    plan_layout(bare, R.ws, &R.pp, &rb);
     prune_layout(hp, E ? E : hp.E, R.d + R.o_prune, R.D);
-    R.D.codes = R.plan->pp.codes;
+    R.D.codes = R.pp.codes;
     R.D.sub = reinterpret_cast<const int32_t *>(R.d + R.o_sub);
     std::vector<char> res(total + 1);
     size_t o = 0;
@@ -862,12 +856,31 @@ int prune_setup(int k, const char *const *seqs, const int32_t *lens, const char 
         if (lens[i]) memcpy(res.data() + o, seqs[i], (size_t)lens[i]);
         o += (size_t)lens[i];
     }
+    ProblemDesc pd;
+    fill_problem_desc(bare, R.pp, 0, pd);
     e = cudaMemcpy(R.d + R.o_res, res.data(), total, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(R.d + R.o_sub, subst, A * A * 4, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(R.pp.prob, &pd, sizeof pd, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(R.pp.amap, amap, 256, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemset(R.D.stats, 0, 16);
     if (e != cudaSuccess) return cuda_error(e, "pruning inputs");
     return MSA_OK;
 }
+
+// The encode step and the pruning kernels, on the set-up's own descriptor.
+cudaError_t prune_analyse(PruneRun &R, const IODesc &io, cudaStream_t s) {
+    cudaError_t e = cudaMemsetAsync(R.ws, 0, R.reset_bytes, s);
+    if (e == cudaSuccess) e = launch_encode(R.pp.prob, 1, R.hp.len_sum, nullptr, io, s);
+    if (e == cudaSuccess) e = launch_prune(R.D, R.D.greedy != 0, s);
+    return e;
+}
+
+// k = 5, 6: the share of a tensor's cells that must be left out for the generic
+// tile kernel, which skips them, to beat the line kernels, which fill everything
+// (one call, k = 5 at 0.78 left out 2.4 against 3.0 ms, k = 6 at 1.0 2.4 against
+// 4.9 ms; of whole tensors the line kernels are 2.3 to 4 times as fast). k = 4: the
+// streamed kernel is faster even at 0.98 left out (1.2 against 1.6 ms).
+constexpr double kPruneTilesShare = 0.65;
 
 }  // namespace
 
@@ -878,34 +891,57 @@ int msa_align_pruned(int k, const char *const *seqs, const int32_t *lens, const 
     PruneRun R;
     int rc = prune_setup(k, seqs, lens, alphabet, subst, nullptr, R);
     if (rc) return rc;
-    const HostPlan &hp = R.plan->hp;
+    const HostPlan &hp = R.hp;
     R.D.gap = gap;
     R.D.greedy = have_lower_bound ? 0 : 1;
     R.D.bound = nullptr;
     cudaError_t e = cudaMemcpy(R.D.lower, &lower_bound, 8, cudaMemcpyHostToDevice);
-    // the fill reads the tiles' flags through the plan's problem descriptor
-    ProblemDesc pd;
-    fill_problem_desc(hp, R.plan->pp, 0, pd);
-    pd.skip = R.D.skip;
-    if (e == cudaSuccess) e = cudaMemcpy(R.plan->pp.prob, &pd, sizeof pd, cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return cuda_error(e, "pruning set-up");
     cudaStream_t s = library_stream(&rc);
     if (rc) return rc;
     msa_device_result *d_res = reinterpret_cast<msa_device_result *>(R.d + R.o_out);
     uint8_t *d_masks = reinterpret_cast<uint8_t *>(R.d + R.o_masks);
-    rc = run_plan(R.plan, R.d + R.o_res, R.D.sub, gap, d_res, d_masks, s, &R.D);
+    e = prune_analyse(R, IODesc{R.d + R.o_res, R.D.sub, d_res, d_masks, gap, 0}, s);
+    if (e != cudaSuccess) return cuda_error(e, "pruning kernels");
+    // The fill: a tile left out saves work, but a fill bound by its chain of waves
+    // gains little from it, and the generic tile kernel that can leave tiles out is
+    // the slowest per cell. k = 2 and 3: always the band and column kernels (k = 3,
+    // 700 / 760 / 800 with 98 % of the tiles left out: 0.64 ms against 6.4 ms).
+    // k = 4: always the streamed kernel; k = 5, 6: the line kernels unless enough is
+    // left out.
+    int kernel = choose_kernel(k, lens, hp.A, kKernelAuto);
+    int64_t st[2] = {0, 0};
+    if (k > 4 && kernel != kKernelTiles) {
+        e = cudaStreamSynchronize(s);
+        if (e == cudaSuccess) e = cudaMemcpy(st, R.D.stats, 16, cudaMemcpyDeviceToHost);
+        if (e != cudaSuccess) return cuda_error(e, "pruning kernels");
+        if ((double)st[1] > kPruneTilesShare * (double)hp.cells) kernel = kKernelTiles;
+    }
+    if (kernel != kKernelTiles && plan_create(k, lens, alphabet, kernel, -1, &R.plan) != MSA_OK) kernel = kKernelTiles;
+    if (kernel == kKernelTiles) {
+        rc = plan_create(k, lens, alphabet, kKernelTiles, -1, &R.plan);
+        if (rc) return rc;
+        // the fill reads the tiles' flags through the plan's problem descriptor
+        ProblemDesc pd;
+        fill_problem_desc(R.plan->hp, R.plan->pp, 0, pd);
+        pd.skip = R.D.skip;
+        e = cudaMemcpy(R.plan->pp.prob, &pd, sizeof pd, cudaMemcpyHostToDevice);
+        if (e != cudaSuccess) return cuda_error(e, "pruning set-up");
+    }
+    rc = msa_plan_execute(R.plan, R.d + R.o_res, R.D.sub, gap, d_res, d_masks, s);
     if (rc) return rc;
     e = cudaStreamSynchronize(s);
     msa_device_result res;
-    int64_t L = 0, st[2] = {0, 0};
+    int64_t L = 0;
     std::vector<uint8_t> masks((size_t)hp.len_sum + 1);
     if (e == cudaSuccess) e = cudaMemcpy(&res, d_res, sizeof res, cudaMemcpyDeviceToHost);
     if (e == cudaSuccess) e = cudaMemcpy(&L, R.D.lower, 8, cudaMemcpyDeviceToHost);
     if (e == cudaSuccess) e = cudaMemcpy(st, R.D.stats, 16, cudaMemcpyDeviceToHost);
     if (e == cudaSuccess) e = cudaMemcpy(masks.data(), d_masks, (size_t)hp.len_sum, cudaMemcpyDeviceToHost);
     if (e != cudaSuccess) return cuda_error(e, "pruning results");
-    // a bound above the optimum leaves out tiles of every optimal alignment: the
-    // corner is then unreachable or its best kept path scores below the bound
+    // A bound above the optimum leaves out tiles of every optimal alignment: the
+    // corner is then unreachable or its best kept path scores below the bound (a
+    // fill of everything finds the optimum itself, below the bound).
     if (have_lower_bound && (res.status != MSA_OK || res.score < lower_bound))
         return set_error(MSA_EINVAL, "lower bound %lld exceeds the optimum", (long long)lower_bound);
     rc = status_error(res.status);
@@ -935,12 +971,10 @@ int msa_tile_bounds(int k, const char *const *seqs, const int32_t *lens, const c
     if (rc) return rc;
     IODesc io{R.d + R.o_res, R.D.sub, reinterpret_cast<msa_device_result *>(R.d + R.o_out),
               reinterpret_cast<uint8_t *>(R.d + R.o_masks), gap, 0};
-    cudaError_t e = cudaMemsetAsync(R.plan->ws, 0, R.plan->reset_bytes, s);
-    if (e == cudaSuccess) e = launch_encode(R.plan->pp.prob, 1, R.plan->hp.len_sum, nullptr, io, s);
-    if (e == cudaSuccess) e = launch_prune(R.D, false, s);
+    cudaError_t e = prune_analyse(R, io, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     msa_device_result st;
-    if (e == cudaSuccess) e = cudaMemcpy(&st, &R.plan->pp.state->istat, sizeof st, cudaMemcpyDeviceToHost);
+    if (e == cudaSuccess) e = cudaMemcpy(&st, &R.pp.state->istat, sizeof st, cudaMemcpyDeviceToHost);
     if (e != cudaSuccess) return cuda_error(e, "tile bounds");
     rc = status_error(st.status);
     if (rc) return rc;

@@ -104,3 +104,45 @@ def test_bound_above_the_optimum_is_reported():
     with pytest.raises(msa.MsaError) as ei:
         msadp.msa_align_pruned(p.seqs, p.alphabet, p.subst, p.gap, lower_bound=want.score + 1000)
     assert ei.value.code == msa.MSA_EINVAL
+
+
+@pytest.mark.parametrize("lens", [(1024, 33), (1023, 31), (1100, 1090), (64, 63), (127, 130), (130, 150, 140), (65, 20, 90, 22),
+                                  (8, 9, 7, 8, 9, 8), (6, 5, 6, 7, 5, 6, 6), (4, 5, 4, 3, 4, 5, 4, 4)])
+def test_passes_boxes_and_mask_rounds(lens):
+    """The edges of the pair tables' passes (1024 rows), warps (128 rows) and chunks
+    (32 columns), of the greedy walk's boxes and of its rounds of 32 masks (k >= 6)."""
+    for seed, related in ((9300, True), (9301, False)):
+        p = inputs.random_problem(seed + len(lens), len(lens), list(lens), alphabet=inputs.PROTEIN, related=related)
+        ext = plan_extents(p.k, p.lens)[0]
+        np.testing.assert_array_equal(msadp.msa_tile_bounds(p.seqs, p.alphabet, p.subst, p.gap, ext),
+                                      oracle.tile_bounds(p.seqs, p.alphabet, p.subst, p.gap, ext).reshape(-1))
+        want = oracle.align_problem(p)
+        score, rows, st = msadp.msa_align_pruned(p.seqs, p.alphabet, p.subst, p.gap)
+        assert (score, rows) == (want.score, want.rows), p.name
+        assert st["lower_bound"] <= want.score
+        # the walk takes the largest U at every step: its score is the oracle's lower-bound walk's, cell by cell
+        assert st["lower_bound"] == greedy_score(p)
+
+
+def greedy_score(p):
+    """The greedy feasible alignment's score from the oracle's pairwise tables."""
+    import itertools
+    k, lens = p.k, p.lens
+    fb = {(i, j): np.add(*oracle.pair_tables(p.seqs[i], p.seqs[j], p.alphabet, p.subst, p.gap)[:2])
+          for i, j in itertools.combinations(range(k), 2)}
+    x, score = [0] * k, 0
+    while x != list(lens):
+        best = None
+        for m in range(1, 1 << k):
+            y = [v + (m >> i & 1) for i, v in enumerate(x)]
+            if any(v > n for v, n in zip(y, lens)):
+                continue
+            u = sum(int(t[y[i], y[j]]) for (i, j), t in fb.items())
+            if best is None or u > best[0]:
+                best = (u, m, y)
+        _, m, x = best
+        for i, j in fb:
+            a, b = m >> i & 1, m >> j & 1
+            score += (int(p.subst[p.alphabet.index(p.seqs[i][x[i] - 1]), p.alphabet.index(p.seqs[j][x[j] - 1])])
+                      if a and b else p.gap if a or b else 0)
+    return score
