@@ -293,8 +293,8 @@ int msa_plan_timings(msa_plan *plan, float out_ms[3]);
  * the size they would need. The first call on each device looks up the array's
  * device address; make that first call before any stream capture. Every call
  * reuses the same array: calls whose GPU work overlaps (different streams or
- * threads) race on it and must be serialised by the caller. Always uses the
- * generic tile fill.
+ * threads) race on it and must be serialised by the caller. Uses the band, column
+ * or line kernel where its working set fits the array, else the generic tile fill.
  */
 #define MSA_NOALLOC_SCRATCH_BYTES (32u * 1024u * 1024u)
 int msa_align_noalloc(int k, const int32_t *lens, const char *alphabet, const char *d_residues,

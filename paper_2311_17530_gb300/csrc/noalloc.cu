@@ -31,21 +31,30 @@ constexpr int kMaxDevices = 64;
 std::mutex g_na_mu;
 void *g_na_ptr[kMaxDevices] = {};
 
-// Wave order of the tiles, built on the device: count tiles per wave, prefix
+// The 256-entry character -> code map, passed by value to the set-up kernel.
+struct AmapBytes {
+    uint8_t m[256];
+};
+
+// One block writes the problem descriptor and the character map into the scratch
+// (both travel as kernel parameters, so no host memory is read after the call
+// returns: no copy from pageable memory, which would block and could not be
+// captured) and builds the wave order of the tiles: count tiles per wave, prefix
 // sums, then scatter (any order inside a wave keeps the order topological).
-__global__ void noalloc_order_kernel(const ProblemDesc *prob, uint64_t *order, int32_t *wave_cnt, int nwaves) {
-    const ProblemDesc &P = *prob;
-    const int64_t nt = P.ntiles;
-    for (int64_t t = threadIdx.x; t < nt; t += blockDim.x) {
-        int64_t rem = t;
+__global__ void noalloc_setup_kernel(const ProblemDesc P, const AmapBytes a, ProblemDesc *prob, uint8_t *amap,
+                                     uint64_t *order, int32_t *wave_cnt, int nwaves) {
+    if (threadIdx.x == 0) *prob = P;
+    for (int i = threadIdx.x; i < 256; i += blockDim.x) amap[i] = a.m[i];
+    auto wave_of = [&](int64_t t) {
         int w = 0;
         for (int i = 0; i < P.k; ++i) {
-            const int64_t c = rem / P.gstride[i];
-            rem -= c * P.gstride[i];
+            const int64_t c = t / P.gstride[i];
+            t -= c * P.gstride[i];
             w += (int)c;
         }
-        atomicAdd(&wave_cnt[w], 1);
-    }
+        return w;
+    };
+    for (int64_t t = threadIdx.x; t < P.ntiles; t += blockDim.x) atomicAdd(&wave_cnt[wave_of(t)], 1);
     __syncthreads();
     if (threadIdx.x == 0) {
         int acc = 0;
@@ -56,29 +65,7 @@ __global__ void noalloc_order_kernel(const ProblemDesc *prob, uint64_t *order, i
         }
     }
     __syncthreads();
-    for (int64_t t = threadIdx.x; t < nt; t += blockDim.x) {
-        int64_t rem = t;
-        int w = 0;
-        for (int i = 0; i < P.k; ++i) {
-            const int64_t c = rem / P.gstride[i];
-            rem -= c * P.gstride[i];
-            w += (int)c;
-        }
-        order[atomicAdd(&wave_cnt[w], 1)] = (uint64_t)t;
-    }
-}
-
-// The 256-entry character -> code map, passed by value to the set-up kernel.
-struct AmapBytes {
-    uint8_t m[256];
-};
-
-// Writes the problem descriptor and the character map into the scratch. Both
-// travel as kernel parameters, so no host memory is read after the call returns
-// (no copy from pageable memory, which would block and could not be captured).
-__global__ void noalloc_setup_kernel(const ProblemDesc d, const AmapBytes a, ProblemDesc *prob, uint8_t *amap) {
-    if (threadIdx.x == 0) *prob = d;
-    for (int i = threadIdx.x; i < 256; i += blockDim.x) amap[i] = a.m[i];
+    for (int64_t t = threadIdx.x; t < P.ntiles; t += blockDim.x) order[atomicAdd(&wave_cnt[wave_of(t)], 1)] = (uint64_t)t;
 }
 
 // Shape, strides and tile grid of the generic tile kernel: the planner's own
@@ -97,6 +84,12 @@ int noalloc_plan(int k, const int32_t *lens, int A, HostPlan &hp) {
     const int rc = plan_shape(k, lens, A, kKernelTiles, hp, err, tile_edge_for(k));
     if (rc) return set_error(rc, "msa_align_noalloc: %s", err.c_str());
     return MSA_OK;
+}
+
+// Bytes of the scratch a plan takes; wave_off: where its wave counters lie.
+size_t noalloc_need(const HostPlan &hp, size_t &wave_off, size_t &reset_bytes) {
+    wave_off = (plan_layout(hp, nullptr, nullptr, &reset_bytes) + 255) & ~(size_t)255;
+    return wave_off + (size_t)hp.waves * 4;
 }
 
 }  // namespace
@@ -118,14 +111,28 @@ extern "C" int msa_align_noalloc(int k, const int32_t *lens, const char *alphabe
     if (rc) return rc;
     if (hp.len_sum > 0 && (!d_residues || !d_masks)) return set_error(MSA_EINVAL, "NULL residues or masks");
 
-    size_t reset_bytes = 0;
-    const size_t layout = plan_layout(hp, nullptr, nullptr, &reset_bytes);
-    const size_t wave_off = (layout + 255) & ~(size_t)255;
-    const size_t need = wave_off + (size_t)hp.waves * 4;
+    // What is accepted is what fits with the generic tile fill.
+    size_t reset_bytes = 0, wave_off = 0;
+    const size_t need = noalloc_need(hp, wave_off, reset_bytes);
     if (need > MSA_NOALLOC_SCRATCH_BYTES)
         return set_error(MSA_ETOOBIG, "msa_align_noalloc: this problem needs %zu bytes of scratch; the static "
                                       "array holds %u bytes",
                          need, (unsigned)MSA_NOALLOC_SCRATCH_BYTES);
+    // The band, column or line kernel where its working set fits too (k = 3 protein,
+    // 120 x 110 x 130, the whole call: 0.24 ms against 0.96 ms with the tile fill). Not the streamed line
+    // kernel, whose faces would have to be cleared at 8 bytes a cell.
+    const int choice = choose_kernel(k, lens, A, kKernelAuto, false);
+    if (choice != kKernelTiles) {
+        HostPlan fast;
+        std::string err;
+        size_t reset2 = 0, wave2 = 0;
+        if (plan_shape(k, lens, A, choice, fast, err, -1, false) == MSA_OK &&
+            noalloc_need(fast, wave2, reset2) <= MSA_NOALLOC_SCRATCH_BYTES) {
+            hp = fast;
+            reset_bytes = reset2;
+            wave_off = wave2;
+        }
+    }
 
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -138,6 +145,8 @@ extern "C" int msa_align_noalloc(int k, const int32_t *lens, const char *alphabe
             void *ptr = nullptr;
             e = cudaGetSymbolAddress(&ptr, g_noalloc_scratch);
             if (e != cudaSuccess) return cuda_error(e, "cudaGetSymbolAddress of the static scratch");
+            e = prepare_kernel_attributes();  // later calls, of any k, may run inside a stream capture
+            if (e != cudaSuccess) return cuda_error(e, "kernel attributes");
             g_na_ptr[dev] = ptr;
         }
         base = static_cast<char *>(g_na_ptr[dev]);
@@ -149,6 +158,9 @@ extern "C" int msa_align_noalloc(int k, const int32_t *lens, const char *alphabe
     int32_t *wave_cnt = reinterpret_cast<int32_t *>(base + wave_off);
     ProblemDesc d;
     fill_problem_desc(hp, pp, 0, d);
+    // tagged faces: the encode step clears them, so that no word of an earlier call
+    // passes for an entry of this one
+    d.clear_faces = tagged_faces(hp.kernel) ? 1 : 0;
     cudaStream_t s = (cudaStream_t)stream;
     int64_t spin_ms;
     {
@@ -162,28 +174,28 @@ extern "C" int msa_align_noalloc(int k, const int32_t *lens, const char *alphabe
     if (e != cudaSuccess) return cuda_error(e, "static scratch set-up");
     AmapBytes am;
     memcpy(am.m, amap, 256);
-    noalloc_setup_kernel<<<1, 256, 0, s>>>(d, am, pp.prob, pp.amap);
+    noalloc_setup_kernel<<<1, 1024, 0, s>>>(d, am, pp.prob, pp.amap, pp.order, wave_cnt, hp.waves);
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_error(e, "set-up kernel launch");
-    noalloc_order_kernel<<<1, 1024, 0, s>>>(pp.prob, pp.order, wave_cnt, hp.waves);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return cuda_error(e, "order kernel launch");
     IODesc io{d_residues, d_subst, d_result, d_masks, gap, 0};
-    e = launch_encode(pp.prob, 1, hp.len_sum, nullptr, io, s);
+    e = launch_encode(pp.prob, 1, hp.len_sum, nullptr, io, s, d.clear_faces ? 64 : 1);
     if (e != cudaSuccess) return cuda_error(e, "encode launch");
     LaunchDesc L;
     memset(&L, 0, sizeof L);
     L.probs = pp.prob;
     L.order = pp.order;
-    L.ntickets = hp.ntiles;
+    L.ntickets = hp.nunits;
     L.done = pp.done;
     L.ticket = &pp.state->ticket;
     L.err = &pp.state->err;
     L.spin_ns = spin_ms * 1000000LL;
     L.withhold = -1;
     L.nprob = 1;
-    e = launch_fill_tiles(k, hp.edge, L, persistent_grid(k, kKernelTiles, hp.ntiles, A, hp.edge), s);
-    if (e != cudaSuccess) return cuda_error(e, "fill launch");
+    L.tab_ints = A * (A + 1);
+    L.epoch = 1;
+    L.corner = hp.check_corner;
+    rc = launch_fill(hp, L, persistent_grid(k, hp.kernel, hp.nunits, A, hp.edge), s);
+    if (rc) return rc;
     e = launch_traceback(pp.prob, 1, L.err, nullptr, io, s);
     if (e != cudaSuccess) return cuda_error(e, "traceback launch");
     return MSA_OK;

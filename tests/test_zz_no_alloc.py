@@ -112,3 +112,14 @@ def test_noalloc_rejects_problems_beyond_its_scratch():
                                 d_result.data_ptr(), d_masks.data_ptr(), _stream())
     assert ei.value.code == msa.MSA_ETOOBIG
     assert "needs" in str(ei.value)
+
+
+@pytest.mark.parametrize("lens", [(0, 0), (0, 5), (127, 128), (129, 40), (1600, 1700), (31, 31, 31), (32, 33, 0), (64, 65, 130),
+                                  (7, 3, 4, 70), (8, 8, 8, 8), (4, 5, 2, 3, 40), (3, 3, 3, 2, 3, 30), (3, 2, 3, 2, 3, 2, 3)])
+def test_noalloc_over_its_kernels(lens):
+    """Band, column, line and tile kernels on the scratch that the call before left
+    behind (an alphabet of 25 letters takes k = 3 to the tile kernel)."""
+    for alphabet in (inputs.DNA, inputs.PROTEIN, inputs.PROTEIN + "BJOUX"):
+        p = inputs.random_problem(46 + len(lens), len(lens), list(lens), alphabet=alphabet, related=True)
+        want = oracle.align_problem(p)
+        assert _noalloc(p) == (want.score, want.rows, 0), (p.name, alphabet)
