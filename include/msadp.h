@@ -170,13 +170,15 @@ int msa_set_stream(void *stream);
  *                       request, in arrival order (default 1)
  *   "fill_kernel"       0: automatic; 1: generic tile kernel; 2: k=3 column kernel;
  *                       3: k=2 band kernel; 4: k=4..6 line kernel (segments of the
- *                       last axis); 5: k=4..6 streamed line kernel (a CTA sweeps a
+ *                       last axis); 5: k=4..8 streamed line kernel (a CTA sweeps a
  *                       super-block of 32-line blocks over the whole last axis; at
  *                       k=6 the whole-column form when the last axis holds at most
- *                       25 positions, the pipelined form otherwise). The automatic
- *                       choice is 5 at k=4,5 and at k=6 for a last axis of at most 25
- *                       positions, else 4 (until msa_autotune picks otherwise); the
- *                       serving loop runs 4 where 5 would be chosen or asked for
+ *                       25 positions, the pipelined form otherwise; at k=7, 8 the
+ *                       whole-column form for at most 13 and 9 positions, else 1).
+ *                       The automatic choice is 5 at k=4,5 and where the whole-column
+ *                       form fits, else 4 at k=6 and 1 at k=7,8 (until msa_autotune
+ *                       or, at k=7,8, msa_set_tile_edge picks otherwise); the serving
+ *                       loop runs 4 (k=7,8: 1) where 5 would be chosen or asked for
  *   "timing"            1: msa_plan_execute records per-stage CUDA events (default 0)
  *   "verify_corner"     1: later plans and requests on the k=3 column kernel record the
  *                       far corner's score during the fill, and the traceback reports
@@ -213,7 +215,7 @@ typedef struct msa_plan_info {
     int64_t tiles;
     int32_t waves;              /* tile hyperplanes (section 3.1, Eq. 2) */
     int32_t fill_kernel;        /* 1 generic tile kernel, 2 k=3 column kernel, 3 k=2 band kernel,
-                                   4 k=4..6 line kernel, 5 k=4..6 streamed line kernel */
+                                   4 k=4..6 line kernel, 5 k=4..8 streamed line kernel */
     void   *d_tb;               /* device pointer of the uint8 traceback tensor: row-major with
                                    tb_strides for the tile kernel (k <= 3) and the band kernel;
                                    tile-major for the tile kernel at k >= 4 and for the line
@@ -368,7 +370,8 @@ int msa_tile_shape(int k, const int32_t *lens, int32_t *out_extent, int32_t *out
  * compiled edges are accepted (k=2: 16 32 64; k=3: 8 12 16; k=4: 4 5 6; k=5: 3 4
  * 5; k=6: 2 3 4; k=7: 2 3; k=8: 2); 0 restores the default (for k = 3 also the
  * automatic choice of the column kernel where it fits, for k = 2 of the band
- * kernel). Later plans and serving batches use the setting. Host-only,
+ * kernel; at k = 7, 8, where an edge that is set selects the tile kernel, of the
+ * streamed line kernel). Later plans and serving batches use the setting. Host-only,
  * thread-safe.
  */
 int msa_set_tile_edge(int k, int32_t edge);

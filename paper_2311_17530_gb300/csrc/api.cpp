@@ -367,7 +367,7 @@ int plan_create(int k, const int32_t *lens, const char *alphabet, int kernel_cho
         e = cudaMemcpy(p->pp.order, p->hp.order.data(), p->hp.order.size() * 8, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(p->pp.amap, amap, 256, cudaMemcpyHostToDevice);
     // tagged faces start with tag 0, which no execution uses
-    if (e == cudaSuccess && tagged_faces(p->hp.kernel)) e = clear_faces(p->hp, p->pp);
+    if (e == cudaSuccess && tagged_faces(p->hp)) e = clear_faces(p->hp, p->pp);
     if (e != cudaSuccess) {
         cudaFree(p->ws);
         delete p;
@@ -425,7 +425,7 @@ int msa_plan_execute(msa_plan *plan, const char *d_residues, const int32_t *d_su
     L.nprob = 1;
     L.tab_ints = plan->hp.A * (plan->hp.A + 1);  // table plus the sentinel column
     L.corner = plan->hp.check_corner;
-    if (tagged_faces(plan->hp.kernel)) {
+    if (tagged_faces(plan->hp)) {
         if (plan->epoch >= 32767) {  // column kernel tags (epoch << 16) + T would wrap: start over from cleared faces
             e = clear_faces(plan->hp, plan->pp, s);
             if (e != cudaSuccess) return cuda_error(e, "face reset");

@@ -174,19 +174,34 @@ int fill_lines_warps_per_cta(int k, int z) {
 cudaError_t launch_fill_stream_k4(const LaunchDesc &L, int grid, cudaStream_t s);
 cudaError_t launch_fill_stream_k5(const LaunchDesc &L, int grid, cudaStream_t s);
 cudaError_t launch_fill_stream_k6(const LaunchDesc &L, int grid, cudaStream_t s, int rho_s);
+cudaError_t launch_fill_stream_k7(const LaunchDesc &L, int grid, cudaStream_t s);
+cudaError_t launch_fill_stream_k8(const LaunchDesc &L, int grid, cudaStream_t s);
 int fill_stream_ctas_k4();
 int fill_stream_ctas_k5();
 int fill_stream_ctas_k6();
+int fill_stream_ctas_k7();
+int fill_stream_ctas_k8();
 
 cudaError_t launch_fill_stream(int k, const LaunchDesc &L, int grid, cudaStream_t s, int rho_s) {
-    return k == 4   ? launch_fill_stream_k4(L, grid, s)
-           : k == 5 ? launch_fill_stream_k5(L, grid, s)
-           : k == 6 ? launch_fill_stream_k6(L, grid, s, rho_s)
-                    : cudaErrorInvalidValue;
+    switch (k) {
+        case 4: return launch_fill_stream_k4(L, grid, s);
+        case 5: return launch_fill_stream_k5(L, grid, s);
+        case 6: return launch_fill_stream_k6(L, grid, s, rho_s);
+        case 7: return launch_fill_stream_k7(L, grid, s);
+        case 8: return launch_fill_stream_k8(L, grid, s);
+        default: return cudaErrorInvalidValue;
+    }
 }
 
 int fill_stream_ctas_per_sm(int k) {
-    return k == 4 ? fill_stream_ctas_k4() : k == 5 ? fill_stream_ctas_k5() : k == 6 ? fill_stream_ctas_k6() : 0;
+    switch (k) {
+        case 4: return fill_stream_ctas_k4();
+        case 5: return fill_stream_ctas_k5();
+        case 6: return fill_stream_ctas_k6();
+        case 7: return fill_stream_ctas_k7();
+        case 8: return fill_stream_ctas_k8();
+        default: return 0;
+    }
 }
 
 cudaError_t col3_attributes();

@@ -1,11 +1,17 @@
-// Whole-column super-block fill for k = 6 with a short last axis (rho_s <= Z):
+// Whole-column super-block fill for k = 6 .. 8 with a short last axis (rho_s <= Z):
 // the line kernel's sweep (fill_lines.cuh: lane l of a warp owns one line of a
-// 32-line block, skewed by the sum of its local coordinates; candidates of the
-// moves that also advance the last axis s are carried from the previous step)
-// on the streamed kernel's super-blocks (fill_lines_stream.cuh: a CTA of 4 warps
-// owns 4 x 4 x 2 x 2 x 2 lines and sweeps them in lockstep, one barrier per
-// step), with the halo exchanged as plain values once per column:
+// 32-line block, skewed by the sum of its local coordinates) on the streamed
+// kernel's super-blocks (fill_lines_stream.cuh: a CTA of 4 warps owns 128 lines --
+// 4 x 4 x 2 x 2 x 2, 2 x 4 x 2 x 2 x 2 x 2, 2^7 -- and sweeps them in lockstep, one
+// barrier per step), with the halo exchanged as plain values once per column:
 //
+// * A step forms the candidate C(m) of every subset m of the line axes (one shared
+//   load, and one add where m has pairs). The moves m + s of the next position cost
+//   C(m) + sum of T_i over m, T_i the pair score of axis i with the last axis there:
+//   their maximum over all m is folded axis by axis, F = max(F(m), F(m + i) + T_i),
+//   one fused add-max per m and nothing to carry but the result (max_over_subsets).
+//   Summing T over every subset, carrying the 2^NA - 1 candidates to the next step
+//   and adding there took 31 + 26 adds and 31 carried registers at k = 6 instead.
 // * Shared memory holds the halo'd super-block (local coordinates -1 .. SB_i - 1)
 //   indexed by POSITION: line h at word sum_i h_i A_i, its position z at word
 //   + z + 1 (word 0 is position -1, "no cell"). At step t lane c reads position
@@ -36,7 +42,9 @@ namespace msadp {
 // Strides (words) of the line axes in the position-indexed super-block box.
 __host__ __device__ constexpr int wide_stride(int K, int i) {
     constexpr int k6[] = {26, 393, 131, 1965, 5905};
-    return k6[i] + 0 * K;
+    constexpr int k7[] = {14, 42, 211, 633, 1901, 5713};
+    constexpr int k8[] = {10, 30, 90, 271, 813, 2449, 7353};
+    return K == 6 ? k6[i] : K == 7 ? k7[i] : k8[i];
 }
 template <int K>
 __host__ __device__ constexpr int wide_move_off(int m) {
@@ -49,7 +57,7 @@ template <int K>
 __host__ __device__ constexpr int wide_v_words() {
     // the last word any line's positions -1 .. Z - 1 use, plus one, plus the 3
     // words past the last position that a face write-back's last group reads
-    int s = kWideZ + 1;
+    int s = wide_z(K) + 1;
     for (int i = 0; i < K - 1; ++i) s += stream_sb(K, i) * wide_stride(K, i);
     return round_up(s + 3, 4);
 }
@@ -72,7 +80,7 @@ struct WideLayout {
     // pair-table rows: positions 0 .. Z - 1, row stride congruent to a line
     // block's skew + 1 mod 32 (lanes of one row read different positions)
     static constexpr int ZS = [] {
-        int s = kWideZ;
+        int s = wide_z(K);
         while (s % 32 != (line_skew_max(K) + 1) % 32) ++s;
         return s;
     }();
@@ -95,6 +103,31 @@ __host__ __device__ constexpr int wide_min_ctas() {
     return c < 1 ? 1 : c;
 }
 
+// Candidates of a position and the fold of the moves that also advance the last
+// axis (see the head of this file). vp: the line's own word of the position; Sp: pair
+// sums over subsets of the line axes; p: pair scores with the next position. acc takes
+// every candidate C(m); the result is max over nonempty m of C(m) + sum of p over m.
+template <int K, int I, int M>
+__device__ __forceinline__ int max_over_subsets(const int32_t *vp, const int (&Sp)[1 << (K - 1)], const int (&p)[K - 1],
+                                                int &acc0, int &acc1) {
+    if constexpr (I == 1) {  // the subsets M and M + {0}
+        const int c1 = vp[-wide_move_off<K>(M | 1)] + Sp[M | 1];
+        if constexpr (M == 0) {
+            acc0 = max(acc0, c1);
+            return c1 + p[0];
+        } else {
+            const int c0 = vp[-wide_move_off<K>(M)] + Sp[M];
+            int &acc = popc_c(M) & 1 ? acc1 : acc0;  // two chains
+            acc = __vimax3_s32(acc, c0, c1);
+            return __viaddmax_s32(c1, p[0], c0);
+        }
+    } else {
+        const int without = max_over_subsets<K, I - 1, M>(vp, Sp, p, acc0, acc1);
+        const int with = max_over_subsets<K, I - 1, M | 1 << (I - 1)>(vp, Sp, p, acc0, acc1);
+        return __viaddmax_s32(with, p[I - 1], without);
+    }
+}
+
 template <int K>
 __global__ void __launch_bounds__(stream_threads<K>(), wide_min_ctas<K>()) fill_lines_wide_kernel(const LaunchDesc L) {
     using LY = WideLayout<K>;
@@ -104,7 +137,7 @@ __global__ void __launch_bounds__(stream_threads<K>(), wide_min_ctas<K>()) fill_
     constexpr int SMAX = stream_skew_max(K);
     constexpr int MASKB = (1 << K) - 1;
     constexpr int HB = 8;  // halo loads in flight per thread
-    static_assert(SMAX < LY::V && wide_v_words<K>() < (1 << 15) && NFL < 128 && M < 32, "geometry");
+    static_assert(SMAX < LY::V && wide_v_words<K>() < (1 << 15) && NFL < 128 && NA < 10, "geometry");
 
     extern __shared__ __align__(16) unsigned char smem_raw[];
     int32_t *sm = reinterpret_cast<int32_t *>(smem_raw);
@@ -350,10 +383,8 @@ __global__ void __launch_bounds__(stream_threads<K>(), wide_min_ctas<K>()) fill_
                 row += stream_sb(K, i);
             }
         }
-        int carry[M + 1];
         int vself = col == 0 && tid == 0 ? 0 : kNeg;
-#pragma unroll
-        for (int m = 1; m <= M; ++m) carry[m] = kNeg + Sp[m];
+        int D = vself;  // best move of the next position that advances the last axis
         const int rows = P.tb_block / 32;
         uint8_t *tbw = P.tb + tile * P.tb_block + lane;
         const int nsteps = rho + SMAX;
@@ -361,26 +392,12 @@ __global__ void __launch_bounds__(stream_threads<K>(), wide_min_ctas<K>()) fill_
             if ((unsigned)(ts - sigw) < (unsigned)(rho + line_skew_max(K))) {
                 const int z = ts - sig;
                 const bool act = (unsigned)z < (unsigned)rho;
-                const int zp = z < 0 ? 0 : (z >= rho ? rho - 1 : z);
+                const int zn = z < -1 ? 0 : (z + 1 >= rho ? rho - 1 : z + 1);
                 int p[NA];
 #pragma unroll
-                for (int i = 0; i < NA; ++i) p[i] = PT[ptoff[i] + zp];
-                int T[M + 1];
-                T[0] = 0;
-#pragma unroll
-                for (int m = 1; m <= M; ++m) T[m] = (m & (m - 1)) ? T[m & (m - 1)] + p[lowbit_c(m)] : p[lowbit_c(m)];
-                const int32_t *vp = V + vbase + z + 1;
-                int acc0 = vself, acc1 = kNeg;
-#pragma unroll
-                for (int m = 1; m <= M; ++m) {
-                    const int cm = vp[-wide_move_off<K>(m)] + Sp[m];
-                    const int cb = carry[m] + T[m];
-                    if (m & 1)
-                        acc0 = __vimax3_s32(acc0, cm, cb);
-                    else
-                        acc1 = __vimax3_s32(acc1, cm, cb);
-                    carry[m] = cm;
-                }
+                for (int i = 0; i < NA; ++i) p[i] = PT[ptoff[i] + zn];
+                int acc0 = D, acc1 = kNeg;
+                const int F = max_over_subsets<K, NA, 0>(V + vbase + z + 1, Sp, p, acc0, acc1);
                 const int acc = max(acc0, acc1);
                 const int tm = (Wl + ts * (1 << NA) - acc) & MASKB;
                 const int val = acc + tm;
@@ -390,6 +407,7 @@ __global__ void __launch_bounds__(stream_threads<K>(), wide_min_ctas<K>()) fill_
                     V[vbase + z + 1] = val;
                     vself = val;
                 }
+                D = max(F, vself);
             }
             __syncthreads();
         }

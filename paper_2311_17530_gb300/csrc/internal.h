@@ -137,7 +137,7 @@ constexpr int kLinesMinK = 4, kLinesMaxK = 6;
 __host__ __device__ constexpr int line_ext(int K, int i) {
     return K == 4 ? (i == 0 ? 2 : 4)   // 2 x 4 x 4
          : K == 5 ? (i == 3 ? 4 : 2)   // 2 x 2 x 2 x 4
-                  : 2;                 // k = 6: 2^5
+                  : i < K - 6 ? 1 : 2; // k = 6: 2^5, k = 7, 8: 1 along the first axes
 }
 constexpr int kMaxLineSegments = 3;
 __host__ __device__ constexpr int line_z_candidate(int k, int idx) {
@@ -167,13 +167,16 @@ __host__ __device__ constexpr int line_skew_max(int K) {
 // kernel, extents line_ext; the warps form a grid of extents stream_wg) over the
 // whole last axis in lockstep, in blocks of stream_block(k) steps; super-blocks
 // exchange faces as (value, epoch) entries indexed by time.
-constexpr int kStreamMinK = 4, kStreamMaxK = 6;
-__host__ __device__ constexpr int stream_block(int K) { return K == 6 ? 4 : 8; }  // steps per block = times per face chunk
-// k = 6: the streamed kernel's whole-column form (fill_lines_wide.cuh) holds a
-// last axis of at most kWideZ positions; longer ones take the pipelined form.
+constexpr int kStreamMinK = 4, kStreamMaxK = 8;
+__host__ __device__ constexpr int stream_block(int K) { return K >= 6 ? 4 : 8; }  // steps per block = times per face chunk
+// k >= 6: the streamed kernel's whole-column form (fill_lines_wide.cuh) holds a last
+// axis of at most wide_z(k) positions (as many as leave room for three CTAs per SM,
+// two at k = 8); longer ones take the pipelined form at k = 6, the generic tile
+// kernel at k = 7, 8.
 constexpr int kWideZ = 25;
+__host__ __device__ constexpr int wide_z(int K) { return K == 6 ? kWideZ : K == 7 ? 13 : K == 8 ? 9 : 0; }
 __host__ __device__ constexpr int stream_wg(int K, int i) {  // warps along line axis i
-    return K == 4 ? 2 : (i < 2 ? 2 : 1);  // k = 4: 2 x 2 x 2; k = 5: 2 x 2 x 1 x 1; k = 6: 2 x 2 x 1 x 1 x 1
+    return K == 4 ? 2 : (i < 2 ? 2 : 1);  // k = 4: 2 x 2 x 2; k >= 5: 2 x 2 x 1 ..
 }
 __host__ __device__ constexpr int stream_warps(int K) {
     int w = 1;

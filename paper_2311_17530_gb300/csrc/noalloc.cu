@@ -160,7 +160,7 @@ extern "C" int msa_align_noalloc(int k, const int32_t *lens, const char *alphabe
     fill_problem_desc(hp, pp, 0, d);
     // tagged faces: the encode step clears them, so that no word of an earlier call
     // passes for an entry of this one
-    d.clear_faces = tagged_faces(hp.kernel) ? 1 : 0;
+    d.clear_faces = tagged_faces(hp) ? 1 : 0;
     cudaStream_t s = (cudaStream_t)stream;
     int64_t spin_ms;
     {

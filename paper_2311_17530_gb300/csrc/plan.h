@@ -20,10 +20,6 @@ enum FillKernel {
     kKernelCount = 6
 };
 
-// Kernels whose faces carry (value, epoch) entries: the plan clears them before
-// the first launch and gives every launch a new epoch.
-inline bool tagged_faces(int kernel) { return kernel == kKernelCol3 || kernel == kKernelStream || kernel == kKernelBand2; }
-
 struct HostPlan {
     int k = 0;
     int A = 0;
@@ -55,6 +51,7 @@ struct HostPlan {
     int32_t lzq = 0;                   // line kernels: entries per line in a tile's (column's) face block
     int32_t edge = 0;              // tile edge of the generic kernel (tile_ext); longest segment of the
                                    // line kernel; 0 for the column and band kernels
+    bool wide = false;             // streamed line kernel: its whole-column form
     int32_t check_corner = 1;      // the fill records the far corner's key and the traceback checks it
                                    // (always, but optional for the column kernel: msa_config "verify_corner")
     int32_t pair_min_sum = 0;
@@ -63,6 +60,12 @@ struct HostPlan {
     std::vector<uint64_t> order;   // ticket -> tile linear index (problem bits added by callers)
     std::vector<int64_t> wave_start;  // order[wave_start[w] .. wave_start[w + 1]) is wave w (tile index sum)
 };
+
+// Plans whose faces carry (value, epoch) entries: the plan clears them before the
+// first launch and gives every launch a new epoch.
+inline bool tagged_faces(const HostPlan &hp) {
+    return hp.kernel == kKernelCol3 || hp.kernel == kKernelBand2 || (hp.kernel == kKernelStream && !hp.wide);
+}
 
 // Tile (or column) extents the planner uses for these lengths, kernel and edge.
 void tile_extents(int k, const int32_t *lens, int kernel, int edge, int32_t *E);

@@ -71,6 +71,7 @@ int msa_set_tile_edge(int k, int32_t edge) {
         return set_error(MSA_EINVAL, "tile edge %d is not compiled for k=%d", edge, k);
     if (k == 3 && edge == 0) set_prefer_tiles_k3(false);  // defaults: the column kernel where it fits
     if (k == 2 && edge == 0) set_prefer_tiles_k2(false);  // defaults: the band kernel
+    if (k > kLinesMaxK && edge == 0) reset_prefer_stream(k);  // defaults: the whole-column form where it fits
     return MSA_OK;
 }
 
@@ -190,7 +191,9 @@ int msa_autotune(int k, const int32_t *lens, int alphabet_size, int32_t repeats,
         int bt = -1;
         for (int i = 0; i < out->ncand; ++i)
             if (out->cand_kernel[i] == kKernelTiles && (bt < 0 || out->cand_ms[i] < out->cand_ms[bt])) bt = i;
-        if (bt >= 0) set_tile_edge(k, out->cand_edge[bt]);
+        // (not at k = 7, 8, where a set edge selects the tile kernel)
+        if (k > kLinesMaxK) set_tile_edge(k, 0);
+        else if (bt >= 0) set_tile_edge(k, out->cand_edge[bt]);
     }
     return MSA_OK;
 }

@@ -167,3 +167,57 @@ def test_automatic_choice_and_serving():
             want = oracle.align(p.seqs, p.alphabet, p.subst, p.gap)
             assert msa.msa_poll(h, p.k, sum(p.lens)) == (want.score, want.rows)
 
+
+
+# k = 7, 8: the whole-column form's super-blocks are 2x4x2x2x2x2 and 2^7 lines, the last
+# axis holds up to 13 and 9 positions
+WIDE_SHAPES = [(7, [1, 3, 1, 1, 1, 1, 12]), (7, [2, 4, 2, 2, 2, 2, 0]), (7, [0, 5, 1, 3, 0, 2, 11]), (7, [3, 8, 2, 3, 2, 4, 5]),
+               (7, [4, 3, 4, 2, 4, 3, 12]), (8, [1, 1, 1, 1, 1, 1, 1, 8]), (8, [2, 2, 1, 2, 0, 2, 2, 7]),
+               (8, [0, 3, 1, 2, 3, 1, 0, 4]), (8, [3, 2, 3, 2, 3, 2, 3, 1])]
+
+
+@pytest.mark.parametrize("k,lens", WIDE_SHAPES)
+@pytest.mark.parametrize("alphabet,related", [(inputs.PROTEIN, True), (inputs.DNA, False)])
+def test_whole_column_form_beyond_k6(k, lens, alphabet, related):
+    """Full tensors, with and without the choice spelled out, in another topological order."""
+    p = inputs.random_problem(7600 + k + sum(lens), k, lens, alphabet=alphabet, related=related)
+    check(p)
+    msa.msa_config("fill_kernel", 0)
+    msa.msa_config("test_shuffle_waves", 5)
+    check(p)
+
+
+@pytest.mark.parametrize("k,lens", [(7, [2, 2, 2, 2, 2, 2, 13]), (8, [1, 1, 2, 1, 1, 2, 1, 9])])
+def test_whole_column_form_limit(k, lens):
+    """One position more than the box holds: the generic tile kernel, also when asked for the
+    streamed one; and a tile edge set by the caller selects it."""
+    msa.msa_config("fill_kernel", 0)
+    p = inputs.random_problem(7700 + k, k, lens, alphabet=inputs.PROTEIN, related=True)
+    want = oracle.align_problem(p)
+    for kernel in (0, 5):
+        msa.msa_config("fill_kernel", kernel)
+        score, rows, status, _, info = run(p)
+        assert (info.fill_kernel, status) == (1, 0) and (score, rows) == (want.score, want.rows)
+    msa.msa_config("fill_kernel", 0)
+    q = inputs.random_problem(7701 + k, k, lens[:-1] + [3], alphabet=inputs.PROTEIN, related=True)
+    assert run(q)[4].fill_kernel == 5
+    msadp.msa_set_tile_edge(k, 2)
+    try:
+        assert run(q)[4].fill_kernel == 1
+    finally:
+        msadp.msa_set_tile_edge(k, 0)
+    assert run(q)[4].fill_kernel == 5
+
+
+def test_whole_column_form_withheld_column():
+    """k = 7, 8: a column that never publishes ends its dependants with a status."""
+    for k, lens in ((7, [3, 4, 2, 2, 2, 2, 6]), (8, [3, 2, 2, 2, 2, 2, 2, 4])):
+        p = inputs.random_problem(7800 + k, k, lens, alphabet=inputs.DNA)
+        msa.msa_config("spin_timeout_ms", 200)
+        msa.msa_config("test_withhold_tile", 0)
+        try:
+            assert run(p)[2] == msa.MSA_ETIMEOUT
+        finally:
+            msa.msa_config("test_withhold_tile", -1)
+            msa.msa_config("spin_timeout_ms", 5000)
+        check(p)
