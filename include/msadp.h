@@ -410,7 +410,7 @@ typedef struct msa_tuning {
 /*
  * Time every compiled tile edge for k (and the column kernel for k = 3, the band
  * kernel for k = 2, each compiled line segment for k = 4..6 and the streamed line
- * kernel for k = 4..6) on a synthetic problem with these lengths over an alphabet
+ * kernel for k = 4..8) on a synthetic problem with these lengths over an alphabet
  * of alphabet_size letters: one warm-up and `repeats` executions each, on the
  * library stream. The fastest becomes the choice for k (msa_set_tile_edge or
  * msa_set_line_segment, and whether the automatic kernel choice takes the band,

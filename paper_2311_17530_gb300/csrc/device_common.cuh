@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 #include "internal.h"
 
 namespace msadp {
@@ -158,5 +160,35 @@ __host__ __device__ constexpr int lowbit_c(int m) {  // index of the lowest set 
     return l;
 }
 __host__ __device__ constexpr int round_up(int x, int a) { return (x + a - 1) / a * a; }
+
+// The line kernels' cell update. C(m) is the candidate of the nonempty subset m of
+// the first I line axes (cand(IntC<m>)); acc takes the maximum over all of them, in
+// two chains. The result is the maximum over them of C(m) + sum of p_i over m, p_i
+// the pair score of axis i with the last axis at the next position: what the moves
+// that also advance the last axis are worth there. It is folded axis by axis,
+// F = max(F(without i), F(with i) + p_i), one fused add-max per subset -- summing p
+// over every subset and keeping every C(m) for the next position costs two adds, half
+// a three-input maximum and a register per subset.
+template <int P>
+using IntC = std::integral_constant<int, P>;
+template <int I, int M, class Cand>
+__device__ __forceinline__ int fold_subsets(const Cand &cand, const int *p, int &acc0, int &acc1) {
+    if constexpr (I == 1) {  // the subsets M and M + {0}
+        const int c1 = cand(IntC<M | 1>{});
+        if constexpr (M == 0) {
+            acc0 = max(acc0, c1);
+            return c1 + p[0];
+        } else {
+            const int c0 = cand(IntC<M>{});
+            int &acc = popc_c(M) & 1 ? acc1 : acc0;
+            acc = __vimax3_s32(acc, c0, c1);
+            return __viaddmax_s32(c1, p[0], c0);
+        }
+    } else {
+        const int without = fold_subsets<I - 1, M>(cand, p, acc0, acc1);
+        const int with = fold_subsets<I - 1, M | 1 << (I - 1)>(cand, p, acc0, acc1);
+        return __viaddmax_s32(with, p[I - 1], without);
+    }
+}
 
 }  // namespace msadp

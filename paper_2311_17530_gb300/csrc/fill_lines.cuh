@@ -18,11 +18,14 @@
 //                                                       constant along the line)
 //   m' + s        : Q(c - e_m', z - 1) + P(m') + T(m', z)   T = pairs of m' with s
 //   s alone       : Q(c, z - 1)                        (no pair)
-// The candidate of m' + s is the previous step's candidate of m' plus T(m', z),
-// so each line keeps the 2^(k-1) - 1 candidates of the previous position in
-// registers ("carried"), P is formed once per tile, and T from k - 1 pair-table
-// lookups per cell. Each step therefore loads one value per line-axis subset
-// m' (2^(k-1) - 1 shared-memory loads), not one per move.
+// The candidate of m' + s is the previous position's candidate of m' plus T(m', z),
+// and T is a sum over the axes of m', so once a position's candidates are known the
+// best of the next position's moves with s is folded axis by axis (fold_subsets) and
+// only that is carried; P is formed once per tile, and the k - 1 pair scores of a
+// position are looked up once. Each step therefore loads one value per line-axis
+// subset m' (2^(k-1) - 1 shared-memory loads), not one per move. (Carrying every
+// candidate and summing T over every subset: 1.51 against 1.46 ms on k4 DNA, 5.46
+// against 5.06 ms on k6 protein.)
 //
 // Scores are packed keys (internal.h): one integer max gives the best value and
 // the lowest move mask among ties; the mask is the traceback byte.
@@ -49,9 +52,8 @@ namespace msadp {
 // ---------------------------------------------------------------------------
 // Geometry (compile-time per k and the longest segment Z).
 
-// The line kernel is compiled for k = 4, 5, 6; at k = 7, 8 a lane would carry
-// 63 or 127 candidates and as many pair sums, more than its registers, and the
-// generic tile kernel runs instead. Block extents, segment candidates, lane
+// The line kernel is compiled for k = 4, 5, 6 (k = 7, 8 have the whole-column form of
+// fill_lines_wide.cuh and the generic tile kernel). Block extents, segment candidates, lane
 // strides and the skew bound are in internal.h (shared with the planner).
 // Shared-memory stride (words) of line axis i in the halo'd line box. Found by
 // exhaustive search for each (k, Z): every stride at least the size of the axes
@@ -417,10 +419,18 @@ __global__ void __launch_bounds__(line_best_warps<K, Z>() * 32) fill_lines_kerne
                     pb += line_ext(K, i) * ZS;
                 }
             }
-            int carry[M + 1];
+            // the moves of the first position that advance the last axis come from
+            // position -1 (lanes that start later fold it as their step before the first)
             int vself = V[vbase];
+            int next;
+            {
+                int p[NA], none0 = kNeg, none1 = kNeg;
 #pragma unroll
-            for (int m = 1; m <= M; ++m) carry[m] = V[vbase - move_line_off<K, Z>(m)] + Sp[m];
+                for (int i = 0; i < NA; ++i) p[i] = PT[ptoff[i]];
+                next = max(vself, fold_subsets<NA, 0>(
+                                      [&](auto m) { return V[vbase - move_line_off<K, Z>(m.value)] + Sp[m.value]; }, p,
+                                      none0, none1));
+            }
             uint8_t *tbblk = P.tb + lin * (int64_t)P.tb_block + lane;
             const int nsteps = Zt + SMAX;
             for (int ts = 0; ts < nsteps; ++ts) {
@@ -428,24 +438,12 @@ __global__ void __launch_bounds__(line_best_warps<K, Z>() * 32) fill_lines_kerne
                 const bool act = (unsigned)z < (unsigned)Zt;
                 const int zz = z + 1;  // word offset of position z
                 const int32_t *vp = V + vbase + zz;
-                int p[NA];
+                int p[NA];  // pair scores of the next position
 #pragma unroll
-                for (int i = 0; i < NA; ++i) p[i] = PT[ptoff[i] + z];
-                int T[M + 1];
-                T[0] = 0;
-#pragma unroll
-                for (int m = 1; m <= M; ++m) T[m] = (m & (m - 1)) ? T[m & (m - 1)] + p[lowbit_c(m)] : p[lowbit_c(m)];
-                int acc0 = vself, acc1 = kNeg;
-#pragma unroll
-                for (int m = 1; m <= M; ++m) {
-                    const int cm = vp[-move_line_off<K, Z>(m)] + Sp[m];
-                    const int cb = carry[m] + T[m];
-                    if (m & 1)
-                        acc0 = __vimax3_s32(acc0, cm, cb);
-                    else
-                        acc1 = __vimax3_s32(acc1, cm, cb);
-                    carry[m] = cm;
-                }
+                for (int i = 0; i < NA; ++i) p[i] = PT[ptoff[i] + z + 1];
+                int acc0 = next, acc1 = kNeg;
+                const int F = fold_subsets<NA, 0>(
+                    [&](auto m) { return vp[-move_line_off<K, Z>(m.value)] + Sp[m.value]; }, p, acc0, acc1);
                 const int acc = max(acc0, acc1);
                 int tm = (Wl + ts * (1 << NA) - acc) & MASKB;
                 int val = acc + tm;
@@ -458,6 +456,7 @@ __global__ void __launch_bounds__(line_best_warps<K, Z>() * 32) fill_lines_kerne
                     V[vbase + zz] = val;
                     vself = val;
                 }
+                next = max(F, vself);
                 __syncwarp();
             }
 

@@ -1,8 +1,11 @@
 // Streamed line fill for k = 4..6: the line kernel's recurrence and lanes
 // (fill_lines.cuh: lane l of a warp owns one line of a 32-line block, skewed by
-// the sum of its local coordinates; candidates of the moves that also advance
-// the last axis s are carried from the previous step), organised for the
-// latency of the hardware:
+// the sum of its local coordinates; the moves that also advance the last axis s are
+// folded from the previous position's candidates), organised for the latency of the
+// hardware. Measured (fill): k4 DNA 110 - 130 0.951 ms, k5 protein 33 - 45 1.395 ms,
+// against 1.021 and 1.577 ms with every candidate carried, the CTA's tables built by
+// one thread and three CTAs of 168 registers per SM at k = 5 (now four of 128: a copy's
+// source is a 4-byte face line, which lets their shared memory fit):
 //
 // * A CTA of W warps owns a SUPER-BLOCK of W line blocks (a grid of extents
 //   stream_wg over the line axes) and sweeps it over the WHOLE last axis in
@@ -114,8 +117,8 @@ struct StreamLayout {
     static constexpr int STAGE = PT + round_up(NROW * ZS, 4);
     static constexpr int NT_ = 32 * stream_warps(K);
     static constexpr int HC = (NH * (stream_block(K) / 2) + NT_ - 1) / NT_;  // halo copies per thread and block
-    static constexpr int HOFS = STAGE + NH * stream_block(K) * 2;  // per copy: source offset (8 bytes)
-    static constexpr int HMETA = HOFS + 2 * HC * NT_;               // ... ring base | time offset << 14
+    static constexpr int HOFS = STAGE + NH * stream_block(K) * 2;  // per copy: source face line
+    static constexpr int HMETA = HOFS + HC * NT_;               // ... ring base | time offset << 14
     static constexpr int HTAB = HMETA + HC * NT_;
     static constexpr int FTAB = HTAB + round_up(NH, 4);
     static constexpr int NB = FTAB + round_up(NFL, 4);
@@ -133,15 +136,59 @@ __host__ __device__ constexpr int stream_threads() {
 }
 // CTAs per SM: what shared memory allows (228 KB per SM, 1 KB reserved per CTA,
 // at most 48 warps) and what a budget of registers per thread allows (the sweep
-// keeps 2^(k-1) carried candidates and pair sums live); the launch bound caps
+// keeps 2^(k-1) pair sums live); the launch bound caps
 // registers to match.
 template <int K>
 __host__ __device__ constexpr int stream_min_ctas() {
     int c = (228 * 1024) / (stream_smem_bytes<K>() + 1024);
     if (c * stream_warps(K) > 48) c = 48 / stream_warps(K);
-    const int regs = K == 4 ? 80 : 168;
+    const int regs = K == 4 ? 80 : K == 5 ? 128 : 168;
     const int cr = 65536 / (regs * stream_threads<K>());
     return c < cr ? c : cr;
+}
+
+// Lines of a super-block and of its halo, numbered in closed form so that all
+// threads fill a CTA's tables (one thread counting them took 0.02 ms at k = 4, 0.09 at
+// k = 6 and 0.2 at k = 8, more than the sweep of a small problem): coordinates of line j (axis 0 most significant);
+// the number of a face line (some c_i = SB_i - 1) among the face lines, else -1; and
+// for halo'd index j (digits h_i in [0, SB_i]) its number among the halo lines (some
+// h_i = 0), else -1.
+template <int K>
+__device__ __forceinline__ void super_line(int j, int (&c)[K - 1]) {
+#pragma unroll
+    for (int i = K - 2; i >= 0; --i) {
+        c[i] = j % stream_sb(K, i);
+        j /= stream_sb(K, i);
+    }
+}
+template <int K>
+__device__ __forceinline__ int face_number(const int (&c)[K - 1]) {
+    int j = 0, inner = 0;  // the line's index; lines before it with every coordinate below SB_i - 1
+    bool prefix = true;    // ... coordinates so far
+#pragma unroll
+    for (int i = 0; i < K - 1; ++i) {
+        j = j * stream_sb(K, i) + c[i];
+        inner = inner * (stream_sb(K, i) - 1) + (prefix ? c[i] : 0);
+        prefix = prefix && c[i] < stream_sb(K, i) - 1;
+    }
+    return prefix ? -1 : j - inner;
+}
+template <int K>
+__device__ __forceinline__ int halo_number(int j, int (&h)[K - 1]) {
+    int rem = j;
+#pragma unroll
+    for (int i = K - 2; i >= 0; --i) {
+        h[i] = rem % (stream_sb(K, i) + 1);
+        rem /= stream_sb(K, i) + 1;
+    }
+    int inner = 0;  // indices before j with every digit >= 1
+    bool prefix = true;
+#pragma unroll
+    for (int i = 0; i < K - 1; ++i) {
+        inner = inner * stream_sb(K, i) + (prefix && h[i] >= 1 ? h[i] - 1 : 0);
+        prefix = prefix && h[i] >= 1;
+    }
+    return prefix ? -1 : j - inner;
 }
 
 __device__ __forceinline__ void cp_async16(void *smem_dst, const void *gsrc) {
@@ -153,9 +200,6 @@ __device__ __forceinline__ void st_relaxed_v2(unsigned long long *p, unsigned lo
 __device__ __forceinline__ unsigned long long tagged(int value, int tag) {
     return (unsigned long long)(unsigned)value | ((unsigned long long)(unsigned)tag << 32);
 }
-
-template <int P>
-using IntC = std::integral_constant<int, P>;
 
 template <int K>
 __global__ void __launch_bounds__(stream_threads<K>(), stream_min_ctas<K>()) fill_lines_stream_kernel(const LaunchDesc L) {
@@ -176,11 +220,11 @@ __global__ void __launch_bounds__(stream_threads<K>(), stream_min_ctas<K>()) fil
     constexpr int PQ = (NROW * U + NT - 1) / NT;  // pair-table entries per thread and refill
     constexpr int C0 = -((NA + U - 1) / U);       // first halo chunk: halo times start at -(k - 1)
     // The ring holds a line's times from t - (k - 1) on plus the next block's U
-    // times; the pair-table ring holds the positions a block reads, bU - SMAX ..
-    // bU + U - 1, and after the block the next U positions replace positions
-    // below (b + 1) U - SMAX.
+    // times; the pair-table ring holds the positions a block reads, bU + 1 - SMAX ..
+    // (b + 1) U, and in the block's step U - 2 the next U positions replace positions
+    // below (b + 1) U - SMAX, which its steps from U - 2 >= 1 on no longer read.
     static_assert(D % U == 0 && NPAR <= 4 && D >= U + NA && SMAX + U <= R && (R & (R - 1)) == 0 && NFL < 128 &&
-                      LY::PT < (1 << 14) && NT % (U / 2) == 0 && SMAX < 32 && M < 32,
+                      U >= 3 && LY::PT < (1 << 14) && NT % (U / 2) == 0 && SMAX < 32 && M < 32,
                   "geometry");
     // ring slot of a time (which may be negative)
     auto rslot = [](int x) { return (D & (D - 1)) == 0 ? x & (D - 1) : ((x % D) + D) % D; };
@@ -192,7 +236,7 @@ __global__ void __launch_bounds__(stream_threads<K>(), stream_min_ctas<K>()) fil
     unsigned long long *stage = reinterpret_cast<unsigned long long *>(sm + LY::STAGE);
     // halo lines: ring base | producer face line << 14 | axes S at -1 << 21 |
     // (the sum of SB_i over S: the producer's time offset) << 26
-    int64_t *hofs = reinterpret_cast<int64_t *>(sm + LY::HOFS);
+    int32_t *hofs = sm + LY::HOFS;
     int32_t *hmeta = sm + LY::HMETA;
     uint32_t *htab = reinterpret_cast<uint32_t *>(sm + LY::HTAB);
     uint32_t *ftab = reinterpret_cast<uint32_t *>(sm + LY::FTAB);  // face lines: ring base
@@ -202,45 +246,31 @@ __global__ void __launch_bounds__(stream_threads<K>(), stream_min_ctas<K>()) fil
     volatile int32_t *misc = sm + LY::MISC;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
-    if (tid == 0) {
-        // face lines of the super-block in line order (coordinates c_i in
-        // [0, SB_i), axis 0 most significant); their numbers index the faces
-        // (fnum: a line's face number, kept in the staging buffer until it is used)
-        int32_t *fnum = reinterpret_cast<int32_t *>(stage);
-        int nf = 0;
-        for (int j = 0; j < NLINES; ++j) {
-            int rem = j, base = 0;
-            bool face = false;
-            for (int i = NA - 1; i >= 0; --i) {
-                const int c = rem % stream_sb(K, i);
-                rem /= stream_sb(K, i);
-                base += (c + 1) * stream_stride(K, i);
-                face = face || c == stream_sb(K, i) - 1;
+    // face lines of the super-block in line order; their numbers index the faces
+    for (int j = tid; j < NLINES; j += NT) {
+        int c[NA], base = 0;
+        super_line<K>(j, c);
+        const int f = face_number<K>(c);
+#pragma unroll
+        for (int i = 0; i < NA; ++i) base += (c[i] + 1) * stream_stride(K, i);
+        if (f >= 0) ftab[f] = (uint32_t)base;
+    }
+    // halo lines
+    for (int j = tid; j < LY::NH + NLINES; j += NT) {
+        int h[NA], c[NA], base = 0;
+        uint32_t S = 0, sbs = 0;
+        const int n = halo_number<K>(j, h);
+        if (n < 0) continue;
+#pragma unroll
+        for (int i = 0; i < NA; ++i) {
+            base += h[i] * stream_stride(K, i);
+            c[i] = h[i] == 0 ? stream_sb(K, i) - 1 : h[i] - 1;  // the line in the super-block that produces it
+            if (h[i] == 0) {
+                S |= 1u << i;
+                sbs += stream_sb(K, i);
             }
-            fnum[j] = face ? nf : -1;
-            if (face) ftab[nf++] = (uint32_t)base;
         }
-        // halo lines (digits h_i in [0, SB_i], some 0): the producer's face line
-        // has c_i = SB_i - 1 where h_i = 0 and h_i - 1 elsewhere
-        int n = 0;
-        int hall = 1;
-        for (int i = 0; i < NA; ++i) hall *= stream_sb(K, i) + 1;
-        for (int j = 0; j < hall; ++j) {
-            int rem = j, base = 0, lp = 0, lstr = 1;
-            uint32_t S = 0, sbs = 0;
-            for (int i = NA - 1; i >= 0; --i) {
-                const int h = rem % (stream_sb(K, i) + 1);
-                rem /= stream_sb(K, i) + 1;
-                base += h * stream_stride(K, i);
-                lp += (h == 0 ? stream_sb(K, i) - 1 : h - 1) * lstr;
-                lstr *= stream_sb(K, i);
-                if (h == 0) {
-                    S |= 1u << i;
-                    sbs += stream_sb(K, i);
-                }
-            }
-            if (S) htab[n++] = (uint32_t)base | (uint32_t)fnum[lp] << 14 | S << 21 | sbs << 26;
-        }
+        htab[n] = (uint32_t)base | (uint32_t)face_number<K>(c) << 14 | S << 21 | sbs << 26;
     }
 
     // this thread's line: warp coordinates in the warp grid, lane coordinates in
@@ -357,21 +387,22 @@ __global__ void __launch_bounds__(stream_threads<K>(), stream_min_ctas<K>()) fil
         // time lies outside [0, ZQ), i.e. outside the producer's sweep).
         const int q2 = tid % (U / 2);  // the same for every copy of this thread
         // this thread's copies, once per column (copy v: pair idx = tid + NT v):
-        // the producer's face entry of time 0 (-1: none), ring base | time offset
+        // the producer's face line (-1: none), ring base | time offset
         // (formed at every copy instead, they cost more than the room they free)
 #pragma unroll
         for (int v = 0; v < HC; ++v)
             if (tid + NT * v < NP) {
                 const uint32_t e = htab[(tid + NT * v) / (U / 2)];
                 const int src = nb[(e >> 21) & 31];
-                hofs[v * NT + tid] = src < 0 ? -1 : (int64_t)src * FB + (int64_t)((e >> 14) & 127) * ZQ;
+                hofs[v * NT + tid] = src < 0 ? -1 : src * NFL + (int)((e >> 14) & 127);
                 hmeta[v * NT + tid] = (int)(e & 0x3FFF) | (2 * q2 + (int)(e >> 26)) << 14;
             }
         auto halo_pair = [&](int v, int &base, int &toff) -> int64_t {
             const int meta = hmeta[v * NT + tid];
             base = meta & 0x3FFF;
             toff = meta >> 14;
-            return hofs[v * NT + tid];
+            const int line = hofs[v * NT + tid];  // face lines of 2 ZQ words: fewer than 2^31 of them fit the GPU
+            return line < 0 ? -1 : (int64_t)line * ZQ;
         };
         auto halo_issue = [&](int c, bool mine) {
             if (mine) {
@@ -552,10 +583,8 @@ __global__ void __launch_bounds__(stream_threads<K>(), stream_min_ctas<K>()) fil
                 row += stream_sb(K, i);
             }
         }
-        int carry[M + 1];
         int vself = col == 0 && tid == 0 ? 0 : kNeg;
-#pragma unroll
-        for (int m = 1; m <= M; ++m) carry[m] = kNeg + Sp[m];
+        int next = vself;  // best move of the next position that advances the last axis
         // this warp's traceback rows: row r = t - (the line block's first skew)
         const int rows = P.tb_block / 32;
         uint8_t *tbw = P.tb + tile * P.tb_block + lane;
@@ -603,24 +632,13 @@ __global__ void __launch_bounds__(stream_threads<K>(), stream_min_ctas<K>()) fil
                     int slp[NA + 1];  // slot of time ts - q
 #pragma unroll
                     for (int q = 0; q <= NA; ++q) slp[q] = own - q < 0 ? own - q + D : own - q;
-                    int p[NA];
+                    int p[NA];  // pair scores of the next position
 #pragma unroll
-                    for (int i = 0; i < NA; ++i) p[i] = ptb[i][s];
-                    int T[M + 1];
-                    T[0] = 0;
-#pragma unroll
-                    for (int m = 1; m <= M; ++m) T[m] = (m & (m - 1)) ? T[m & (m - 1)] + p[lowbit_c(m)] : p[lowbit_c(m)];
-                    int acc0 = vself, acc1 = kNeg;  // two independent max chains
-#pragma unroll
-                    for (int m = 1; m <= M; ++m) {
-                        const int cm = vb[slp[popc_c(m)] - stream_move_off<K>(m)] + Sp[m];
-                        const int cb = carry[m] + T[m];
-                        if (m & 1)
-                            acc0 = __vimax3_s32(acc0, cm, cb);
-                        else
-                            acc1 = __vimax3_s32(acc1, cm, cb);
-                        carry[m] = cm;
-                    }
+                    for (int i = 0; i < NA; ++i) p[i] = ptb[i][s + 1];
+                    int acc0 = next, acc1 = kNeg;  // two independent max chains
+                    const int F = fold_subsets<NA, 0>(
+                        [&](auto m) { return vb[slp[popc_c(m.value)] - stream_move_off<K>(m.value)] + Sp[m.value]; }, p,
+                        acc0, acc1);
                     const int acc_all = max(acc0, acc1);
                     const int tm = (Wb0 + s * (1 << NA) - acc_all) & MASKB;
                     const int val = acc_all + tm;
@@ -629,12 +647,15 @@ __global__ void __launch_bounds__(stream_threads<K>(), stream_min_ctas<K>()) fil
                         vb[own] = val;
                         vself = val;
                     }
+                    next = max(F, vself);
                 }
+                // the block's last step reads the next block's first position; the
+                // positions replaced lie below every position this block still reads
+                if (s == U - 2 && refill) pt_store((b + 1) * U);
                 __syncthreads();
             };
 #pragma unroll
             for (int s = 0; s < U; ++s) step(s);
-            if (refill) pt_store((b + 1) * U);
             face_write(b);
             __syncthreads();  // the block's face stores precede the count in program order (a hint)
             if (tid == 0 && tagout != 0) st_relaxed(prog + col, b + 1);

@@ -5,13 +5,10 @@
 // 4 x 4 x 2 x 2 x 2, 2 x 4 x 2 x 2 x 2 x 2, 2^7 -- and sweeps them in lockstep, one
 // barrier per step), with the halo exchanged as plain values once per column:
 //
-// * A step forms the candidate C(m) of every subset m of the line axes (one shared
-//   load, and one add where m has pairs). The moves m + s of the next position cost
-//   C(m) + sum of T_i over m, T_i the pair score of axis i with the last axis there:
-//   their maximum over all m is folded axis by axis, F = max(F(m), F(m + i) + T_i),
-//   one fused add-max per m and nothing to carry but the result (max_over_subsets).
-//   Summing T over every subset, carrying the 2^NA - 1 candidates to the next step
-//   and adding there took 31 + 26 adds and 31 carried registers at k = 6 instead.
+// * The cell update is the shared fold (fold_subsets): one load, one add where a
+//   subset has pairs, one fused add-max and half a three-input maximum per subset,
+//   only the result carried to the next position. Carrying every candidate instead
+//   was 4.88 against 4.39 ms (k6 protein, 18 - 24 residues).
 // * Shared memory holds the halo'd super-block (local coordinates -1 .. SB_i - 1)
 //   indexed by POSITION: line h at word sum_i h_i A_i, its position z at word
 //   + z + 1 (word 0 is position -1, "no cell"). At step t lane c reads position
@@ -103,31 +100,6 @@ __host__ __device__ constexpr int wide_min_ctas() {
     return c < 1 ? 1 : c;
 }
 
-// Candidates of a position and the fold of the moves that also advance the last
-// axis (see the head of this file). vp: the line's own word of the position; Sp: pair
-// sums over subsets of the line axes; p: pair scores with the next position. acc takes
-// every candidate C(m); the result is max over nonempty m of C(m) + sum of p over m.
-template <int K, int I, int M>
-__device__ __forceinline__ int max_over_subsets(const int32_t *vp, const int (&Sp)[1 << (K - 1)], const int (&p)[K - 1],
-                                                int &acc0, int &acc1) {
-    if constexpr (I == 1) {  // the subsets M and M + {0}
-        const int c1 = vp[-wide_move_off<K>(M | 1)] + Sp[M | 1];
-        if constexpr (M == 0) {
-            acc0 = max(acc0, c1);
-            return c1 + p[0];
-        } else {
-            const int c0 = vp[-wide_move_off<K>(M)] + Sp[M];
-            int &acc = popc_c(M) & 1 ? acc1 : acc0;  // two chains
-            acc = __vimax3_s32(acc, c0, c1);
-            return __viaddmax_s32(c1, p[0], c0);
-        }
-    } else {
-        const int without = max_over_subsets<K, I - 1, M>(vp, Sp, p, acc0, acc1);
-        const int with = max_over_subsets<K, I - 1, M | 1 << (I - 1)>(vp, Sp, p, acc0, acc1);
-        return __viaddmax_s32(with, p[I - 1], without);
-    }
-}
-
 template <int K>
 __global__ void __launch_bounds__(stream_threads<K>(), wide_min_ctas<K>()) fill_lines_wide_kernel(const LaunchDesc L) {
     using LY = WideLayout<K>;
@@ -154,35 +126,26 @@ __global__ void __launch_bounds__(stream_threads<K>(), wide_min_ctas<K>()) fill_
     // box bases, then every halo line (some digit h_i = 0) with its base, the
     // number of its producer's face line (c_i = SB_i - 1 where h_i = 0, h_i - 1
     // elsewhere) and the subset S of axes at -1 (which neighbour produces it).
-    if (tid == 0) {
-        int32_t *fnum = V;  // a line's face number (-1: none), kept in the box until it is used
-        int nf = 0;
-        for (int j = 0; j < NT; ++j) {
-            int rem = j, base = 0;
-            bool face = false;
-            for (int i = NA - 1; i >= 0; --i) {
-                const int c = rem % stream_sb(K, i);
-                rem /= stream_sb(K, i);
-                base += (c + 1) * wide_stride(K, i);
-                face = face || c == stream_sb(K, i) - 1;
-            }
-            fnum[j] = face ? nf : -1;
-            if (face) ftab[nf++] = base;
+    for (int j = tid; j < NT; j += NT) {
+        int c[NA], base = 0;
+        super_line<K>(j, c);
+        const int f = face_number<K>(c);
+#pragma unroll
+        for (int i = 0; i < NA; ++i) base += (c[i] + 1) * wide_stride(K, i);
+        if (f >= 0) ftab[f] = base;
+    }
+    for (int j = tid; j < NHL; j += NT) {
+        int h[NA], c[NA], base = 0;
+        uint32_t S = 0;
+        const int n = halo_number<K>(j, h);
+        if (n < 0) continue;
+#pragma unroll
+        for (int i = 0; i < NA; ++i) {
+            base += h[i] * wide_stride(K, i);
+            c[i] = h[i] == 0 ? stream_sb(K, i) - 1 : h[i] - 1;
+            if (h[i] == 0) S |= 1u << i;
         }
-        int n = 0;
-        for (int j = 0; j < NHL; ++j) {
-            int rem = j, base = 0, lp = 0, lstr = 1;
-            uint32_t S = 0;
-            for (int i = NA - 1; i >= 0; --i) {
-                const int h = rem % (stream_sb(K, i) + 1);
-                rem /= stream_sb(K, i) + 1;
-                base += h * wide_stride(K, i);
-                lp += (h == 0 ? stream_sb(K, i) - 1 : h - 1) * lstr;
-                lstr *= stream_sb(K, i);
-                if (h == 0) S |= 1u << i;
-            }
-            if (S) hdesc[n++] = (uint32_t)base | (uint32_t)fnum[lp] << 15 | S << 22;
-        }
+        hdesc[n] = (uint32_t)base | (uint32_t)face_number<K>(c) << 15 | S << 22;
     }
 
     // this thread's line: warp and lane coordinates, box base, skew
@@ -397,7 +360,9 @@ __global__ void __launch_bounds__(stream_threads<K>(), wide_min_ctas<K>()) fill_
 #pragma unroll
                 for (int i = 0; i < NA; ++i) p[i] = PT[ptoff[i] + zn];
                 int acc0 = D, acc1 = kNeg;
-                const int F = max_over_subsets<K, NA, 0>(V + vbase + z + 1, Sp, p, acc0, acc1);
+                const int32_t *vp = V + vbase + z + 1;
+                const int F = fold_subsets<NA, 0>(
+                    [&](auto m) { return vp[-wide_move_off<K>(m.value)] + Sp[m.value]; }, p, acc0, acc1);
                 const int acc = max(acc0, acc1);
                 const int tm = (Wl + ts * (1 << NA) - acc) & MASKB;
                 const int val = acc + tm;
