@@ -284,3 +284,13 @@ def test_shuffled_orders_over_a_poisoned_traceback(kernel, k, lens, seed):
         msa.msa_config("test_poison_tb", 0)
         msa.msa_config("test_shuffle_waves", 0)
         msa.msa_config("fill_kernel", 0)
+
+
+@pytest.mark.parametrize("lens", [(1, 1), (3, 2), (4, 3), (126, 14), (127, 15), (128, 16), (129, 17), (255, 271),
+                                  (1, 400), (400, 1)])
+def test_k2_band_kernel_edges(lens):
+    """One below, at and above the edges of a lane's 4 rows, a band's 128 rows and a
+    block of 16 columns."""
+    for related in (False, True):
+        check_problem(inputs.random_problem(9100 + sum(lens) + related, 2, list(lens), alphabet=inputs.DNA,
+                                            related=related))
