@@ -253,11 +253,10 @@ __host__ __device__ constexpr int mask_of_tag(int t) { return t == 7 ? 1 : t == 
 __host__ __device__ constexpr int64_t tb_col_bytes(int rho2) { return (int64_t)(nsteps(rho2) + U) * W * 32 * R; }
 }  // namespace c3
 
-// Traceback box edge D for the row-major layout with k <= 3 (the box [x-D, x] is
-// staged in shared memory, rows along the last axis in 16-byte granules, so a
-// staged row holds at most round_up(D + 16, 16) bytes); larger k reads cells
-// directly.
-__host__ __device__ constexpr int traceback_box(int k) { return k == 2 ? 192 : 28; }
+// Traceback box edge D for the row-major layout at k = 3 (the box [x-D, x] is staged
+// in shared memory, rows along the last axis in 16-byte granules, so a staged row
+// holds at most round_up(D + 16, 16) bytes).
+constexpr int kTracebackBox = 28;
 constexpr int kTracebackSmem = 224 * 1024;  // two 112 KB windows (column layout)
 // The traceback tensor's last axis is padded to this many bytes (16-byte rows).
 constexpr int kTbRowAlign = 16;

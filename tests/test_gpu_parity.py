@@ -294,3 +294,11 @@ def test_k2_band_kernel_edges(lens):
     for related in (False, True):
         check_problem(inputs.random_problem(9100 + sum(lens) + related, 2, list(lens), alphabet=inputs.DNA,
                                             related=related))
+
+
+@pytest.mark.parametrize("lens", [(1500, 1480), (1450, 330), (330, 1450), (1700, 40), (40, 1700)])
+def test_k2_strip_walk(lens):
+    """Paths longer than one traceback strip, along, above and below the diagonal."""
+    for related in (False, True):
+        check_problem(inputs.random_problem(9200 + sum(lens) + related, 2, list(lens), alphabet=inputs.DNA,
+                                            related=related))
