@@ -676,7 +676,7 @@ int msa_near_optimal(int k, const char *const *seqs, const int32_t *lens, const 
     const size_t o_res = take(total + 16), o_sub = take((size_t)A * A * 4), o_out = take(sizeof(msa_device_result)),
                  o_mask1 = take(total + 16), o_masks = take((size_t)max_count * total + 16),
                  o_ncols = take((size_t)max_count * 4), o_scores = take((size_t)max_count * 8), o_cm = take(8),
-                 o_work = take(near_optimal_work_bytes(k, (int64_t)total));
+                 o_work = take(near_optimal_work_bytes(k, (int64_t)total, max_count));
     char *d = nullptr;
     cudaError_t e = cudaMalloc(&d, off);
     if (e != cudaSuccess) {

@@ -310,7 +310,8 @@ int col3_smem_bytes(int alphabet_size);
 // Outputs of the near-optimal enumeration (near_optimal.cu), device memory:
 // masks max_count x len_sum (first column first), ncols and scores per alignment,
 // count_more[2] = {alignments stored, 1 when more were left (2: walk inconsistent)};
-// work holds near_optimal_work_bytes of tables and stack (0: they fit in shared memory).
+// work holds near_optimal_work_bytes of the walk's history, or of tables and stack beyond
+// shared memory.
 struct NearOut {
     uint8_t *masks;
     int32_t *ncols;
@@ -318,7 +319,7 @@ struct NearOut {
     int32_t *count_more;
     unsigned char *work;
 };
-size_t near_optimal_work_bytes(int k, int64_t len_sum);
+size_t near_optimal_work_bytes(int k, int64_t len_sum, int32_t max_count);
 cudaError_t launch_near_optimal(int k, int64_t len_sum, const ProblemDesc *d_prob, IODesc io, int64_t delta,
                                 int32_t max_count, NearOut o, cudaStream_t s);
 

@@ -17,7 +17,7 @@
 // exactly (and in 32 bits: every sum compared below is the score of an alignment,
 // which the encode step's range check keeps in range).
 //
-// One warp walks, and what bounds it is the chain of one node: residue codes and
+// In the depth-first form one warp walks, and what bounds it is the chain of one node: residue codes and
 // offsets from shared memory, one score per lane, a ballot. At a node every mask is
 // judged at once, a lane per mask (and 32 masks per round), and the set that
 // qualifies goes on the stack, so going back costs no judging: the lanes look 32
@@ -25,8 +25,11 @@
 // with one ballot per axis. The offset of a cell is a sum of one term per axis in
 // every layout of the scores, so the terms are tabulated per coordinate once.
 // 256 alignments of 120 x 110 x 130 (9,100 moves followed): 24.6 ms when the walk
-// went back one column at a time, judging again, with positions in local memory.
+// went back one column at a time, judging again, with positions in local memory;
+// 2.4 ms now, 0.105 ms level by level (near_beam_kernel, the form for shorter sequences).
 #include "device_common.cuh"
+
+#include <algorithm>
 
 namespace msadp {
 
@@ -245,6 +248,237 @@ __global__ void __launch_bounds__(kNearThreads) near_optimal_kernel(const Proble
     }
 }
 
+// The same enumeration level by level: every partial alignment that qualifies leads to
+// at least one alignment, so of the partial alignments of d columns, in order, only the
+// first max_count can be the start of one of the first max_count alignments. They are
+// kept as slots in shared memory; at each level a group of 2^k lanes per slot judges
+// its masks, and a count over the ballots lays the children down in order (a slot that
+// has reached the origin is carried on as it is). A level is one chain of loads, a
+// ballot and a barrier, as a node of the depth-first walk is, but takes all slots: 256
+// alignments of 120 x 110 x 130, 143 levels: 0.105 against 2.4 ms node by node. A level
+// costs more than a node, though, and the walk judges only the cells of the alignments
+// it stores, which on long sequences differ in their last few columns. So up to
+// kBeamLength residues this way (300 x 300, 30 alignments: 0.187 against 0.376 ms;
+// 120 x 110 x 130, all 660 of up to 2,000: 0.485 against 9.96) and the walk beyond (800 x
+// 700 unrelated, 90: 0.621 against 0.455 ms; 5000 x 4800, 512: 12.2 against 7.64), and
+// beyond kBeamRounds rounds of a CTA's lanes per level.
+//
+// A slot carries its last up to 8 masks packed in a word and its ancestor's slot at the
+// level the word began; every 8 levels the two go to the history, from which each
+// alignment's columns are read back at the end, 8 at a time.
+constexpr int kBeamThreads = 1024, kBeamRounds = 16, kBeamLength = 1024;
+__host__ __device__ constexpr int beam_group(int K) { return K < 5 ? 1 << K : 32; }  // lanes judging a slot
+__host__ __device__ constexpr int beam_slots(int K) { return kBeamThreads / beam_group(K); }  // slots a round takes
+__host__ __device__ constexpr int beam_words(int K) { return (K + 4) | 1; }  // position, score, ancestor, two words of masks (odd: no bank conflicts)
+__host__ __device__ constexpr size_t beam_history_rows(int64_t len_sum) { return (size_t)len_sum / 8 + 1; }
+size_t beam_tables(int k, int64_t len_sum) { return ((size_t)len_sum + k) * 8 + (((size_t)len_sum + 15) & ~(size_t)15) + 16; }
+size_t beam_state(int k, int32_t max_count) { return (size_t)2 * beam_words(k) * max_count * 4; }
+bool beam_fits(int k, int64_t len_sum, int32_t max_count) {
+    return max_count <= kBeamRounds * beam_slots(k) && len_sum <= kBeamLength &&
+           beam_tables(k, len_sum) + beam_state(k, max_count) <= (size_t)kNearSmem;
+}
+
+template <int K>
+__global__ void __launch_bounds__(kBeamThreads) near_beam_kernel(const ProblemDesc *probs, IODesc io, int64_t delta,
+                                                                 int32_t max_count, NearOut o) {
+    constexpr int NW = near_words(K), NM = 1 << K, NP = K * (K - 1) / 2;
+    constexpr int GW = beam_group(K), SPW = 32 / GW, NS = beam_words(K);
+    extern __shared__ __align__(16) unsigned char near_smem[];
+    __shared__ int sub[MSA_MAX_ALPHABET * MSA_MAX_ALPHABET];
+    __shared__ int counts[2][32];
+    __shared__ int dead;  // a slot away from the origin that no move leads on from
+    const ProblemDesc &P = probs[0];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    int nthreads = blockDim.x, nwarps = nthreads / 32;
+    const int A = P.A, total = P.len_sum;
+    if (ld_volatile(&P.istat->status) != 0) {  // the fill did not complete: nothing to enumerate
+        if (tid < 2) o.count_more[tid] = 0;
+        return;
+    }
+    int64_t *off = reinterpret_cast<int64_t *>(near_smem);
+    int *state = reinterpret_cast<int *>(off + total + K);
+    uint8_t *codes = reinterpret_cast<uint8_t *>(state + 2 * (size_t)NS * max_count);
+    int cofs[K], at[K];
+#pragma unroll
+    for (int i = 0; i < K; ++i) {
+        cofs[i] = P.cofs[i];
+        at[i] = cofs[i] + i;
+        for (int v = tid; v < P.rho[i]; v += nthreads) off[at[i] + v] = axis_offset(P, i, v);
+    }
+    for (int c = tid; c < total; c += nthreads) codes[c] = P.codes[c];
+    for (int c = tid; c < A * A; c += nthreads) sub[c] = io.subst[c];
+    if (tid < 64) counts[tid >> 5][lane] = 0;
+    auto slot_words = [&](int buf, int slot) { return state + (buf * max_count + slot) * NS; };
+    if (tid == 0) {
+        dead = 0;
+        for (int w = 0; w < NS; ++w) state[w] = w < K ? P.len[w] : 0;
+    }
+    __syncthreads();
+
+    if (max_count <= SPW) {  // one warp takes every level
+        if (warp > 0) return;
+        nthreads = 32, nwarps = 1;
+    }
+    const int gap = io.gap, u = gap * (K - 1);
+    const int32_t *Q = P.Q;
+    int thr;
+    {
+        int S = 0, W = 0;
+        int64_t corner = 0;
+#pragma unroll
+        for (int i = 0; i < K; ++i) {
+            S += P.len[i];
+            W += P.len[i] << i;
+            corner += off[at[i] + P.len[i]];
+        }
+        const int opt = ((Q[corner] - W) >> K) + u * S;
+        thr = delta > (int64_t)opt - INT32_MIN ? INT32_MIN : (int)(opt - delta);
+    }
+    uint64_t *hwords = reinterpret_cast<uint64_t *>(o.work);
+    int32_t *hprev = reinterpret_cast<int32_t *>(hwords + beam_history_rows(total) * max_count);
+    int n = 1, level = 0, more_left = 0, cur = 0, cb = 0;
+    // (every level but the last lowers the sum of every unfinished slot's coordinates)
+    while (level <= total) {
+        int base = 0, live = 0, more = 0;
+        const bool flush = (level & 7) == 7;
+        for (int s0 = 0; s0 < n && !more; s0 += nwarps * SPW) {
+            const int first = s0 + warp * SPW, slot = first + lane / GW;
+            unsigned mine[NW];
+            int sps[NW];
+            int x[K], acc = 0, S = 0, cnt = 0;
+#pragma unroll
+            for (int w = 0; w < NW; ++w) mine[w] = 0;
+            if (first < n) {
+                const int *st = slot_words(cur, min(slot, n - 1));
+                int W = 0, open = 0, code[K];
+#pragma unroll
+                for (int i = 0; i < K; ++i) {
+                    x[i] = st[i];
+                    S += x[i];
+                    W += x[i] << i;
+                    open |= (x[i] > 0) << i;
+                    code[i] = codes[min(cofs[i] + max(x[i] - 1, 0), total - 1)];  // at x_i = 0 unused, but a code
+                }
+                acc = st[K];
+                int pair[NP];
+                {
+                    int p = 0;
+#pragma unroll
+                    for (int i = 0; i < K; ++i)
+#pragma unroll
+                        for (int j = i + 1; j < K; ++j) pair[p++] = sub[code[i] * A + code[j]] - 2 * gap;
+                }
+#pragma unroll
+                for (int w = 0; w < NW; ++w) {
+                    const int m = 32 * w + lane % GW;
+                    const bool ok = slot < n && m > 0 && m < NM && (m & ~open) == 0;
+                    int sp = u * __popc(m);
+                    int p = 0;
+                    int64_t g = 0;
+#pragma unroll
+                    for (int i = 0; i < K; ++i) {
+                        const int bi = (m >> i) & 1;
+                        g += off[at[i] + x[i] - (ok ? bi : 0)];
+#pragma unroll
+                        for (int j = i + 1; j < K; ++j, ++p)
+                            if (bi & (m >> j)) sp += pair[p];
+                    }
+                    sps[w] = sp;
+                    bool hit = false;
+                    if (ok) {
+                        const int h = ((Q[g] - (W - m)) >> K) + u * (S - __popc(m));
+                        hit = h + sp + acc >= thr;
+                        live |= hit;
+                    } else if (m == 0 && slot < n) {
+                        hit = S == 0;  // finished: carried on
+                    }
+                    mine[w] = __ballot_sync(kFull, hit);
+                    cnt += __popc(mine[w]);
+                }
+                unsigned any = 0;
+#pragma unroll
+                for (int w = 0; w < NW; ++w) any |= mine[w] >> (lane & ~(GW - 1));
+                if (slot < n && (any & (GW == 32 ? kFull : (1u << GW % 32) - 1)) == 0) dead = 1;
+            }
+            if (lane == 0) counts[cb][warp] = cnt;
+            __syncthreads();
+            const int c = counts[cb][lane];
+            int idx = base + (int)__reduce_add_sync(kFull, (unsigned)(lane < warp ? c : 0));
+            base += (int)__reduce_add_sync(kFull, (unsigned)c);
+            cb ^= 1;
+            more = base > max_count || (base == max_count && s0 + nwarps * SPW < n);
+            if (cnt == 0) continue;
+#pragma unroll
+            for (int w = 0; w < NW; ++w) {
+                const int i0 = idx + __popc(mine[w] & ((1u << lane) - 1));
+                idx += __popc(mine[w]);
+                if (!((mine[w] >> lane) & 1) || i0 >= max_count) continue;
+                const int m = 32 * w + lane % GW;
+                const int *st = slot_words(cur, slot);
+                int *child = slot_words(cur ^ 1, i0);
+#pragma unroll
+                for (int i = 0; i < K; ++i) child[i] = x[i] - ((m >> i) & 1);
+                child[K] = acc + (m ? sps[w] : 0);
+                uint2 packed = make_uint2((unsigned)st[K + 2], (unsigned)st[K + 3]);
+                const unsigned put = (unsigned)m << 8 * (level & 3);
+                if (level & 4)
+                    packed.y |= put;
+                else
+                    packed.x |= put;
+                int from = st[K + 1];
+                if (flush) {
+                    const size_t h = (size_t)(level >> 3) * max_count + i0;
+                    hwords[h] = (uint64_t)packed.y << 32 | packed.x;
+                    hprev[h] = from;
+                    packed = make_uint2(0, 0);
+                    from = i0;
+                }
+                child[K + 1] = from;
+                child[K + 2] = (int)packed.x;
+                child[K + 3] = (int)packed.y;
+            }
+        }
+        n = min(base, max_count);
+        cur ^= 1;
+        ++level;
+        more_left |= more;
+        if (!__syncthreads_or(live)) break;
+    }
+    // every slot stands at the origin: its columns, first (the last move) to last
+    for (int slot = tid; slot < n; slot += nthreads) {
+        uint8_t *dst = o.masks + (int64_t)slot * total;
+        const int *st = slot_words(cur, slot);
+        uint64_t w = (uint64_t)(unsigned)st[K + 3] << 32 | (unsigned)st[K + 2];
+        int from = st[K + 1], c = 0;
+        for (int row = (level >> 3) - 1;; --row) {
+            for (; w; w <<= 8)
+                if (w >> 56) dst[c++] = (uint8_t)(w >> 56);
+            if (row < 0) break;
+            const size_t h = (size_t)row * max_count + from;
+            w = hwords[h];
+            from = hprev[h];
+        }
+        o.ncols[slot] = c;
+        o.scores[slot] = st[K];
+    }
+    if (tid == 0) {
+        o.count_more[0] = n;
+        o.count_more[1] = dead ? 2 : more_left;  // 2: an inconsistent tensor
+    }
+}
+
+template <int K>
+cudaError_t launch_beam(const ProblemDesc *d_prob, IODesc io, int64_t delta, int64_t len_sum, int32_t max_count, NearOut o,
+                        cudaStream_t s) {
+    cudaError_t e = cudaFuncSetAttribute(near_beam_kernel<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, kNearSmem);
+    if (e != cudaSuccess) return e;
+    // as many warps as a level may fill (eight at least, for the tables and the columns)
+    const int warps = std::min(kBeamThreads / 32, std::max(8, (max_count * beam_group(K) + 31) / 32));
+    near_beam_kernel<K><<<1, 32 * warps, beam_tables(K, len_sum) + beam_state(K, max_count), s>>>(d_prob, io, delta,
+                                                                                                 max_count, o);
+    return cudaGetLastError();
+}
+
 template <int K>
 cudaError_t launch_near(const ProblemDesc *d_prob, IODesc io, int64_t delta, int32_t max_count, NearOut o, size_t bytes,
                         cudaStream_t s) {
@@ -257,7 +491,8 @@ cudaError_t launch_near(const ProblemDesc *d_prob, IODesc io, int64_t delta, int
 
 }  // namespace
 
-size_t near_optimal_work_bytes(int k, int64_t len_sum) {
+size_t near_optimal_work_bytes(int k, int64_t len_sum, int32_t max_count) {
+    if (beam_fits(k, len_sum, max_count)) return beam_history_rows(len_sum) * max_count * 12;
     const size_t b = near_bytes(k, len_sum);
     return b <= (size_t)kNearSmem ? 0 : b;
 }
@@ -265,6 +500,15 @@ size_t near_optimal_work_bytes(int k, int64_t len_sum) {
 cudaError_t launch_near_optimal(int k, int64_t len_sum, const ProblemDesc *d_prob, IODesc io, int64_t delta,
                                 int32_t max_count, NearOut o, cudaStream_t s) {
     const size_t bytes = near_bytes(k, len_sum);
+    if (beam_fits(k, len_sum, max_count)) switch (k) {
+            case 2: return launch_beam<2>(d_prob, io, delta, len_sum, max_count, o, s);
+            case 3: return launch_beam<3>(d_prob, io, delta, len_sum, max_count, o, s);
+            case 4: return launch_beam<4>(d_prob, io, delta, len_sum, max_count, o, s);
+            case 5: return launch_beam<5>(d_prob, io, delta, len_sum, max_count, o, s);
+            case 6: return launch_beam<6>(d_prob, io, delta, len_sum, max_count, o, s);
+            case 7: return launch_beam<7>(d_prob, io, delta, len_sum, max_count, o, s);
+            case 8: return launch_beam<8>(d_prob, io, delta, len_sum, max_count, o, s);
+        }
     switch (k) {
         case 2: return launch_near<2>(d_prob, io, delta, max_count, o, bytes, s);
         case 3: return launch_near<3>(d_prob, io, delta, max_count, o, bytes, s);

@@ -82,3 +82,16 @@ def test_more_masks_than_lanes(lens):
 def test_stack_beyond_shared_memory():
     """Sequences whose tables and stack do not fit in shared memory (kept in global memory)."""
     check(inputs.random_problem(8600, 2, [4700, 4650], alphabet=inputs.PROTEIN, related=True), 2, 40)
+
+
+@pytest.mark.parametrize("max_count", [1, 4, 5, 127, 128, 129, 2047, 2048, 2049])
+def test_level_by_level_and_walk_caps(max_count):
+    """k = 3: one below, at and above the slots of a warp, of a round of the CTA's lanes and of the most
+    rounds a level takes (the depth-first walk beyond)."""
+    check(inputs.random_problem(8700, 3, [9, 8, 10], table=PAPER_TABLE, gap=-1), 5, max_count)
+
+
+@pytest.mark.parametrize("lens", [(512, 512), (512, 513), (1020, 4), (0, 1024)])
+def test_level_by_level_longest(lens):
+    """The longest sequences that go level by level, and one residue more."""
+    check(inputs.random_problem(8800, 2, list(lens), alphabet=inputs.PROTEIN, related=True), 1, 20)
