@@ -81,8 +81,9 @@ int msa_align(int k, const char *const *seqs, const int32_t *lens, const char *a
  * Every alignment scoring at least OPT - delta (delta >= 0; delta = 0: every
  * optimal alignment), the further optimal and near-optimal solutions the paper
  * proposes to retrieve by forking at equally ranked paths or within a user
- * threshold (section 6). The fill keeps every cell's score (the generic tile
- * kernel); a walk on the device from the far corner follows a move only when the
+ * threshold (section 6). The fill keeps every cell's score (the band and column
+ * kernels in a form that does, or the generic tile kernel); a walk on the device
+ * from the far corner follows a move only when the
  * best completion through its predecessor still reaches OPT - delta, trying the
  * moves of each column in increasing mask order, so alignments come in
  * increasing lexicographic order of their reversed column sequence (for

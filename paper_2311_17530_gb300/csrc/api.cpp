@@ -172,6 +172,7 @@ size_t plan_layout(const HostPlan &hp, char *base, PlanPointers *pp, size_t *res
     char *tb = take((size_t)hp.tb_dev_bytes + 16);
     char *Q = take((size_t)hp.qelems * 4 + 16);
     char *aux = take((size_t)hp.aux_elems * 4 + 16);
+    char *kept = take(hp.keep ? (size_t)hp.kept_elems * 4 + 16 : 0);
     if (pp && base) {
         LaunchState *ls = reinterpret_cast<LaunchState *>(hdr);
         pp->state = ls;
@@ -185,6 +186,7 @@ size_t plan_layout(const HostPlan &hp, char *base, PlanPointers *pp, size_t *res
         pp->tb = reinterpret_cast<uint8_t *>(tb);
         pp->Q = reinterpret_cast<int32_t *>(Q);
         pp->aux = reinterpret_cast<int32_t *>(aux);
+        pp->kept = hp.keep ? reinterpret_cast<int32_t *>(kept) : nullptr;
     }
     return off;
 }
@@ -228,6 +230,7 @@ void fill_problem_desc(const HostPlan &hp, const PlanPointers &pp, int64_t tile_
     d.Q = pp.Q;
     d.aux = pp.aux;
     d.tb = pp.tb;
+    d.kept = pp.kept;
     d.qcorner = pp.qcorner;
     d.istat = &pp.state->istat;
 }
@@ -329,7 +332,8 @@ int msa_plan_create(int k, const int32_t *lens, const char *alphabet, msa_plan *
 
 namespace msadp {
 
-int plan_create(int k, const int32_t *lens, const char *alphabet, int kernel_choice, int edge, msa_plan **out_plan) {
+int plan_create(int k, const int32_t *lens, const char *alphabet, int kernel_choice, int edge, msa_plan **out_plan,
+                bool keep_scores) {
     if (!out_plan) return set_error(MSA_EINVAL, "out_plan is NULL");
     *out_plan = nullptr;
     uint8_t amap[256];
@@ -344,9 +348,10 @@ int plan_create(int k, const int32_t *lens, const char *alphabet, int kernel_cho
         delete p;
         return set_error(rc, "%s", err.c_str());
     }
+    p->hp.keep = keep_scores;
     {
         std::lock_guard<std::mutex> g(settings_mutex());
-        p->hp.check_corner = p->hp.kernel != kKernelCol3 || settings().verify_corner ? 1 : 0;
+        p->hp.check_corner = p->hp.kernel != kKernelCol3 || keep_scores || settings().verify_corner ? 1 : 0;
     }
     strncpy(p->alphabet, alphabet, MSA_MAX_ALPHABET);
     p->ws_bytes = plan_layout(p->hp, nullptr, nullptr, &p->reset_bytes);
@@ -425,6 +430,7 @@ int msa_plan_execute(msa_plan *plan, const char *d_residues, const int32_t *d_su
     L.nprob = 1;
     L.tab_ints = plan->hp.A * (plan->hp.A + 1);  // table plus the sentinel column
     L.corner = plan->hp.check_corner;
+    L.keep = plan->hp.keep;
     if (tagged_faces(plan->hp)) {
         if (plan->epoch >= 32767) {  // column kernel tags (epoch << 16) + T would wrap: start over from cleared faces
             e = clear_faces(plan->hp, plan->pp, s);
@@ -655,34 +661,56 @@ int msa_near_optimal(int k, const char *const *seqs, const int32_t *lens, const 
     if (rc) return rc;
     if (delta < 0 || max_count < 1 || !out_masks || !out_ncols || !out_scores || !out_count || !out_more)
         return set_error(MSA_EINVAL, "delta < 0, max_count < 1 or a NULL output pointer");
-    // the generic tile kernel keeps every cell's score, which the walk reads
-    msa_plan *plan = nullptr;
-    rc = plan_create(k, lens, alphabet, kKernelTiles, -1, &plan);
-    if (rc) return rc;
-    const int A = plan->hp.A;
-    const size_t total = (size_t)plan->hp.len_sum;
-    if ((double)max_count * (double)(total + 1) > (double)(1LL << 36)) {
-        msa_plan_destroy(plan);
-        return set_error(MSA_ETOOBIG, "max_count x (sum of lengths) is beyond the supported output size");
+    // A kernel that keeps every cell's score, which the walk reads: for k = 2, 3 the band
+    // and column kernels where they are the choice for one alignment (120 x 110 x 130:
+    // 0.089 against 0.89 ms of the generic tile kernel, 800 x 760: 0.110 against 1.35), unless
+    // their layouts' padding doubles the scores; else, and where memory does not hold
+    // both, the generic tile kernel.
+    const size_t A = strlen(alphabet);
+    int keep = kKernelTiles;
+    if (k <= 3) {
+        HostPlan shape;
+        std::string err;
+        if (plan_shape(k, lens, (int)A, kKernelAuto, shape, err) == MSA_OK &&
+            shape.kept_elems <= 2 * shape.cells + (16 << 20))
+            keep = shape.kernel;
     }
-    // one device buffer: inputs, the single-alignment outputs, the enumeration's
-    // outputs and its stack
-    size_t off = 0;
-    auto take = [&](size_t bytes) {
-        const size_t o = off;
-        off = (off + bytes + 255) & ~(size_t)255;
-        return o;
-    };
-    const size_t o_res = take(total + 16), o_sub = take((size_t)A * A * 4), o_out = take(sizeof(msa_device_result)),
-                 o_mask1 = take(total + 16), o_masks = take((size_t)max_count * total + 16),
-                 o_ncols = take((size_t)max_count * 4), o_scores = take((size_t)max_count * 8), o_cm = take(8),
-                 o_work = take(near_optimal_work_bytes(k, (int64_t)total, max_count));
+    msa_plan *plan = nullptr;
+    size_t total = 0, o_res = 0, o_sub = 0, o_out = 0, o_mask1 = 0, o_masks = 0, o_ncols = 0, o_scores = 0, o_cm = 0,
+           o_work = 0;
     char *d = nullptr;
-    cudaError_t e = cudaMalloc(&d, off);
-    if (e != cudaSuccess) {
+    cudaError_t e = cudaSuccess;
+    for (int kernel = keep;; kernel = kKernelTiles) {
+        rc = plan_create(k, lens, alphabet, kernel, -1, &plan, kernel != kKernelTiles);
+        if (rc == MSA_ENOMEM && kernel != kKernelTiles) continue;
+        if (rc) return rc;
+        total = (size_t)plan->hp.len_sum;
+        if ((double)max_count * (double)(total + 1) > (double)(1LL << 36)) {
+            msa_plan_destroy(plan);
+            return set_error(MSA_ETOOBIG, "max_count x (sum of lengths) is beyond the supported output size");
+        }
+        // one device buffer: inputs, the single-alignment outputs, the enumeration's
+        // outputs and its history or stack
+        size_t off = 0;
+        auto take = [&](size_t bytes) {
+            const size_t o = off;
+            off = (off + bytes + 255) & ~(size_t)255;
+            return o;
+        };
+        o_res = take(total + 16);
+        o_sub = take(A * A * 4);
+        o_out = take(sizeof(msa_device_result));
+        o_mask1 = take(total + 16);
+        o_masks = take((size_t)max_count * total + 16);
+        o_ncols = take((size_t)max_count * 4);
+        o_scores = take((size_t)max_count * 8);
+        o_cm = take(8);
+        o_work = take(near_optimal_work_bytes(k, (int64_t)total, max_count));
+        e = cudaMalloc(&d, off);
+        if (e == cudaSuccess) break;
         cudaGetLastError();
         msa_plan_destroy(plan);
-        return set_error(MSA_ENOMEM, "near-optimal buffers: %s", cudaGetErrorString(e));
+        if (kernel == kKernelTiles) return set_error(MSA_ENOMEM, "near-optimal buffers: %s", cudaGetErrorString(e));
     }
     std::vector<char> res(total + 1);
     size_t o = 0;

@@ -39,6 +39,7 @@ struct PlanPointers {
     uint8_t *amap = nullptr;
     uint8_t *codes = nullptr;
     int32_t *tab = nullptr;
+    int32_t *kept = nullptr;
     int32_t *qcorner = nullptr;
     uint8_t *tb = nullptr;
     int32_t *Q = nullptr;
@@ -58,7 +59,9 @@ int validate_request(int k, const char *const *seqs, const int32_t *lens, const 
 int status_error(int status);
 int persistent_grid(int k, int kernel, int64_t units, int A, int edge);
 // msa_plan_create with an explicit kernel choice and tile edge (edge < 0: tuned).
-int plan_create(int k, const int32_t *lens, const char *alphabet, int kernel_choice, int edge, msa_plan **out_plan);
+// keep_scores (column and band kernels): the fill keeps every cell's score.
+int plan_create(int k, const int32_t *lens, const char *alphabet, int kernel_choice, int edge, msa_plan **out_plan,
+                bool keep_scores = false);
 size_t plan_layout(const HostPlan &hp, char *base, PlanPointers *pp, size_t *reset_bytes);
 void fill_problem_desc(const HostPlan &hp, const PlanPointers &pp, int64_t tile_base, ProblemDesc &d);
 int launch_fill(const HostPlan &hp, const LaunchDesc &L, int grid, cudaStream_t s);

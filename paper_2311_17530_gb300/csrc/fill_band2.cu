@@ -116,6 +116,11 @@ __device__ __forceinline__ void band_tile(BandState &g, const int (&t)[4][R], co
                   0x03030303u;
 }
 
+// KEEP: every cell's best candidate, V plus tag, is kept for the near-optimal walk, by
+// step, row of the lane and lane (band2_kept_term): each 16-byte store of a warp is one
+// run (row-major, a line per lane, 5000 x 4800 took 1.83 against 0.69 ms; the fill without
+// KEEP 0.54).
+template <bool KEEP>
 __global__ void __launch_bounds__(kBandWarps * 32) fill_band2_kernel(const LaunchDesc L) {
     __shared__ BandSmem sms[kBandWarps];
     const int lane = threadIdx.x & 31;
@@ -170,6 +175,10 @@ __global__ void __launch_bounds__(kBandWarps * 32) fill_band2_kernel(const Launc
 #pragma unroll
         for (int q = 0; q < R; ++q)
             tbp[q] = P.tb + (int64_t)(i0 + q < rho0 ? i0 + q : 0) * P.tbstride[0] - 4 * lane;  // + 4 t: this lane's group
+        int *kept = KEEP ? P.kept + (int64_t)band * band2_kept_steps(rho1) * (128 * R) + lane * 4 : nullptr;
+        auto keep = [&](int q, int t, const int (&v)[4]) {
+            *reinterpret_cast<int4 *>(kept + (int64_t)t * (128 * R) + q * 128) = make_int4(v[0], v[1], v[2], v[3]);
+        };
         bool row_in[R];
 #pragma unroll
         for (int q = 0; q < R; ++q) row_in[q] = i0 + q < rho0;
@@ -248,7 +257,10 @@ __global__ void __launch_bounds__(kBandWarps * 32) fill_band2_kernel(const Launc
                         band_tile(g, te, up, t == 0 && band == 0, mask, acc, [&](int c, int v) { last[c] = v; });
 #pragma unroll
                         for (int q = 0; q < R; ++q)
-                            if (row_in[q]) *reinterpret_cast<uint32_t *>(tbp[q] + 4 * s) = mask[q];
+                            if (row_in[q]) {
+                                *reinterpret_cast<uint32_t *>(tbp[q] + 4 * s) = mask[q];
+                                if constexpr (KEEP) keep(q, t, acc[q]);
+                            }
                         if (grp == gc && corner_lane) {
                             int v = 0;  // a select chain: an index would put the registers in memory
 #pragma unroll
@@ -268,7 +280,10 @@ __global__ void __launch_bounds__(kBandWarps * 32) fill_band2_kernel(const Launc
                     });
 #pragma unroll
                     for (int q = 0; q < R; ++q)
-                        if (row_in[q]) *reinterpret_cast<uint32_t *>(tbp[q] + 4 * s) = mask[q];
+                        if (row_in[q]) {
+                            *reinterpret_cast<uint32_t *>(tbp[q] + 4 * s) = mask[q];
+                            if constexpr (KEEP) keep(q, t, acc[q]);
+                        }
                 }
                 if (lane == 31) *reinterpret_cast<int4 *>(&sm.below[((t - 31) >> 2) & 1][4 * ((t - 31) & 3)]) =
                     make_int4(last[0], last[1], last[2], last[3]);
@@ -296,13 +311,16 @@ __global__ void __launch_bounds__(kBandWarps * 32) fill_band2_kernel(const Launc
 }  // namespace
 
 cudaError_t launch_fill_band2(const LaunchDesc &L, int grid, cudaStream_t s) {
-    fill_band2_kernel<<<grid, kBandWarps * 32, 0, s>>>(L);
+    if (L.keep)
+        fill_band2_kernel<true><<<grid, kBandWarps * 32, 0, s>>>(L);
+    else
+        fill_band2_kernel<false><<<grid, kBandWarps * 32, 0, s>>>(L);
     return cudaGetLastError();
 }
 
 int fill_band2_ctas_per_sm() {
     int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fill_band2_kernel, kBandWarps * 32, 0) != cudaSuccess)
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fill_band2_kernel<false>, kBandWarps * 32, 0) != cudaSuccess)
         return 0;
     return n;
 }

@@ -223,6 +223,7 @@ struct C3Blk {
     unsigned long long *f1o;        // this lane's entry of F1[T0 ..][wR ..]
     const int *p02;                 // p02r[w][0][(T0 + 2 - wR - lane) mod SQ]
     const int *p12;                 // p12r[(T0 + 2 - wR) mod SP][lane]
+    int *kept;                      // kept scores of (T0, w, lane): R / 4 runs of 4 words (kernels that keep them)
 };
 
 // Every HF steps a warp handles HF x R = 32 entries, one a lane: of face F1, and of
@@ -255,7 +256,7 @@ __device__ __forceinline__ void c3_load_face(C3St &g, const int *fr, int wR) {
 // One step. Everything with a latency is started a step or more before its use:
 // the shuffles of this step's values (for the next step) as soon as they exist,
 // the staged face a step ahead, row -1 a chunk ahead with one vote per chunk.
-template <int s>
+template <int s, bool KEEP>
 __device__ __forceinline__ void c3_step(C3St &g, const C3Ln &c, const C3Fill &f, const C3Blk &b, int T0, int lane,
                                         C3Smem &sm, const LaunchDesc &L) {
     constexpr int R = c3::R, H = c3::U, M = R - 1;
@@ -302,6 +303,11 @@ __device__ __forceinline__ void c3_step(C3St &g, const C3Ln &c, const C3Fill &f,
         *reinterpret_cast<uint32_t *>(b.tbp + s * (c3::W * 32 * R)) = pk[0];
     else
         *reinterpret_cast<uint2 *>(b.tbp + s * (c3::W * 32 * R)) = make_uint2(pk[0], pk[R / 4 - 1]);
+    if constexpr (KEEP) {
+#pragma unroll
+        for (int r = 0; r < R; r += 4)
+            *reinterpret_cast<int4 *>(b.kept + s * (c3::W * 32 * R) + r * 32) = make_int4(acc[r], acc[r + 1], acc[r + 2], acc[r + 3]);
+    }
     // a p02 entry of the next block: looked up in the first of HF steps, stored in the last
     if constexpr (s % HF == 0) g.q = c3_fill_load(f, T + H);
     if constexpr (s % HF == HF - 1) c3_fill_store(f, T - HF + 1 + H, g.q);
@@ -344,10 +350,10 @@ __device__ __forceinline__ void c3_step(C3St &g, const C3Ln &c, const C3Fill &f,
 
 // A step of the block that holds the far corner's CTA time (kernels that record
 // the corner): the plain step, then the corner's lane stores its row's key.
-template <int s>
+template <int s, bool KEEP>
 __device__ __forceinline__ void c3_capture_step(C3St &g, const C3Ln &c, const C3Fill &f, const C3Blk &b, int T0,
                                                 int lane, C3Smem &sm, const LaunchDesc &L) {
-    c3_step<s>(g, c, f, b, T0, lane, sm, L);
+    c3_step<s, KEEP>(g, c, f, b, T0, lane, sm, L);
     if (T0 + s == c.ctime) {
         int v = g.V[0];  // a select chain: a loop with a dynamic index would put the registers in memory
 #pragma unroll
@@ -357,13 +363,13 @@ __device__ __forceinline__ void c3_capture_step(C3St &g, const C3Ln &c, const C3
 }
 
 // The unrolled steps of a block.
-template <bool CAP, int... S>
+template <bool CAP, bool KEEP, int... S>
 __device__ __forceinline__ void c3_steps(C3St &g, const C3Ln &c, const C3Fill &f, const C3Blk &b, int T0, int lane,
                                          C3Smem &sm, const LaunchDesc &L, std::integer_sequence<int, S...>) {
     if constexpr (CAP)
-        (c3_capture_step<S>(g, c, f, b, T0, lane, sm, L), ...);
+        (c3_capture_step<S, KEEP>(g, c, f, b, T0, lane, sm, L), ...);
     else
-        (c3_step<S>(g, c, f, b, T0, lane, sm, L), ...);
+        (c3_step<S, KEEP>(g, c, f, b, T0, lane, sm, L), ...);
 }
 
 struct C3Col {
@@ -527,8 +533,13 @@ __device__ __forceinline__ bool c3_block_wait(C3Smem &sm, const C3Ln &c, int w, 
 
 // CAP: the warp that computes the far corner records its key for the traceback's
 // cross-check; the block holding it runs a capturing copy of the steps (which
-// costs registers, so plain launches use the kernel without it).
-template <bool CAP>
+// costs registers, so plain launches use the kernel without it). KEEP: every cell's
+// best candidate, V plus tag, is kept for the near-optimal walk (c3::kept_term): the
+// traceback's layout with a word for its byte and a lane's rows in runs of four, so
+// that each 16-byte store of a warp is one run (120 x 110 x 130: 0.089 ms, 0.085 without
+// KEEP; 0.225 with CAP's second copy of the steps to record the corner, instruction
+// fetch, so the corner's lane reads its own store back instead).
+template <bool CAP, bool KEEP>
 __global__ void __launch_bounds__(c3::THREADS, c3::CTAS) fill_col3_kernel(const LaunchDesc L) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C3Smem &sm = *reinterpret_cast<C3Smem *>(smem_raw);
@@ -673,6 +684,7 @@ __global__ void __launch_bounds__(c3::THREADS, c3::CTAS) fill_col3_kernel(const 
             b.rout = ringout + (lastw ? 0 : (-c3::U & (c3::SI - 1)) * 32);
             b.f1row = &sm.f1r[-c3::U & (c3::SF - 1)][0];
             b.tbp = tbw;
+            b.kept = KEEP ? P.kept + (int64_t)lin * c3::tb_col_bytes(P.rho[2]) + w * (32 * c3::R) + lane * 4 : nullptr;
             b.f1o = cc.f1dst + (int64_t)c.f1t * c3::WR + c.wR + lane % c3::R;
             b.p02 = &sm.p02r[w][0][(-c3::U + 2 - c.wR - lane) & (c3::SQ - 1)][0];
             b.p12 = &sm.p12r[(-c3::U + 2 - c.wR) & (c3::SP - 1)][lane];
@@ -689,14 +701,22 @@ __global__ void __launch_bounds__(c3::THREADS, c3::CTAS) fill_col3_kernel(const 
                 n.rout = lastw ? b.rout + c3::U * 32 : ringout + (Tn & (c3::SI - 1)) * 32;
                 n.f1row = &sm.f1r[Tn & (c3::SF - 1)][0];
                 n.tbp = b.tbp + c3::U * (c3::W * 32 * c3::R);
+                n.kept = KEEP ? b.kept + c3::U * (c3::W * 32 * c3::R) : nullptr;
                 n.f1o = b.f1o + c3::U * c3::WR;
                 n.p02 = &sm.p02r[w][0][(Tn + 2 - c.wR - lane) & (c3::SQ - 1)][0];
                 n.p12 = &sm.p12r[(Tn + 2 - c.wR) & (c3::SP - 1)][lane];
                 if (!CAP || T0 != T0c)
-                    c3_steps<false>(g, c, f, b, T0, lane, sm, L, std::make_integer_sequence<int, c3::U>{});
+                    c3_steps<false, KEEP>(g, c, f, b, T0, lane, sm, L, std::make_integer_sequence<int, c3::U>{});
                 else
-                    c3_steps<true>(g, c, f, b, T0, lane, sm, L, std::make_integer_sequence<int, c3::U>{});
+                    c3_steps<true, KEEP>(g, c, f, b, T0, lane, sm, L, std::make_integer_sequence<int, c3::U>{});
                 b = n;
+            }
+            if constexpr (KEEP) {  // the corner's lane has its score from its own store
+                if (c.ctime != (int)0x80000000) {
+                    const int64_t at = c3::kept_term(0, P.len[0], NB, P.rho[2]) + c3::kept_term(1, P.len[1], NB, P.rho[2]) +
+                                       c3::kept_term(2, P.len[2], NB, P.rho[2]);
+                    __stcg(c.qcorner, (*reinterpret_cast<volatile int *>(P.kept + at) & ~7) + c.wcorner);
+                }
             }
             __syncwarp();
             if (lane == 0) st_release_shared(&sm.prog[w], 1 << 30);
@@ -717,11 +737,10 @@ int col3_smem_bytes(int alphabet_size) {
 cudaError_t col3_attributes() {
     static DeviceOnce once;
     return once.run([] {
-        cudaError_t e = cudaFuncSetAttribute(fill_col3_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             col3_smem_bytes(c3::MAXA));
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(fill_col3_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     col3_smem_bytes(c3::MAXA));
+        cudaError_t e = cudaSuccess;
+        for (auto kernel : {fill_col3_kernel<false, false>, fill_col3_kernel<true, false>, fill_col3_kernel<false, true>})
+            if (e == cudaSuccess)
+                e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, col3_smem_bytes(c3::MAXA));
         return e;
     });
 }
@@ -729,7 +748,7 @@ cudaError_t col3_attributes() {
 int fill_col3_ctas_per_sm(int smem) {
     if (col3_attributes() != cudaSuccess) return 0;
     int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fill_col3_kernel<false>, c3::THREADS, smem) != cudaSuccess)
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fill_col3_kernel<false, false>, c3::THREADS, smem) != cudaSuccess)
         return 0;
     return n;
 }
@@ -738,10 +757,12 @@ cudaError_t launch_fill_col3(const LaunchDesc &L, int grid, int smem, cudaStream
     cudaError_t e = col3_attributes();
     if (e != cudaSuccess) return e;
     if (smem > col3_smem_bytes(c3::MAXA)) return cudaErrorInvalidValue;
-    if (L.corner)
-        fill_col3_kernel<true><<<grid, c3::THREADS, smem, s>>>(L);
+    if (L.keep)
+        fill_col3_kernel<false, true><<<grid, c3::THREADS, smem, s>>>(L);
+    else if (L.corner)
+        fill_col3_kernel<true, false><<<grid, c3::THREADS, smem, s>>>(L);
     else
-        fill_col3_kernel<false><<<grid, c3::THREADS, smem, s>>>(L);
+        fill_col3_kernel<false, false><<<grid, c3::THREADS, smem, s>>>(L);
     return cudaGetLastError();
 }
 

@@ -69,6 +69,8 @@ struct ProblemDesc {
     uint8_t *tb;                 // traceback tensor
     int32_t *qcorner;            // packed key of the far corner
     msa_device_result *istat;    // internal status block (reset before every run)
+    int32_t *kept;               // column and band kernels that keep every cell's score: H' shifted by k plus
+                                 // a tag (c3::kept_term, band2_kept_term; nullptr: faces only)
     const uint8_t *skip;         // generic tile kernel: per tile, nonzero = left out by the
                                  // pruning bound (nullptr: every tile is filled)
 };
@@ -97,6 +99,7 @@ struct LaunchDesc {
     int32_t tab_ints;        // column kernel: shared-memory ints of the replicated table
     int32_t epoch;           // column and streamed line kernels: tag of this launch's face entries (>= 1)
     int32_t corner;          // column kernel: record the far corner's key (the traceback checks it)
+    int32_t keep;            // column and band kernels: keep every cell's score (ProblemDesc::kept)
 };
 
 // Tile shapes of the generic kernel. A shape is named by its edge E: the tile
@@ -200,6 +203,15 @@ __host__ __device__ constexpr int stream_face_lines(int K) {  // lines of a supe
 
 // k = 2 band kernel: rows per lane (a band is 32 of them per lane, 32 lanes).
 constexpr int kBand2RowsPerLane = 4;
+// Kept scores of a band: by step (lanes skewed by one group of four columns), row of the
+// lane, lane and column of the group; a sum of one term per axis.
+__host__ __device__ constexpr int64_t band2_kept_steps(int rho1) { return (rho1 + 15) / 16 * 4 + 31; }
+__host__ __device__ constexpr int64_t band2_kept_term(int axis, int v, int rho1) {
+    constexpr int R = kBand2RowsPerLane;
+    const int lane = v / R % 32;
+    return axis == 0 ? v / (32 * R) * band2_kept_steps(rho1) * (128 * R) + lane * (128 * R + 4) + v % R * 128
+                     : (int64_t)(v / 4) * (128 * R) + v % 4;
+}
 
 // k = 3 column kernel geometry (shared by the planner and the kernel).
 //
@@ -250,6 +262,16 @@ __host__ __device__ constexpr int face1_rows(int rho2) { return nsteps(rho2) + U
 // R bytes. A byte is the tag of the winning move (fill_col3.cu): tags 7 5 4 3 2 1 0
 // are the masks 1 .. 7, tag 6 is no move; the origin's byte is not read.
 __host__ __device__ constexpr int mask_of_tag(int t) { return t == 7 ? 1 : t == 6 ? 0 : 7 - t; }
+// Kept scores: (((T + U)*W + w)*R/4 + r / 4)*128 + l*4 + r mod 4 words into the column's
+// tb_col_bytes words, a sum of one term per axis (G1: columns along axis 1).
+__host__ __device__ constexpr int64_t tb_col_bytes(int rho2);
+__host__ __device__ constexpr int64_t kept_term(int axis, int v, int G1, int rho2) {
+    constexpr int64_t time = W * 32 * R;
+    const int rho = v % WR, r = rho % R;
+    return axis == 0   ? v / WR * G1 * tb_col_bytes(rho2) + rho * time + rho / R * (32 * R) + r / 4 * 128 + r % 4
+           : axis == 1 ? v / 32 * tb_col_bytes(rho2) + v % 32 * (time + 4)
+                       : (v + U) * time;
+}
 __host__ __device__ constexpr int64_t tb_col_bytes(int rho2) { return (int64_t)(nsteps(rho2) + U) * W * 32 * R; }
 }  // namespace c3
 

@@ -11,11 +11,13 @@
 // H being the forward tensor: H(p) is the best any completion through p can add,
 // so every qualifying alignment is reached and no other one is produced.
 //
-// The fill is the generic tile kernel, which keeps the packed key of every cell:
+// The fill is the column or band kernel in the form that keeps every cell's score, or
+// the generic tile kernel, which keeps the packed key of every cell:
 // Q(x) = H'(x) 2^k + W(x) with H'(x) = H(x) - gap (k - 1) |x|_1 and
 // W(x) = sum_i 2^i x_i, so H(x) = (Q(x) - W(x)) / 2^k + gap (k - 1) |x|_1
 // exactly (and in 32 bits: every sum compared below is the score of an alignment,
-// which the encode step's range check keeps in range).
+// which the encode step's range check keeps in range). The other two keep
+// H'(x) 2^k plus a tag below 2^k, so there W is left out.
 //
 // In the depth-first form one warp walks, and what bounds it is the chain of one node: residue codes and
 // offsets from shared memory, one score per lane, a ballot. At a node every mask is
@@ -26,7 +28,8 @@
 // every layout of the scores, so the terms are tabulated per coordinate once.
 // 256 alignments of 120 x 110 x 130 (9,100 moves followed): 24.6 ms when the walk
 // went back one column at a time, judging again, with positions in local memory;
-// 2.4 ms now, 0.105 ms level by level (near_beam_kernel, the form for shorter sequences).
+// 2.4 ms now, and level by level less again (near_beam_kernel, the form for shorter
+// sequences).
 #include "device_common.cuh"
 
 #include <algorithm>
@@ -39,8 +42,10 @@ constexpr int kNearThreads = 256;
 constexpr int kNearSmem = 160 * 1024;  // tables and stack beyond this stay in global memory
 
 // Term of coordinate v of axis i in the element offset of a cell's score: row-major
-// (qstride) for k <= 3, tile-major (the traceback's layout 2) for k >= 4.
+// (qstride) for k <= 3, tile-major (the traceback's layout 2) for k >= 4; the layouts of
+// the kernels that keep scores.
 __device__ __forceinline__ int64_t axis_offset(const ProblemDesc &P, int i, int v) {
+    if (P.kept) return P.k == 2 ? band2_kept_term(i, v, P.rho[1]) : c3::kept_term(i, v, P.G[1], P.rho[2]);
     if (P.tb_layout != 2) return (int64_t)v * P.qstride[i];
     const int q = v / P.E[i];
     return (int64_t)q * P.gstride[i] * P.tb_block + (int64_t)(v - q * P.E[i]) * P.lst[i];
@@ -101,8 +106,9 @@ __global__ void __launch_bounds__(kNearThreads) near_optimal_kernel(const Proble
         W += x[i] << i;
         corner += off[at[i] + x[i]];
     }
-    const int32_t *Q = P.Q;
-    const int opt = ((Q[corner] - W) >> K) + u * S;
+    const int32_t *Q = P.kept ? P.kept : P.Q;
+    const int withw = P.kept ? 0 : -1;  // the scores' W part
+    const int opt = ((Q[corner] - (W & withw)) >> K) + u * S;
     // OPT - delta (no alignment scores below the 32-bit range)
     const int thr = delta > (int64_t)opt - INT32_MIN ? INT32_MIN : (int)(opt - delta);
     int d = 0, count = 0, more = 0;
@@ -160,7 +166,7 @@ __global__ void __launch_bounds__(kNearThreads) near_optimal_kernel(const Proble
                 }
                 bool hit = false;
                 if (ok) {
-                    const int h = ((Q[g] - (W - m)) >> K) + u * (S - __popc(m));
+                    const int h = ((Q[g] - ((W - m) & withw)) >> K) + u * (S - __popc(m));
                     hit = h + sp + acc >= thr;
                 }
                 mine[w] = __ballot_sync(kFull, hit);
@@ -255,7 +261,7 @@ __global__ void __launch_bounds__(kNearThreads) near_optimal_kernel(const Proble
 // its masks, and a count over the ballots lays the children down in order (a slot that
 // has reached the origin is carried on as it is). A level is one chain of loads, a
 // ballot and a barrier, as a node of the depth-first walk is, but takes all slots: 256
-// alignments of 120 x 110 x 130, 143 levels: 0.105 against 2.4 ms node by node. A level
+// alignments of 120 x 110 x 130, 143 levels: 0.263 against 3.62 ms node by node. A level
 // costs more than a node, though, and the walk judges only the cells of the alignments
 // it stores, which on long sequences differ in their last few columns. So up to
 // kBeamLength residues this way (300 x 300, 30 alignments: 0.187 against 0.376 ms;
@@ -320,7 +326,8 @@ __global__ void __launch_bounds__(kBeamThreads) near_beam_kernel(const ProblemDe
         nthreads = 32, nwarps = 1;
     }
     const int gap = io.gap, u = gap * (K - 1);
-    const int32_t *Q = P.Q;
+    const int32_t *Q = P.kept ? P.kept : P.Q;
+    const int withw = P.kept ? 0 : -1;  // the scores' W part
     int thr;
     {
         int S = 0, W = 0;
@@ -331,7 +338,7 @@ __global__ void __launch_bounds__(kBeamThreads) near_beam_kernel(const ProblemDe
             W += P.len[i] << i;
             corner += off[at[i] + P.len[i]];
         }
-        const int opt = ((Q[corner] - W) >> K) + u * S;
+        const int opt = ((Q[corner] - (W & withw)) >> K) + u * S;
         thr = delta > (int64_t)opt - INT32_MIN ? INT32_MIN : (int)(opt - delta);
     }
     uint64_t *hwords = reinterpret_cast<uint64_t *>(o.work);
@@ -386,7 +393,7 @@ __global__ void __launch_bounds__(kBeamThreads) near_beam_kernel(const ProblemDe
                     sps[w] = sp;
                     bool hit = false;
                     if (ok) {
-                        const int h = ((Q[g] - (W - m)) >> K) + u * (S - __popc(m));
+                        const int h = ((Q[g] - ((W - m) & withw)) >> K) + u * (S - __popc(m));
                         hit = h + sp + acc >= thr;
                         live |= hit;
                     } else if (m == 0 && slot < n) {

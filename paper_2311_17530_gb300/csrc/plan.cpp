@@ -372,6 +372,7 @@ int plan_shape(int k, const int32_t *lens, int A, int kernel_choice, HostPlan &h
         // (value, tag) entries of two words
         hp.face0_stride = 2 * round_up64(hp.rho[1], 32);
         hp.qelems = hp.ntiles * hp.face0_stride;
+        hp.kept_elems = hp.ntiles * band2_kept_steps(hp.rho[1]) * (128 * kBand2RowsPerLane);
     }
 
     if (hp.kernel == kKernelCol3) {  // faces between columns
@@ -383,7 +384,7 @@ int plan_shape(int k, const int32_t *lens, int A, int kernel_choice, HostPlan &h
         hp.qelems = nt * hp.face0_stride;
         hp.aux_elems = nt * hp.face1_stride;
         hp.tb_layout = 1;
-        hp.tb_dev_bytes = nt * c3::tb_col_bytes(rho2);
+        hp.tb_dev_bytes = hp.kept_elems = nt * c3::tb_col_bytes(rho2);
     }
     return MSA_OK;
 }

@@ -52,6 +52,8 @@ struct HostPlan {
     int32_t edge = 0;              // tile edge of the generic kernel (tile_ext); longest segment of the
                                    // line kernel; 0 for the column and band kernels
     bool wide = false;             // streamed line kernel: its whole-column form
+    bool keep = false;             // column and band kernels: every cell's score is kept
+    int64_t kept_elems = 0;        // words these scores take
     int32_t check_corner = 1;      // the fill records the far corner's key and the traceback checks it
                                    // (always, but optional for the column kernel: msa_config "verify_corner")
     int32_t pair_min_sum = 0;

@@ -95,3 +95,12 @@ def test_level_by_level_and_walk_caps(max_count):
 def test_level_by_level_longest(lens):
     """The longest sequences that go level by level, and one residue more."""
     check(inputs.random_problem(8800, 2, list(lens), alphabet=inputs.PROTEIN, related=True), 1, 20)
+
+
+@pytest.mark.parametrize("lens", [(127, 15), (128, 16), (129, 33), (31, 31, 7), (32, 32, 8), (33, 31, 40), (31, 33, 70),
+                                  (3, 3, 100), (64, 2, 3)])
+def test_scores_kept_by_the_band_and_column_kernels(lens):
+    """Edges of the bands, the groups of columns and the 32 x 32 columns the kept scores are laid out by."""
+    for delta in (0, 2):
+        check(inputs.random_problem(8900 + sum(lens), len(lens), list(lens), alphabet=inputs.PROTEIN, related=True),
+              delta, 60)
