@@ -213,6 +213,7 @@ void fill_problem_desc(const HostPlan &hp, const PlanPointers &pp, int64_t tile_
     }
     d.tb_block = hp.tb_block;
     d.lzq = hp.lzq;
+    d.chain = hp.chain;
     d.tile_base = tile_base;
     d.ntiles = hp.ntiles;
     d.has_qcorner = hp.check_corner;

@@ -174,8 +174,8 @@ int fill_lines_warps_per_cta(int k, int z) {
 cudaError_t launch_fill_stream_k4(const LaunchDesc &L, int grid, cudaStream_t s);
 cudaError_t launch_fill_stream_k5(const LaunchDesc &L, int grid, cudaStream_t s);
 cudaError_t launch_fill_stream_k6(const LaunchDesc &L, int grid, cudaStream_t s, int rho_s);
-cudaError_t launch_fill_stream_k7(const LaunchDesc &L, int grid, cudaStream_t s);
-cudaError_t launch_fill_stream_k8(const LaunchDesc &L, int grid, cudaStream_t s);
+cudaError_t launch_fill_stream_k7(const LaunchDesc &L, int grid, cudaStream_t s, int rho_s);
+cudaError_t launch_fill_stream_k8(const LaunchDesc &L, int grid, cudaStream_t s, int rho_s);
 int fill_stream_ctas_k4();
 int fill_stream_ctas_k5();
 int fill_stream_ctas_k6();
@@ -187,8 +187,8 @@ cudaError_t launch_fill_stream(int k, const LaunchDesc &L, int grid, cudaStream_
         case 4: return launch_fill_stream_k4(L, grid, s);
         case 5: return launch_fill_stream_k5(L, grid, s);
         case 6: return launch_fill_stream_k6(L, grid, s, rho_s);
-        case 7: return launch_fill_stream_k7(L, grid, s);
-        case 8: return launch_fill_stream_k8(L, grid, s);
+        case 7: return launch_fill_stream_k7(L, grid, s, rho_s);
+        case 8: return launch_fill_stream_k8(L, grid, s, rho_s);
         default: return cudaErrorInvalidValue;
     }
 }

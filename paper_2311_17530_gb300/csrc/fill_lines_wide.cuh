@@ -17,18 +17,34 @@
 //   by exhaustive search, footprint within 1 % of the unpadded box).
 // * A column waits for the completion flags of its face neighbours along the
 //   line axes (their own waits make the diagonal neighbours complete as well),
-//   loads its 547 halo lines' positions in 16-byte groups from their producers'
-//   faces, sweeps rho_s + SMAX steps, writes its upper-face lines back (every
-//   position, line-major), and publishes its flag with a release store after a
-//   CTA barrier. Per halo value that is a quarter of a 16-byte load and one
-//   shared store, against a tagged 8-byte entry, its check and its ring store
-//   per value in the pipelined form; a column cannot start before its
+//   loads its halo lines (547 at k = 6) from their producers' faces, sweeps
+//   rho_s + SMAX steps, writes its upper-face lines back, and publishes its flag with
+//   a release store after a CTA barrier. Per halo value that is a quarter of a
+//   16-byte load and one shared store, against a tagged 8-byte entry, its check and
+//   its ring store per value in the pipelined form; a column cannot start before its
 //   producers have finished theirs, which on a last axis of 25 positions costs
 //   less than the per-block exchange.
+// * A face holds its lines side by side in groups of four positions: neighbouring
+//   lanes load neighbouring lines, each thread a line, with the loads of two to five
+//   lines in flight and the pair sums formed meanwhile. Line by line (consecutive
+//   groups of a line on neighbouring lanes, stores to shared memory four words apart)
+//   the halo took 22,000 of a column's 53,000 cycles, 16,000 now.
+// * A ticket is a unit of one or more super-blocks along axis J = k - 2, filled one
+//   after the other: the lines at h_J = SB_J become the next one's lines at h_J = 0
+//   in shared memory, and the pair sums and tables without axis J stay (the planner's
+//   wide_chain says when this pays).
+//
+// Measured (fill, against the form without the last two): 18 - 24 residues at k = 6
+// 4.33 -> 3.67 ms, 8 each 0.163 -> 0.146; 9 - 12 at k = 7 1.26 -> 1.00; 8 each at k = 8
+// 8.5 -> 5.5. A step is 184 issue cycles of a warp and 12 warps fill an SM, so a sweep
+// is bound by the integer pipe while three CTAs sweep together (530 - 600 cycles a
+// step); over a whole column it is at half of that rate, the rest being the halo's
+// latency. A CTA barrier only every 2 / 4 / 8 steps, with the warps that many steps
+// apart, was slower (4.42 / 4.51 / 4.74 at k = 6): the sweep gets longer.
 //
 // Global memory: the traceback bytes of each line block (layout 3 spanning the
 // whole last axis, as the streamed kernel), the faces of each super-block: its
-// upper-face lines, line-major, ZQ = rho_s rounded up to 4 positions each.
+// upper-face lines by groups of four positions, rho_s rounded up to 4 of them.
 #pragma once
 
 #include "device_common.cuh"
@@ -100,7 +116,10 @@ __host__ __device__ constexpr int wide_min_ctas() {
     return c < 1 ? 1 : c;
 }
 
-template <int K>
+// SHORT: at most kWideShort positions a line, so that more lines' loads fit in flight
+// (4^6 cells, four waves of super-blocks: 0.0270 against 0.0343 ms).
+constexpr int kWideShort = 12;
+template <int K, bool SHORT>
 __global__ void __launch_bounds__(stream_threads<K>(), wide_min_ctas<K>()) fill_lines_wide_kernel(const LaunchDesc L) {
     using LY = WideLayout<K>;
     constexpr int NA = K - 1;
@@ -108,8 +127,12 @@ __global__ void __launch_bounds__(stream_threads<K>(), wide_min_ctas<K>()) fill_
     constexpr int NT = LY::NT, NH = LY::NH, NHL = LY::NHL, NFL = LY::NFL, NROW = LY::NROW, ZS = LY::ZS;
     constexpr int SMAX = stream_skew_max(K);
     constexpr int MASKB = (1 << K) - 1;
-    constexpr int HB = 8;  // halo loads in flight per thread
-    static_assert(SMAX < LY::V && wide_v_words<K>() < (1 << 15) && NFL < 128 && NA < 10, "geometry");
+    constexpr int NQM = ((SHORT ? kWideShort : wide_z(K)) + 3) / 4;  // groups of 4 positions of a line, at most
+    constexpr int J = NA - 1, SBJ = stream_sb(K, J);  // the axis a unit of work runs along
+    constexpr int NC = NHL / (SBJ + 1);            // lines with h_J = 0, all of them halo
+    constexpr int CZ = wide_z(K) > 16 ? 32 : 16;   // lanes copying one line's positions
+    constexpr int HB = NQM >= 7 ? 2 : NQM >= 4 ? 3 : 5;           // ... whose loads are in flight together
+    static_assert(SMAX < LY::V && wide_v_words<K>() < (1 << 15) && NFL <= NT && NFL < 128 && NA < 10, "geometry");
 
     extern __shared__ __align__(16) unsigned char smem_raw[];
     int32_t *sm = reinterpret_cast<int32_t *>(smem_raw);
@@ -134,11 +157,23 @@ __global__ void __launch_bounds__(stream_threads<K>(), wide_min_ctas<K>()) fill_
         for (int i = 0; i < NA; ++i) base += (c[i] + 1) * wide_stride(K, i);
         if (f >= 0) ftab[f] = base;
     }
+    // Position -1 of every line, which no column changes, is set here too.
+    for (int j = tid; j < NHL; j += NT) {
+        int rem = j, base = 0;
+#pragma unroll
+        for (int i = NA - 1; i >= 0; --i) {
+            base += (rem % (stream_sb(K, i) + 1)) * wide_stride(K, i);
+            rem /= stream_sb(K, i) + 1;
+        }
+        V[base] = kNeg;
+    }
     for (int j = tid; j < NHL; j += NT) {
         int h[NA], c[NA], base = 0;
         uint32_t S = 0;
-        const int n = halo_number<K>(j, h);
+        int n = halo_number<K>(j, h);
         if (n < 0) continue;
+        // the lines with h_J = 0 last (every SBJ + 1st line of the box)
+        n = h[J] == 0 ? NH - NC + j / (SBJ + 1) : n - (j / (SBJ + 1) + 1);
 #pragma unroll
         for (int i = 0; i < NA; ++i) {
             base += h[i] * wide_stride(K, i);
@@ -184,7 +219,7 @@ __global__ void __launch_bounds__(stream_threads<K>(), wide_min_ctas<K>()) fill_
         const uint64_t ent = L.order[t];
         const int pidx = (int)(ent >> 32);
         const ProblemDesc &P = L.probs[pidx];
-        const int col = (int)(uint32_t)ent;  // super-block index
+        int col = (int)(uint32_t)ent;  // the unit's first super-block
         if (pidx != cached_prob) {
             cached_prob = pidx;
             cached_live = ld_volatile(&P.istat->status) == 0;
@@ -210,187 +245,221 @@ __global__ void __launch_bounds__(stream_threads<K>(), wide_min_ctas<K>()) fill_
         const int NQ = ZQ / 4;
         const int64_t FB = (int64_t)NFL * ZQ;
         const int32_t *Fq = P.Q;
-        int32_t *Fo = P.Q + (int64_t)col * FB;
         int32_t *const done = L.done + P.tile_base;
 
-        int64_t tile = 0;
-        bool has_tile = true;
-#pragma unroll
-        for (int i = 0; i < NA; ++i) {
-            const int g = sco[i] * stream_wg(K, i) + cw[i];
-            has_tile = has_tile && g < P.G[i];
-            tile += (int64_t)g * P.gstride[i];
-        }
-
-        // neighbour super-blocks, pair-table rows' residue codes, position -1 of
-        // every box line
-        for (int S = tid; S <= M; S += NT) {
-            int n = col;
-            bool in = true;
-#pragma unroll
-            for (int i = 0; i < NA; ++i)
-                if ((S >> i) & 1) {
-                    in = in && sco[i] > 0;
-                    n -= (int)P.sgstride[i];
-                }
-            nb[S] = in ? n : -1;
-        }
-        if (tid < NROW) {
-            int x = 0, len = 0, cof = 0, row = 0;
+        // super-blocks of this unit: up to P.chain of them along axis J
+        const int jend = min(sco[J] + P.chain, (P.G[J] + stream_wg(K, J) - 1) / stream_wg(K, J));
+        int Sp[M + 1], cd[NA];
+        bool first = true;
+        while (true) {
+            int32_t *Fo = P.Q + (int64_t)col * FB;
+            const int nh = first ? NH : NH - NC;  // halo lines to load
+            int64_t tile = 0;
+            bool has_tile = true;
 #pragma unroll
             for (int i = 0; i < NA; ++i) {
-                if (tid >= row && tid < row + stream_sb(K, i)) {
-                    x = o[i] + tid - row;
-                    len = P.len[i];
-                    cof = P.cofs[i];
-                }
-                row += stream_sb(K, i);
+                const int g = sco[i] * stream_wg(K, i) + cw[i];
+                has_tile = has_tile && g < P.G[i];
+                tile += (int64_t)g * P.gstride[i];
             }
-            crow[tid] = (x >= 1 && x <= len) ? codes[cof + x - 1] : 0;
-        }
-        for (int j = tid; j < NHL; j += NT) {
-            int rem = j, base = 0;
-#pragma unroll
-            for (int i = NA - 1; i >= 0; --i) {
-                base += (rem % (stream_sb(K, i) + 1)) * wide_stride(K, i);
-                rem /= stream_sb(K, i) + 1;
-            }
-            V[base] = kNeg;
-        }
-        // this line's pair sums over subsets of the line axes
-        int Sp[M + 1];
-        {
-            int cd[NA];
-#pragma unroll
-            for (int i = 0; i < NA; ++i) {
-                const int x = o[i] + cl[i];
-                cd[i] = (x >= 1 && x <= P.len[i]) ? codes[P.cofs[i] + x - 1] : 0;
-            }
-            Sp[0] = 0;
-#pragma unroll
-            for (int h = 0; h < NA; ++h) {
-                int Rs[1 << (NA - 1)];
-                Rs[0] = 0;
-#pragma unroll
-                for (int r = 1; r < (1 << h); ++r) Rs[r] = Rs[r & (r - 1)] + __ldg(tab + cd[lowbit_c(r)] * A + cd[h]);
-#pragma unroll
-                for (int r = 0; r < (1 << h); ++r) Sp[r | (1 << h)] = Sp[r] + Rs[r];
-            }
-        }
-        __syncthreads();  // nb and crow are read below
-        // pair tables of the last axis against every line axis, positions 0 .. rho - 1
-        for (int it = tid; it < NROW * rho; it += NT) {
-            const int row = it / rho, z = it - row * rho;
-            const int cz = z >= 1 ? codes[cofs + z - 1] : 0;
-            PT[row * ZS + z] = __ldg(tab + crow[row] * A + cz);
-        }
-        // face neighbours along the line axes (one lane each); their completion
-        // implies that of every diagonal neighbour
-        if (warp == 0) {
-            bool ok = true;
-            if (lane < NA && sco[lane] > 0) ok = wait_at_least(done + nb[1 << lane], 1, L.err, L.spin_ns);
-            ok = __all_sync(kFull, ok);
-            if (lane == 0) misc[1] = ok;
-        }
-        __syncthreads();  // the waiting lanes' acquires precede every thread's halo loads
-        if (!misc[1]) {
-            if (tid == 0) atomicCAS(L.err, 0, MSA_ETIMEOUT);
-            break;
-        }
 
-        // the halo: positions 0 .. rho - 1 of every halo line, 4 at a time
-        for (int i0 = 0; i0 < NH * NQ; i0 += NT * HB) {
-            int4 val[HB];
-            int dst[HB];
+            // neighbour super-blocks, pair-table rows' residue codes
+            for (int S = tid; S <= M; S += NT) {
+                int n = col;
+                bool in = true;
 #pragma unroll
-            for (int u = 0; u < HB; ++u) {
-                const int it = i0 + NT * u + tid;
-                dst[u] = -1;
-                val[u] = make_int4(kNeg, kNeg, kNeg, kNeg);
-                if (it < NH * NQ) {
-                    const int j = it / NQ, q = it - j * NQ;
+                for (int i = 0; i < NA; ++i)
+                    if ((S >> i) & 1) {
+                        in = in && sco[i] > 0;
+                        n -= (int)P.sgstride[i];
+                    }
+                nb[S] = in ? n : -1;
+            }
+            if (tid < NROW) {
+                int x = 0, len = 0, cof = 0, row = 0;
+#pragma unroll
+                for (int i = 0; i < NA; ++i) {
+                    if (tid >= row && tid < row + stream_sb(K, i)) {
+                        x = o[i] + tid - row;
+                        len = P.len[i];
+                        cof = P.cofs[i];
+                    }
+                    row += stream_sb(K, i);
+                }
+                crow[tid] = (x >= 1 && x <= len) ? codes[cof + x - 1] : 0;
+            }
+            __syncthreads();  // nb and crow are read below
+            // face neighbours along the line axes (one lane of warp 0 each; their completion
+            // implies that of every diagonal neighbour), and meanwhile the pair tables of the
+            // last axis against every line axis, positions 0 .. rho - 1
+            if (warp == 0) {
+                bool ok = true;
+                if (lane < NA && sco[lane] > 0 && (first || lane != J))
+                    ok = wait_at_least(done + nb[1 << lane], 1, L.err, L.spin_ns);
+                ok = __all_sync(kFull, ok);
+                if (lane == 0) misc[1] = ok;
+            } else {
+                for (int z = lane; z < rho; z += 32) {
+                    const int cz = z >= 1 ? codes[cofs + z - 1] : 0;
+                    for (int row = (first ? 0 : NROW - SBJ) + warp - 1; row < NROW; row += NT / 32 - 1)
+                        PT[row * ZS + z] = __ldg(tab + crow[row] * A + cz);
+                }
+            }
+            __syncthreads();  // the waiting lanes' acquires precede every thread's halo loads
+            if (!misc[1]) {
+                if (tid == 0) atomicCAS(L.err, 0, MSA_ETIMEOUT);
+                return;
+            }
+
+            // The halo: positions 0 .. rho - 1 of every halo line, a line per thread and turn
+            // (neighbouring lanes read neighbouring lines of one face, 16 bytes each), HB
+            // lines' loads in flight; the first of them fly while the pair sums are formed.
+            int4 hv[HB][NQM];
+            int hdst[HB];
+            auto halo_load = [&](int s0) {
+#pragma unroll
+                for (int u = 0; u < HB; ++u) {
+                    const int j = (s0 + u) * NT + tid;
+                    hdst[u] = -1;
+                    if (j >= nh) continue;
                     const uint32_t e = hdesc[j];
                     const int src = nb[e >> 22];
-                    dst[u] = (int)(e & 0x7FFF) + 1 + 4 * q;
-                    if (src >= 0)
-                        val[u] = __ldcg(reinterpret_cast<const int4 *>(Fq + (int64_t)src * FB +
-                                                                       (int)((e >> 15) & 127) * ZQ + 4 * q));
+                    hdst[u] = (int)(e & 0x7FFF) + 1;
+                    const int4 *p = reinterpret_cast<const int4 *>(Fq + (int64_t)src * FB) + (int)((e >> 15) & 127);
+#pragma unroll
+                    for (int q = 0; q < NQM; ++q) {
+                        hv[u][q] = make_int4(kNeg, kNeg, kNeg, kNeg);
+                        if (src >= 0 && q < NQ) hv[u][q] = __ldcg(p + q * NFL);
+                    }
                 }
-            }
+            };
+            auto halo_store = [&]() {
 #pragma unroll
-            for (int u = 0; u < HB; ++u)
-                if (dst[u] >= 0) {
-                    const int it = i0 + NT * u + tid;
-                    const int n = rho - 4 * (it - (it / NQ) * NQ);  // positions left on the line
-                    V[dst[u]] = val[u].x;
-                    if (n > 1) V[dst[u] + 1] = val[u].y;
-                    if (n > 2) V[dst[u] + 2] = val[u].z;
-                    if (n > 3) V[dst[u] + 3] = val[u].w;
+                for (int u = 0; u < HB; ++u) {
+                    if (hdst[u] < 0) continue;
+                    int32_t *d = V + hdst[u];
+#pragma unroll
+                    for (int q = 0; q < NQM; ++q) {
+                        if (4 * q < rho) d[4 * q] = hv[u][q].x;
+                        if (4 * q + 1 < rho) d[4 * q + 1] = hv[u][q].y;
+                        if (4 * q + 2 < rho) d[4 * q + 2] = hv[u][q].z;
+                        if (4 * q + 3 < rho) d[4 * q + 3] = hv[u][q].w;
+                    }
                 }
-        }
-        __syncthreads();
-
-        // The sweep: rho + SMAX steps, one barrier each. Every lane reads its own
-        // skewed position, in range or not (a read below position -1 or past the
-        // last position feeds only candidates that are overwritten or never
-        // stored); the origin's lane starts from H(0) = 0 as its previous position.
-        int Wl = -sig * (1 << NA);  // W(x) = Wl + t 2^NA at step t
+            };
+            halo_load(0);
+                // this line's pair sums over subsets of the line axes; along the unit only
+                // those with axis J change
+                const int xj = o[J] + cl[J];
+                const int cj = (xj >= 1 && xj <= P.len[J]) ? codes[P.cofs[J] + xj - 1] : 0;
+                if (first) {
+                    Sp[0] = 0;
 #pragma unroll
-        for (int i = 0; i < NA; ++i) Wl += (o[i] + cl[i]) << i;
-        int ptoff[NA];
-        {
-            int row = 0;
+                    for (int i = 0; i < J; ++i) {
+                        const int x = o[i] + cl[i];
+                        cd[i] = (x >= 1 && x <= P.len[i]) ? codes[P.cofs[i] + x - 1] : 0;
+                    }
 #pragma unroll
-            for (int i = 0; i < NA; ++i) {
-                ptoff[i] = (row + cl[i]) * ZS;
-                row += stream_sb(K, i);
-            }
-        }
-        int vself = col == 0 && tid == 0 ? 0 : kNeg;
-        int D = vself;  // best move of the next position that advances the last axis
-        const int rows = P.tb_block / 32;
-        uint8_t *tbw = P.tb + tile * P.tb_block + lane;
-        const int nsteps = rho + SMAX;
-        for (int ts = 0; ts < nsteps; ++ts) {
-            if ((unsigned)(ts - sigw) < (unsigned)(rho + line_skew_max(K))) {
-                const int z = ts - sig;
-                const bool act = (unsigned)z < (unsigned)rho;
-                const int zn = z < -1 ? 0 : (z + 1 >= rho ? rho - 1 : z + 1);
-                int p[NA];
+                    for (int h = 0; h < J; ++h) {
+                        int Rs[1 << (NA - 1)];
+                        Rs[0] = 0;
 #pragma unroll
-                for (int i = 0; i < NA; ++i) p[i] = PT[ptoff[i] + zn];
-                int acc0 = D, acc1 = kNeg;
-                const int32_t *vp = V + vbase + z + 1;
-                const int F = fold_subsets<NA, 0>(
-                    [&](auto m) { return vp[-wide_move_off<K>(m.value)] + Sp[m.value]; }, p, acc0, acc1);
-                const int acc = max(acc0, acc1);
-                const int tm = (Wl + ts * (1 << NA) - acc) & MASKB;
-                const int val = acc + tm;
-                const int r = ts - sigw;
-                if (has_tile && r < rows) tbw[(int64_t)r * 32] = (uint8_t)tm;
-                if (act) {
-                    V[vbase + z + 1] = val;
-                    vself = val;
+                        for (int r = 1; r < (1 << h); ++r) Rs[r] = Rs[r & (r - 1)] + __ldg(tab + cd[lowbit_c(r)] * A + cd[h]);
+#pragma unroll
+                        for (int r = 0; r < (1 << h); ++r) Sp[r | (1 << h)] = Sp[r] + Rs[r];
+                    }
                 }
-                D = max(F, vself);
+                {
+                    int Rs[1 << J];
+                    Rs[0] = 0;
+#pragma unroll
+                    for (int r = 1; r < (1 << J); ++r) Rs[r] = Rs[r & (r - 1)] + __ldg(tab + cd[lowbit_c(r)] * A + cj);
+#pragma unroll
+                    for (int r = 0; r < (1 << J); ++r) Sp[r | (1 << J)] = Sp[r] + Rs[r];
+                }
+            halo_store();
+#pragma unroll 1
+            for (int s0 = HB; s0 * NT < nh; s0 += HB) {
+                halo_load(s0);
+                halo_store();
             }
             __syncthreads();
-        }
 
-        // faces for the successors: every position of the upper-face lines
-        for (int it = tid; it < NFL * NQ; it += NT) {
-            const int f = it / NQ, q = it - f * NQ;
-            const int32_t *s = V + ftab[f] + 1 + 4 * q;
-            *reinterpret_cast<int4 *>(Fo + (int64_t)f * ZQ + 4 * q) = make_int4(s[0], s[1], s[2], s[3]);
-        }
-        {
-            bool corner = true;
+            // The sweep: rho + SMAX steps, one barrier each. Every lane reads its own
+            // skewed position, in range or not (a read below position -1 or past the
+            // last position feeds only candidates that are overwritten or never
+            // stored); the origin's lane starts from H(0) = 0 as its previous position.
+            int Wl = -sig * (1 << NA);  // W(x) = Wl + t 2^NA at step t
 #pragma unroll
-            for (int i = 0; i < NA; ++i) corner = corner && o[i] + cl[i] == P.len[i];
-            if (corner) *P.qcorner = V[vbase + rho];
+            for (int i = 0; i < NA; ++i) Wl += (o[i] + cl[i]) << i;
+            int ptoff[NA];
+            {
+                int row = 0;
+#pragma unroll
+                for (int i = 0; i < NA; ++i) {
+                    ptoff[i] = (row + cl[i]) * ZS;
+                    row += stream_sb(K, i);
+                }
+            }
+            int vself = col == 0 && tid == 0 ? 0 : kNeg;
+            int D = vself;  // best move of the next position that advances the last axis
+            const int rows = P.tb_block / 32;
+            uint8_t *tbw = P.tb + tile * P.tb_block + lane;
+            const int nsteps = rho + SMAX;
+            for (int ts = 0; ts < nsteps; ++ts) {
+                if ((unsigned)(ts - sigw) < (unsigned)(rho + line_skew_max(K))) {
+                    const int z = ts - sig;
+                    const bool act = (unsigned)z < (unsigned)rho;
+                    const int zn = z < -1 ? 0 : (z + 1 >= rho ? rho - 1 : z + 1);
+                    int p[NA];
+#pragma unroll
+                    for (int i = 0; i < NA; ++i) p[i] = PT[ptoff[i] + zn];
+                    int acc0 = D, acc1 = kNeg;
+                    const int32_t *vp = V + vbase + z + 1;
+                    const int F = fold_subsets<NA, 0>(
+                        [&](auto m) { return vp[-wide_move_off<K>(m.value)] + Sp[m.value]; }, p, acc0, acc1);
+                    const int acc = max(acc0, acc1);
+                    const int tm = (Wl + ts * (1 << NA) - acc) & MASKB;
+                    const int val = acc + tm;
+                    const int r = ts - sigw;
+                    if (has_tile && r < rows) tbw[(int64_t)r * 32] = (uint8_t)tm;
+                    if (act) {
+                        V[vbase + z + 1] = val;
+                        vself = val;
+                    }
+                    D = max(F, vself);
+                }
+                __syncthreads();
+            }
+
+            // faces for the successors: every position of the upper-face lines
+            if (tid < NFL) {
+                const int32_t *v = V + ftab[tid] + 1;
+                int4 *dst = reinterpret_cast<int4 *>(Fo) + tid;
+                for (int q = 0; q < NQ; ++q, v += 4) dst[q * NFL] = make_int4(v[0], v[1], v[2], v[3]);
+            }
+            // the next super-block's lines with h_J = 0 are this one's with h_J = SB_J
+            const bool more = sco[J] + 1 < jend;
+            if (more)
+                for (int m = tid / CZ; m < NC; m += NT / CZ) {
+                    int32_t *to = V + (hdesc[NH - NC + m] & 0x7FFF) + 1;
+                    const int z = tid % CZ;
+                    if (z < rho) to[z] = to[SBJ * wide_stride(K, J) + z];
+                }
+            {
+                bool corner = true;
+#pragma unroll
+                for (int i = 0; i < NA; ++i) corner = corner && o[i] + cl[i] == P.len[i];
+                if (corner) *P.qcorner = V[vbase + rho];
+            }
+            __syncthreads();  // every thread's face stores precede the release
+            if (tid == 0 && (int64_t)t != L.withhold) st_release(done + col, 1);
+            if (!more) break;
+            first = false;
+            col += (int)P.sgstride[J];
+            ++sco[J];
+            o[J] += SBJ;
         }
-        __syncthreads();  // every thread's face stores precede the release
-        if (tid == 0 && (int64_t)t != L.withhold) st_release(done + col, 1);
     }
 }
 
@@ -398,16 +467,23 @@ template <int K>
 cudaError_t wide_attributes() {
     static DeviceOnce once;
     return once.run([] {
-        return cudaFuncSetAttribute(fill_lines_wide_kernel<K>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    wide_smem_bytes<K>());
+        cudaError_t e = cudaFuncSetAttribute(fill_lines_wide_kernel<K, true>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, wide_smem_bytes<K>());
+        if (e == cudaSuccess && wide_z(K) > kWideShort)
+            e = cudaFuncSetAttribute(fill_lines_wide_kernel<K, (wide_z(K) <= kWideShort)>,
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, wide_smem_bytes<K>());
+        return e;
     });
 }
 
 template <int K>
-cudaError_t launch_wide(const LaunchDesc &L, int grid, cudaStream_t s) {
+cudaError_t launch_wide(const LaunchDesc &L, int grid, cudaStream_t s, int rho_s) {
     cudaError_t e = wide_attributes<K>();
     if (e != cudaSuccess) return e;
-    fill_lines_wide_kernel<K><<<grid, stream_threads<K>(), wide_smem_bytes<K>(), s>>>(L);
+    if (rho_s <= kWideShort)
+        fill_lines_wide_kernel<K, true><<<grid, stream_threads<K>(), wide_smem_bytes<K>(), s>>>(L);
+    else
+        fill_lines_wide_kernel<K, (wide_z(K) <= kWideShort)><<<grid, stream_threads<K>(), wide_smem_bytes<K>(), s>>>(L);
     return cudaGetLastError();
 }
 
@@ -415,8 +491,8 @@ template <int K>
 int wide_ctas() {
     if (wide_attributes<K>() != cudaSuccess) return 0;
     int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fill_lines_wide_kernel<K>, stream_threads<K>(),
-                                                      wide_smem_bytes<K>()) != cudaSuccess)
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fill_lines_wide_kernel<K, (wide_z(K) <= kWideShort)>,
+                                                      stream_threads<K>(), wide_smem_bytes<K>()) != cudaSuccess)
         return 0;
     return n;
 }

@@ -4,7 +4,7 @@
 
 namespace msadp {
 
-cudaError_t launch_fill_stream_k7(const LaunchDesc &L, int grid, cudaStream_t s) { return launch_wide<7>(L, grid, s); }
+cudaError_t launch_fill_stream_k7(const LaunchDesc &L, int grid, cudaStream_t s, int rho_s) { return launch_wide<7>(L, grid, s, rho_s); }
 int fill_stream_ctas_k7() { return wide_ctas<7>(); }
 
 }  // namespace msadp

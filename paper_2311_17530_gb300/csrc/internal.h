@@ -49,6 +49,7 @@ struct ProblemDesc {
     int32_t w_corner;            // W(len)
     int32_t len_sum;
     int32_t has_qcorner;         // the fill records the corner's packed key (cross-check)
+    int32_t chain;               // streamed line kernel's whole-column form: super-blocks of a unit of work
     int32_t lzq;                 // line kernels: entries per line in a tile's (column's) face block
     int32_t tb_block;            // tile-major layouts: traceback bytes per tile
     int32_t lst[MSA_MAX_K];      // tile-major layouts: byte stride of axis i inside a tile's block

@@ -263,12 +263,24 @@ bool score_and_traceback_layout(HostPlan &hp) {
         // (the whole-column form: words, every position)
         hp.wide = stream && z <= wide_z(k);
         if (hp.wide) hp.lzq = (z + 3) / 4 * 4;
-        hp.qelems = stream ? hp.nunits * stream_face_lines(k) * hp.lzq * (hp.wide ? 1 : 2) : hp.ntiles * 32 * hp.lzq;
+        hp.qelems = stream ? hp.sgstride[0] * hp.SG[0] * stream_face_lines(k) * hp.lzq * (hp.wide ? 1 : 2) : hp.ntiles * 32 * hp.lzq;
         hp.tb_layout = 3;
         hp.tb_dev_bytes = hp.ntiles * hp.tb_block;
         if (hp.qelems >= (1LL << 38) || hp.tb_dev_bytes >= (1LL << 40)) return false;
     }
     return true;
+}
+
+// Super-blocks along axis k - 2 that one unit of the whole-column form covers: all of
+// them where the faces are more than about twice the L2 cache, for a face is read again
+// up to k - 1 waves of super-blocks later, and a unit keeps two fifths of its next halo
+// (18 - 24 residues at k = 6, 1.04 GB of faces: 4.15 -> 3.67 ms; 9^8 cells, 476 MB: 5.70
+// -> 5.49; 18 - 21 at k = 6, 345 MB: 1.52 -> 1.50); below, one: a unit's super-blocks
+// follow one another, and the waves are long as it is (17^6 cells, 173 MB: 0.76 with
+// one, 0.86 with all; 9^6: 0.146, 0.202).
+static int wide_chain(int k, int64_t super_blocks, const int32_t *SG, int rho_s) {
+    const int64_t face_bytes = super_blocks * stream_face_lines(k) * round_up64(rho_s, 4) * 4;
+    return face_bytes >= (1LL << 28) ? SG[k - 2] : 1;
 }
 
 int plan_shape(int k, const int32_t *lens, int A, int kernel_choice, HostPlan &hp, std::string &err, int edge,
@@ -359,6 +371,10 @@ int plan_shape(int k, const int32_t *lens, int A, int kernel_choice, HostPlan &h
         nu *= hp.SG[i];
     }
     hp.nunits = nu;
+    if (hp.kernel == kKernelStream && lens[k - 1] + 1 <= wide_z(k)) {
+        hp.chain = wide_chain(k, nu, hp.SG, lens[k - 1] + 1);
+        hp.nunits = nu / hp.SG[k - 2] * ((hp.SG[k - 2] + hp.chain - 1) / hp.chain);
+    }
     int gsum = 0;
     for (int i = 0; i < k; ++i) gsum += hp.SG[i];
     hp.waves = gsum - k + 1;
@@ -417,30 +433,39 @@ int make_plan(int k, const int32_t *lens, int A, int kernel_choice, HostPlan &hp
 
     // ticket order: by wave, then by linear tile index (counting sort); the wave
     // of each tile follows its grid coordinates, stepped like an odometer (last
-    // axis fastest) instead of decoded from the linear index
-    std::vector<int64_t> cnt(hp.waves + 1, 0);
+    // axis fastest) instead of decoded from the linear index. A unit of several
+    // super-blocks along axis k - 2 is listed by its first one, in the wave of that.
+    const int64_t waves = hp.waves;
+    const int cj = k - 2;  // the axis of the units' super-blocks
+    std::vector<int64_t> cnt(waves + 1, 0);
     std::vector<int32_t> wave_of(nt);
+    std::vector<uint64_t> tile_of(nt);
     {
         int c[MSA_MAX_K] = {};
         int w = 0;
+        int64_t tile = 0;
         for (int64_t t = 0; t < nt; ++t) {
             wave_of[t] = w;
+            tile_of[t] = tile;
             cnt[w + 1]++;
             for (int i = k - 1; i >= 0; --i) {
-                if (c[i] + 1 < hp.SG[i]) {
-                    ++c[i];
-                    ++w;
+                const int step = i == cj ? hp.chain : 1;
+                if (c[i] + step < hp.SG[i]) {
+                    c[i] += step;
+                    w += step;
+                    tile += step * hp.sgstride[i];
                     break;
                 }
+                tile -= c[i] * hp.sgstride[i];
                 w -= c[i];
                 c[i] = 0;
             }
         }
     }
-    for (int w = 0; w < hp.waves; ++w) cnt[w + 1] += cnt[w];
+    for (int w = 0; w < waves; ++w) cnt[w + 1] += cnt[w];
     hp.wave_start = cnt;
     hp.order.assign(nt, 0);
-    for (int64_t t = 0; t < nt; ++t) hp.order[cnt[wave_of[t]]++] = (uint64_t)t;
+    for (int64_t t = 0; t < nt; ++t) hp.order[cnt[wave_of[t]]++] = (uint64_t)tile_of[t];
     shuffle_within_waves(hp);
     return MSA_OK;
 }

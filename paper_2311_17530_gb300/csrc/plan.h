@@ -52,6 +52,7 @@ struct HostPlan {
     int32_t edge = 0;              // tile edge of the generic kernel (tile_ext); longest segment of the
                                    // line kernel; 0 for the column and band kernels
     bool wide = false;             // streamed line kernel: its whole-column form
+    int32_t chain = 1;             // ... super-blocks along axis k - 2 that one ticket covers
     bool keep = false;             // column and band kernels: every cell's score is kept
     int64_t kept_elems = 0;        // words these scores take
     int32_t check_corner = 1;      // the fill records the far corner's key and the traceback checks it

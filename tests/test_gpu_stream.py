@@ -221,3 +221,16 @@ def test_whole_column_form_withheld_column():
             msa.msa_config("test_withhold_tile", -1)
             msa.msa_config("spin_timeout_ms", 5000)
         check(p)
+
+
+@pytest.mark.parametrize("k,lens", [(6, [27, 31, 26, 27, 28, 2]), (7, [15, 14, 13, 14, 15, 15, 4])])
+def test_units_of_several_super_blocks(k, lens):
+    """Faces beyond 256 MB: a unit of work is every super-block along axis k - 2 (the last one ragged).
+    The whole traceback tensor against the generic tile kernel's."""
+    p = inputs.random_problem(4700 + k, k, lens, alphabet=inputs.DNA, related=True)
+    got = run(p)
+    msa.msa_config("fill_kernel", 1)
+    want = run(p)
+    assert (got[4].fill_kernel, want[4].fill_kernel) == (5, 1)
+    assert got[:3] == want[:3] and got[2] == 0
+    np.testing.assert_array_equal(got[3], want[3])
