@@ -569,7 +569,7 @@ def measure_extensions(reps: int = 3):
             "optimum": score, "same_result_as_msa_align": (s2, r2) == (score, rows),
             "tiles": st["tiles"], "tiles_skipped": st["tiles_skipped"], "cells_skipped": st["cells_skipped"],
             "cells": st["cells"], "fraction_skipped": st["cells_skipped"] / max(1, st["cells"]),
-            "note": "host-buffer call: pairwise tables, bound, greedy feasible alignment, pruned generic-tile fill, "
+            "note": "host-buffer call: pairwise tables, bound, greedy feasible alignment, fill (the fastest for the shape), "
                     "traceback, with per-call allocation and copies"}
     q = inputs.random_problem(17, 3, [120, 110, 130], alphabet=inputs.PROTEIN, related=True)
     for delta in (0, 3):
