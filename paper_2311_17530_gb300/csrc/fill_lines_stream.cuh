@@ -2,53 +2,49 @@
 // (fill_lines.cuh: lane l of a warp owns one line of a 32-line block, skewed by
 // the sum of its local coordinates; the moves that also advance the last axis s are
 // folded from the previous position's candidates), organised for the latency of the
-// hardware. Measured (fill): k4 DNA 110 - 130 0.951 ms, k5 protein 33 - 45 1.395 ms,
-// against 1.021 and 1.577 ms with every candidate carried, the CTA's tables built by
-// one thread and three CTAs of 168 registers per SM at k = 5 (now four of 128: a copy's
-// source is a 4-byte face line, which lets their shared memory fit):
+// hardware. Measured (fill), with the exchange on warps of its own against inside the
+// sweep: k5 protein 33 - 45 1.097 against 1.402 ms, 15^5 0.100 / 0.159, 31^5 0.407 / 0.594;
+// k4 DNA 110 - 130 0.948 / 0.946, 61 - 64 0.189 / 0.237, 41^4 0.106 / 0.147, 21^4 0.050 /
+// 0.066.
 //
-// * A CTA of W warps owns a SUPER-BLOCK of W line blocks (a grid of extents
+// * A CTA of W sweeping warps owns a SUPER-BLOCK of W line blocks (a grid of extents
 //   stream_wg over the line axes) and sweeps it over the WHOLE last axis in
-//   lockstep: at step t every lane of the CTA computes position z = t - sigma of
+//   lockstep: at step t every lane of the sweep computes position z = t - sigma of
 //   its line, sigma being the sum of the line's coordinates inside the
-//   super-block, and a CTA barrier ends the step. Every predecessor line of the
-//   super-block then holds position z at time t - |m'|, so warps exchange
+//   super-block, and a barrier of the sweep's warps ends the step. Every predecessor
+//   line of the super-block then holds position z at time t - |m'|, so warps exchange
 //   nothing but shared memory; only super-blocks talk through global memory.
 //   The skew, the set-up and the ticket are paid once per super-block column.
 // * Super-blocks are handed out in wave order of their grid (section 3: blocks
-//   whose coordinates sum to w form wave w). After each block of U steps a
-//   super-block publishes what its upper-face lines held at those U TIMES, as
-//   (value, tag) 8-byte entries (the tag is the launch's epoch), then a count
-//   of published blocks (a plain relaxed store). Publishing by time makes a
-//   block's data complete as soon as the block ends; a consumer's halo time tau
-//   is its producer's time tau + SB_S (the super-block extents along the axes
-//   S in which the producer lies below).
-// * A consumer loads its producers' counts at a block's start and, once they
-//   cover the next block's halo, copies it into a staging buffer during the
-//   sweep (16-byte cp.async copies through L2); at the block's end it accepts
-//   the entries once every one carries the epoch, copying again otherwise (a
-//   bounded wait). The counts only spare the memory system from copies that
-//   would fail: correctness rests on the tags, so no fence or release/acquire
-//   pair is needed. An aligned 8-byte entry is written by one store and read
-//   whole, and each entry is written once per launch; earlier launches left
-//   smaller epochs (the plan clears the faces before the first launch and when
-//   epochs wrap).
+//   whose coordinates sum to w form wave w). What a super-block's upper-face lines held
+//   at the U TIMES of a block goes out as (value, tag) 8-byte entries (the tag is the
+//   launch's epoch). Publishing by time makes a block's data complete as soon as the
+//   block ends; a consumer's halo time tau is its producer's time tau + SB_S (the
+//   super-block extents along the axes S in which the producer lies below).
+// * Separate warps of the CTA do that exchange: they write the swept blocks' faces and
+//   bring the halo of the blocks to come, loading entries until all carry the epoch (a
+//   bounded wait), while the sweep runs; the sweep only looks, two steps before a block
+//   ends, whether the next block's halo is there. In the sweeping warps themselves
+//   (copies into a staging buffer during a block, tag checks and ring stores at its
+//   end) the exchange took 106 of a step's 181 instructions at k = 5 and stood between
+//   the blocks. Correctness rests on the tags, so no fence or release/acquire pair is
+//   needed between CTAs: an aligned 8-byte entry is written by one store and read
+//   whole, each entry is written once per launch, and earlier launches left smaller
+//   epochs (the plan clears the faces before the first launch and when epochs wrap).
 //
 // Shared memory per CTA:
-//   V      a ring of D words per line of the halo'd super-block (local
+//   V      a ring of three blocks' times per line of the halo'd super-block (local
 //          coordinates -1 .. SB_i - 1), indexed by time: position z of line c sits
-//          in slot (z + sigma(c)) mod D. At step t every lane reads slot
-//          (t - |m'|) mod D of its predecessor line c - e_m' (one slot for all
-//          lanes) and writes slot t mod D of its own line, so the 32 accesses of
-//          a warp are conflict-free when sum_i c_i A_i is distinct mod 32 over a
-//          line block (strides A_i found by exhaustive search, below).
-//   PT     an R-position ring of the pair tables of s against every line axis.
-//   stage  the halo of the next block: U times of every halo line.
+//          in slot (z + sigma(c)) mod 3U. At step t every lane reads its predecessor
+//          line c - e_m' at time t - |m'| and writes its own line's slot of time t: a
+//          constant offset from the block's slots or from those of the block before, so
+//          the steps are unrolled once. The 32 accesses of a warp are conflict-free when
+//          sum_i c_i A_i is distinct mod 32 over a line block (strides A_i found by
+//          exhaustive search, below). The third block's slots take the arriving halo.
+//   PT     an R-position ring of the pair tables of s against every line axis, refilled
+//          by the exchanging warps.
 //   tables of the halo and face lines, the neighbour super-block of every
 //          subset of the line axes, the residue code of every pair-table row.
-// Blocks of U = 8 steps and a D = 16 slot ring for k = 4, 5; for k = 6 (547 halo
-// lines around 128, so the ring and staging per CTA are large) U = 4 and D = 12,
-// which leaves room for three CTAs per SM instead of two.
 //
 // Global memory: the traceback bytes of each line block (a tile of the line
 // kernel's layout 3 spanning the whole last axis: cell (c, z) at
@@ -62,18 +58,16 @@
 
 namespace msadp {
 
-// Ring slots per line: a line's times from t - (k - 1) on plus the next block's
-// U times, so D >= U + k - 1, and a whole number of blocks, so that every slot a
-// step touches is a constant within a block of known parity b mod (D / U).
-__host__ __device__ constexpr int stream_ring_d(int K) { return K == 6 ? 12 : 16; }
-// Pair-table ring positions: a block reads positions bU - SMAX .. bU + U - 1.
-__host__ __device__ constexpr int stream_pt_ring(int K) { return K == 6 ? 16 : 32; }
+// Ring slots per line: the block being swept, the one before and the one whose halo arrives.
+__host__ __device__ constexpr int stream_ring_d(int K) { return 3 * stream_block(K); }
+// Pair-table ring positions: two blocks and the skew of a super-block at least.
+__host__ __device__ constexpr int stream_pt_ring(int K) { return K == 4 ? 64 : 32; }
 
 // Ring stride (words) of line axis i over the halo'd super-block: the smallest
 // footprint with every line's D slots disjoint and sum_i c_i A_i distinct mod 32
 // over a warp's line block.
 __host__ __device__ constexpr int stream_stride(int K, int i) {
-    constexpr int k4[] = {16, 81, 732}, k5[] = {16, 81, 406, 1220}, k6[] = {12, 61, 306, 920, 2768};
+    constexpr int k4[] = {217, 24, 1086}, k5[] = {362, 1812, 121, 24}, k6[] = {24, 362, 121, 1812, 5456};
     return K == 4 ? k4[i] : K == 5 ? k5[i] : k6[i];
 }
 template <int K>
@@ -101,6 +95,9 @@ __host__ __device__ constexpr int stream_ring_words() {
     for (int i = 0; i < K - 1; ++i) s += stream_sb(K, i) * stream_stride(K, i);
     return round_up(s, 4);
 }
+// Warps of a CTA that exchange the faces: half or all of the sweep's. k = 4 with 4 / 8: 20^4
+// 0.0527 / 0.0494 ms, 40^4 0.112 / 0.106; k = 5 with 1 / 2 / 4 / 8: 2.31 / 1.38 / 1.10 / 1.23.
+__host__ __device__ constexpr int stream_xwarps(int K) { return K == 4 ? 8 : 4; }
 // Shared memory of a CTA, in 4-byte words (every part 16-byte aligned).
 template <int K>
 struct StreamLayout {
@@ -114,17 +111,13 @@ struct StreamLayout {
     static constexpr int NT = 32 * stream_warps(K);
     static constexpr int V = 0;
     static constexpr int PT = V + stream_ring_words<K>();
-    static constexpr int STAGE = PT + round_up(NROW * ZS, 4);
-    static constexpr int NT_ = 32 * stream_warps(K);
-    static constexpr int HC = (NH * (stream_block(K) / 2) + NT_ - 1) / NT_;  // halo copies per thread and block
-    static constexpr int HOFS = STAGE + NH * stream_block(K) * 2;  // per copy: source face line
-    static constexpr int HMETA = HOFS + HC * NT_;               // ... ring base | time offset << 14
-    static constexpr int HTAB = HMETA + HC * NT_;
+    static constexpr int HSRC = PT + round_up(NROW * ZS, 4);  // per halo line: its producer's face line (-1: none)
+    static constexpr int HTAB = HSRC + round_up(NH, 4);
     static constexpr int FTAB = HTAB + round_up(NH, 4);
     static constexpr int NB = FTAB + round_up(NFL, 4);
     static constexpr int CROW = NB + round_up(1 << (K - 1), 4);
-    static constexpr int MISC = CROW + round_up(NROW, 4);  // ticket, verdicts
-    static constexpr int WORDS = MISC + 8;
+    static constexpr int MISC = CROW + round_up(NROW, 4);  // ticket, progress, verdicts
+    static constexpr int WORDS = MISC + 8 + round_up(stream_xwarps(K), 4);
 };
 template <int K>
 __host__ __device__ constexpr int stream_smem_bytes() {
@@ -134,16 +127,18 @@ template <int K>
 __host__ __device__ constexpr int stream_threads() {
     return 32 * stream_warps(K);
 }
-// CTAs per SM: what shared memory allows (228 KB per SM, 1 KB reserved per CTA,
-// at most 48 warps) and what a budget of registers per thread allows (the sweep
-// keeps 2^(k-1) pair sums live); the launch bound caps
-// registers to match.
+// The streamed kernel's CTA: the sweep's warps and those that exchange the faces.
+template <int K>
+__host__ __device__ constexpr int stream_cta_threads() {
+    return stream_threads<K>() + 32 * stream_xwarps(K);
+}
+// CTAs per SM: what shared memory allows (228 KB per SM, 1 KB reserved per CTA)
+// and what leaves the sweep its registers (it keeps 2^(k-1) pair sums live). k = 4 with a
+// third CTA (56 registers): 0.941 against 0.949 ms, but 40^4 0.126 against 0.112; k = 5 with
+// a fourth (64): 1.063 against 1.099, but 20^5 0.184 against 0.171.
 template <int K>
 __host__ __device__ constexpr int stream_min_ctas() {
-    int c = (228 * 1024) / (stream_smem_bytes<K>() + 1024);
-    if (c * stream_warps(K) > 48) c = 48 / stream_warps(K);
-    const int regs = K == 4 ? 80 : K == 5 ? 128 : 168;
-    const int cr = 65536 / (regs * stream_threads<K>());
+    const int c = (228 * 1024) / (stream_smem_bytes<K>() + 1024), cr = K == 4 ? 2 : 3;
     return c < cr ? c : cr;
 }
 
@@ -191,8 +186,39 @@ __device__ __forceinline__ int halo_number(int j, int (&h)[K - 1]) {
     return prefix ? -1 : j - inner;
 }
 
-__device__ __forceinline__ void cp_async16(void *smem_dst, const void *gsrc) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(smem_dst)), "l"(gsrc) : "memory");
+__device__ __forceinline__ ulonglong2 ld_relaxed_v2(const unsigned long long *p) {
+    ulonglong2 v;
+    asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ int ld_acquire_shared(const int32_t *p) {
+    int v;
+    asm volatile("ld.acquire.cta.shared.u32 %0, [%1];" : "=r"(v) : "r"(smem_u32(p)) : "memory");
+    return v;
+}
+__device__ __forceinline__ void st_release_shared(int32_t *p, int v) {
+    asm volatile("st.release.cta.shared.u32 [%0], %1;" ::"r"(smem_u32(p)), "r"(v) : "memory");
+}
+// The barrier of the sweep's warps.
+template <int N>
+__device__ __forceinline__ void sweep_barrier() {
+    asm volatile("bar.sync 1, %0;" ::"n"(N) : "memory");
+}
+// Bounded wait of a sweep warp for the exchanging warp (whose own waits are bounded and
+// which then sets `failed`); the same in every lane.
+static __device__ __noinline__ bool stream_wait(const int32_t *landed, int n, int need, volatile int32_t *failed, int64_t spin_ns) {
+    uint64_t t0 = 0;
+    for (int polls = 0;; ++polls) {
+        if (__all_sync(kFull, ld_acquire_shared(landed + (threadIdx.x & 31) % n) >= need)) return true;
+        if ((polls & 15) == 15) {
+            if (t0 == 0) t0 = global_ns();
+            if (__any_sync(kFull, *failed != 0 || (int64_t)(global_ns() - t0) > 2 * spin_ns + 1000000000)) {
+                *failed = 1;
+                return false;
+            }
+        }
+        __nanosleep(32);
+    }
 }
 __device__ __forceinline__ void st_relaxed_v2(unsigned long long *p, unsigned long long a, unsigned long long b) {
     asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(p), "l"(a), "l"(b) : "memory");
@@ -202,48 +228,44 @@ __device__ __forceinline__ unsigned long long tagged(int value, int tag) {
 }
 
 template <int K>
-__global__ void __launch_bounds__(stream_threads<K>(), stream_min_ctas<K>()) fill_lines_stream_kernel(const LaunchDesc L) {
+__global__ void __launch_bounds__(stream_cta_threads<K>(), stream_min_ctas<K>()) fill_lines_stream_kernel(const LaunchDesc L) {
     constexpr int NA = K - 1;
     constexpr int M = (1 << NA) - 1;
-    constexpr int NT = stream_threads<K>();
-    constexpr int NLINES = NT;
+    constexpr int NS = stream_threads<K>(), NT = stream_cta_threads<K>();  // threads of the sweep, of the CTA
+    constexpr int NLINES = NS;
     constexpr int SMAX = stream_skew_max(K);
-    constexpr int U = stream_block(K), D = stream_ring_d(K), R = stream_pt_ring(K);
-    constexpr int NPAR = D / U;  // block parities: slot of time bU + s is ((b mod NPAR) U + s) mod D
+    constexpr int U = stream_block(K), R = stream_pt_ring(K);
     constexpr int MASKB = (1 << K) - 1;
     using LY = StreamLayout<K>;
     constexpr int NH = LY::NH, NFL = LY::NFL, NROW = LY::NROW, ZS = LY::ZS;
-    constexpr int NP = NH * (U / 2);              // halo copies (two entries each) per block
-    constexpr int HC = LY::HC;                    // ... per thread
-    constexpr int NF = NFL * (U / 2);             // face stores (two entries each) per block
-    constexpr int FC = (NF + NT - 1) / NT;        // ... per thread
-    constexpr int PQ = (NROW * U + NT - 1) / NT;  // pair-table entries per thread and refill
-    constexpr int C0 = -((NA + U - 1) / U);       // first halo chunk: halo times start at -(k - 1)
-    // The ring holds a line's times from t - (k - 1) on plus the next block's U
-    // times; the pair-table ring holds the positions a block reads, bU + 1 - SMAX ..
-    // (b + 1) U, and in the block's step U - 2 the next U positions replace positions
-    // below (b + 1) U - SMAX, which its steps from U - 2 >= 1 on no longer read.
-    static_assert(D % U == 0 && NPAR <= 4 && D >= U + NA && SMAX + U <= R && (R & (R - 1)) == 0 && NFL < 128 &&
-                      U >= 3 && LY::PT < (1 << 14) && NT % (U / 2) == 0 && SMAX < 32 && M < 32,
+    constexpr int LQ = U / 2, LG = 32 / LQ;        // lanes per line (two entries each), lines per load of the warp
+    constexpr int NX = stream_xwarps(K);
+    constexpr int HB = K == 4 ? 3 : 8;            // loads in flight per lane of an exchanging warp
+    constexpr int PQ = (NROW * U + 32 * NX - 1) / (32 * NX);  // pair-table entries per lane and chunk
+    constexpr int NBATCH = (NH + NX * LG * HB - 1) / (NX * LG * HB);  // batches of a chunk per exchanging warp
+    // The ring holds three blocks of a line's times: the one being swept, the one before
+    // (read up to k - 1 times back) and the one whose halo is arriving. The pair-table
+    // ring: while block c - 1 is swept, it reads positions from (c - 1) U + 1 - SMAX on, and
+    // chunk c's positions cU + 1 .. (c + 1) U replace those R below.
+    static_assert(stream_ring_d(K) == 3 * U && U >= NA && U % 2 == 0 && 32 % LQ == 0 && (R & (R - 1)) == 0 &&
+                      2 * U + SMAX <= R && LY::PT < (1 << 14) && NFL < 128 && M < 32,
                   "geometry");
-    // ring slot of a time (which may be negative)
-    auto rslot = [](int x) { return (D & (D - 1)) == 0 ? x & (D - 1) : ((x % D) + D) % D; };
 
     extern __shared__ __align__(16) unsigned char smem_raw[];
     int32_t *sm = reinterpret_cast<int32_t *>(smem_raw);
     int32_t *V = sm + LY::V;
     int32_t *PT = sm + LY::PT;
-    unsigned long long *stage = reinterpret_cast<unsigned long long *>(sm + LY::STAGE);
+    int32_t *hsrc = sm + LY::HSRC;
     // halo lines: ring base | producer face line << 14 | axes S at -1 << 21 |
     // (the sum of SB_i over S: the producer's time offset) << 26
-    int32_t *hofs = sm + LY::HOFS;
-    int32_t *hmeta = sm + LY::HMETA;
     uint32_t *htab = reinterpret_cast<uint32_t *>(sm + LY::HTAB);
     uint32_t *ftab = reinterpret_cast<uint32_t *>(sm + LY::FTAB);  // face lines: ring base
     int32_t *nb = sm + LY::NB;
     int32_t *crow = sm + LY::CROW;
-    // [0] ticket, [2] poll verdict, [3] / [4] the two count checkpoints' verdicts
+    // [0] ticket, [1] blocks swept, [2] the waiting path's verdict, [3] failed, [4] [5] verdicts on
+    // the next block's chunk (by block parity), [8 ..] chunks of the halo in place, per exchanging warp
     volatile int32_t *misc = sm + LY::MISC;
+    int32_t *const swept = sm + LY::MISC + 1, *const landed = sm + LY::MISC + 8;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
     // face lines of the super-block in line order; their numbers index the faces
@@ -340,7 +362,6 @@ __global__ void __launch_bounds__(stream_threads<K>(), stream_min_ctas<K>()) fil
         const int64_t FB = (int64_t)NFL * ZQ;  // face entries per super-block
         unsigned long long *Fq = reinterpret_cast<unsigned long long *>(P.Q);
         unsigned long long *Fo = Fq + (int64_t)col * FB;
-        int32_t *const prog = L.done + P.tile_base;  // published blocks per super-block
 
         // this warp's tile (line block) for the traceback, or none past the grid
         int64_t tile = 0;
@@ -379,297 +400,206 @@ __global__ void __launch_bounds__(stream_threads<K>(), stream_min_ctas<K>()) fil
             crow[tid] = (x >= 1 && x <= len) ? codes[cof + x - 1] : 0;
         }
         for (int i = tid; i < LY::PT; i += NT) V[i] = kNeg;
+        if (tid < 7 + NX) misc[1 + tid] = 0;
         __syncthreads();  // nb, crow and the ring are read by every thread below
 
-        // Halo copies of the consumer times [cU, cU + U): pair idx = (halo line j,
-        // q2) holds times cU + 2 q2 and + 1, copied from the producer's face line
-        // at those times + SB_S (none where there is no producer or the producer
-        // time lies outside [0, ZQ), i.e. outside the producer's sweep).
-        const int q2 = tid % (U / 2);  // the same for every copy of this thread
-        // this thread's copies, once per column (copy v: pair idx = tid + NT v):
-        // the producer's face line (-1: none), ring base | time offset
-        // (formed at every copy instead, they cost more than the room they free)
-#pragma unroll
-        for (int v = 0; v < HC; ++v)
-            if (tid + NT * v < NP) {
-                const uint32_t e = htab[(tid + NT * v) / (U / 2)];
+        if (tid >= NS) {
+            // The exchanging warp. Chunk c of the halo is the consumer times [cU, cU + U):
+            // four lanes per line load the producer's entries at those times + SB_S, 16 bytes
+            // (two entries) each, again until both carry this launch's epoch, and store the
+            // values into the ring (kNeg where there is no producer or its sweep does not
+            // reach). A chunk may arrive once block c - 2 is swept; a swept block's faces go
+            // out before anything else.
+            const int q2 = lane % LQ, xw = (tid - NS) >> 5, sub = lane / LQ + LG * xw;
+            // (each warp's own lines: those with j / LG mod NX = xw)
+            for (int j = lane % LG + LG * xw; j < NH; j += LG * NX) {
+                const uint32_t e = htab[j];
                 const int src = nb[(e >> 21) & 31];
-                hofs[v * NT + tid] = src < 0 ? -1 : src * NFL + (int)((e >> 14) & 127);
-                hmeta[v * NT + tid] = (int)(e & 0x3FFF) | (2 * q2 + (int)(e >> 26)) << 14;
+                hsrc[j] = src < 0 ? -1 : src * NFL + (int)((e >> 14) & 127);
             }
-        auto halo_pair = [&](int v, int &base, int &toff) -> int64_t {
-            const int meta = hmeta[v * NT + tid];
-            base = meta & 0x3FFF;
-            toff = meta >> 14;
-            const int line = hofs[v * NT + tid];  // face lines of 2 ZQ words: fewer than 2^31 of them fit the GPU
-            return line < 0 ? -1 : (int64_t)line * ZQ;
-        };
-        auto halo_issue = [&](int c, bool mine) {
-            if (mine) {
-#pragma unroll
-                for (int v = 0; v < HC; ++v) {
-                    const int idx = tid + NT * v;
-                    if (idx < NP) {
-                        int base, toff;
-                        const int64_t o = halo_pair(v, base, toff);
-                        const int tp = c * U + toff;
-                        if (o >= 0 && (unsigned)tp < (unsigned)ZQ) cp_async16(stage + 2 * idx, Fq + o + tp);
+            __syncwarp();
+            int out = 0, chunk = -1, batch = 0, tables = -2;  // next block out, next chunk and batch in
+            uint64_t t0 = 0;
+            for (int polls = 0; out < nblk;) {
+                const int done = ld_acquire_shared(swept);
+                bool moved = false;
+                if (done > out) {  // face times [out U, out U + U) of the upper-face lines
+                    const int sl = out % 3 * U + 2 * q2, tt = out * U + 2 * q2;
+                    for (int f = sub; f < NFL; f += LG * NX) {
+                        const int32_t *v = V + ftab[f] + sl;
+                        st_relaxed_v2(Fo + (int64_t)f * ZQ + tt, tagged(v[0], tagout), tagged(v[1], tagout));
                     }
-                }
-            }
-            asm volatile("cp.async.commit_group;" ::: "memory");
-        };
-        auto sb_of = [](uint32_t S) {
-            int s = 0;
+                    ++out;
+                    moved = true;
+                } else if (chunk < nblk && done >= chunk - 1) {
+                    ulonglong2 x[HB];
+                    bool ok = true;
+                    const int tc = chunk * U + 2 * q2;
 #pragma unroll
-            for (int i = 0; i < NA; ++i)
-                if ((S >> i) & 1) s += stream_sb(K, i);
-            return s;
-        };
-        // Warp 0's lanes 1 .. M watch one producer each (subset S = lane). The
-        // counts cover consumer chunk c (times [cU, cU + U)) once producer S has
-        // published the blocks holding its times up to cU + U - 1 + SB_S.
-        const int my_src = warp == 0 && lane >= 1 && lane <= M ? nb[lane] : -1;
-        const int my_ahead = 1 + (U - 1 + sb_of((uint32_t)lane)) / U;
-        auto count_ok = [&](int cnt, int c) { return cnt >= min(nblk, c + my_ahead); };
-        // Wait (bounded) until the counts cover chunk c; every thread gets the verdict.
-        uint64_t t0 = 0;
-        auto halo_ready = [&](int c) -> bool {
-            if (warp == 0) {
-                bool ready = false;
-                for (int polls = 0;; ++polls) {
-                    ready = __all_sync(kFull, my_src < 0 || count_ok(ld_relaxed(prog + my_src), c));
-                    if (ready) break;
-                    if (t0 == 0) t0 = global_ns();
-                    if (ld_volatile(L.err) != 0 || (int64_t)(global_ns() - t0) > L.spin_ns) break;
-                    __nanosleep(polls < 8 ? 32 : 128);
-                }
-                if (lane == 0) misc[2] = ready;
-            }
-            __syncthreads();
-            return misc[2] != 0;
-        };
-        // Accept chunk c: store the staged entries into the ring once all carry
-        // this launch's tag. Copies not yet issued wait for the counts; entries
-        // that fail the tag check are copied again. Bounded.
-        auto halo_accept = [&](int c, bool issued) -> bool {
-            t0 = 0;
-            bool mine = true;
-            for (int tries = 0;; ++tries) {
-                if (!issued) {
-                    if (!halo_ready(c)) return false;
-                    halo_issue(c, mine);
-                }
-                asm volatile("cp.async.wait_all;" ::: "memory");  // each thread reads only its own copies
-                bool ok = true;
-#pragma unroll
-                for (int v = 0; v < HC; ++v) {
-                    const int idx = tid + NT * v;
-                    if (idx < NP) {
-                        const int tc = c * U + 2 * q2;
-                        int base, toff;
-                        const int64_t o = halo_pair(v, base, toff);
-                        const int tp = c * U + toff;
-                        int v0 = kNeg, v1 = kNeg;
-                        if (o >= 0 && (unsigned)tp < (unsigned)ZQ) {
-                            const ulonglong2 x = *reinterpret_cast<const ulonglong2 *>(stage + 2 * idx);
-                            ok = ok && (int)(x.x >> 32) == epoch && (int)(x.y >> 32) == epoch;
-                            v0 = (int)(unsigned)x.x;
-                            v1 = (int)(unsigned)x.y;
+                    for (int u = 0; u < HB; ++u) {
+                        const int j = (batch * HB + u) * LG * NX + sub;
+                        x[u] = make_ulonglong2(tagged(kNeg, epoch), tagged(kNeg, epoch));
+                        if (j < NH) {
+                            const int line = hsrc[j], tp = tc + (int)(htab[j] >> 26);
+                            if (line >= 0 && (unsigned)tp < (unsigned)ZQ)
+                                x[u] = ld_relaxed_v2(Fq + (int64_t)line * ZQ + tp);
                         }
-                        const int sl = rslot(tc);  // tc is even and D even: sl + 1 is the slot of tc + 1
-                        V[base + sl] = v0;
-                        V[base + sl + 1] = v1;
+                    }
+                    if (tables < chunk) {  // meanwhile the pair tables of positions cU + 1 .. (c + 1) U
+                        int pent[PQ];
+#pragma unroll
+                        for (int u = 0; u < PQ; ++u) {
+                            const int it = tid - NS + 32 * NX * u, p = chunk * U + 1 + it % U;
+                            pent[u] = it < NROW * U && p >= 1 && p <= lens ? codes[cofs + p - 1] : 0;
+                        }
+#pragma unroll
+                        for (int u = 0; u < PQ; ++u) {
+                            const int it = tid - NS + 32 * NX * u;
+                            if (it < NROW * U) pent[u] = __ldg(tab + crow[it / U] * A + pent[u]);
+                        }
+#pragma unroll
+                        for (int u = 0; u < PQ; ++u) {
+                            const int it = tid - NS + 32 * NX * u, p = chunk * U + 1 + it % U;
+                            if (it < NROW * U) {
+                                PT[it / U * ZS + (p & (R - 1))] = pent[u];
+                                PT[it / U * ZS + (p & (R - 1)) + R] = pent[u];
+                            }
+                        }
+                        tables = chunk;
+                    }
+#pragma unroll
+                    for (int u = 0; u < HB; ++u)
+                        ok = ok && (int)(x[u].x >> 32) == epoch && (int)(x[u].y >> 32) == epoch;
+                    if (__all_sync(kFull, ok)) {
+                        const int sl = (chunk + 3) % 3 * U + 2 * q2;
+#pragma unroll
+                        for (int u = 0; u < HB; ++u) {
+                            const int j = (batch * HB + u) * LG * NX + sub;
+                            if (j < NH) {
+                                int32_t *v = V + (htab[j] & 0x3FFF) + sl;
+                                v[0] = (int)(unsigned)x[u].x;
+                                v[1] = (int)(unsigned)x[u].y;
+                            }
+                        }
+                        if (++batch == NBATCH) {
+                            batch = 0;
+                            ++chunk;
+                            __syncwarp();
+                            if (lane == 0) st_release_shared(landed + xw, chunk);  // chunks below this one
+                        }
+                        moved = true;
                     }
                 }
-                if (__syncthreads_and(ok)) return true;
-                bool expired = false;
-                if (tid == 0) {
+                if (moved) {
+                    polls = 0;
+                    t0 = 0;
+                    continue;
+                }
+                if ((++polls & 15) == 0) {
                     if (t0 == 0) t0 = global_ns();
-                    expired = ld_volatile(L.err) != 0 || (int64_t)(global_ns() - t0) > L.spin_ns;
+                    if (__any_sync(kFull, misc[3] != 0 || ld_volatile(L.err) != 0 ||
+                                              (int64_t)(global_ns() - t0) > L.spin_ns)) {
+                        misc[3] = 1;
+                        break;
+                    }
                 }
-                if (__syncthreads_or(expired)) return false;  // no copy is in flight here
-                __nanosleep(32);
-                issued = false;
-                mine = !ok;
+                __nanosleep(polls < 64 ? 32 : 128);
             }
-        };
-        // face times [bU, bU + U) of the upper-face lines
-        auto face_write = [&](int b) {
+        } else {
+            int Sp[M + 1];
+            {
+                int cd[NA];
 #pragma unroll
-            for (int v = 0; v < FC; ++v) {
-                const int idx = tid + NT * v;
-                if (idx < NF) {
-                    const int f = idx / (U / 2), tt = b * U + 2 * (idx % (U / 2));
-                    const int base = (int)ftab[f], sl = rslot(tt);
-                    st_relaxed_v2(Fo + (int64_t)f * ZQ + tt, tagged(V[base + sl], tagout),
-                                  tagged(V[base + sl + 1], tagout));
+                for (int i = 0; i < NA; ++i) {
+                    const int x = o[i] + cl[i];
+                    cd[i] = (x >= 1 && x <= P.len[i]) ? codes[P.cofs[i] + x - 1] : 0;
                 }
-            }
-        };
-        // pair tables of positions [p0, p0 + U): codes, then entries (in place), then stores
-        int pent[PQ];
-        auto pt_codes = [&](int p0) {
+                Sp[0] = 0;
 #pragma unroll
-            for (int u = 0; u < PQ; ++u) {
-                const int it = tid + NT * u, p = p0 + it % U;
-                pent[u] = (it < NROW * U && p >= 1 && p <= lens) ? codes[cofs + p - 1] : 0;
-            }
-        };
-        auto pt_entries = [&]() {
+                for (int h = 0; h < NA; ++h) {
+                    int Rs[1 << (NA - 1)];
+                    Rs[0] = 0;
 #pragma unroll
-            for (int u = 0; u < PQ; ++u) {
-                const int it = tid + NT * u;
-                if (it < NROW * U) pent[u] = __ldg(tab + crow[it / U] * A + pent[u]);
-            }
-        };
-        auto pt_store = [&](int p0) {
+                    for (int r = 1; r < (1 << h); ++r) Rs[r] = Rs[r & (r - 1)] + __ldg(tab + cd[lowbit_c(r)] * A + cd[h]);
 #pragma unroll
-            for (int u = 0; u < PQ; ++u) {
-                const int it = tid + NT * u, p = p0 + it % U;
-                if (it < NROW * U && p < rho) {
-                    PT[(it / U) * ZS + (p & (R - 1))] = pent[u];
-                    PT[(it / U) * ZS + (p & (R - 1)) + R] = pent[u];
+                    for (int r = 0; r < (1 << h); ++r) Sp[r | (1 << h)] = Sp[r] + Rs[r];
                 }
             }
-        };
-
-        // Halo times [C0 U, U): one poll of the counts covers every initial chunk
-        // (a halo line with a -1 coordinate holds positions >= 0 at negative
-        // times); the first chunk's copies fly while this line's pair sums and the
-        // first pair-table positions are formed.
-        bool ok = halo_ready(0);
-        if (ok) halo_issue(C0, true);
-        pt_codes(0);
-        int Sp[M + 1];
-        {
-            int cd[NA];
+            // The sweep. The origin's lane starts from H(0) = 0 as its "previous
+            // position", which makes its key 0 with no move.
+            int Wl = -sig * (1 << NA);  // W(x) = Wl + t 2^NA at step t
 #pragma unroll
-            for (int i = 0; i < NA; ++i) {
-                const int x = o[i] + cl[i];
-                cd[i] = (x >= 1 && x <= P.len[i]) ? codes[P.cofs[i] + x - 1] : 0;
+            for (int i = 0; i < NA; ++i) Wl += (o[i] + cl[i]) << i;
+            int32_t *ptrow[NA];
+            {
+                int row = 0;
+#pragma unroll
+                for (int i = 0; i < NA; ++i) {
+                    ptrow[i] = PT + (row + cl[i]) * ZS;
+                    row += stream_sb(K, i);
+                }
             }
-            Sp[0] = 0;
+            int vself = col == 0 && tid == 0 ? 0 : kNeg;
+            int next = vself;  // best move of the next position that advances the last axis
+            uint8_t *tbw = P.tb + tile * P.tb_block + lane - sigw * 32;  // this warp's traceback rows, by step
+            int32_t *cur = vb, *prev = vb + 2 * U;  // the ring's slots of this block and the one before
+            bool go = false;                        // this block's chunk is in place
+            for (int b = 0; b < nblk; ++b) {
+                if (!go) {  // uniform over the sweep's warps
+                    if (warp == 0) {
+                        const bool r = stream_wait(landed, NX, b + 1, misc + 3, L.spin_ns);
+                        if (lane == 0) misc[2] = r;
+                    }
+                    sweep_barrier<NS>();
+                    if (!misc[2]) break;
+                }
+                const int Wb0 = Wl + b * U * (1 << NA);
+                const int zp0 = (b * U - sig) & (R - 1);
+                const int32_t *ptb[NA];
 #pragma unroll
-            for (int h = 0; h < NA; ++h) {
-                int Rs[1 << (NA - 1)];
-                Rs[0] = 0;
+                for (int i = 0; i < NA; ++i) ptb[i] = ptrow[i] + zp0;
 #pragma unroll
-                for (int r = 1; r < (1 << h); ++r) Rs[r] = Rs[r & (r - 1)] + __ldg(tab + cd[lowbit_c(r)] * A + cd[h]);
+                for (int s = 0; s < U; ++s) {
+                    const int ts = b * U + s;
+                    // a warp none of whose lanes holds a cell at this step skips it (every
+                    // thread still meets the step's one barrier)
+                    if ((unsigned)(ts - sigw) < (unsigned)(rho + line_skew_max(K))) {
+                        const bool act = (unsigned)(ts - sig) < (unsigned)rho;
+                        int p[NA];  // pair scores of the next position
 #pragma unroll
-                for (int r = 0; r < (1 << h); ++r) Sp[r | (1 << h)] = Sp[r] + Rs[r];
+                        for (int i = 0; i < NA; ++i) p[i] = ptb[i][s + 1];
+                        int acc0 = next, acc1 = kNeg;  // two independent max chains
+                        const int F = fold_subsets<NA, 0>(
+                            [&](auto m) {  // the predecessor line's value popc(m) times ago
+                                constexpr int q = popc_c(m.value), off = stream_move_off<K>(m.value);
+                                return (s >= q ? cur[s - q - off] : prev[s - q + U - off]) + Sp[m.value];
+                            },
+                            p, acc0, acc1);
+                        const int acc_all = max(acc0, acc1);
+                        const int tm = (Wb0 + s * (1 << NA) - acc_all) & MASKB;
+                        const int val = acc_all + tm;
+                        if (has_tile) tbw[s * 32] = (uint8_t)tm;
+                        if (act) {
+                            cur[s] = val;
+                            vself = val;
+                        }
+                        next = max(F, vself);
+                    }
+                    if (s == U - 2 && warp == 0) {
+                        const bool r = __all_sync(kFull, ld_acquire_shared(landed + lane % NX) >= b + 2);
+                        if (lane == 0) misc[4 + (b & 1)] = r;
+                    }
+                    sweep_barrier<NS>();
+                }
+                if (tid == 0) st_release_shared(swept, b + 1);
+                go = misc[4 + (b & 1)] != 0;
+                tbw += U * 32;
+                prev = cur;
+                cur = cur == vb + 2 * U ? vb : cur + U;
             }
-        }
-        pt_entries();
-        pt_store(0);
-        if (ok) ok = halo_accept(C0, true);
-        for (int c = C0 + 1; c <= 0 && ok; ++c) {
-            halo_issue(c, true);
-            ok = halo_accept(c, true);
         }
         __syncthreads();
-
-        // The sweep. The origin's lane starts from H(0) = 0 as its "previous
-        // position", which makes its key 0 with no move.
-        int Wl = -sig * (1 << NA);  // W(x) = Wl + t 2^NA at step t
-#pragma unroll
-        for (int i = 0; i < NA; ++i) Wl += (o[i] + cl[i]) << i;
-        int32_t *ptrow[NA];
-        {
-            int row = 0;
-#pragma unroll
-            for (int i = 0; i < NA; ++i) {
-                ptrow[i] = PT + (row + cl[i]) * ZS;
-                row += stream_sb(K, i);
-            }
-        }
-        int vself = col == 0 && tid == 0 ? 0 : kNeg;
-        int next = vself;  // best move of the next position that advances the last axis
-        // this warp's traceback rows: row r = t - (the line block's first skew)
-        const int rows = P.tb_block / 32;
-        uint8_t *tbw = P.tb + tile * P.tb_block + lane;
-
-        // One block of U steps, unrolled: PAR = b mod NPAR makes every ring slot a
-        // constant.
-        // Warp 0 judges the counts at steps J1 and J2 (each verdict in its own
-        // word), every thread reads a verdict after that step's barrier and
-        // issues the next chunk's copies.
-        constexpr int J1 = U / 4, J2 = U / 2 + U / 8;
-        static_assert(J1 < J2 && J2 + 1 < U, "checkpoints");
-        auto block = [&](int b, auto par) {
-            constexpr int PAR = decltype(par)::value;
-            const bool want = b + 1 < nblk;  // the next block needs chunk b + 1
-            int cnt = 0x7fffffff;
-            if (want && my_src >= 0) cnt = ld_relaxed(prog + my_src);
-            const bool refill = (b + 1) * U < rho;
-            if (refill) pt_codes((b + 1) * U);
-            bool issued = false;
-            const int Wb0 = Wl + b * U * (1 << NA);
-            const int r0 = b * U - sigw;  // traceback row of step bU
-            const int zp0 = (b * U - sig) & (R - 1);
-            constexpr int sl0 = PAR * U;  // ring slot of time bU
-            const int32_t *ptb[NA];
-#pragma unroll
-            for (int i = 0; i < NA; ++i) ptb[i] = ptrow[i] + zp0;
-            auto step = [&](int s) {
-                if ((s == J1 || s == J2) && want && !issued && warp == 0) {
-                    const bool r = __all_sync(kFull, my_src < 0 || count_ok(cnt, b + 1));
-                    if (lane == 0) misc[s == J1 ? 3 : 4] = r;
-                    if (!r && my_src >= 0) cnt = ld_relaxed(prog + my_src);
-                }
-                if ((s == J1 + 1 || s == J2 + 1) && want && !issued) {
-                    issued = misc[s == J1 + 1 ? 3 : 4] != 0;
-                    if (issued) halo_issue(b + 1, true);
-                }
-                if (s == U / 2 - 1 && refill) pt_entries();
-                const int ts = b * U + s;
-                // a warp none of whose lanes holds a cell at this step skips it (every
-                // thread still meets the step's one barrier)
-                if ((unsigned)(ts - sigw) < (unsigned)(rho + line_skew_max(K))) {
-                    const int z = ts - sig;
-                    const bool act = (unsigned)z < (unsigned)rho;
-                    const int own = sl0 + s < D ? sl0 + s : sl0 + s - D;  // slot of time ts
-                    int slp[NA + 1];  // slot of time ts - q
-#pragma unroll
-                    for (int q = 0; q <= NA; ++q) slp[q] = own - q < 0 ? own - q + D : own - q;
-                    int p[NA];  // pair scores of the next position
-#pragma unroll
-                    for (int i = 0; i < NA; ++i) p[i] = ptb[i][s + 1];
-                    int acc0 = next, acc1 = kNeg;  // two independent max chains
-                    const int F = fold_subsets<NA, 0>(
-                        [&](auto m) { return vb[slp[popc_c(m.value)] - stream_move_off<K>(m.value)] + Sp[m.value]; }, p,
-                        acc0, acc1);
-                    const int acc_all = max(acc0, acc1);
-                    const int tm = (Wb0 + s * (1 << NA) - acc_all) & MASKB;
-                    const int val = acc_all + tm;
-                    if (has_tile && (unsigned)(r0 + s) < (unsigned)rows) tbw[(int64_t)(r0 + s) * 32] = (uint8_t)tm;
-                    if (act) {
-                        vb[own] = val;
-                        vself = val;
-                    }
-                    next = max(F, vself);
-                }
-                // the block's last step reads the next block's first position; the
-                // positions replaced lie below every position this block still reads
-                if (s == U - 2 && refill) pt_store((b + 1) * U);
-                __syncthreads();
-            };
-#pragma unroll
-            for (int s = 0; s < U; ++s) step(s);
-            face_write(b);
-            __syncthreads();  // the block's face stores precede the count in program order (a hint)
-            if (tid == 0 && tagout != 0) st_relaxed(prog + col, b + 1);
-            if (want) ok = halo_accept(b + 1, issued);
-        };
-        for (int b = 0; b < nblk && ok; b += NPAR) {
-            block(b, IntC<0>{});
-            if constexpr (NPAR > 1)
-                if (b + 1 < nblk && ok) block(b + 1, IntC<1 % NPAR>{});
-            if constexpr (NPAR > 2)
-                if (b + 2 < nblk && ok) block(b + 2, IntC<2 % NPAR>{});
-            if constexpr (NPAR > 3)
-                if (b + 3 < nblk && ok) block(b + 3, IntC<3 % NPAR>{});
-        }
+        const bool ok = misc[3] == 0;
         if (!ok) {
             if (tid == 0) atomicCAS(L.err, 0, MSA_ETIMEOUT);
             break;
@@ -679,7 +609,7 @@ __global__ void __launch_bounds__(stream_threads<K>(), stream_min_ctas<K>()) fil
             bool corner = true;
 #pragma unroll
             for (int i = 0; i < NA; ++i) corner = corner && o[i] + cl[i] == P.len[i];
-            if (corner) *P.qcorner = V[vbase + rslot(lens + sig)];
+            if (corner && tid < NS) *P.qcorner = V[vbase + (lens + sig) % (3 * U)];
         }
     }
 }
@@ -697,7 +627,7 @@ template <int K>
 cudaError_t launch_stream(const LaunchDesc &L, int grid, cudaStream_t s) {
     cudaError_t e = stream_attributes<K>();
     if (e != cudaSuccess) return e;
-    fill_lines_stream_kernel<K><<<grid, stream_threads<K>(), stream_smem_bytes<K>(), s>>>(L);
+    fill_lines_stream_kernel<K><<<grid, stream_cta_threads<K>(), stream_smem_bytes<K>(), s>>>(L);
     return cudaGetLastError();
 }
 
@@ -705,7 +635,7 @@ template <int K>
 int stream_ctas() {
     if (stream_attributes<K>() != cudaSuccess) return 0;
     int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fill_lines_stream_kernel<K>, stream_threads<K>(),
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fill_lines_stream_kernel<K>, stream_cta_threads<K>(),
                                                       stream_smem_bytes<K>()) != cudaSuccess)
         return 0;
     return n;

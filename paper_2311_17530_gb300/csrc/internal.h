@@ -172,7 +172,7 @@ __host__ __device__ constexpr int line_skew_max(int K) {
 // whole last axis in lockstep, in blocks of stream_block(k) steps; super-blocks
 // exchange faces as (value, epoch) entries indexed by time.
 constexpr int kStreamMinK = 4, kStreamMaxK = 8;
-__host__ __device__ constexpr int stream_block(int K) { return K >= 6 ? 4 : 8; }  // steps per block = times per face chunk
+__host__ __device__ constexpr int stream_block(int K) { return K >= 7 ? 4 : 8; }  // steps per block = times per face chunk
 // k >= 6: the streamed kernel's whole-column form (fill_lines_wide.cuh) holds a last
 // axis of at most wide_z(k) positions (as many as leave room for three CTAs per SM,
 // two at k = 8); longer ones take the pipelined form at k = 6, the generic tile

@@ -234,3 +234,11 @@ def test_units_of_several_super_blocks(k, lens):
     assert (got[4].fill_kernel, want[4].fill_kernel) == (5, 1)
     assert got[:3] == want[:3] and got[2] == 0
     np.testing.assert_array_equal(got[3], want[3])
+
+
+@pytest.mark.parametrize("last", [0, 6, 7, 8, 14, 15, 16, 22, 23, 24, 31, 32])
+@pytest.mark.parametrize("k,lens", [(4, [5, 9, 8]), (5, [5, 4, 2, 5]), (6, [4, 5, 2, 3, 2])])
+def test_blocks_and_ring_of_the_last_axis(k, lens, last):
+    """One position below, at and above one, two, three and four blocks of 8 (the ring holds three), over
+    several super-blocks along every line axis."""
+    check(inputs.random_problem(4800 + last, k, lens + [last], alphabet=inputs.PROTEIN, related=True))
