@@ -4,7 +4,7 @@
 // folded from the previous position's candidates), organised for the latency of the
 // hardware. Measured (fill), with the exchange on warps of its own against inside the
 // sweep: k5 protein 33 - 45 1.097 against 1.402 ms, 15^5 0.100 / 0.159, 31^5 0.407 / 0.594;
-// k4 DNA 110 - 130 0.948 / 0.946, 61 - 64 0.189 / 0.237, 41^4 0.106 / 0.147, 21^4 0.050 /
+// k4 DNA 110 - 130 0.898 / 0.946, 61 - 64 0.184 / 0.237, 41^4 0.103 / 0.147, 21^4 0.050 /
 // 0.066.
 //
 // * A CTA of W sweeping warps owns a SUPER-BLOCK of W line blocks (a grid of extents
@@ -558,39 +558,48 @@ __global__ void __launch_bounds__(stream_cta_threads<K>(), stream_min_ctas<K>())
                 const int32_t *ptb[NA];
 #pragma unroll
                 for (int i = 0; i < NA; ++i) ptb[i] = ptrow[i] + zp0;
+                auto steps = [&](auto check) {
+                    constexpr bool CHECK = decltype(check)::value != 0;
 #pragma unroll
-                for (int s = 0; s < U; ++s) {
-                    const int ts = b * U + s;
-                    // a warp none of whose lanes holds a cell at this step skips it (every
-                    // thread still meets the step's one barrier)
-                    if ((unsigned)(ts - sigw) < (unsigned)(rho + line_skew_max(K))) {
-                        const bool act = (unsigned)(ts - sig) < (unsigned)rho;
-                        int p[NA];  // pair scores of the next position
+                    for (int s = 0; s < U; ++s) {
+                        const int ts = b * U + s;
+                        // a warp none of whose lanes holds a cell at this step skips it (every
+                        // thread still meets the step's one barrier)
+                        if (!CHECK || (unsigned)(ts - sigw) < (unsigned)(rho + line_skew_max(K))) {
+                            const bool act = !CHECK || (unsigned)(ts - sig) < (unsigned)rho;
+                            int p[NA];  // pair scores of the next position
 #pragma unroll
-                        for (int i = 0; i < NA; ++i) p[i] = ptb[i][s + 1];
-                        int acc0 = next, acc1 = kNeg;  // two independent max chains
-                        const int F = fold_subsets<NA, 0>(
-                            [&](auto m) {  // the predecessor line's value popc(m) times ago
-                                constexpr int q = popc_c(m.value), off = stream_move_off<K>(m.value);
-                                return (s >= q ? cur[s - q - off] : prev[s - q + U - off]) + Sp[m.value];
-                            },
-                            p, acc0, acc1);
-                        const int acc_all = max(acc0, acc1);
-                        const int tm = (Wb0 + s * (1 << NA) - acc_all) & MASKB;
-                        const int val = acc_all + tm;
-                        if (has_tile) tbw[s * 32] = (uint8_t)tm;
-                        if (act) {
-                            cur[s] = val;
-                            vself = val;
+                            for (int i = 0; i < NA; ++i) p[i] = ptb[i][s + 1];
+                            int acc0 = next, acc1 = kNeg;  // two independent max chains
+                            const int F = fold_subsets<NA, 0>(
+                                [&](auto m) {  // the predecessor line's value popc(m) times ago
+                                    constexpr int q = popc_c(m.value), off = stream_move_off<K>(m.value);
+                                    return (s >= q ? cur[s - q - off] : prev[s - q + U - off]) + Sp[m.value];
+                                },
+                                p, acc0, acc1);
+                            const int acc_all = max(acc0, acc1);
+                            const int tm = (Wb0 + s * (1 << NA) - acc_all) & MASKB;
+                            const int val = acc_all + tm;
+                            if (has_tile) tbw[s * 32] = (uint8_t)tm;
+                            if (act) {
+                                cur[s] = val;
+                                vself = val;
+                            }
+                            next = max(F, vself);
                         }
-                        next = max(F, vself);
+                        if (s == U - 2 && warp == 0) {
+                            const bool r = __all_sync(kFull, ld_acquire_shared(landed + lane % NX) >= b + 2);
+                            if (lane == 0) misc[4 + (b & 1)] = r;
+                        }
+                        sweep_barrier<NS>();
                     }
-                    if (s == U - 2 && warp == 0) {
-                        const bool r = __all_sync(kFull, ld_acquire_shared(landed + lane % NX) >= b + 2);
-                        if (lane == 0) misc[4 + (b & 1)] = r;
-                    }
-                    sweep_barrier<NS>();
-                }
+                };
+                // most blocks: every lane of the warp on a cell in every step (without the checks
+                // 0.948 -> 0.898 ms on k4 DNA, a fifth of a step's instructions)
+                if (b * U >= sigw + line_skew_max(K) && (b + 1) * U <= sigw + rho)
+                    steps(IntC<0>{});
+                else
+                    steps(IntC<1>{});
                 if (tid == 0) st_release_shared(swept, b + 1);
                 go = misc[4 + (b & 1)] != 0;
                 tbw += U * 32;
