@@ -96,6 +96,7 @@ struct C3Smem {
     int32_t ctl[2];
     int32_t cur_prob;
     int32_t pad[3];
+    int32_t corner[c3::R];                       // the far corner's lane's rows at the corner's CTA time
 };
 
 int col3_warps_per_cta() { return c3::W + 2; }
@@ -256,7 +257,7 @@ __device__ __forceinline__ void c3_load_face(C3St &g, const int *fr, int wR) {
 // One step. Everything with a latency is started a step or more before its use:
 // the shuffles of this step's values (for the next step) as soon as they exist,
 // the staged face a step ahead, row -1 a chunk ahead with one vote per chunk.
-template <int s, bool KEEP>
+template <int s, bool CAP, bool KEEP>
 __device__ __forceinline__ void c3_step(C3St &g, const C3Ln &c, const C3Fill &f, const C3Blk &b, int T0, int lane,
                                         C3Smem &sm, const LaunchDesc &L) {
     constexpr int R = c3::R, H = c3::U, M = R - 1;
@@ -290,6 +291,13 @@ __device__ __forceinline__ void c3_step(C3St &g, const C3Ln &c, const C3Fill &f,
         g.S[r] = __shfl_up_sync(kFull, g.V[r], 1);
     }
     g.SM = __shfl_up_sync(kFull, VMn, 1);
+    if constexpr (CAP) {  // one lane of the launch, once
+        if (T == c.ctime) {
+#pragma unroll
+            for (int r = 0; r < R; r += 4)
+                *reinterpret_cast<int4 *>(sm.corner + r) = make_int4(g.V[r], g.V[r + 1], g.V[r + 2], g.V[r + 3]);
+        }
+    }
     // outputs: last row to the warp below (or face F0), traceback bytes, lane 31 to face F1
     st_entry(b.rout + s * 32, pack_entry(g.V[R - 1], c.tagout + T));
     c3_load_face(g, b.f1row + (s + 1) * c3::F1S, c.wR);
@@ -348,28 +356,11 @@ __device__ __forceinline__ void c3_step(C3St &g, const C3Ln &c, const C3Fill &f,
     }
 }
 
-// A step of the block that holds the far corner's CTA time (kernels that record
-// the corner): the plain step, then the corner's lane stores its row's key.
-template <int s, bool KEEP>
-__device__ __forceinline__ void c3_capture_step(C3St &g, const C3Ln &c, const C3Fill &f, const C3Blk &b, int T0,
-                                                int lane, C3Smem &sm, const LaunchDesc &L) {
-    c3_step<s, KEEP>(g, c, f, b, T0, lane, sm, L);
-    if (T0 + s == c.ctime) {
-        int v = g.V[0];  // a select chain: a loop with a dynamic index would put the registers in memory
-#pragma unroll
-        for (int r = 1; r < c3::R; ++r) v = c.crow == r ? g.V[r] : v;
-        __stcg(c.qcorner, v + c.wcorner);
-    }
-}
-
 // The unrolled steps of a block.
 template <bool CAP, bool KEEP, int... S>
 __device__ __forceinline__ void c3_steps(C3St &g, const C3Ln &c, const C3Fill &f, const C3Blk &b, int T0, int lane,
                                          C3Smem &sm, const LaunchDesc &L, std::integer_sequence<int, S...>) {
-    if constexpr (CAP)
-        (c3_capture_step<S, KEEP>(g, c, f, b, T0, lane, sm, L), ...);
-    else
-        (c3_step<S, KEEP>(g, c, f, b, T0, lane, sm, L), ...);
+    (c3_step<S, CAP, KEEP>(g, c, f, b, T0, lane, sm, L), ...);
 }
 
 struct C3Col {
@@ -531,14 +522,16 @@ __device__ __forceinline__ bool c3_block_wait(C3Smem &sm, const C3Ln &c, int w, 
 
 }  // namespace
 
-// CAP: the warp that computes the far corner records its key for the traceback's
-// cross-check; the block holding it runs a capturing copy of the steps (which
-// costs registers, so plain launches use the kernel without it). KEEP: every cell's
+// CAP: the lane that computes the far corner lays its rows out in shared memory at the
+// corner's CTA time and records the corner's key at the column's end, for the
+// traceback's cross-check: a comparison and two predicated stores per step, 0.703 ms at
+// 700 x 760 x 800 and 0.107 at 128^3 (plain launches, without it, 0.640 and 0.099). A
+// second copy of the block's steps with the capture, for the corner's block only, was
+// 1.96 and 0.232 (instruction fetch). KEEP: every cell's
 // best candidate, V plus tag, is kept for the near-optimal walk (c3::kept_term): the
 // traceback's layout with a word for its byte and a lane's rows in runs of four, so
 // that each 16-byte store of a warp is one run (120 x 110 x 130: 0.089 ms, 0.085 without
-// KEEP; 0.225 with CAP's second copy of the steps to record the corner, instruction
-// fetch, so the corner's lane reads its own store back instead).
+// KEEP); the corner's lane reads its own store back.
 template <bool CAP, bool KEEP>
 __global__ void __launch_bounds__(c3::THREADS, c3::CTAS) fill_col3_kernel(const LaunchDesc L) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -673,12 +666,6 @@ __global__ void __launch_bounds__(c3::THREADS, c3::CTAS) fill_col3_kernel(const 
 
             unsigned long long *ringout = lastw ? cc.f0dst + lane : &sm.ring[w + 1][0][lane];
             unsigned char *tbw = P.tb + (int64_t)lin * c3::tb_col_bytes(P.rho[2]) + (w * 32 + lane) * c3::R;
-            // the block of the corner's CTA time, the same in every lane of its warp
-            int T0c = -2 * c3::U;
-            if (CAP) {
-                const int ct = __shfl_sync(kFull, c.ctime, (P.len[1] - 32 * cc.B) & 31);
-                if (ct != (int)0x80000000) T0c = ct / c3::U * c3::U;
-            }
             C3Blk b;
             b.rin2 = &sm.ring[w][-c3::U & (c3::SI - 1)][lane];
             b.rout = ringout + (lastw ? 0 : (-c3::U & (c3::SI - 1)) * 32);
@@ -705,12 +692,10 @@ __global__ void __launch_bounds__(c3::THREADS, c3::CTAS) fill_col3_kernel(const 
                 n.f1o = b.f1o + c3::U * c3::WR;
                 n.p02 = &sm.p02r[w][0][(Tn + 2 - c.wR - lane) & (c3::SQ - 1)][0];
                 n.p12 = &sm.p12r[(Tn + 2 - c.wR) & (c3::SP - 1)][lane];
-                if (!CAP || T0 != T0c)
-                    c3_steps<false, KEEP>(g, c, f, b, T0, lane, sm, L, std::make_integer_sequence<int, c3::U>{});
-                else
-                    c3_steps<true, KEEP>(g, c, f, b, T0, lane, sm, L, std::make_integer_sequence<int, c3::U>{});
+                c3_steps<CAP, KEEP>(g, c, f, b, T0, lane, sm, L, std::make_integer_sequence<int, c3::U>{});
                 b = n;
             }
+            if (CAP && c.ctime != (int)0x80000000) __stcg(c.qcorner, sm.corner[c.crow] + c.wcorner);
             if constexpr (KEEP) {  // the corner's lane has its score from its own store
                 if (c.ctime != (int)0x80000000) {
                     const int64_t at = c3::kept_term(0, P.len[0], NB, P.rho[2]) + c3::kept_term(1, P.len[1], NB, P.rho[2]) +
