@@ -217,6 +217,7 @@ void fill_problem_desc(const HostPlan &hp, const PlanPointers &pp, int64_t tile_
     d.tile_base = tile_base;
     d.ntiles = hp.ntiles;
     d.has_qcorner = hp.check_corner;
+    d.qelems = hp.qelems;
     d.face0_stride = hp.face0_stride;
     d.face1_stride = hp.face1_stride;
     d.face0_rows = hp.face0_rows;

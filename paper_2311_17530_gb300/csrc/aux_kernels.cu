@@ -14,10 +14,10 @@ __global__ void encode_kernel(const ProblemDesc *probs, const IODesc *io_arr, IO
     const IODesc io = io_arr ? io_arr[p] : io1;
     msa_device_result *st = P.istat;
     if (P.clear_faces) {
-        // Column-kernel faces in a reused region: tag 0 everywhere, so that no
-        // stale word can pass for an entry of this launch (the fill runs after this
-        // kernel on the same stream). Face sizes are multiples of 64 ints.
-        const int64_t n0 = P.face0_stride * P.ntiles / 4, n1 = P.face1_stride * P.ntiles / 4;
+        // Tagged faces in a reused region: tag 0 everywhere, so that no stale word can
+        // pass for an entry of this launch (the fill runs after this kernel on the same
+        // stream). Face sizes are multiples of 16 ints.
+        const int64_t n0 = P.qelems / 4, n1 = P.face1_stride * P.ntiles / 4;
         const int4 z = make_int4(0, 0, 0, 0);
         for (int64_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n0; i += (int64_t)gridDim.x * blockDim.x)
             reinterpret_cast<int4 *>(P.Q)[i] = z;

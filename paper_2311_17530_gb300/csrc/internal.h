@@ -59,6 +59,7 @@ struct ProblemDesc {
     int32_t face1_rows;          // column kernel: skewed rows per axis-1 face
     int32_t tb_layout;           // 0: row-major (tbstride); 1: column-blocked (column kernel);
                                  // 2, 3: tile-major (generic tile kernel, line kernel)
+    int64_t qelems;              // words of Q
     int32_t clear_faces;         // the encode step zeroes the column kernel's faces first (serving:
                                  // the arena region may hold stale words of other requests)
     const uint8_t *amap;         // device 256-entry char -> code map (0xFF: invalid)

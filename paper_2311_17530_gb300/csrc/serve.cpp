@@ -214,11 +214,25 @@ int Server::submit(const msa_request *req, uint64_t *out) {
     }
     r->subst.assign(req->subst, req->subst + (size_t)r->A * r->A);
     std::string err;
-    // the streamed line kernel stays out of serving: its faces would have to be
-    // cleared in every reused arena region (8 bytes per cell); the line kernel
-    // synchronises by flags instead
+    // The streamed line kernel at k = 4, 5 where it is the choice for a plan: clearing its
+    // faces in the reused arena region (4 bytes a cell, in the encode step) costs less than
+    // the segmented line kernel's fill takes longer. A burst of 256 mixed requests: 7.5 ms
+    // against 9.1, their fills at k = 4 2.7 against 4.1, encoding 0.54 against 0.11; 8
+    // requests 0.87 against 1.1. k = 6 stays with the segmented kernel (the whole-column
+    // form's launch depends on the request's last axis), and so does a request whose
+    // streamed working set the arena could not hold.
     const int choice = cfg.fill_kernel == kKernelStream ? kKernelLines : (int)cfg.fill_kernel;
-    rc = make_plan(r->k, r->lens.data(), r->A, choice, r->hp, err, -1, false);
+    bool streamed = false;
+    if (r->k <= 5 && choose_kernel(r->k, r->lens.data(), r->A, (int)cfg.fill_kernel, true) == kKernelStream &&
+        make_plan(r->k, r->lens.data(), r->A, kKernelStream, r->hp, err, -1) == MSA_OK) {
+        size_t rb = 0, cap = (size_t)cfg.budget_mb << 20;
+        {
+            std::lock_guard<std::mutex> lk(mu_);
+            if (started_) cap = arena_bytes_;
+        }
+        streamed = plan_layout(r->hp, nullptr, nullptr, &rb) + Arena::kAlign <= cap;
+    }
+    if (!streamed) rc = make_plan(r->k, r->lens.data(), r->A, choice, r->hp, err, -1, false);
     if (rc) {
         delete r;
         return set_error(rc, "%s", err.c_str());
@@ -420,7 +434,7 @@ int Server::launch(Slot &sl, std::vector<ServeReq *> &batch, const Settings &cfg
         }
         Group &g = groups.back();
         g.count++;
-        g.tickets += hp.ntiles;
+        g.tickets += hp.nunits;
         g.tiles += hp.ntiles;
         g.maxA = std::max(g.maxA, hp.A);
     }
@@ -490,7 +504,7 @@ int Server::launch(Slot &sl, std::vector<ServeReq *> &batch, const Settings &cfg
     msa_device_result *distat = reinterpret_cast<msa_device_result *>(D + off_istat);
     msa_device_result *dres = reinterpret_cast<msa_device_result *>(D + sl.off_results);
     int64_t max_ncode = 1;
-    bool clear = false;
+    bool clear = false, streamed = false;
     for (Group &g : groups) {
         int64_t tile_base = 0;
         for (int j = 0; j < g.count; ++j) {
@@ -502,6 +516,7 @@ int Server::launch(Slot &sl, std::vector<ServeReq *> &batch, const Settings &cfg
             fill_problem_desc(r->hp, pp, tile_base, hdesc[i]);
             hdesc[i].clear_faces = tagged_faces(r->hp) ? 1 : 0;
             clear = clear || tagged_faces(r->hp);
+            streamed = streamed || r->hp.kernel == kKernelStream;
             tile_base += r->hp.ntiles;
             hdesc[i].amap = reinterpret_cast<uint8_t *>(D + off_amap + (size_t)i * 256);
             hdesc[i].istat = distat + i;
@@ -557,7 +572,7 @@ int Server::launch(Slot &sl, std::vector<ServeReq *> &batch, const Settings &cfg
     int rc = MSA_OK;
     if (e == cudaSuccess) e = cudaMemcpyAsync(D, H, in_bytes, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(D + off_state, 0, zero_bytes, s);
-    if (e == cudaSuccess) e = launch_encode(ddesc, n, max_ncode, dio, IODesc{}, s, clear ? 32 : 1);
+    if (e == cudaSuccess) e = launch_encode(ddesc, n, max_ncode, dio, IODesc{}, s, clear ? (streamed ? 128 : 32) : 1);
     for (size_t gi = 0; gi < groups.size() && e == cudaSuccess; ++gi) {
         const Group &g = groups[gi];
         LaunchDesc L;
@@ -577,6 +592,7 @@ int Server::launch(Slot &sl, std::vector<ServeReq *> &batch, const Settings &cfg
         e = g.kernel == kKernelCol3    ? launch_fill_col3(L, g.grid, col3_smem_bytes(g.maxA), s)
           : g.kernel == kKernelBand2 ? launch_fill_band2(L, g.grid, s)
           : g.kernel == kKernelLines ? launch_fill_lines(g.k, g.edge, L, g.grid, s)
+          : g.kernel == kKernelStream ? launch_fill_stream(g.k, L, g.grid, s, 0)
                                      : launch_fill_tiles(g.k, g.edge, L, g.grid, s);
     }
     if (e == cudaSuccess) e = launch_traceback(ddesc, n, &dstate[0].err, dio, IODesc{}, s);

@@ -242,3 +242,19 @@ def test_blocks_and_ring_of_the_last_axis(k, lens, last):
     """One position below, at and above one, two, three and four blocks of 8 (the ring holds three), over
     several super-blocks along every line axis."""
     check(inputs.random_problem(4800 + last, k, lens + [last], alphabet=inputs.PROTEIN, related=True))
+
+
+@pytest.mark.parametrize("k", [4, 5])
+def test_serving_in_reused_arena_regions(k):
+    """The streamed kernel in serving: bursts of requests of changing sizes, whose faces fall on what
+    earlier requests left in the arena."""
+    msa.msa_config("fill_kernel", 0)
+    for burst in range(3):
+        probs = [inputs.random_problem(4900 + 10 * burst + i, k, [5 + (3 * i + burst) % 9, 8 + i, 11 - i, 7 + 9 * i, 30][5 - k:],
+                                       related=True) for i in range(5)]
+        probs += [inputs.random_problem(4950 + burst, 3, [40, 35 + burst, 50]), inputs.random_problem(4960 + burst, 2, [150, 90])]
+        handles = [msa.msa_submit(p.seqs, p.alphabet, p.subst, p.gap) for p in probs]
+        msa.msa_drain()
+        for h, p in zip(handles, probs):
+            want = oracle.align(p.seqs, p.alphabet, p.subst, p.gap)
+            assert msa.msa_poll(h, p.k, sum(p.lens)) == (want.score, want.rows)
