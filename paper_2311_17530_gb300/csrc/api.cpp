@@ -905,12 +905,14 @@ cudaError_t prune_analyse(PruneRun &R, const IODesc &io, cudaStream_t s) {
     return e;
 }
 
-// k = 5, 6: the share of a tensor's cells that must be left out for the generic
-// tile kernel, which skips them, to beat the line kernels, which fill everything
-// (one call, k = 5 at 0.78 left out 2.4 against 3.0 ms, k = 6 at 1.0 2.4 against
-// 4.9 ms; of whole tensors the line kernels are 2.3 to 4 times as fast). k = 4: the
-// streamed kernel is faster even at 0.98 left out (1.2 against 1.6 ms).
-constexpr double kPruneTilesShare = 0.65;
+// k >= 5: the generic tile kernel, which skips what is left out, against the line
+// kernels, which fill everything several times as fast per cell: the tiles' own chain of
+// waves takes 1.2 to 2.5 ms, so they win only where much is left out of a large tensor.
+// One call, ms with tiles / lines: k = 6, 87 M cells with 1.0 left out 2.5 / 3.3; k = 5,
+// 116 M, 0.95 2.48 / 2.57; 100 M, 0.78 2.49 / 2.50; but 34 M, 0.97 1.64 / 1.34; k = 6, 47 M,
+// 0.65 2.28 / 1.71; k = 7, 36 M, 1.0 2.66 / 1.81.
+constexpr double kPruneTilesShare = 0.78;
+constexpr int64_t kPruneTilesCells = 80000000;
 
 }  // namespace
 
@@ -937,11 +939,11 @@ int msa_align_pruned(int k, const char *const *seqs, const int32_t *lens, const 
     // gains little from it, and the generic tile kernel that can leave tiles out is
     // the slowest per cell. k = 2 and 3: always the band and column kernels (k = 3,
     // 700 / 760 / 800 with 98 % of the tiles left out: 0.64 ms against 6.4 ms).
-    // k = 4: always the streamed kernel; k = 5, 6: the line kernels unless enough is
-    // left out.
+    // k = 4: always the streamed kernel; k >= 5: the line kernels unless enough of a large
+    // tensor is left out.
     int kernel = choose_kernel(k, lens, hp.A, kKernelAuto);
     int64_t st[2] = {0, 0};
-    if (k > 4 && kernel != kKernelTiles) {
+    if (k > 4 && kernel != kKernelTiles && hp.cells >= kPruneTilesCells) {
         e = cudaStreamSynchronize(s);
         if (e == cudaSuccess) e = cudaMemcpy(st, R.D.stats, 16, cudaMemcpyDeviceToHost);
         if (e != cudaSuccess) return cuda_error(e, "pruning kernels");

@@ -119,7 +119,7 @@ extern "C" int msa_align_noalloc(int k, const int32_t *lens, const char *alphabe
                                       "array holds %u bytes",
                          need, (unsigned)MSA_NOALLOC_SCRATCH_BYTES);
     // The band, column or line kernel where its working set fits too (k = 3 protein,
-    // 120 x 110 x 130, the whole call: 0.24 ms against 0.96 ms with the tile fill). Not the streamed line
+    // 120 x 110 x 130, the whole call: 0.14 ms against 0.96 ms with the tile fill). Not the streamed line
     // kernel, whose faces would have to be cleared at 8 bytes a cell.
     const int choice = choose_kernel(k, lens, A, kKernelAuto, false);
     if (choice != kKernelTiles) {

@@ -124,8 +124,8 @@ int choose_kernel(int k, const int32_t *lens, int A, int requested, bool allow_s
     if (requested == kKernelTiles) return kKernelTiles;
     if (requested == kKernelStream && k >= kStreamMinK && k <= kLinesMaxK) return kKernelStream;
     // k = 7, 8: the whole-column form where the last axis fits its box (k = 7, 12 x 10 x
-    // 13 x 11 x 10 x 12 x 11 cells: 1.38 against 4.84 ms of the generic tile kernel; 9^8:
-    // 8.5 against 26.6 ms)
+    // 13 x 11 x 10 x 12 x 11 cells: 1.00 against 4.84 ms of the generic tile kernel; 9^8:
+    // 5.5 against 26.6 ms)
     if (k > kLinesMaxK && stream_fits(k, lens) &&
         (requested == kKernelStream ||
          (requested == kKernelAuto && allow_stream && prefer_stream(k) && !tile_edge_set(k))))

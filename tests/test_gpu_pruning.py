@@ -146,3 +146,13 @@ def greedy_score(p):
             score += (int(p.subst[p.alphabet.index(p.seqs[i][x[i] - 1]), p.alphabet.index(p.seqs[j][x[j] - 1])])
                       if a and b else p.gap if a or b else 0)
     return score
+
+
+@pytest.mark.parametrize("k,lens", [(6, [20, 20, 21, 22, 20, 21]), (5, [40, 39, 41, 40, 38])])
+def test_large_tensors_with_most_tiles_left_out(k, lens):
+    """Beyond 8e7 cells with most of them left out the generic tile kernel fills the rest: the same
+    score and alignment as the fill of every cell."""
+    p = inputs.random_problem(9950 + k, k, lens, alphabet=inputs.PROTEIN, related=True)
+    score, rows, stats = msadp.msa_align_pruned(p.seqs, p.alphabet, p.subst, p.gap)
+    assert stats["cells"] >= 8e7 and stats["cells_skipped"] > 0.8 * stats["cells"]
+    assert (score, rows) == msa.msa_align(p.seqs, p.alphabet, p.subst, p.gap)
