@@ -18,10 +18,6 @@ __device__ __forceinline__ int ld_acquire(const int32_t *p) {
     return v;
 }
 
-__device__ __forceinline__ void st_relaxed(int32_t *p, int v) {
-    asm volatile("st.relaxed.gpu.global.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
-}
-
 __device__ __forceinline__ void st_release(int32_t *p, int v) {
     asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
