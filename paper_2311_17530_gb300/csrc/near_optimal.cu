@@ -364,7 +364,7 @@ __global__ void __launch_bounds__(kBeamThreads) near_beam_kernel(const ProblemDe
                     S += x[i];
                     W += x[i] << i;
                     open |= (x[i] > 0) << i;
-                    code[i] = codes[min(cofs[i] + max(x[i] - 1, 0), total - 1)];  // at x_i = 0 unused, but a code
+                    code[i] = x[i] > 0 ? codes[cofs[i] + x[i] - 1] : 0;  // (no residue to read where all are empty)
                 }
                 acc = st[K];
                 int pair[NP];

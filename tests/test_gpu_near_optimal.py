@@ -104,3 +104,12 @@ def test_scores_kept_by_the_band_and_column_kernels(lens):
     for delta in (0, 2):
         check(inputs.random_problem(8900 + sum(lens), len(lens), list(lens), alphabet=inputs.PROTEIN, related=True),
               delta, 60)
+
+
+@pytest.mark.parametrize("k", range(2, 9))
+def test_every_sequence_empty(k):
+    """No residue at all: one alignment of no columns, level by level (its only slot stands at the
+    origin, where there is no residue code to read) and by the depth-first walk (max_count = 2049)."""
+    for max_count in (1, 4, 2049):
+        p = inputs.random_problem(9000 + k, k, [0] * k, alphabet=inputs.PROTEIN)
+        assert check(p, 3, max_count) == [(0, [], [""] * k)]
