@@ -951,7 +951,8 @@ int msa_align_pruned(int k, const char *const *seqs, const int32_t *lens, const 
     }
     if (kernel != kKernelTiles && plan_create(k, lens, alphabet, kernel, -1, &R.plan) != MSA_OK) kernel = kKernelTiles;
     if (kernel == kKernelTiles) {
-        rc = plan_create(k, lens, alphabet, kKernelTiles, -1, &R.plan);
+        // with the edge the flags were made for (the tuned one may have changed since)
+        rc = plan_create(k, lens, alphabet, kKernelTiles, hp.edge, &R.plan);
         if (rc) return rc;
         // the fill reads the tiles' flags through the plan's problem descriptor
         ProblemDesc pd;

@@ -1,0 +1,142 @@
+// Host check of the library's device calls (compiled by tests/test_host_calls.py): api.cpp,
+// plan.cpp and tune.cpp linked against a CUDA runtime and kernel launchers of this file.
+// Device memory is host memory; a launcher only notes what it was asked for. Modes:
+//   pruned    the fill of a pruned call gets the flags of its own tile grid, also when the
+//             tuned tile edge changes while the call runs
+#include <cuda_runtime.h>
+
+#include <cstdio>
+#include <cstdlib>
+#include <cstring>
+#include <string>
+#include <vector>
+
+#include "api_internal.h"
+
+using namespace msadp;
+
+static int g_bad = 0;
+#define CHECK(cond, ...)                                            \
+    do {                                                            \
+        if (!(cond)) {                                              \
+            printf("line %d: %s: ", __LINE__, #cond);               \
+            printf(__VA_ARGS__);                                    \
+            printf("\n");                                           \
+            ++g_bad;                                                \
+        }                                                           \
+    } while (0)
+
+// ---------------------------------------------------------------------------
+// The runtime.
+
+extern "C" {
+cudaError_t cudaGetDevice(int *d) { return *d = 0, cudaSuccess; }
+cudaError_t cudaDeviceGetAttribute(int *v, cudaDeviceAttr, int) { return *v = 152, cudaSuccess; }
+cudaError_t cudaGetLastError() { return cudaSuccess; }
+const char *cudaGetErrorString(cudaError_t) { return "error"; }
+cudaError_t cudaMalloc(void **p, size_t n) { return (*p = calloc(n + 1, 1)) ? cudaSuccess : cudaErrorMemoryAllocation; }
+cudaError_t cudaFree(void *p) { return free(p), cudaSuccess; }
+cudaError_t cudaHostAlloc(void **p, size_t n, unsigned) { return cudaMalloc(p, n); }
+cudaError_t cudaFreeHost(void *p) { return cudaFree(p); }
+cudaError_t cudaMemcpy(void *d, const void *s, size_t n, cudaMemcpyKind) { return memcpy(d, s, n), cudaSuccess; }
+cudaError_t cudaMemcpyAsync(void *d, const void *s, size_t n, cudaMemcpyKind, cudaStream_t) { return memcpy(d, s, n), cudaSuccess; }
+cudaError_t cudaMemset(void *d, int v, size_t n) { return memset(d, v, n), cudaSuccess; }
+cudaError_t cudaMemsetAsync(void *d, int v, size_t n, cudaStream_t) { return memset(d, v, n), cudaSuccess; }
+cudaError_t cudaStreamCreateWithFlags(cudaStream_t *s, unsigned) { return *s = (cudaStream_t)0x10, cudaSuccess; }
+cudaError_t cudaStreamSynchronize(cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaDeviceSynchronize() { return cudaSuccess; }
+cudaError_t cudaEventCreate(cudaEvent_t *e) { return *e = (cudaEvent_t)0x20, cudaSuccess; }
+cudaError_t cudaEventDestroy(cudaEvent_t) { return cudaSuccess; }
+cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaEventSynchronize(cudaEvent_t) { return cudaSuccess; }
+cudaError_t cudaEventElapsedTime(float *ms, cudaEvent_t, cudaEvent_t) { return *ms = 1, cudaSuccess; }
+}
+
+// ---------------------------------------------------------------------------
+// The kernel launchers.
+
+static PruneDesc g_prune;           // of the last analysis
+static int g_edge_after_prune = 0;  // tile edge another thread sets once the analysis is enqueued
+static int g_tile_fills = 0;
+
+namespace msadp {
+cudaError_t launch_encode(const ProblemDesc *, int, int, const IODesc *, IODesc, cudaStream_t, int) { return cudaSuccess; }
+cudaError_t launch_traceback(const ProblemDesc *, int, const int32_t *, const IODesc *, IODesc, cudaStream_t) { return cudaSuccess; }
+cudaError_t launch_prune(const PruneDesc &D, bool, cudaStream_t) {
+    g_prune = D;
+    if (g_edge_after_prune) set_tile_edge(D.k, g_edge_after_prune);
+    return cudaSuccess;
+}
+cudaError_t launch_fill_tiles(int k, int edge, const LaunchDesc &L, int, cudaStream_t) {
+    ++g_tile_fills;
+    const ProblemDesc &P = L.probs[0];
+    if (P.skip) {
+        CHECK(P.skip == g_prune.skip, "flags of another call");
+        CHECK(P.ntiles == g_prune.ntiles && L.ntickets == g_prune.ntiles, "k=%d: %lld tiles filled, flags of %lld", k,
+              (long long)P.ntiles, (long long)g_prune.ntiles);
+        for (int i = 0; i < k; ++i)
+            CHECK(tile_ext(k, edge, i) == g_prune.E[i] && P.E[i] == g_prune.E[i], "k=%d axis %d: extent %d, flags for %d", k, i,
+                  P.E[i], g_prune.E[i]);
+    }
+    return cudaSuccess;
+}
+cudaError_t launch_fill_col3(const LaunchDesc &, int, int, cudaStream_t) { return cudaSuccess; }
+cudaError_t launch_fill_band2(const LaunchDesc &, int, cudaStream_t) { return cudaSuccess; }
+cudaError_t launch_fill_lines(int, int, const LaunchDesc &, int, cudaStream_t) { return cudaSuccess; }
+cudaError_t launch_fill_stream(int, const LaunchDesc &, int, cudaStream_t, int) { return cudaSuccess; }
+size_t near_optimal_work_bytes(int, int64_t, int32_t) { return 0; }
+cudaError_t launch_near_optimal(int, int64_t, const ProblemDesc *, IODesc, int64_t, int32_t, NearOut, cudaStream_t) { return cudaSuccess; }
+int fill_tiles_ctas_per_sm(int, int) { return 1; }
+int fill_tiles_warps_per_cta(int, int) { return 1; }
+int fill_col3_ctas_per_sm(int) { return 1; }
+int fill_lines_ctas_per_sm(int, int) { return 1; }
+int fill_lines_warps_per_cta(int, int) { return 1; }
+int fill_stream_ctas_per_sm(int) { return 1; }
+int fill_band2_ctas_per_sm() { return 1; }
+int fill_band2_warps_per_cta() { return 2; }
+int col3_smem_bytes(int) { return 1; }
+}  // namespace msadp
+
+// ---------------------------------------------------------------------------
+
+struct Problem {
+    int k;
+    std::vector<std::string> text;
+    std::vector<const char *> seqs;
+    std::vector<int32_t> lens, table;
+    std::string alphabet;
+    Problem(std::vector<int32_t> lens_, int letters) : k((int)lens_.size()), lens(std::move(lens_)) {
+        alphabet = std::string("ABCDEFGHIJKLMNOPQRSTUVWXYZ").substr(0, (size_t)letters);
+        for (int32_t n : lens) text.push_back(std::string((size_t)n, 'A'));
+        for (auto &t : text) seqs.push_back(t.c_str());
+        table.assign((size_t)letters * letters, 1);
+    }
+};
+
+static void pruned() {
+    // k = 3 with 25 letters and k = 7, 8 with a long last axis take the tile kernel
+    struct { std::vector<int32_t> lens; int letters, edge; } cases[] = {
+        {{40, 41, 39}, 25, 8}, {{40, 41, 39}, 25, 16}, {{3, 4, 3, 2, 3, 4, 20}, 4, 3}};
+    for (auto &c : cases) {
+        Problem p(c.lens, c.letters);
+        std::string out((size_t)p.k * 400, '\0');
+        int32_t score = 0;
+        g_tile_fills = 0;
+        g_edge_after_prune = c.edge;
+        const int rc = msa_align_pruned(p.k, p.seqs.data(), p.lens.data(), p.alphabet.c_str(), p.table.data(), -1, 0, 0, &score,
+                                        &out[0], nullptr);
+        CHECK(rc == MSA_OK, "%s", msa_last_error());
+        CHECK(g_tile_fills == 1, "%d fills by the tile kernel", g_tile_fills);
+        CHECK(tile_edge_for(p.k) == c.edge, "the edge did not change");
+        g_edge_after_prune = 0;
+        msa_set_tile_edge(p.k, 0);
+    }
+}
+
+int main(int argc, char **argv) {
+    const std::string mode = argc > 1 ? argv[1] : "";
+    if (mode == "pruned") pruned();
+    else CHECK(false, "unknown mode");
+    if (!g_bad) printf("ok\n");
+    return g_bad != 0;
+}
