@@ -240,7 +240,6 @@ void fill_problem_desc(const HostPlan &hp, const PlanPointers &pp, int64_t tile_
 cudaError_t clear_faces(const HostPlan &hp, const PlanPointers &pp, cudaStream_t s) {
     cudaError_t e = cudaMemsetAsync(pp.Q, 0, (size_t)hp.qelems * 4, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(pp.aux, 0, (size_t)hp.aux_elems * 4, s);
-    if (e == cudaSuccess && s == nullptr) e = cudaDeviceSynchronize();
     return e;
 }
 
@@ -374,7 +373,10 @@ int plan_create(int k, const int32_t *lens, const char *alphabet, int kernel_cho
         e = cudaMemcpy(p->pp.order, p->hp.order.data(), p->hp.order.size() * 8, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(p->pp.amap, amap, 256, cudaMemcpyHostToDevice);
     // tagged faces start with tag 0, which no execution uses
-    if (e == cudaSuccess && tagged_faces(p->hp)) e = clear_faces(p->hp, p->pp);
+    if (e == cudaSuccess && tagged_faces(p->hp)) e = clear_faces(p->hp, p->pp, nullptr);
+    // these writes may still be on their way, and an execution's stream need not wait for
+    // the default one
+    if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
     if (e != cudaSuccess) {
         cudaFree(p->ws);
         delete p;
@@ -720,10 +722,11 @@ int msa_near_optimal(int k, const char *const *seqs, const int32_t *lens, const 
         if (lens[i]) memcpy(res.data() + o, seqs[i], (size_t)lens[i]);
         o += (size_t)lens[i];
     }
+    // (copies on the call's own stream: its kernels do not wait for the default one)
     cudaStream_t s = library_stream(&rc);
     if (!rc) {
-        e = cudaMemcpy(d + o_res, res.data(), total, cudaMemcpyHostToDevice);
-        if (e == cudaSuccess) e = cudaMemcpy(d + o_sub, subst, (size_t)A * A * 4, cudaMemcpyHostToDevice);
+        e = cudaMemcpyAsync(d + o_res, res.data(), total, cudaMemcpyHostToDevice, s);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(d + o_sub, subst, (size_t)A * A * 4, cudaMemcpyHostToDevice, s);
         if (e != cudaSuccess) rc = cuda_error(e, "near-optimal inputs");
     }
     if (!rc)
@@ -759,6 +762,7 @@ int msa_near_optimal(int k, const char *const *seqs, const int32_t *lens, const 
         *out_count = cm[0];
         *out_more = cm[1];
     }
+    if (rc) cudaStreamSynchronize(s);  // nothing may read the inputs' host memory any more
     cudaFree(d);
     msa_plan_destroy(plan);
     return rc;
@@ -829,18 +833,24 @@ struct PruneRun {
     size_t reset_bytes = 0;
     char *ws = nullptr;
     char *d = nullptr;
+    cudaStream_t s = nullptr;  // of the whole call: its copies, too, for a kernel here does not wait for the default stream
     PruneDesc D;
     size_t o_res = 0, o_sub = 0, o_out = 0, o_masks = 0, o_prune = 0, o_ws = 0;
+    std::vector<char> res;  // host memory of copies, kept until the stream is done
+    ProblemDesc desc, fill_desc;
+    uint8_t amap[256];
     ~PruneRun() {
-        if (d) cudaFree(d);
+        if (d) {
+            cudaStreamSynchronize(s);
+            cudaFree(d);
+        }
         if (plan) msa_plan_destroy(plan);
     }
 };
 
 int prune_setup(int k, const char *const *seqs, const int32_t *lens, const char *alphabet, const int32_t *subst,
                 const int32_t *E, PruneRun &R) {
-    uint8_t amap[256];
-    int rc = validate_request(k, seqs, lens, alphabet, subst, amap);
+    int rc = validate_request(k, seqs, lens, alphabet, subst, R.amap);
     if (rc) return rc;
     for (int i = 0; i < k; ++i)
         if (lens[i] > 16383) return set_error(MSA_ETOOBIG, "pruning takes sequences of at most 16383 residues");
@@ -868,6 +878,8 @@ int prune_setup(int k, const char *const *seqs, const int32_t *lens, const char 
     R.o_masks = take(total + 16);
     R.o_ws = take(wbytes);
     R.o_prune = take(pbytes);
+    R.s = library_stream(&rc);
+    if (rc) return rc;
     cudaError_t e = cudaMalloc(&R.d, off);
     if (e != cudaSuccess) {
         cudaGetLastError();
@@ -880,28 +892,27 @@ int prune_setup(int k, const char *const *seqs, const int32_t *lens, const char 
     prune_layout(hp, E ? E : hp.E, R.d + R.o_prune, R.D);
     R.D.codes = R.pp.codes;
     R.D.sub = reinterpret_cast<const int32_t *>(R.d + R.o_sub);
-    std::vector<char> res(total + 1);
+    R.res.resize(total + 1);
     size_t o = 0;
     for (int i = 0; i < k; ++i) {
-        if (lens[i]) memcpy(res.data() + o, seqs[i], (size_t)lens[i]);
+        if (lens[i]) memcpy(R.res.data() + o, seqs[i], (size_t)lens[i]);
         o += (size_t)lens[i];
     }
-    ProblemDesc pd;
-    fill_problem_desc(bare, R.pp, 0, pd);
-    e = cudaMemcpy(R.d + R.o_res, res.data(), total, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(R.d + R.o_sub, subst, A * A * 4, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(R.pp.prob, &pd, sizeof pd, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(R.pp.amap, amap, 256, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemset(R.D.stats, 0, 16);
+    fill_problem_desc(bare, R.pp, 0, R.desc);
+    e = cudaMemcpyAsync(R.d + R.o_res, R.res.data(), total, cudaMemcpyHostToDevice, R.s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(R.d + R.o_sub, subst, A * A * 4, cudaMemcpyHostToDevice, R.s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(R.pp.prob, &R.desc, sizeof R.desc, cudaMemcpyHostToDevice, R.s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(R.pp.amap, R.amap, 256, cudaMemcpyHostToDevice, R.s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(R.D.stats, 0, 16, R.s);
     if (e != cudaSuccess) return cuda_error(e, "pruning inputs");
     return MSA_OK;
 }
 
 // The encode step and the pruning kernels, on the set-up's own descriptor.
-cudaError_t prune_analyse(PruneRun &R, const IODesc &io, cudaStream_t s) {
-    cudaError_t e = cudaMemsetAsync(R.ws, 0, R.reset_bytes, s);
-    if (e == cudaSuccess) e = launch_encode(R.pp.prob, 1, R.hp.len_sum, nullptr, io, s);
-    if (e == cudaSuccess) e = launch_prune(R.D, R.D.greedy != 0, s);
+cudaError_t prune_analyse(PruneRun &R, const IODesc &io) {
+    cudaError_t e = cudaMemsetAsync(R.ws, 0, R.reset_bytes, R.s);
+    if (e == cudaSuccess) e = launch_encode(R.pp.prob, 1, R.hp.len_sum, nullptr, io, R.s);
+    if (e == cudaSuccess) e = launch_prune(R.D, R.D.greedy != 0, R.s);
     return e;
 }
 
@@ -927,13 +938,12 @@ int msa_align_pruned(int k, const char *const *seqs, const int32_t *lens, const 
     R.D.gap = gap;
     R.D.greedy = have_lower_bound ? 0 : 1;
     R.D.bound = nullptr;
-    cudaError_t e = cudaMemcpy(R.D.lower, &lower_bound, 8, cudaMemcpyHostToDevice);
+    cudaStream_t s = R.s;
+    cudaError_t e = cudaMemcpyAsync(R.D.lower, &lower_bound, 8, cudaMemcpyHostToDevice, s);
     if (e != cudaSuccess) return cuda_error(e, "pruning set-up");
-    cudaStream_t s = library_stream(&rc);
-    if (rc) return rc;
     msa_device_result *d_res = reinterpret_cast<msa_device_result *>(R.d + R.o_out);
     uint8_t *d_masks = reinterpret_cast<uint8_t *>(R.d + R.o_masks);
-    e = prune_analyse(R, IODesc{R.d + R.o_res, R.D.sub, d_res, d_masks, gap, 0}, s);
+    e = prune_analyse(R, IODesc{R.d + R.o_res, R.D.sub, d_res, d_masks, gap, 0});
     if (e != cudaSuccess) return cuda_error(e, "pruning kernels");
     // The fill: a tile left out saves work, but a fill bound by its chain of waves
     // gains little from it, and the generic tile kernel that can leave tiles out is
@@ -955,10 +965,9 @@ int msa_align_pruned(int k, const char *const *seqs, const int32_t *lens, const 
         rc = plan_create(k, lens, alphabet, kKernelTiles, hp.edge, &R.plan);
         if (rc) return rc;
         // the fill reads the tiles' flags through the plan's problem descriptor
-        ProblemDesc pd;
-        fill_problem_desc(R.plan->hp, R.plan->pp, 0, pd);
-        pd.skip = R.D.skip;
-        e = cudaMemcpy(R.plan->pp.prob, &pd, sizeof pd, cudaMemcpyHostToDevice);
+        fill_problem_desc(R.plan->hp, R.plan->pp, 0, R.fill_desc);
+        R.fill_desc.skip = R.D.skip;
+        e = cudaMemcpyAsync(R.plan->pp.prob, &R.fill_desc, sizeof R.fill_desc, cudaMemcpyHostToDevice, s);
         if (e != cudaSuccess) return cuda_error(e, "pruning set-up");
     }
     rc = msa_plan_execute(R.plan, R.d + R.o_res, R.D.sub, gap, d_res, d_masks, s);
@@ -1000,12 +1009,10 @@ int msa_tile_bounds(int k, const char *const *seqs, const int32_t *lens, const c
     R.D.gap = gap;
     R.D.greedy = 0;
     R.D.skip = nullptr;
-    cudaStream_t s = library_stream(&rc);
-    if (rc) return rc;
     IODesc io{R.d + R.o_res, R.D.sub, reinterpret_cast<msa_device_result *>(R.d + R.o_out),
               reinterpret_cast<uint8_t *>(R.d + R.o_masks), gap, 0};
-    cudaError_t e = prune_analyse(R, io, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    cudaError_t e = prune_analyse(R, io);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(R.s);
     msa_device_result st;
     if (e == cudaSuccess) e = cudaMemcpy(&st, &R.pp.state->istat, sizeof st, cudaMemcpyDeviceToHost);
     if (e != cudaSuccess) return cuda_error(e, "tile bounds");

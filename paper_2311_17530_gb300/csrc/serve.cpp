@@ -329,6 +329,7 @@ void Server::run() {
     if (e == cudaSuccess) e = cudaMalloc(&arena_base_, arena_bytes_);
     // face entries must start with a tag no launch uses
     if (e == cudaSuccess) e = cudaMemset(arena_base_, 0, arena_bytes_);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);  // the slots' streams do not wait for the default one
     for (int i = 0; i < kSlots && e == cudaSuccess; ++i)
         e = cudaStreamCreateWithFlags(&slots_[i].s, cudaStreamNonBlocking);
     std::unique_lock<std::mutex> lk(mu_);

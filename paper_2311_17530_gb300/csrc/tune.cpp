@@ -130,6 +130,7 @@ int msa_autotune(int k, const int32_t *lens, int alphabet_size, int32_t repeats,
     if (e == cudaSuccess) e = cudaMalloc(&b.masks, (size_t)total + 16);
     if (e == cudaSuccess) e = cudaMemcpy(b.res, res.data(), res.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(b.sub, sub.data(), sub.size() * 4, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);  // the library stream does not wait for the default one
     if (e != cudaSuccess) {
         cudaGetLastError();
         return set_error(MSA_ENOMEM, "autotune buffers: %s", cudaGetErrorString(e));

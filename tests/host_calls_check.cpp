@@ -3,7 +3,12 @@
 // Device memory is host memory; a launcher only notes what it was asked for. Modes:
 //   pruned    the fill of a pruned call gets the flags of its own tile grid, also when the
 //             tuned tile edge changes while the call runs
+//   ordering  no kernel is launched on a stream while a write of the default stream, which
+//             that stream does not wait for, may still be on its way; host memory that an
+//             asynchronous copy reads stays as it is until the copy's stream is waited for;
+//             no result is read before that
 #include <cuda_runtime.h>
+#include <malloc.h>
 
 #include <cstdio>
 #include <cstdlib>
@@ -29,6 +34,25 @@ static int g_bad = 0;
 // ---------------------------------------------------------------------------
 // The runtime.
 
+static int g_default_writes = 0;  // writes of the default stream that nothing has waited for
+static bool g_busy = false;       // work on another stream that nothing has waited for
+struct Source {
+    const char *at;
+    std::vector<char> bytes;
+};
+static std::vector<Source> g_sources;  // host memory of its copies
+
+static void stream_work(const char *what) {
+    CHECK(g_default_writes == 0, "%s with %d writes of the default stream on their way", what, g_default_writes);
+    g_busy = true;
+}
+static void wait_streams() {
+    for (const Source &s : g_sources)
+        CHECK(memcmp(s.at, s.bytes.data(), s.bytes.size()) == 0, "a copy's source changed before the copy was waited for");
+    g_sources.clear();
+    g_busy = false;
+}
+
 extern "C" {
 cudaError_t cudaGetDevice(int *d) { return *d = 0, cudaSuccess; }
 cudaError_t cudaDeviceGetAttribute(int *v, cudaDeviceAttr, int) { return *v = 152, cudaSuccess; }
@@ -38,17 +62,45 @@ cudaError_t cudaMalloc(void **p, size_t n) { return (*p = calloc(n + 1, 1)) ? cu
 cudaError_t cudaFree(void *p) { return free(p), cudaSuccess; }
 cudaError_t cudaHostAlloc(void **p, size_t n, unsigned) { return cudaMalloc(p, n); }
 cudaError_t cudaFreeHost(void *p) { return cudaFree(p); }
-cudaError_t cudaMemcpy(void *d, const void *s, size_t n, cudaMemcpyKind) { return memcpy(d, s, n), cudaSuccess; }
-cudaError_t cudaMemcpyAsync(void *d, const void *s, size_t n, cudaMemcpyKind, cudaStream_t) { return memcpy(d, s, n), cudaSuccess; }
-cudaError_t cudaMemset(void *d, int v, size_t n) { return memset(d, v, n), cudaSuccess; }
-cudaError_t cudaMemsetAsync(void *d, int v, size_t n, cudaStream_t) { return memset(d, v, n), cudaSuccess; }
+// A copy from pageable memory and a memset may return before the device has them; work on
+// a non-blocking stream does not wait for the default stream's (every stream but it here).
+cudaError_t cudaMemcpy(void *d, const void *s, size_t n, cudaMemcpyKind kind) {
+    if (kind == cudaMemcpyDeviceToHost) {
+        CHECK(!g_busy, "results read before their stream is done");
+        g_default_writes = 0;  // waits for the default stream
+    } else {
+        ++g_default_writes;
+    }
+    return memcpy(d, s, n), cudaSuccess;
+}
+cudaError_t cudaMemsetAsync(void *d, int v, size_t n, cudaStream_t s) {
+    if (s) stream_work("memset");
+    else ++g_default_writes;
+    return memset(d, v, n), cudaSuccess;
+}
+cudaError_t cudaMemset(void *d, int v, size_t n) { return cudaMemsetAsync(d, v, n, nullptr); }
+cudaError_t cudaMemcpyAsync(void *d, const void *s, size_t n, cudaMemcpyKind kind, cudaStream_t stream) {
+    if (!stream) return cudaMemcpy(d, s, n, kind);
+    stream_work("copy");
+    if (kind == cudaMemcpyHostToDevice && n)
+        g_sources.push_back({(const char *)s, std::vector<char>((const char *)s, (const char *)s + n)});
+    return memcpy(d, s, n), cudaSuccess;
+}
+cudaError_t cudaStreamSynchronize(cudaStream_t s) {
+    if (s) wait_streams();
+    else g_default_writes = 0;
+    return cudaSuccess;
+}
+cudaError_t cudaDeviceSynchronize() {
+    wait_streams();
+    g_default_writes = 0;
+    return cudaSuccess;
+}
 cudaError_t cudaStreamCreateWithFlags(cudaStream_t *s, unsigned) { return *s = (cudaStream_t)0x10, cudaSuccess; }
-cudaError_t cudaStreamSynchronize(cudaStream_t) { return cudaSuccess; }
-cudaError_t cudaDeviceSynchronize() { return cudaSuccess; }
 cudaError_t cudaEventCreate(cudaEvent_t *e) { return *e = (cudaEvent_t)0x20, cudaSuccess; }
 cudaError_t cudaEventDestroy(cudaEvent_t) { return cudaSuccess; }
 cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) { return cudaSuccess; }
-cudaError_t cudaEventSynchronize(cudaEvent_t) { return cudaSuccess; }
+cudaError_t cudaEventSynchronize(cudaEvent_t) { return wait_streams(), cudaSuccess; }
 cudaError_t cudaEventElapsedTime(float *ms, cudaEvent_t, cudaEvent_t) { return *ms = 1, cudaSuccess; }
 }
 
@@ -59,15 +111,23 @@ static PruneDesc g_prune;           // of the last analysis
 static int g_edge_after_prune = 0;  // tile edge another thread sets once the analysis is enqueued
 static int g_tile_fills = 0;
 
-namespace msadp {
-cudaError_t launch_encode(const ProblemDesc *, int, int, const IODesc *, IODesc, cudaStream_t, int) { return cudaSuccess; }
-cudaError_t launch_traceback(const ProblemDesc *, int, const int32_t *, const IODesc *, IODesc, cudaStream_t) { return cudaSuccess; }
-cudaError_t launch_prune(const PruneDesc &D, bool, cudaStream_t) {
-    g_prune = D;
-    if (g_edge_after_prune) set_tile_edge(D.k, g_edge_after_prune);
+static cudaError_t kernel(cudaStream_t s) {
+    if (s) stream_work("kernel");
     return cudaSuccess;
 }
-cudaError_t launch_fill_tiles(int k, int edge, const LaunchDesc &L, int, cudaStream_t) {
+
+namespace msadp {
+cudaError_t launch_encode(const ProblemDesc *, int, int, const IODesc *, IODesc, cudaStream_t s, int) { return kernel(s); }
+cudaError_t launch_traceback(const ProblemDesc *, int, const int32_t *, const IODesc *, IODesc io, cudaStream_t s) {
+    *io.result = msa_device_result{};
+    return kernel(s);
+}
+cudaError_t launch_prune(const PruneDesc &D, bool, cudaStream_t s) {
+    g_prune = D;
+    if (g_edge_after_prune) set_tile_edge(D.k, g_edge_after_prune);
+    return kernel(s);
+}
+cudaError_t launch_fill_tiles(int k, int edge, const LaunchDesc &L, int, cudaStream_t s) {
     ++g_tile_fills;
     const ProblemDesc &P = L.probs[0];
     if (P.skip) {
@@ -78,14 +138,14 @@ cudaError_t launch_fill_tiles(int k, int edge, const LaunchDesc &L, int, cudaStr
             CHECK(tile_ext(k, edge, i) == g_prune.E[i] && P.E[i] == g_prune.E[i], "k=%d axis %d: extent %d, flags for %d", k, i,
                   P.E[i], g_prune.E[i]);
     }
-    return cudaSuccess;
+    return kernel(s);
 }
-cudaError_t launch_fill_col3(const LaunchDesc &, int, int, cudaStream_t) { return cudaSuccess; }
-cudaError_t launch_fill_band2(const LaunchDesc &, int, cudaStream_t) { return cudaSuccess; }
-cudaError_t launch_fill_lines(int, int, const LaunchDesc &, int, cudaStream_t) { return cudaSuccess; }
-cudaError_t launch_fill_stream(int, const LaunchDesc &, int, cudaStream_t, int) { return cudaSuccess; }
+cudaError_t launch_fill_col3(const LaunchDesc &, int, int, cudaStream_t s) { return kernel(s); }
+cudaError_t launch_fill_band2(const LaunchDesc &, int, cudaStream_t s) { return kernel(s); }
+cudaError_t launch_fill_lines(int, int, const LaunchDesc &, int, cudaStream_t s) { return kernel(s); }
+cudaError_t launch_fill_stream(int, const LaunchDesc &, int, cudaStream_t s, int) { return kernel(s); }
 size_t near_optimal_work_bytes(int, int64_t, int32_t) { return 0; }
-cudaError_t launch_near_optimal(int, int64_t, const ProblemDesc *, IODesc, int64_t, int32_t, NearOut, cudaStream_t) { return cudaSuccess; }
+cudaError_t launch_near_optimal(int, int64_t, const ProblemDesc *, IODesc, int64_t, int32_t, NearOut, cudaStream_t s) { return kernel(s); }
 int fill_tiles_ctas_per_sm(int, int) { return 1; }
 int fill_tiles_warps_per_cta(int, int) { return 1; }
 int fill_col3_ctas_per_sm(int) { return 1; }
@@ -133,9 +193,47 @@ static void pruned() {
     }
 }
 
+static void ordering() {
+    mallopt(M_PERTURB, 0xa5);  // freed memory changes at once
+    for (int k = 2; k <= 8; ++k) {
+        const int n = k == 2 ? 700 : k == 3 ? 40 : k < 6 ? 9 : 4;
+        Problem p(std::vector<int32_t>((size_t)k, n), k == 3 ? 20 : 4);
+        const int A = (int)p.alphabet.size();
+        std::string out((size_t)k * (size_t)(k * n + 1), '\0');
+        int32_t score = 0, ncols[4], count = 0, more = 0;
+        int64_t scores[4];
+        std::vector<uint8_t> masks((size_t)4 * k * n + 16);
+        // plans of every kernel, executed on a stream of the caller's
+        for (int kernel = 0; kernel <= 5; ++kernel) {
+            msa_config("fill_kernel", kernel);
+            msa_plan *plan = nullptr;
+            CHECK(msa_plan_create(k, p.lens.data(), p.alphabet.c_str(), &plan) == MSA_OK, "%s", msa_last_error());
+            msa_device_result res;
+            msa_plan_execute(plan, p.seqs[0], p.table.data(), -1, &res, masks.data(), (void *)0x30);
+            cudaStreamSynchronize((cudaStream_t)0x30);
+            msa_plan_destroy(plan);
+        }
+        msa_config("fill_kernel", 0);
+        CHECK(msa_align(k, p.seqs.data(), p.lens.data(), p.alphabet.c_str(), p.table.data(), -1, &score, &out[0]) == MSA_OK, "%s",
+              msa_last_error());
+        for (int given = 0; given < 2; ++given)
+            CHECK(msa_align_pruned(k, p.seqs.data(), p.lens.data(), p.alphabet.c_str(), p.table.data(), -1, given, -5, &score,
+                                   &out[0], nullptr) == MSA_OK, "%s", msa_last_error());
+        const std::vector<int32_t> ext((size_t)k, 100);
+        std::vector<int64_t> bounds(64);  // at most 7 x 7 tiles
+        CHECK(msa_tile_bounds(k, p.seqs.data(), p.lens.data(), p.alphabet.c_str(), p.table.data(), -1, ext.data(),
+                              bounds.data()) == MSA_OK, "%s", msa_last_error());
+        CHECK(msa_near_optimal(k, p.seqs.data(), p.lens.data(), p.alphabet.c_str(), p.table.data(), -1, 1, 4, masks.data(), ncols,
+                               scores, &count, &more) == MSA_OK, "%s", msa_last_error());
+        msa_tuning t;
+        CHECK(msa_autotune(k, p.lens.data(), A, 1, &t) == MSA_OK, "%s", msa_last_error());
+    }
+}
+
 int main(int argc, char **argv) {
     const std::string mode = argc > 1 ? argv[1] : "";
     if (mode == "pruned") pruned();
+    else if (mode == "ordering") ordering();
     else CHECK(false, "unknown mode");
     if (!g_bad) printf("ok\n");
     return g_bad != 0;

@@ -27,3 +27,7 @@ def check(tmp_path_factory):
 
 def test_pruned_fill_takes_the_flags_of_its_own_grid(check):
     check("pruned")
+
+
+def test_device_work_is_ordered_after_the_copies_it_reads(check):
+    check("ordering")
