@@ -415,7 +415,9 @@ typedef struct msa_tuning {
  * of alphabet_size letters: one warm-up and `repeats` executions each, on the
  * library stream. The fastest becomes the choice for k (msa_set_tile_edge or
  * msa_set_line_segment, and whether the automatic kernel choice takes the band,
- * column, line or streamed line kernel).
+ * column, line or streamed line kernel). A kernel that cannot take these lengths (the
+ * column kernel; at k = 6..8 the whole-column form beyond its last axis) is not timed,
+ * and shapes it can take keep it.
  * Allocates device memory; synchronous.
  */
 int msa_autotune(int k, const int32_t *lens, int alphabet_size, int32_t repeats, msa_tuning *out);

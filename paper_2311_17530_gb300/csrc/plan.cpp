@@ -38,13 +38,6 @@ int tile_edge_for(int k) {
     return g_edge[k] ? g_edge[k] : tile_edge_default(k);
 }
 
-// A tile edge set for k = 7, 8 selects the generic tile kernel (the only one there
-// until it was given a whole-column form).
-static bool tile_edge_set(int k) {
-    std::lock_guard<std::mutex> g(g_tune_mu);
-    return g_edge[k] != 0;
-}
-
 int set_tile_edge(int k, int edge) {
     if (k < 2 || k > MSA_MAX_K || (edge != 0 && !tile_edge_valid(k, edge))) return MSA_EINVAL;
     std::lock_guard<std::mutex> g(g_tune_mu);
@@ -128,16 +121,15 @@ int choose_kernel(int k, const int32_t *lens, int A, int requested, bool allow_s
     // 5.5 against 26.6 ms)
     if (k > kLinesMaxK && stream_fits(k, lens) &&
         (requested == kKernelStream ||
-         (requested == kKernelAuto && allow_stream && prefer_stream(k) && !tile_edge_set(k))))
+         (requested == kKernelAuto && allow_stream && prefer_stream(k))))
+        return kKernelStream;
+    // at k = 6 only the whole-column form (last axis of at most kWideZ) beats the line kernel
+    if (k >= kLinesMinK && k <= kLinesMaxK && requested == kKernelAuto && allow_stream && prefer_stream(k) &&
+        stream_fits(k, lens) && (k != 6 || lens[k - 1] + 1 <= kWideZ))
         return kKernelStream;
     if (k >= kLinesMinK && k <= kLinesMaxK &&
-        (requested == kKernelLines || requested == kKernelStream || (requested == kKernelAuto && !prefer_tiles_lines(k)))) {
-        // at k = 6 only the whole-column form (last axis of at most kWideZ) beats the line kernel
-        if (requested == kKernelAuto && allow_stream && prefer_stream(k) && stream_fits(k, lens) &&
-            (k != 6 || lens[k - 1] + 1 <= kWideZ))
-            return kKernelStream;
+        (requested == kKernelLines || requested == kKernelStream || (requested == kKernelAuto && !prefer_tiles_lines(k))))
         return kKernelLines;
-    }
     if (k == 2 && (requested == kKernelBand2 || (requested == kKernelAuto && !prefer_tiles_k2()))) return kKernelBand2;
     if (col3_fits(k, lens, A) && (requested == kKernelCol3 || !prefer_tiles_k3())) return kKernelCol3;
     return kKernelTiles;

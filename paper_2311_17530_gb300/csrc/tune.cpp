@@ -1,8 +1,8 @@
 // Autotuner of the tile shape: the paper fixes its partition size S by hand
 // (section 3.2's example uses S = 3); here each k has a few compiled tile edges
 // (tile_edge_candidate) and, for k = 3, the column kernel (k = 2: the band
-// kernel; k = 4 .. 6: the line kernel's compiled segment lengths, and at k = 4, 5
-// its streamed form). msa_autotune times
+// kernel; k = 4 .. 6: the line kernel's compiled segment lengths; k = 4 .. 8: its
+// streamed form). msa_autotune times
 // every candidate on a synthetic problem of the caller's shape -- plan creation,
 // then repeated executions of encode, fill and traceback between CUDA events --
 // and makes the fastest the choice for k in every later plan and serving batch.
@@ -71,7 +71,10 @@ int msa_set_tile_edge(int k, int32_t edge) {
         return set_error(MSA_EINVAL, "tile edge %d is not compiled for k=%d", edge, k);
     if (k == 3 && edge == 0) set_prefer_tiles_k3(false);  // defaults: the column kernel where it fits
     if (k == 2 && edge == 0) set_prefer_tiles_k2(false);  // defaults: the band kernel
-    if (k > kLinesMaxK && edge == 0) reset_prefer_stream(k);  // defaults: the whole-column form where it fits
+    if (k > kLinesMaxK) {  // an edge selects the tile kernel; defaults: the whole-column form where it fits
+        if (edge) set_prefer_stream(k, false);
+        else reset_prefer_stream(k);
+    }
     return MSA_OK;
 }
 
@@ -83,7 +86,7 @@ int msa_get_tile_edge(int k, int32_t *out_edge) {
 
 int msa_set_line_segment(int k, int32_t z) {
     if (set_line_z(k, z) != MSA_OK) return set_error(MSA_EINVAL, "line segment %d is not compiled for k=%d", z, k);
-    if (z == 0) {  // defaults: the line kernel for k = 4 .. 6, streamed at k = 4, 5
+    if (z == 0) {  // defaults: the line kernel for k = 4 .. 6, streamed where that is the choice
         set_prefer_tiles_lines(k, false);
         reset_prefer_stream(k);
     }
@@ -164,38 +167,24 @@ int msa_autotune(int k, const int32_t *lens, int alphabet_size, int32_t repeats,
         if (best < 0 || ms < out->cand_ms[best]) best = i;
     }
     out->best = best;
-    // the winner becomes the choice for k
-    if (out->cand_kernel[best] == kKernelTiles) {
-        set_tile_edge(k, out->cand_edge[best]);
-        if (k == 3) set_prefer_tiles_k3(true);
-        if (k == 2) set_prefer_tiles_k2(true);
-        set_prefer_tiles_lines(k, true);
-        set_prefer_stream(k, false);
-    } else {
-        if (k == 3) set_prefer_tiles_k3(false);
-        if (k == 2) set_prefer_tiles_k2(false);
-        if (out->cand_kernel[best] == kKernelLines) {
-            set_line_z(k, out->cand_edge[best]);
-            set_prefer_tiles_lines(k, false);
-            set_prefer_stream(k, false);
-        }
-        if (out->cand_kernel[best] == kKernelStream) {
-            set_prefer_tiles_lines(k, false);
-            set_prefer_stream(k, true);
-            // the best segmented candidate stays the choice where the streamed one cannot run (serving)
-            int bl = -1;
-            for (int i = 0; i < out->ncand; ++i)
-                if (out->cand_kernel[i] == kKernelLines && (bl < 0 || out->cand_ms[i] < out->cand_ms[bl])) bl = i;
-            if (bl >= 0) set_line_z(k, out->cand_edge[bl]);
-        }
-        // the best generic edge stays the fallback for shapes the column kernel cannot take
-        int bt = -1;
+    // The winner becomes the choice for k, among the forms that were timed: a shape the
+    // column kernel or the whole-column form cannot take says nothing of those it can (k = 7
+    // tuned on a last axis of 20, then plans of 11: 1.03 ms in the whole-column form, 4.9 in
+    // the tile kernel). The best tile edge stays the fallback for the former, the best line
+    // segment for where the streamed form cannot run (serving at k = 6).
+    auto fastest = [&](int kernel) {
+        int b = -1;
         for (int i = 0; i < out->ncand; ++i)
-            if (out->cand_kernel[i] == kKernelTiles && (bt < 0 || out->cand_ms[i] < out->cand_ms[bt])) bt = i;
-        // (not at k = 7, 8, where a set edge selects the tile kernel)
-        if (k > kLinesMaxK) set_tile_edge(k, 0);
-        else if (bt >= 0) set_tile_edge(k, out->cand_edge[bt]);
-    }
+            if (out->cand_kernel[i] == kernel && (b < 0 || out->cand_ms[i] < out->cand_ms[b])) b = i;
+        return b;
+    };
+    const int won = out->cand_kernel[best], tiles = fastest(kKernelTiles), lines = fastest(kKernelLines);
+    if (tiles >= 0) set_tile_edge(k, out->cand_edge[tiles]);
+    if (lines >= 0 && won != kKernelTiles) set_line_z(k, out->cand_edge[lines]);
+    if (k == 2) set_prefer_tiles_k2(won == kKernelTiles);
+    if (fastest(kKernelCol3) >= 0) set_prefer_tiles_k3(won == kKernelTiles);
+    if (lines >= 0) set_prefer_tiles_lines(k, won == kKernelTiles);
+    if (fastest(kKernelStream) >= 0 && (k < 6 || lens[k - 1] + 1 <= wide_z(k))) set_prefer_stream(k, won == kKernelStream);
     return MSA_OK;
 }
 

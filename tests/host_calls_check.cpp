@@ -7,6 +7,7 @@
 //             that stream does not wait for, may still be on its way; host memory that an
 //             asynchronous copy reads stays as it is until the copy's stream is waited for;
 //             no result is read before that
+//   tuning    what the autotuner timed decides for the shapes it could time, and for no other
 #include <cuda_runtime.h>
 #include <malloc.h>
 
@@ -34,6 +35,7 @@ static int g_bad = 0;
 // ---------------------------------------------------------------------------
 // The runtime.
 
+static float g_ms = 1;            // what events are apart
 static int g_default_writes = 0;  // writes of the default stream that nothing has waited for
 static bool g_busy = false;       // work on another stream that nothing has waited for
 struct Source {
@@ -101,7 +103,7 @@ cudaError_t cudaEventCreate(cudaEvent_t *e) { return *e = (cudaEvent_t)0x20, cud
 cudaError_t cudaEventDestroy(cudaEvent_t) { return cudaSuccess; }
 cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaEventSynchronize(cudaEvent_t) { return wait_streams(), cudaSuccess; }
-cudaError_t cudaEventElapsedTime(float *ms, cudaEvent_t, cudaEvent_t) { return *ms = 1, cudaSuccess; }
+cudaError_t cudaEventElapsedTime(float *ms, cudaEvent_t, cudaEvent_t) { return *ms = g_ms, cudaSuccess; }
 }
 
 // ---------------------------------------------------------------------------
@@ -110,6 +112,8 @@ cudaError_t cudaEventElapsedTime(float *ms, cudaEvent_t, cudaEvent_t) { return *
 static PruneDesc g_prune;           // of the last analysis
 static int g_edge_after_prune = 0;  // tile edge another thread sets once the analysis is enqueued
 static int g_tile_fills = 0;
+static float g_cost[kKernelCount];  // ms of a fill by kernel, more the further a tile edge is from g_best_edge
+static int g_best_edge = 0;
 
 static cudaError_t kernel(cudaStream_t s) {
     if (s) stream_work("kernel");
@@ -129,6 +133,7 @@ cudaError_t launch_prune(const PruneDesc &D, bool, cudaStream_t s) {
 }
 cudaError_t launch_fill_tiles(int k, int edge, const LaunchDesc &L, int, cudaStream_t s) {
     ++g_tile_fills;
+    g_ms = g_cost[kKernelTiles] + 0.01f * (float)abs(edge - g_best_edge);
     const ProblemDesc &P = L.probs[0];
     if (P.skip) {
         CHECK(P.skip == g_prune.skip, "flags of another call");
@@ -140,10 +145,10 @@ cudaError_t launch_fill_tiles(int k, int edge, const LaunchDesc &L, int, cudaStr
     }
     return kernel(s);
 }
-cudaError_t launch_fill_col3(const LaunchDesc &, int, int, cudaStream_t s) { return kernel(s); }
-cudaError_t launch_fill_band2(const LaunchDesc &, int, cudaStream_t s) { return kernel(s); }
-cudaError_t launch_fill_lines(int, int, const LaunchDesc &, int, cudaStream_t s) { return kernel(s); }
-cudaError_t launch_fill_stream(int, const LaunchDesc &, int, cudaStream_t s, int) { return kernel(s); }
+cudaError_t launch_fill_col3(const LaunchDesc &, int, int, cudaStream_t s) { return g_ms = g_cost[kKernelCol3], kernel(s); }
+cudaError_t launch_fill_band2(const LaunchDesc &, int, cudaStream_t s) { return g_ms = g_cost[kKernelBand2], kernel(s); }
+cudaError_t launch_fill_lines(int, int, const LaunchDesc &, int, cudaStream_t s) { return g_ms = g_cost[kKernelLines], kernel(s); }
+cudaError_t launch_fill_stream(int, const LaunchDesc &, int, cudaStream_t s, int) { return g_ms = g_cost[kKernelStream], kernel(s); }
 size_t near_optimal_work_bytes(int, int64_t, int32_t) { return 0; }
 cudaError_t launch_near_optimal(int, int64_t, const ProblemDesc *, IODesc, int64_t, int32_t, NearOut, cudaStream_t s) { return kernel(s); }
 int fill_tiles_ctas_per_sm(int, int) { return 1; }
@@ -230,10 +235,83 @@ static void ordering() {
     }
 }
 
+// Tunes on `lens` with the tile, line, column and streamed kernels' times, the tile kernel's
+// best at `edge`.
+static void tune(const std::vector<int32_t> &lens, float tiles, float lines, float column, float stream, int edge) {
+    g_cost[kKernelTiles] = tiles;
+    g_cost[kKernelLines] = lines;
+    g_cost[kKernelCol3] = column;
+    g_cost[kKernelStream] = stream;
+    g_best_edge = edge;
+    msa_tuning t;
+    CHECK(msa_autotune((int)lens.size(), lens.data(), 20, 1, &t) == MSA_OK, "%s", msa_last_error());
+}
+static int chosen(const std::vector<int32_t> &lens, int A = 20) { return choose_kernel((int)lens.size(), lens.data(), A, kKernelAuto); }
+static void defaults(int k) {
+    msa_set_tile_edge(k, 0);
+    msa_set_line_segment(k, 0);
+}
+
+static void tuning() {
+    for (int k = 7; k <= 8; ++k) {
+        std::vector<int32_t> shrt((size_t)k, 3), lng((size_t)k, 2);
+        lng.back() = 20;  // beyond the whole-column form
+        const int other = tile_edge_candidate(k, 1) > 0 ? tile_edge_candidate(k, 1) : tile_edge_candidate(k, 0);
+        tune(lng, 5, 0, 0, 1, other);
+        CHECK(chosen(shrt) == kKernelStream && chosen(lng) == kKernelTiles && tile_edge_for(k) == other, "k=%d", k);
+        tune(shrt, 5, 0, 0, 1, other);
+        CHECK(chosen(shrt) == kKernelStream && chosen(lng) == kKernelTiles && tile_edge_for(k) == other, "k=%d", k);
+        tune(shrt, 1, 0, 0, 5, other);
+        CHECK(chosen(shrt) == kKernelTiles, "k=%d", k);
+        tune(lng, 1, 0, 0, 5, other);  // leaves that choice
+        CHECK(chosen(shrt) == kKernelTiles, "k=%d", k);
+        defaults(k);
+        CHECK(chosen(shrt) == kKernelStream && tile_edge_for(k) == tile_edge_default(k), "k=%d", k);
+        msa_set_tile_edge(k, tile_edge_candidate(k, 0));  // an edge of the caller's selects the tile kernel
+        CHECK(chosen(shrt) == kKernelTiles, "k=%d", k);
+        tune(lng, 5, 0, 0, 1, other);
+        CHECK(chosen(shrt) == kKernelTiles, "k=%d", k);
+        defaults(k);
+    }
+    const std::vector<int32_t> s6 = {3, 3, 3, 3, 3, 24}, l6 = {3, 3, 3, 3, 3, 25};
+    for (float tiles : {5.f, 1.f}) {  // the last axis beyond the whole-column form, lines or tiles the fastest
+        tune(l6, tiles, 2, 0, 3, 3);
+        CHECK(chosen(s6) == kKernelStream && chosen(l6) == (tiles > 2 ? kKernelLines : kKernelTiles), "k=6");
+        defaults(6);
+    }
+    tune(l6, 5, 2, 0, 1, 3);
+    CHECK(chosen(s6) == kKernelStream && chosen(l6) == kKernelLines, "k=6");
+    tune(s6, 5, 1, 0, 2, 3);
+    CHECK(chosen(s6) == kKernelLines && chosen(l6) == kKernelLines, "k=6");
+    tune(s6, 1, 5, 0, 2, 3);
+    CHECK(chosen(s6) == kKernelTiles && chosen(l6) == kKernelTiles, "k=6");
+    defaults(6);
+    for (int k = 4; k <= 5; ++k) {
+        const std::vector<int32_t> lens((size_t)k, 9);
+        CHECK(chosen(lens) == kKernelStream, "k=%d", k);
+        tune(lens, 5, 1, 0, 2, 4);
+        CHECK(chosen(lens) == kKernelLines, "k=%d", k);
+        tune(lens, 1, 2, 0, 2, 4);
+        CHECK(chosen(lens) == kKernelTiles, "k=%d", k);
+        tune(lens, 5, 2, 0, 1, 4);
+        CHECK(chosen(lens) == kKernelStream, "k=%d", k);
+        defaults(k);
+    }
+    const std::vector<int32_t> s3 = {9, 9, 9}, l3 = {1, 1, 5000};
+    tune(l3, 1, 0, 0, 0, 8);  // a last axis the column kernel does not take
+    CHECK(chosen(s3) == kKernelCol3 && chosen(l3) == kKernelTiles && tile_edge_for(3) == 8, "k=3");
+    tune(s3, 1, 0, 2, 0, 8);
+    CHECK(chosen(s3) == kKernelTiles, "k=3");
+    tune(s3, 2, 0, 1, 0, 16);
+    CHECK(chosen(s3) == kKernelCol3 && tile_edge_for(3) == 16, "k=3");
+    defaults(3);
+}
+
 int main(int argc, char **argv) {
     const std::string mode = argc > 1 ? argv[1] : "";
     if (mode == "pruned") pruned();
     else if (mode == "ordering") ordering();
+    else if (mode == "tuning") tuning();
     else CHECK(false, "unknown mode");
     if (!g_bad) printf("ok\n");
     return g_bad != 0;

@@ -31,3 +31,7 @@ def test_pruned_fill_takes_the_flags_of_its_own_grid(check):
 
 def test_device_work_is_ordered_after_the_copies_it_reads(check):
     check("ordering")
+
+
+def test_tuning_decides_for_the_shapes_it_could_time(check):
+    check("tuning")
