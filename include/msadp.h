@@ -116,7 +116,8 @@ int msa_near_optimal(int k, const char *const *seqs, const int32_t *lens, const 
  * bound -- the sum over pairs of the largest fwd + bwd over the tile's rectangle
  * -- is below a lower bound L on the optimum holds no cell of an optimal
  * alignment: the fill may leave it out, and does (with that kernel) where this is
- * faster than a kernel that fills every cell. The score and alignment equal
+ * faster than a kernel that fills every cell, where no other kernel takes the shape
+ * and with msa_config("fill_kernel", 1). The score and alignment equal
  * msa_align's (the same tie rule) whenever L does not exceed the optimum.
  *
  *   have_lower_bound  0: L is the score of a feasible alignment the device builds

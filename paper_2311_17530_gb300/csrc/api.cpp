@@ -950,8 +950,13 @@ int msa_align_pruned(int k, const char *const *seqs, const int32_t *lens, const 
     // the slowest per cell. k = 2 and 3: always the band and column kernels (k = 3,
     // 700 / 760 / 800 with 98 % of the tiles left out: 0.64 ms against 6.4 ms).
     // k = 4: always the streamed kernel; k >= 5: the line kernels unless enough of a large
-    // tensor is left out.
-    int kernel = choose_kernel(k, lens, hp.A, kKernelAuto);
+    // tensor is left out. msa_config("fill_kernel", 1) asks for the tile kernel.
+    int kernel;
+    {
+        std::lock_guard<std::mutex> g(settings_mutex());
+        kernel = settings().fill_kernel == kKernelTiles ? kKernelTiles : kKernelAuto;
+    }
+    kernel = choose_kernel(k, lens, hp.A, kernel);
     int64_t st[2] = {0, 0};
     if (k > 4 && kernel != kKernelTiles && hp.cells >= kPruneTilesCells) {
         e = cudaStreamSynchronize(s);

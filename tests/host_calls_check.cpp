@@ -2,7 +2,7 @@
 // plan.cpp and tune.cpp linked against a CUDA runtime and kernel launchers of this file.
 // Device memory is host memory; a launcher only notes what it was asked for. Modes:
 //   pruned    the fill of a pruned call gets the flags of its own tile grid, also when the
-//             tuned tile edge changes while the call runs
+//             tuned tile edge changes while the call runs; fill_kernel = 1 gives every k that fill
 //   ordering  no kernel is launched on a stream while a write of the default stream, which
 //             that stream does not wait for, may still be on its way; host memory that an
 //             asynchronous copy reads stays as it is until the copy's stream is waited for;
@@ -111,7 +111,7 @@ cudaError_t cudaEventElapsedTime(float *ms, cudaEvent_t, cudaEvent_t) { return *
 
 static PruneDesc g_prune;           // of the last analysis
 static int g_edge_after_prune = 0;  // tile edge another thread sets once the analysis is enqueued
-static int g_tile_fills = 0;
+static int g_tile_fills = 0, g_skipping_fills = 0;
 static float g_cost[kKernelCount];  // ms of a fill by kernel, more the further a tile edge is from g_best_edge
 static int g_best_edge = 0;
 
@@ -136,6 +136,7 @@ cudaError_t launch_fill_tiles(int k, int edge, const LaunchDesc &L, int, cudaStr
     g_ms = g_cost[kKernelTiles] + 0.01f * (float)abs(edge - g_best_edge);
     const ProblemDesc &P = L.probs[0];
     if (P.skip) {
+        ++g_skipping_fills;
         CHECK(P.skip == g_prune.skip, "flags of another call");
         CHECK(P.ntiles == g_prune.ntiles && L.ntickets == g_prune.ntiles, "k=%d: %lld tiles filled, flags of %lld", k,
               (long long)P.ntiles, (long long)g_prune.ntiles);
@@ -196,6 +197,18 @@ static void pruned() {
         g_edge_after_prune = 0;
         msa_set_tile_edge(p.k, 0);
     }
+    for (int k = 2; k <= 8; ++k)
+        for (int kernel : {0, 1}) {
+            Problem p(std::vector<int32_t>((size_t)k, 4), 4);
+            std::string out((size_t)k * 400, '\0');
+            int32_t score = 0;
+            g_skipping_fills = 0;
+            msa_config("fill_kernel", kernel);
+            CHECK(msa_align_pruned(k, p.seqs.data(), p.lens.data(), p.alphabet.c_str(), p.table.data(), -1, 0, 0, &score, &out[0],
+                                   nullptr) == MSA_OK, "%s", msa_last_error());
+            CHECK(g_skipping_fills == kernel, "k=%d: %d fills leave tiles out with fill_kernel = %d", k, g_skipping_fills, kernel);
+        }
+    msa_config("fill_kernel", 0);
 }
 
 static void ordering() {

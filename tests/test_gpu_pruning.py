@@ -156,3 +156,29 @@ def test_large_tensors_with_most_tiles_left_out(k, lens):
     score, rows, stats = msadp.msa_align_pruned(p.seqs, p.alphabet, p.subst, p.gap)
     assert stats["cells"] >= 8e7 and stats["cells_skipped"] > 0.8 * stats["cells"]
     assert (score, rows) == msa.msa_align(p.seqs, p.alphabet, p.subst, p.gap)
+
+
+SKIPPING = [(150, 170), (300, 40), (45, 40, 50), (60, 64, 58), (20, 22, 19, 24), (9, 11, 10, 12, 8), (7, 8, 6, 7, 8, 6),
+            (5, 6, 4, 5, 6, 5, 4), (3, 4, 3, 4, 3, 4, 3, 2)]
+
+
+@pytest.mark.parametrize("related", [True, False])
+@pytest.mark.parametrize("lens", SKIPPING)
+def test_fill_that_leaves_tiles_out(lens, related):
+    """The tile kernel's fill without the tiles the bound rules out, for every k: the device's bound, the
+    optimum, a bound that rules out nothing, and bounds above the optimum, which leave the corner
+    unreachable or its best remaining path below the bound."""
+    p = inputs.random_problem(9500 + sum(lens) + related, len(lens), list(lens), alphabet=inputs.PROTEIN, related=related)
+    want = oracle.align_problem(p)
+    msa.msa_config("fill_kernel", 1)
+    try:
+        for bound in (None, want.score, -(1 << 40)):
+            score, rows, st = msadp.msa_align_pruned(p.seqs, p.alphabet, p.subst, p.gap, lower_bound=bound)
+            assert (score, rows) == (want.score, want.rows), bound
+        assert st["tiles_skipped"] == 0
+        for above in (1, 50, 1 << 40):
+            with pytest.raises(msa.MsaError) as ei:
+                msadp.msa_align_pruned(p.seqs, p.alphabet, p.subst, p.gap, lower_bound=want.score + above)
+            assert ei.value.code == msa.MSA_EINVAL
+    finally:
+        msa.msa_config("fill_kernel", 0)
