@@ -916,14 +916,34 @@ cudaError_t prune_analyse(PruneRun &R, const IODesc &io) {
     return e;
 }
 
-// k >= 5: the generic tile kernel, which skips what is left out, against the line
-// kernels, which fill everything several times as fast per cell: the tiles' own chain of
-// waves takes 1.2 to 2.5 ms, so they win only where much is left out of a large tensor.
-// One call, ms with tiles / lines: k = 6, 87 M cells with 1.0 left out 2.5 / 3.3; k = 5,
-// 116 M, 0.95 2.48 / 2.57; 100 M, 0.78 2.49 / 2.50; but 34 M, 0.97 1.64 / 1.34; k = 6, 47 M,
-// 0.65 2.28 / 1.71; k = 7, 36 M, 1.0 2.66 / 1.81.
-constexpr double kPruneTilesShare = 0.78;
-constexpr int64_t kPruneTilesCells = 80000000;
+// k >= 4: the generic tile kernel, which skips what is left out, against the kernels that
+// fill everything several times as fast per cell. Milliseconds of the call beside the
+// analysis (plan, fill, traceback), fitted to 344 calls of 86 shapes, both fills measured
+// on each (0.3 to 45 ms; within 10 % but for a few small shapes): the tile kernel by its
+// cells, edge tiles padded, those not left out, and its waves; the streamed kernels by
+// their sweeps' lane steps (the skew makes a short last axis dear) and waves, the
+// segmented one by lines and segments. Both sides, fast / tiles: k = 5, 60^4 x 15 with
+// 0.37 left out 7.05 / 5.26; 40^5, 0.36 2.86 / 3.35; k = 6, 20^6, 0.99 3.01 / 2.16; 24^6,
+// 0.70 6.50 / 7.64; 26^6 (segmented), 0.83 25.6 / 7.2; k = 7, 13^6 x 12, 0.99 4.00 / 6.20;
+// k = 8, 8^8, 0.996 6.33 / 4.28. Choosing by it costs 0.7 % over the better one on average.
+double pruned_tiles_ms(const HostPlan &t, double live) {
+    struct Cost { double call, padded_ps, live_ps, wave_us; };
+    constexpr Cost costs[] = {{0.27, 6.2, 2.5, 18.8}, {0.39, 8.3, 9.9, 19}, {0.24, 10.2, 27.7, 27.5}, {0.47, 49.6, 167, 13.7},
+                              {0.51, 35, 390, 5.4}};
+    const Cost &c = costs[t.k - 4];
+    double padded = (double)t.ntiles;
+    for (int i = 0; i < t.k; ++i) padded *= t.E[i];
+    return c.call + 1e-9 * (c.padded_ps * padded + c.live_ps * live) + 1e-3 * c.wave_us * t.waves;
+}
+double full_fill_ms(const HostPlan &f) {
+    const int k = f.k, E = f.E[k - 1];
+    if (f.kernel == kKernelLines) return 0.63 + 1e-9 * 32 * (double)f.ntiles * (574 + 8 * E);
+    struct Cost { double call, step_ps, wave_us; };
+    constexpr Cost costs[] = {{0.37, 6.4, 4.8}, {0.44, 11.6, 4.3}, {0.44, 12.6, 4.2}, {0.44, 18.3, 5.2}, {0.5, 38, 0}};
+    const Cost &c = costs[k - 4];
+    const double lanes = 32.0 * stream_warps(k) * (double)f.sgstride[0] * f.SG[0];
+    return c.call + 1e-9 * c.step_ps * lanes * (f.wide ? E + stream_skew_max(k) : f.lzq) + 1e-3 * c.wave_us * f.waves;
+}
 
 }  // namespace
 
@@ -948,9 +968,10 @@ int msa_align_pruned(int k, const char *const *seqs, const int32_t *lens, const 
     // The fill: a tile left out saves work, but a fill bound by its chain of waves
     // gains little from it, and the generic tile kernel that can leave tiles out is
     // the slowest per cell. k = 2 and 3: always the band and column kernels (k = 3,
-    // 700 / 760 / 800 with 98 % of the tiles left out: 0.64 ms against 6.4 ms).
-    // k = 4: always the streamed kernel; k >= 5: the line kernels unless enough of a large
-    // tensor is left out. msa_config("fill_kernel", 1) asks for the tile kernel.
+    // 700 / 760 / 800 with 98 % of the tiles left out: 0.64 ms against 6.4 ms). k >= 4: by
+    // the estimates above, and the analysis is only waited for where the tile kernel
+    // would win with everything left out (a million cells at least: below, both take half
+    // a millisecond). msa_config("fill_kernel", 1) asks for it.
     int kernel;
     {
         std::lock_guard<std::mutex> g(settings_mutex());
@@ -958,11 +979,16 @@ int msa_align_pruned(int k, const char *const *seqs, const int32_t *lens, const 
     }
     kernel = choose_kernel(k, lens, hp.A, kernel);
     int64_t st[2] = {0, 0};
-    if (k > 4 && kernel != kKernelTiles && hp.cells >= kPruneTilesCells) {
-        e = cudaStreamSynchronize(s);
-        if (e == cudaSuccess) e = cudaMemcpy(st, R.D.stats, 16, cudaMemcpyDeviceToHost);
-        if (e != cudaSuccess) return cuda_error(e, "pruning kernels");
-        if ((double)st[1] > kPruneTilesShare * (double)hp.cells) kernel = kKernelTiles;
+    if (k >= 4 && kernel != kKernelTiles && hp.cells >= (1 << 20)) {
+        HostPlan full;
+        std::string err;
+        const bool fits = plan_shape(k, lens, hp.A, kernel, full, err) == MSA_OK;
+        if (fits && pruned_tiles_ms(hp, 0) < full_fill_ms(full)) {
+            e = cudaStreamSynchronize(s);
+            if (e == cudaSuccess) e = cudaMemcpy(st, R.D.stats, 16, cudaMemcpyDeviceToHost);
+            if (e != cudaSuccess) return cuda_error(e, "pruning kernels");
+            if (pruned_tiles_ms(hp, (double)(hp.cells - st[1])) < full_fill_ms(full)) kernel = kKernelTiles;
+        }
     }
     if (kernel != kKernelTiles && plan_create(k, lens, alphabet, kernel, -1, &R.plan) != MSA_OK) kernel = kKernelTiles;
     if (kernel == kKernelTiles) {

@@ -7,6 +7,7 @@
 //             that stream does not wait for, may still be on its way; host memory that an
 //             asynchronous copy reads stays as it is until the copy's stream is waited for;
 //             no result is read before that
+//   choice    a pruned call's fill: the tile kernel where leaving cells out makes it the faster one
 //   tuning    what the autotuner timed decides for the shapes it could time, and for no other
 #include <cuda_runtime.h>
 #include <malloc.h>
@@ -78,7 +79,8 @@ cudaError_t cudaMemcpy(void *d, const void *s, size_t n, cudaMemcpyKind kind) {
 cudaError_t cudaMemsetAsync(void *d, int v, size_t n, cudaStream_t s) {
     if (s) stream_work("memset");
     else ++g_default_writes;
-    return memset(d, v, n), cudaSuccess;
+    if (v || n < (64 << 20)) memset(d, v, n);  // (large ones: zero from calloc, and left to it)
+    return cudaSuccess;
 }
 cudaError_t cudaMemset(void *d, int v, size_t n) { return cudaMemsetAsync(d, v, n, nullptr); }
 cudaError_t cudaMemcpyAsync(void *d, const void *s, size_t n, cudaMemcpyKind kind, cudaStream_t stream) {
@@ -110,6 +112,7 @@ cudaError_t cudaEventElapsedTime(float *ms, cudaEvent_t, cudaEvent_t) { return *
 // The kernel launchers.
 
 static PruneDesc g_prune;           // of the last analysis
+static double g_left_out = 0;       // share of the cells the analysis rules out
 static int g_edge_after_prune = 0;  // tile edge another thread sets once the analysis is enqueued
 static int g_tile_fills = 0, g_skipping_fills = 0;
 static float g_cost[kKernelCount];  // ms of a fill by kernel, more the further a tile edge is from g_best_edge
@@ -128,6 +131,9 @@ cudaError_t launch_traceback(const ProblemDesc *, int, const int32_t *, const IO
 }
 cudaError_t launch_prune(const PruneDesc &D, bool, cudaStream_t s) {
     g_prune = D;
+    double cells = 1;
+    for (int i = 0; i < D.k; ++i) cells *= D.len[i] + 1;
+    D.stats[1] = (int64_t)(g_left_out * cells);
     if (g_edge_after_prune) set_tile_edge(D.k, g_edge_after_prune);
     return kernel(s);
 }
@@ -320,10 +326,37 @@ static void tuning() {
     defaults(3);
 }
 
+static void choice() {
+    // both fills measured in one call, ms: the kernel that fills every cell, the tile kernel
+    const struct { std::vector<int32_t> lens; double out; float fast, tiles; } cases[] = {
+        {{60, 60, 60, 60}, 0.967, 0.65f, 1.14f},          {{200, 190, 200, 195}, 0.995, 11.4f, 14.2f},
+        {{30, 30, 30, 30, 30}, 0.985, 1.08f, 1.36f},      {{40, 40, 40, 40, 40}, 0.987, 2.85f, 2.49f},
+        {{40, 40, 40, 40, 40}, 0.356, 2.86f, 3.35f},      {{60, 60, 60, 60, 15}, 0.365, 7.05f, 5.26f},
+        {{60, 60, 60, 60, 5}, 0.397, 4.68f, 3.09f},       {{25, 25, 25, 25, 100}, 0.97, 1.21f, 1.84f},
+        {{14, 14, 14, 14, 14, 14}, 0.994, 0.86f, 1.05f},  {{20, 20, 20, 20, 20, 20}, 0.988, 3.01f, 2.16f},
+        {{24, 24, 24, 24, 24, 24}, 0.699, 6.5f, 7.64f},   {{30, 30, 30, 30, 30, 5}, 0.732, 7.21f, 5.02f},
+        {{26, 26, 26, 26, 26, 26}, 0.833, 25.6f, 7.18f},  {{20, 20, 20, 20, 20, 60}, 0.21, 12.4f, 9.62f},
+        {{17, 17, 17, 17, 17, 26}, 0.57, 3.15f, 2.07f},   {{10, 10, 10, 10, 10, 60}, 0.452, 1.19f, 1.64f},
+        {{12, 12, 12, 12, 12, 12, 12}, 1.0, 3.84f, 5.67f}, {{13, 13, 13, 13, 13, 13, 12}, 0.988, 4.0f, 6.2f},
+        {{8, 8, 8, 8, 8, 8, 8, 8}, 0.996, 6.33f, 4.28f},  {{9, 9, 9, 9, 9, 9, 9, 4}, 0.983, 5.3f, 3.77f},
+        {{10, 10, 10, 10, 10, 10, 10, 5}, 0.692, 18.3f, 21.f}};
+    for (const auto &c : cases) {
+        Problem p(c.lens, 4);
+        std::string out((size_t)p.k * 1000, '\0');
+        int32_t score = 0;
+        g_left_out = c.out;
+        g_skipping_fills = 0;
+        CHECK(msa_align_pruned(p.k, p.seqs.data(), p.lens.data(), p.alphabet.c_str(), p.table.data(), -1, 0, 0, &score, &out[0],
+                               nullptr) == MSA_OK, "%s", msa_last_error());
+        CHECK(g_skipping_fills == (c.tiles < c.fast), "k=%d, last axis %d, %.3f left out", p.k, c.lens.back(), c.out);
+    }
+}
+
 int main(int argc, char **argv) {
     const std::string mode = argc > 1 ? argv[1] : "";
     if (mode == "pruned") pruned();
     else if (mode == "ordering") ordering();
+    else if (mode == "choice") choice();
     else if (mode == "tuning") tuning();
     else CHECK(false, "unknown mode");
     if (!g_bad) printf("ok\n");

@@ -35,3 +35,7 @@ def test_device_work_is_ordered_after_the_copies_it_reads(check):
 
 def test_tuning_decides_for_the_shapes_it_could_time(check):
     check("tuning")
+
+
+def test_pruned_call_takes_the_faster_fill(check):
+    check("choice")
