@@ -78,7 +78,7 @@ cudaError_t launch_encode(const ProblemDesc *d_probs, int nprob, int max_ncode,
     int bx = (max_ncode + 255) / 256;
     if (bx < min_blocks) bx = min_blocks;
     if (bx < 1) bx = 1;
-    if (bx > 64) bx = 64;
+    if (bx > kEncodeBlocks) bx = kEncodeBlocks;
     encode_kernel<<<dim3(bx, nprob), 256, 0, s>>>(d_probs, io_array, io_single);
     return cudaGetLastError();
 }

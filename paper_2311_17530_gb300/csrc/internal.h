@@ -313,6 +313,7 @@ class DeviceOnce {
 // Kernel entry points (host wrappers), defined in the .cu files.
 // A kernel reads its per-problem IODesc from io_array[p] when io_array is set,
 // else from io_single (single-problem executions pass it by value).
+constexpr int kEncodeBlocks = 64;  // most blocks per problem
 cudaError_t launch_encode(const ProblemDesc *d_probs, int nprob, int max_ncode,
                           const IODesc *io_array, IODesc io_single, cudaStream_t s, int min_blocks = 1);
 cudaError_t launch_fill_tiles(int k, int edge, const LaunchDesc &L, int grid, cudaStream_t s);

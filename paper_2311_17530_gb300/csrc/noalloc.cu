@@ -178,7 +178,7 @@ extern "C" int msa_align_noalloc(int k, const int32_t *lens, const char *alphabe
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_error(e, "set-up kernel launch");
     IODesc io{d_residues, d_subst, d_result, d_masks, gap, 0};
-    e = launch_encode(pp.prob, 1, hp.len_sum, nullptr, io, s, d.clear_faces ? 64 : 1);
+    e = launch_encode(pp.prob, 1, hp.len_sum, nullptr, io, s, d.clear_faces ? kEncodeBlocks : 1);
     if (e != cudaSuccess) return cuda_error(e, "encode launch");
     LaunchDesc L;
     memset(&L, 0, sizeof L);

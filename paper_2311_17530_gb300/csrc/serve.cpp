@@ -573,7 +573,7 @@ int Server::launch(Slot &sl, std::vector<ServeReq *> &batch, const Settings &cfg
     int rc = MSA_OK;
     if (e == cudaSuccess) e = cudaMemcpyAsync(D, H, in_bytes, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(D + off_state, 0, zero_bytes, s);
-    if (e == cudaSuccess) e = launch_encode(ddesc, n, max_ncode, dio, IODesc{}, s, clear ? (streamed ? 128 : 32) : 1);
+    if (e == cudaSuccess) e = launch_encode(ddesc, n, max_ncode, dio, IODesc{}, s, clear ? (streamed ? kEncodeBlocks : 32) : 1);
     for (size_t gi = 0; gi < groups.size() && e == cudaSuccess; ++gi) {
         const Group &g = groups[gi];
         LaunchDesc L;
