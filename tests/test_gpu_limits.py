@@ -67,3 +67,33 @@ def test_largest_alphabet_generic_and_line_kernels(kernel, k, lens):
 
 def test_long_pair():
     run_full(inputs.random_problem(5300, 2, [3000, 2500], related=True))
+
+
+def near_limit_problem(lens, sign):
+    """Scores at the int32 limit: the gap as large as the device's range check lets it be (the pair
+    scores near 2 gap, so that a pair's share beside the gaps stays small), all scores near sign * 2^31."""
+    k, pair_min = len(lens), sum(min(a, b) for i, a in enumerate(lens) for b in lens[i + 1:])
+    table = np.where(np.eye(4, dtype=bool), 5, -4)
+    gap = sign * ((2**31 - 2 - 5 * pair_min) // ((k - 1) * sum(lens)))
+    p = inputs.random_problem(5400 + sum(lens), k, lens, table=table, gap=gap, related=True)
+    p.subst = (table + 2 * gap).astype(np.int32)
+    return p
+
+
+@pytest.mark.parametrize("sign", [-1, 1])
+@pytest.mark.parametrize("lens", [[60, 57], [700, 650], [30, 28, 33], [14, 12, 15, 13], [6, 5, 7, 6, 5, 6]])
+def test_scores_at_the_int32_limit(lens, sign):
+    """The enumeration (level by level, and depth first beyond 1024 residues or 2048 alignments) and the
+    pruned call with its greedy bound keep scores and bounds in 32 bits: exact up to the range check."""
+    p = near_limit_problem(lens, sign)
+    want = oracle.align_problem(p)
+    assert abs(want.score) > 2**31 - 2**17
+    for delta, count in ((0, 30), (3, 30), (1 << 40, 30), (2, 2049)):
+        got, more = msadp.msa_near_optimal(p.seqs, p.alphabet, p.subst, p.gap, delta, count)
+        exp, emore = oracle.align_near_optimal(p.seqs, p.alphabet, p.subst, p.gap, delta, count)
+        assert more == emore and [g[:2] for g in got] == [(e.score, e.masks) for e in exp], (delta, count)
+    score, rows, st = msadp.msa_align_pruned(p.seqs, p.alphabet, p.subst, p.gap)
+    assert (score, rows) == (want.score, want.rows) and want.score - 2**20 < st["lower_bound"] <= want.score
+    ext = [4] * p.k
+    np.testing.assert_array_equal(msadp.msa_tile_bounds(p.seqs, p.alphabet, p.subst, p.gap, ext),
+                                  oracle.tile_bounds(p.seqs, p.alphabet, p.subst, p.gap, ext).reshape(-1))
