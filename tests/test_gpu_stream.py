@@ -258,3 +258,8 @@ def test_serving_in_reused_arena_regions(k):
         for h, p in zip(handles, probs):
             want = oracle.align(p.seqs, p.alphabet, p.subst, p.gap)
             assert msa.msa_poll(h, p.k, sum(p.lens)) == (want.score, want.rows)
+
+
+def test_units_of_several_super_blocks_k8():
+    """k = 8, 9^8 cells: faces of 476 MB, a unit every super-block along axis 6 (the last one ragged)."""
+    test_units_of_several_super_blocks(8, [8] * 8)
