@@ -180,12 +180,14 @@ int msa_set_stream(void *stream);
  *                       The automatic choice is 5 at k=4,5 and where the whole-column
  *                       form fits, else 4 at k=6 and 1 at k=7,8 (until msa_autotune
  *                       or, at k=7,8, msa_set_tile_edge picks otherwise); the serving
- *                       loop runs 4 (k=7,8: 1) where 5 would be chosen or asked for
+ *                       loop runs 5 at k=4,5 for requests its memory can hold that way,
+ *                       else 4, and 4 (k=7,8: 1) at k>=6; 1 also gives msa_align_pruned
+ *                       the fill that leaves tiles out
  *   "timing"            1: msa_plan_execute records per-stage CUDA events (default 0)
  *   "verify_corner"     1: later plans and requests on the k=3 column kernel record the
  *                       far corner's score during the fill, and the traceback reports
  *                       MSA_ECUDA when the rescored alignment disagrees with it (about
- *                       3 % slower); the other fill kernels always do (default 0)
+ *                       10 % slower); the other fill kernels always do (default 0)
  *   "test_withhold_tile" test hook: the tile with this ticket never publishes its
  *                       completion, so its dependants time out (default -1: off)
  *   "test_poison_tb"    test hook: 1 makes msa_plan_execute fill the plan's traceback
@@ -222,7 +224,8 @@ typedef struct msa_plan_info {
                                    tb_strides for the tile kernel (k <= 3) and the band kernel;
                                    tile-major for the tile kernel at k >= 4 and for the line
                                    kernels; for the k=3 column kernel a column-blocked layout
-                                   (msa_plan_read_tb returns row-major) */
+                                   of move tags, not masks (msa_plan_read_tb returns row-major
+                                   masks) */
 } msa_plan_info;
 
 /* Result block written on the device by msa_plan_execute. */
@@ -418,7 +421,8 @@ typedef struct msa_tuning {
  * msa_set_line_segment, and whether the automatic kernel choice takes the band,
  * column, line or streamed line kernel). A kernel that cannot take these lengths (the
  * column kernel; at k = 6..8 the whole-column form beyond its last axis) is not timed,
- * and shapes it can take keep it.
+ * and shapes it can take keep it; at k = 6 beyond 25 positions the streamed line kernel
+ * is timed, but a plan runs it only with msa_config("fill_kernel", 5).
  * Allocates device memory; synchronous.
  */
 int msa_autotune(int k, const int32_t *lens, int alphabet_size, int32_t repeats, msa_tuning *out);

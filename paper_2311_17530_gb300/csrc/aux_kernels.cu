@@ -60,9 +60,9 @@ __global__ void encode_kernel(const ProblemDesc *probs, const IODesc *io_arr, IO
         if (sbad & 1) atomicCAS(&st->status, 0, MSA_EINVAL);
         // |H'| <= maxp * sum_{i<j} min(len_i, len_j); a candidate adds at most
         // C(k,2) * maxp; keys carry the factor 2^B and the potential W <= W(len).
-        // The margin 4 * (len_sum + 64) keeps the k = 3 column kernel's skew cells
-        // (x2 < 0, seeded at kNeg, tie bits adding at most 7 per cell along a path
-        // of at most len_sum + 63 cells) strictly below every valid key.
+        // The margin 4 * (len_sum + 64) covers what the kernels add to a key beside pair
+        // scores and W: a candidate's tag (at most 7, cut off before the next cell), in the
+        // cells outside the tensor that the column and band kernels compute as well.
         const int64_t npairs = (int64_t)P.k * (P.k - 1) / 2;
         const int64_t key_bound = (int64_t)smax * (P.pair_min_sum + npairs) * ((int64_t)1 << B) + P.w_corner +
                                   4 * ((int64_t)P.len_sum + 64);

@@ -90,7 +90,9 @@ __host__ __device__ constexpr int line_v_words() {
     return round_up(top + 4, 4);
 }
 // Pair-table row stride: at least Z + skew_max (a lane reads its row at positions
-// -skew_max .. Z + skew_max - 1, unclamped, in the sweep), and congruent to
+// -skew_max + 1 .. Z + skew_max, unclamped, in the sweep; the last of them is the word
+// after the shortest row: the next row's first, after the last row the neighbour
+// table's), and congruent to
 // skew_max + 1 mod 32, so that lanes reading row c_i at position t - sum c hit
 // distinct banks unless they read the same word.
 template <int K, int Z>

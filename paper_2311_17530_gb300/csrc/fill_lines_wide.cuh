@@ -348,35 +348,35 @@ __global__ void __launch_bounds__(stream_threads<K>(), wide_min_ctas<K>()) fill_
                 }
             };
             halo_load(0);
-                // this line's pair sums over subsets of the line axes; along the unit only
-                // those with axis J change
-                const int xj = o[J] + cl[J];
-                const int cj = (xj >= 1 && xj <= P.len[J]) ? codes[P.cofs[J] + xj - 1] : 0;
-                if (first) {
-                    Sp[0] = 0;
+            // this line's pair sums over subsets of the line axes; along the unit only
+            // those with axis J change
+            const int xj = o[J] + cl[J];
+            const int cj = (xj >= 1 && xj <= P.len[J]) ? codes[P.cofs[J] + xj - 1] : 0;
+            if (first) {
+                Sp[0] = 0;
 #pragma unroll
-                    for (int i = 0; i < J; ++i) {
-                        const int x = o[i] + cl[i];
-                        cd[i] = (x >= 1 && x <= P.len[i]) ? codes[P.cofs[i] + x - 1] : 0;
-                    }
-#pragma unroll
-                    for (int h = 0; h < J; ++h) {
-                        int Rs[1 << (NA - 1)];
-                        Rs[0] = 0;
-#pragma unroll
-                        for (int r = 1; r < (1 << h); ++r) Rs[r] = Rs[r & (r - 1)] + __ldg(tab + cd[lowbit_c(r)] * A + cd[h]);
-#pragma unroll
-                        for (int r = 0; r < (1 << h); ++r) Sp[r | (1 << h)] = Sp[r] + Rs[r];
-                    }
+                for (int i = 0; i < J; ++i) {
+                    const int x = o[i] + cl[i];
+                    cd[i] = (x >= 1 && x <= P.len[i]) ? codes[P.cofs[i] + x - 1] : 0;
                 }
-                {
-                    int Rs[1 << J];
+#pragma unroll
+                for (int h = 0; h < J; ++h) {
+                    int Rs[1 << (NA - 1)];
                     Rs[0] = 0;
 #pragma unroll
-                    for (int r = 1; r < (1 << J); ++r) Rs[r] = Rs[r & (r - 1)] + __ldg(tab + cd[lowbit_c(r)] * A + cj);
+                    for (int r = 1; r < (1 << h); ++r) Rs[r] = Rs[r & (r - 1)] + __ldg(tab + cd[lowbit_c(r)] * A + cd[h]);
 #pragma unroll
-                    for (int r = 0; r < (1 << J); ++r) Sp[r | (1 << J)] = Sp[r] + Rs[r];
+                    for (int r = 0; r < (1 << h); ++r) Sp[r | (1 << h)] = Sp[r] + Rs[r];
                 }
+            }
+            {
+                int Rs[1 << J];
+                Rs[0] = 0;
+#pragma unroll
+                for (int r = 1; r < (1 << J); ++r) Rs[r] = Rs[r & (r - 1)] + __ldg(tab + cd[lowbit_c(r)] * A + cj);
+#pragma unroll
+                for (int r = 0; r < (1 << J); ++r) Sp[r | (1 << J)] = Sp[r] + Rs[r];
+            }
             halo_store();
 #pragma unroll 1
             for (int s0 = HB; s0 * NT < nh; s0 += HB) {

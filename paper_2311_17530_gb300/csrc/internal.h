@@ -60,8 +60,8 @@ struct ProblemDesc {
     int32_t tb_layout;           // 0: row-major (tbstride); 1: column-blocked (column kernel);
                                  // 2, 3: tile-major (generic tile kernel, line kernel)
     int64_t qelems;              // words of Q
-    int32_t clear_faces;         // the encode step zeroes the column kernel's faces first (serving:
-                                 // the arena region may hold stale words of other requests)
+    int32_t clear_faces;         // the encode step zeroes the tagged faces first (serving and the
+                                 // no-allocation call: the region may hold stale words)
     const uint8_t *amap;         // device 256-entry char -> code map (0xFF: invalid)
     uint8_t *codes;              // device codes
     int32_t *tab;                // device scaled pair table ((sub - 2 gap) << B)

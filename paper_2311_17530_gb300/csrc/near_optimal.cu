@@ -26,10 +26,10 @@
 // depths at a time for the deepest one with a mask left and count the moves to undo
 // with one ballot per axis. The offset of a cell is a sum of one term per axis in
 // every layout of the scores, so the terms are tabulated per coordinate once.
-// 256 alignments of 120 x 110 x 130 (9,100 moves followed): 24.6 ms when the walk
-// went back one column at a time, judging again, with positions in local memory;
-// 2.4 ms now, and level by level less again (near_beam_kernel, the form for shorter
-// sequences).
+// 256 alignments within 3 of the optimum of a related 120 x 110 x 130 triple: 37.9 ms when
+// the walk went back one column at a time, judging again, with positions in local memory;
+// 3.58 ms depth first now, 0.32 level by level (near_beam_kernel, the form for shorter
+// sequences, which this problem takes).
 #include "device_common.cuh"
 
 #include <algorithm>
@@ -261,7 +261,7 @@ __global__ void __launch_bounds__(kNearThreads) near_optimal_kernel(const Proble
 // its masks, and a count over the ballots lays the children down in order (a slot that
 // has reached the origin is carried on as it is). A level is one chain of loads, a
 // ballot and a barrier, as a node of the depth-first walk is, but takes all slots: 256
-// alignments of 120 x 110 x 130, 143 levels: 0.263 against 3.62 ms node by node. A level
+// alignments of another such triple, 143 levels: 0.263 against 3.62 ms node by node. A level
 // costs more than a node, though, and the walk judges only the cells of the alignments
 // it stores, which on long sequences differ in their last few columns. So up to
 // kBeamLength residues this way (300 x 300, 30 alignments: 0.187 against 0.376 ms;

@@ -123,7 +123,10 @@ int choose_kernel(int k, const int32_t *lens, int A, int requested, bool allow_s
         (requested == kKernelStream ||
          (requested == kKernelAuto && allow_stream && prefer_stream(k))))
         return kKernelStream;
-    // at k = 6 only the whole-column form (last axis of at most kWideZ) beats the line kernel
+    // At k = 6 only the whole-column form (last axis of at most kWideZ). The pipelined one
+    // was slower than the line kernel when the line was drawn (6.69 against 5.45 ms on k6
+    // protein) and is not now (last axis 26: 6.62 against 10.17 ms, 61: 0.40 / 0.64 on 11^5
+    // lines); it runs on request.
     if (k >= kLinesMinK && k <= kLinesMaxK && requested == kKernelAuto && allow_stream && prefer_stream(k) &&
         stream_fits(k, lens) && (k != 6 || lens[k - 1] + 1 <= kWideZ))
         return kKernelStream;

@@ -89,8 +89,8 @@ int line_z_for(int k);
 int set_line_z(int k, int z);
 bool prefer_tiles_lines(int k);
 void set_prefer_tiles_lines(int k, bool v);
-// k = 4, 5: whether the automatic choice of the line kernel takes its streamed
-// form (one column per warp over the whole last axis); reset restores the default.
+// k = 4, 5, and k = 6 .. 8 where the whole-column form fits: whether the automatic
+// choice takes the streamed line kernel; reset restores the default.
 bool prefer_stream(int k);
 void set_prefer_stream(int k, bool v);
 void reset_prefer_stream(int k);
@@ -106,7 +106,8 @@ bool score_and_traceback_layout(HostPlan &hp);
 // everything of make_plan that needs no heap memory. Returns MSA_OK or an MSA_E*
 // code with `err` set; edge < 0 takes the current tuned edge for k.
 // allow_stream = false keeps the automatic choice off the streamed line kernel
-// (serving, whose arena regions are reused without clearing faces).
+// (serving at k >= 6, and at k = 4, 5 where its arena cannot hold the faces; the
+// no-allocation call).
 int plan_shape(int k, const int32_t *lens, int A, int kernel_choice, HostPlan &hp, std::string &err, int edge = -1,
                bool allow_stream = true);
 

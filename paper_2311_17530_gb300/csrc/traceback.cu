@@ -15,15 +15,18 @@
 //   * row-major layout, k = 2: a strip along the diagonal staged by the CTA (walk_pair);
 //   * row-major layout, k = 3: boxes [x - D, x] staged by the CTA (rows of the last axis
 //     copied in 16-byte granules);
-//   * k >= 4 (row-major or tile-major; short paths, large boxes): no staging; warp 0
+//   * k >= 4, tile-major: the blocks of the tiles around the current one staged by the
+//     CTA (walk_tiles), or windows of the line tiles that span the last axis (walk_lines);
+//   * k = 7, 8 whole-column tiles: no staging, one load per move (walk_chain);
+//   * k >= 4 otherwise (row-major, or tiles too large to stage): no staging; warp 0
 //     loads the traceback bytes of the current cell and of all its predecessors
 //     in one round trip, which fixes two moves.
 // The walk records only the masks (last column first). The score is computed
 // afterwards by the whole CTA: each thread takes a contiguous run of columns,
 // the per-axis move counts are prefix-summed to give each column's position, and
 // the column scores u*|m| + sum over moved pairs of (sub - 2 gap) are added up.
-// For the generic tile kernel the sum is cross-checked against the corner's
-// packed key.
+// The sum is cross-checked against the corner's packed key where the fill recorded it
+// (the column kernel: on request).
 #include "api_internal.h"
 #include "device_common.cuh"
 
