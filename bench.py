@@ -570,7 +570,8 @@ def measure_extensions(reps: int = 3):
             "tiles": st["tiles"], "tiles_skipped": st["tiles_skipped"], "cells_skipped": st["cells_skipped"],
             "cells": st["cells"], "fraction_skipped": st["cells_skipped"] / max(1, st["cells"]),
             "note": "host-buffer call: pairwise tables, bound, greedy feasible alignment, fill (the fastest for the shape), "
-                    "traceback, with per-call allocation and copies"}
+                    "traceback, with per-call allocation and copies; skipped: what the bound rules out, which the fills of "
+                    "these two shapes (column and streamed kernel) fill all the same"}
     q = inputs.random_problem(17, 3, [120, 110, 130], alphabet=inputs.PROTEIN, related=True)
     for delta in (0, 3):
         msadp.msa_near_optimal(q.seqs, q.alphabet, q.subst, q.gap, delta, 256)
